@@ -30,7 +30,7 @@
  *   - State layout: four float32 planes x | x_dot | theta | theta_dot; element i of
  *     plane p is planes[p * plane_stride + i]. Vector (16-byte) access is used when
  *     planes is 16-byte aligned and plane_stride is a multiple of 4; any other
- *     layout takes a scalar path with identical results.
+ *     layout takes a path of 4-byte accesses with identical results.
  *   - Environment i of a batch has global id env_offset + i; all hashing uses the
  *     global id, so results do not depend on how environments are sharded.
  *
@@ -345,7 +345,7 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * "rollout_ctas_per_sm" (0 = default: one 32*ept-environment task per warp and as many
  * CTAs as that takes; k > 0 = persistent grid of k CTAs per SM looping over tasks), "step_block"
  * (32..256, default 64), "step_vec_min_envs" (batches smaller than this use the one-env-per-thread
- * step kernel even when the four-envs-per-thread vector form is possible; default 262144),
+ * step kernel instead of the four-envs-per-thread forms; default 262144),
  * "step_pdl" (1 = default: the step kernels and the ladder's one-op kernels are launched with
  * programmatic stream serialization, so that a launch is set up — and, in the fused step, the
  * actions hashed — while the launch before it still runs; 0 = plain launches).

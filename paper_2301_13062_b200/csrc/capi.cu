@@ -373,10 +373,12 @@ static int step_impl(cp_state *state, const uint8_t *action, cp_state *out_state
     fill_step_params(p, state, out_state, action, reward, done);
     p.ep_len = ep_len;
     p.max_steps = max_steps;
-    const bool vec = state->n >= cp::g_tuning.step_vec_min_envs && state_vec_ok(state) && state_vec_ok(out_state) &&
-                     (!reward || is_aligned(reward, 16)) && (!done || is_aligned(done, 4)) &&
-                     (!action || is_aligned(action, 4)) && (!ep_len || is_aligned(ep_len, 16));
-    cudaError_t e = cp::launch_step(p, vec, tl_stream);
+    const bool vec_ok = state_vec_ok(state) && state_vec_ok(out_state) &&
+                        (!reward || is_aligned(reward, 16)) && (!done || is_aligned(done, 4)) &&
+                        (!action || is_aligned(action, 4)) && (!ep_len || is_aligned(ep_len, 16));
+    const bool large = state->n >= cp::g_tuning.step_vec_min_envs;
+    cudaError_t e = large && !vec_ok ? cp::launch_step_strided(p, tl_stream)
+                                     : cp::launch_step(p, large && vec_ok, tl_stream);
     if (e != cudaSuccess) return cuda_fail(e, "step launch");
     advance(state, out_state, 1);
     return CP_OK;
