@@ -86,7 +86,7 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
 cudaError_t launch_rollout_contracted(RolloutParams &p, int policy, bool streams, cudaStream_t s);
 // the producer-assisted kernel for very small batches, and whether a call is one it covers
 bool rollout_assisted_applies(const RolloutParams &p, int policy, bool streams);
-cudaError_t launch_rollout_assisted(RolloutParams &p, bool contracted, cudaStream_t s);
+cudaError_t launch_rollout_assisted(RolloutParams &p, int policy, bool contracted, cudaStream_t s);
 // the deferred-restart kernel (large batches, no per-step streams), and whether a call is one it covers
 bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams);
 cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracted, cudaStream_t s);

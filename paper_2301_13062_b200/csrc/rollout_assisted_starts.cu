@@ -1,0 +1,12 @@
+// The producer-assisted kernel (rollout_assisted.cuh) for supplied start states.
+#include "rollout_assisted.cuh"
+
+namespace cp {
+
+void launch_assisted_starts(const RolloutParams &p, int policy, bool contracted, cudaStream_t s) {
+    if (policy == 0) launch_assisted_pairs<0, true>(p, true, contracted, s);
+    else if (policy == 1) launch_assisted_pairs<1, true>(p, true, contracted, s);
+    else launch_assisted_pairs<6, true>(p, true, contracted, s);
+}
+
+}  // namespace cp

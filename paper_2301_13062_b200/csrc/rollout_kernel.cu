@@ -20,8 +20,8 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
                             (policy == 0 || policy == 1 || policy == 6 || network);
     if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams))
         return launch_rollout_deferred(p, policy, contracted, s);
-    // very small batches with hashed actions: a helper warp per stepping warp (rollout_assisted.cu)
-    if (rollout_assisted_applies(p, policy, streams)) return launch_rollout_assisted(p, contracted, s);
+    // very small batches, unless a network acts: a helper warp per stepping warp (rollout_assisted.cu)
+    if (rollout_assisted_applies(p, policy, streams)) return launch_rollout_assisted(p, policy, contracted, s);
     if (contracted) return launch_rollout_contracted(p, policy, streams, s);
     return launch_rollout_arith<false>(p, policy, streams, s);
 }

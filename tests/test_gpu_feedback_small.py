@@ -1,0 +1,95 @@
+"""Small batches under feedback policies or from supplied start states: the producer-assisted kernel
+(linear policies, supplied starts) must give the bits of the general kernel's per-lane shape, which
+the other files pin to the oracle. Sizes: around the 32 environments of a bit-plane word, odd warp
+tasks. Horizons: around the hand-overs of 16 and 32 steps."""
+import numpy as np
+import pytest
+
+from tests import gpu_helpers as H
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+LINEAR, MLP, PER_ENV = 1, 2, 6
+ALL = ("reward_stream", "done_bits", "action_bits", "trajectory")
+
+
+@pytest.fixture(scope="module")
+def cp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_13062_b200 import binding, build
+    build.build()
+    binding.lib()
+    torch.cuda.set_device(0)
+    return binding
+
+
+def policy_of(cp, kind, n, seed=3):
+    from paper_2301_13062_b200 import inputs
+    if kind == PER_ENV:
+        return cp.policy(kind, torch.from_numpy(inputs.per_env_linear_weights(n, seed)).cuda())
+    return cp.policy(kind, inputs.policy_weights(kind, seed))
+
+
+def rollout(cp, coop, kind, n, T, streams=(), limit=0, contracted=False, starts=None, given=None, spread=None):
+    from paper_2301_13062_b200 import inputs
+    words = (n + 31) // 32
+    shapes = {"done_bits": ((T, words), torch.int32), "action_bits": ((T, words), torch.int32),
+              "reward_stream": ((T, n), torch.float32), "trajectory": ((T, 4, n), torch.float32)}
+    out = {"ep_return_sum": torch.full((n,), -1.0, device="cuda"),
+           "ep_count": torch.full((n,), -1, dtype=torch.int32, device="cuda"),
+           "totals": torch.zeros(2, dtype=torch.int64, device="cuda")}
+    for name in streams:
+        out[name] = torch.full(shapes[name][0], 7, dtype=shapes[name][1], device="cuda")
+    kw = {"policy": policy_of(cp, kind, n) if kind else None, "max_episode_steps": limit, "action_bits_in": given,
+          "arithmetic": cp.CP_ARITH_CONTRACTED if contracted else cp.CP_ARITH_EXACT, "start_states_in": starts}
+    with H.rollout_shape(cp, 1 if coop else 0, coop):
+        if spread:  # a batch in the middle of its episodes
+            planes = torch.from_numpy(inputs.random_states(n, 5, spread)).cuda()
+            ep_len = torch.arange(n, dtype=torch.int32, device="cuda") % 37
+            cp.cp_rollout_ex(T=T, state=cp.cp_wrap(planes, n, 9, t=11, env_offset=6), ep_len=ep_len, **kw, **out)
+            out["planes"], out["ep_len"] = planes, ep_len
+        else:
+            out["final_state"] = torch.zeros(4, n, device="cuda")
+            cp.cp_rollout_ex(n_envs=n, T=T, seed=9, t0=11, env_offset=6, **kw, **out)
+    torch.cuda.synchronize()
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+def assert_same_bits(a, b):
+    for k in a:
+        assert np.array_equal(a[k].view(np.uint32) if a[k].dtype == np.float32 else a[k],
+                              b[k].view(np.uint32) if b[k].dtype == np.float32 else b[k]), k
+
+
+def start_rows(T, n):
+    rng = np.random.default_rng(17)
+    s = rng.uniform(-0.3, 0.3, (T, 4, n)).astype(np.float32)  # angles on both sides of the polynomial range
+    s[:, 2, ::7] = rng.uniform(-3, 3, s[:, 2, ::7].shape)
+    s[T // 2, 0, ::5] = np.inf
+    s[T // 3, 3, ::5] = np.nan
+    return torch.from_numpy(s).cuda()
+
+
+@pytest.mark.parametrize("kind", [LINEAR, PER_ENV])
+@pytest.mark.parametrize("n,T", [(1, 15), (33, 32), (2049, 33), (4737, 16), (4801, 65)])
+@pytest.mark.parametrize("contracted", [False, True])
+def test_linear_policies(cp, kind, n, T, contracted):
+    for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("reward_stream", "done_bits"), 0, "edge"),
+                                   (("action_bits", "trajectory"), 9, None)):
+        args = dict(streams=streams, limit=limit, spread=spread, contracted=contracted)
+        assert_same_bits(rollout(cp, 4, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
+        assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
+
+
+@pytest.mark.parametrize("kind", [0, LINEAR, PER_ENV, MLP])
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("n,T", [(1, 17), (33, 1), (1000, 16), (4801, 47)])
+def test_supplied_starts(cp, kind, given, n, T):
+    bits = torch.from_numpy(np.random.default_rng(2).integers(-2**31, 2**31, (T, (n + 31) // 32)).astype(np.int32)).cuda()
+    for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("reward_stream", "done_bits"), 0, None),
+                                   (("done_bits",), 0, "edge")):
+        args = dict(streams=streams, limit=limit, spread=spread, starts=start_rows(T, n), given=bits if given else None)
+        assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
