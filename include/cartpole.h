@@ -332,7 +332,8 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * actions only, otherwise as 2), 4 = a helper warp per stepping warp hashes every step's action
  * and start state ahead into shared memory, or fetches the supplied ones (hashed or supplied
  * actions and the linear policies; otherwise as 2), 2, 3 and 4 only with one environment per
- * thread; 0 = default: helper warps for up to ten warps of environments per SM, per lane for
+ * thread; 0 = default: helper warps for up to ten warps of environments per SM, the hidden units
+ * of a network spread over several lanes for up to two warps per scheduler, per lane for
  * other batches too small to fill the GPU (ahead for the smaller ones), deferred (5) from one
  * 64-environment warp per scheduler on (37,888 environments on 148 SMs) where that form applies,
  * by the warp otherwise;

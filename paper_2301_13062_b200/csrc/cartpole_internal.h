@@ -91,6 +91,9 @@ cudaError_t launch_rollout_assisted(RolloutParams &p, int policy, bool contracte
 bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams);
 cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracted, cudaStream_t s);
 cudaError_t launch_rollout_deferred_wide(RolloutParams &p, int policy, bool contracted, cudaStream_t s);  // policies 4, 5, 7
+// the lane-split kernel of the network policies: lanes per environment it would use for a call, 0 = not its call
+int rollout_lanes_for(const RolloutParams &p, int policy, bool streams);
+cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s);
 // the MLP policies (kinds 2, 4, 5, 7), canonical and contracted arithmetic; mode and shape as
 // chosen by launch_rollout_arith
 cudaError_t launch_rollout_networks(RolloutParams &p, int policy, int mode, int shape, cudaStream_t s);

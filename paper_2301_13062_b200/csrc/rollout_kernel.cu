@@ -13,6 +13,9 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // 131,072 0.163 / 0.251; linear policy 47,360 0.088 / 0.100, 131,072 0.154 / 0.212; network
     // 56,832 0.483 / 0.427, 75,776 0.483 / 0.545. rollout_coop = 5 forces it wherever it
     // applies, any other forced shape keeps the other kernels.
+    // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
+    // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
+    if (const int lanes = rollout_lanes_for(p, policy, streams)) return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
     const int64_t warps64 = (p.n + 63) / 64;
     const bool network = policy == 2 || policy == 4 || policy == 5 || policy == 7;
     const bool enough = network ? warps64 >= (int64_t)sm_count() * 7 : warps64 >= (int64_t)sm_count() * 4;

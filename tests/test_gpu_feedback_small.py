@@ -1,7 +1,9 @@
 """Small batches under feedback policies or from supplied start states: the producer-assisted kernel
-(linear policies, supplied starts) must give the bits of the general kernel's per-lane shape, which
-the other files pin to the oracle. Sizes: around the 32 environments of a bit-plane word, odd warp
-tasks. Horizons: around the hand-overs of 16 and 32 steps."""
+(linear policies, supplied starts) and the network kernel that spreads hidden units over lanes. Both
+must give the bits of the general kernel's per-lane shape, which the other files pin to the oracle.
+Sizes: around the 32 environments of a bit-plane word, odd warp tasks, and either side of the bounds
+at which the network kernel takes more lanes or leaves the call (148 SMs: 1,184, 2,368, 4,736 and
+9,472 environments). Horizons: around the 32-step hand-overs of both kernels."""
 import numpy as np
 import pytest
 
@@ -11,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-LINEAR, MLP, PER_ENV = 1, 2, 6
+LINEAR, MLP, MLP32, MLP64, PER_ENV, DEEP = 1, 2, 4, 5, 6, 7
 ALL = ("reward_stream", "done_bits", "action_bits", "trajectory")
 
 
@@ -71,6 +73,25 @@ def start_rows(T, n):
     s[T // 2, 0, ::5] = np.inf
     s[T // 3, 3, ::5] = np.nan
     return torch.from_numpy(s).cuda()
+
+
+@pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
+@pytest.mark.parametrize("n,T", [(1, 33), (31, 64), (33, 5), (1184, 40), (1185, 31), (2369, 32), (4737, 31),
+                                 (9465, 65), (9472, 33), (9473, 33)])
+def test_networks(cp, kind, n, T):
+    for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("done_bits",), 0, "edge"), (("trajectory",), 9, None)):
+        args = dict(streams=streams, limit=limit, spread=spread)
+        assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
+
+
+@pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
+@pytest.mark.parametrize("n", [97, 1500, 4097])
+def test_networks_contracted_and_supplied_starts(cp, kind, n):
+    for streams in ((), ALL):
+        args = dict(streams=streams, limit=15, contracted=True)
+        assert_same_bits(rollout(cp, 0, kind, n, 50, **args), rollout(cp, 2, kind, n, 50, **args))
+        args = dict(streams=streams, starts=start_rows(50, n), spread="edge")
+        assert_same_bits(rollout(cp, 0, kind, n, 50, **args), rollout(cp, 2, kind, n, 50, **args))
 
 
 @pytest.mark.parametrize("kind", [LINEAR, PER_ENV])
