@@ -23,6 +23,8 @@ def cp():
 
 def step(cp, min_envs, n, pad, given, limit, in_place, wanted, offset):
     from paper_2301_13062_b200 import inputs
+    if (n + pad) % 4 == 0:
+        offset = 1                                                  # or the float4 form would take the call
     z = np.concatenate([inputs.random_states(n - n // 3, 4, "wide"), inputs.random_states(n // 3, 5, "edge")], 1) if n > 3 \
         else inputs.random_states(n, 4, "edge")
     store = torch.zeros(4 * (n + pad) + 1, device="cuda")          # planes from the first float on, or from the second
