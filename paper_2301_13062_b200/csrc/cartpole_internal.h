@@ -90,6 +90,8 @@ cudaError_t launch_rollout_assisted(RolloutParams &p, int policy, bool contracte
 // the deferred-restart kernel (large batches, no per-step streams), and whether a call is one it covers
 bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams);
 cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracted, cudaStream_t s);
+// policies 0, 1, 3 (supplied actions), 6 where actions or start states are the caller's data
+cudaError_t launch_rollout_deferred_data(RolloutParams &p, int policy, int k, bool contracted, cudaStream_t s);
 cudaError_t launch_rollout_deferred_wide(RolloutParams &p, int policy, bool contracted, cudaStream_t s);  // policies 4, 5, 7
 // the lane-split kernel of the network policies: lanes per environment it would use for a call, 0 = not its call
 int rollout_lanes_for(const RolloutParams &p, int policy, bool streams);

@@ -9,7 +9,9 @@ namespace cp {
 bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams) {
     // per-step outputs: none, or exactly the reward plane + done bitmask
     const bool outputs_ok = !streams || (p.reward_stream && p.done_bits && !p.action_bits && !p.trajectory);
-    if (!outputs_ok || p.action_bits_in || p.start_in) return false;
+    if (!outputs_ok) return false;
+    if (p.action_bits_in) return true;  // supplied actions replace whatever policy was named
+    if (p.start_in) return policy == 0 || policy == 1 || policy == 6;
     if (is_wide_network(policy)) return !streams && !p.max_steps;
     return policy == 0 || policy == 1 || policy == 2 || policy == 6;
 }
@@ -24,12 +26,14 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
     // the passes come closer together (us per step of 1,048,576 envs at K = 2 / 4 / 6, hashed
     // actions: T = 16: 3.39 / 3.65 / 4.03, T = 64: 2.41 / 2.38 / 2.45, T = 256: 2.17 / 2.02 / 2.00;
     // below 12 steps the general kernel is as fast or faster and keeps the call).
-    // The shared linear policy's 80-step episodes leave a pass little to do, so long launches
-    // space them further (with the reward plane and done bits, K = 4 / 6 / 8: 1,048,576 x 500
-    // 1.076 / 1.041 / 1.027 ms, 4,194,304 x 1,000 8.45 / 8.12 / 7.97 ms; without them 4,194,304 x
-    // 1,000 7.05 / 7.01 ms at K = 6 / 8; at 200 steps K = 6 is ahead, and so it is at every length
-    // with hashed actions: 4,194,304 x 1,000 with streams 9.11 / 8.57 / 8.90 ms).
-    const int by_length = p.T < 48u ? 2 : p.T < 192u ? 4 : (policy == 1 && p.T >= 384u) ? 8 : 6;
+    // 8 trips between passes, which the shared linear policy once had from 384 steps on, suit a policy
+    // whose episodes last 80 steps (1,048,576 x 400, with the reward plane and done bits, K = 6 / 8:
+    // 835 / 833 us) and cost most policies drawn at random, which push one way and fall after 9 or 10
+    // steps (1,009 / 1,359 us, without outputs 902 / 1,154). 5 and 10 trips fit such episodes
+    // better (981, 935) and others worse (31-step mixtures 949 at 6; 1,080, 1,199). Choosing in the
+    // kernel, by counting the waiting slots every second trip or after every pass, cost 6 to 14 % of
+    // every launch.
+    const int by_length = p.T < 48u ? 2 : p.T < 192u ? 4 : 6;
     const int k = g_tuning.rollout_defer > 0 ? g_tuning.rollout_defer : (is_network(policy) ? 3 : by_length);
     // the action hash folds the time's upper half into the lower one: nothing to do below 2^16
     const bool short_times = (uint64_t)p.t0 + p.T <= 65536u;
@@ -38,6 +42,7 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
         static_assert(sizeof(p.w) >= 2 * 450 * sizeof(float), "the launch parameters hold the largest policy twice");
         for (int i = count - 1; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
     }
+    if (p.action_bits_in || p.start_in) return launch_rollout_deferred_data(p, p.action_bits_in ? 3 : policy, k, contracted, s);
     switch (policy) {
         case 0: return short_times ? launch_limit<0, true>(p, k, contracted, s) : launch_limit<0, false>(p, k, contracted, s);
         case 1: return launch_limit<1, false>(p, k, contracted, s);

@@ -23,8 +23,8 @@
 // the price is idle slots (about 7 % at K = 4 with the random policy's 22-step episodes) and a
 // ragged end.
 //
-// Scope: hashed actions, the shared linear policy, the shared 4-16-2 tanh network or one linear
-// policy per environment; either arithmetic; with or without the episode step limit; per-step
+// Scope: hashed or supplied actions, the shared linear policy, the shared 4-16-2 tanh network or one
+// linear policy per environment; hashed start states, or (but for the network) supplied ones; either arithmetic; with or without the episode step limit; per-step
 // outputs either none or exactly the reward plane + done bitmask (the action bitmask and the
 // trajectory are rows of global time that half the lanes would have to touch every step). The
 // wider and deeper networks (4-32-2, 4-64-2, 4-16-16-2) too, for the plain call: no step limit,
@@ -135,12 +135,17 @@ constexpr uint32_t kClearApartFrom = 192u;
 // fold16(t) == t.
 template <int POLICY, bool SHORT, bool CONTRACT>
 __device__ __forceinline__ void deferred_actions(const RolloutParams &p, const FoldedKeys (&ka)[2],
-                                                 const LinearW *own, const uint32_t (&t)[2], const StatePair &zz,
-                                                 uint32_t &sb0, uint32_t &sb1) {
+                                                 const LinearW *own, const uint32_t (&t)[2], const bool (&act)[2],
+                                                 uint32_t (&window)[2], const StatePair &zz, uint32_t &sb0, uint32_t &sb1) {
     const f32x2 *pairs = reinterpret_cast<const f32x2 *>(p.w);
     if (POLICY == 0) {
         sb0 = action_signbit_folded(ka[0], SHORT ? t[0] : fold16(t[0]));
         sb1 = action_signbit_folded(ka[1], SHORT ? t[1] : fold16(t[1]));
+    } else if (POLICY == 3) {  // the next action is the window's top bit (load_windows)
+        sb0 = window[0] & 0x80000000u;
+        sb1 = window[1] & 0x80000000u;
+        if (act[0]) window[0] <<= 1;  // a waiting slot's clock stands still, and so does its window
+        if (act[1]) window[1] <<= 1;
     } else if (POLICY == 1) {
         linear_action_pair(pairs, zz, sb0, sb1);
     } else if (POLICY == 2) {
@@ -159,10 +164,36 @@ __device__ __forceinline__ void deferred_actions(const RolloutParams &p, const F
     }
 }
 
+// 32x32 bit transpose over a warp: in, lane l holds row l; out, bit r of lane l is bit l of row r.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
+    uint32_t m = 0x0000ffffu;
+#pragma unroll
+    for (uint32_t j = 16u; j != 0u; j >>= 1, m ^= m << j) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+        x = (lane & j) ? (x & ~m) | ((y >> j) & m) : (x & m) | ((y & m) << j);
+    }
+    return x;
+}
+
+// Supplied actions in this kernel: the caller's rows hold one step of 32 environments per word, and the
+// environments of a warp stand at different steps, so reading rows lane by lane would be a gather in
+// every trip. Instead a warp reads 32 rows at a time, one per lane, transposes the 32x32 bits, and
+// keeps the last kRing such blocks in shared memory: one word per environment with its next 32
+// actions. Every 32 trips or so a lane takes 32 actions from its clock on out of two such words.
+// An environment more than kRing - 1 blocks behind the warp's first one (never seen with
+// actions drawn at random) collects its bits from the caller's rows itself.
+// What bounds it: the float32 pipe, as with hashed actions (1,048,576 x 250: 490 us, hashed 475; the
+// general kernel, which reads a word per warp and step, 617), and with supplied start states the
+// gather of 16 bytes per episode from rows that no two environments of a warp share at a time:
+// latency, so these instances ask for three CTAs per SM (200,003 x 250, supplied actions and
+// start states, at 1 / 2 / 3: 236 / 171 / 140 us; the general kernel 290).
+constexpr int kRing = 8;
+
 // POLICY: 0 hashed actions, 1 shared linear policy, 2 / 4 / 5 / 7 a shared tanh network (is_network),
 // 6 one linear policy per environment.
 // K: trips between restart passes. LIMIT: episodes are cut off after p.max_steps steps.
 // RD: the reward plane and the done bitmask are written (see the comment at reward_row).
+// START_IN: finished environments continue from the caller's start states, which may hold any angle.
 // CONTRACT: the contracted arithmetic (euler_step_contracted_pair, tanh_contracted_pair).
 // One CTA per SM is all the launch bounds ask for, which lets the assembler take the registers it
 // wants (77-96 instead of the 58-64 it settles for when left to aim at occupancy): the kernel is
@@ -173,8 +204,10 @@ __device__ __forceinline__ void deferred_actions(const RolloutParams &p, const F
 // (The network policies are the exception: their hidden units are latency — exp2 and
 // reciprocal on the special-function pipe — that only more resident warps hide: 16,777,216 x
 // 200 takes 53.1 / 41.1 / 39.9 / 39.4 / 40.8 ms at 1 / 2 / 3 / 4 / 5 CTAs per SM.)
-template <int POLICY, int K, bool SHORT, bool LIMIT, bool RD, bool CONTRACT>
-__global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : 1) rollout_deferred_kernel(const __grid_constant__ RolloutParams p) {
+template <int POLICY, int K, bool SHORT, bool LIMIT, bool RD, bool CONTRACT, bool START_IN = false>
+__global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || START_IN ? 3 : 1) rollout_deferred_kernel(const __grid_constant__ RolloutParams p) {
+    constexpr bool GIVEN = POLICY == 3;
+    __shared__ uint32_t s_ring[GIVEN ? 8 : 1][GIVEN ? kRing : 1][2][32];
     const uint32_t lane = threadIdx.x & 31u;
     const int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     unsigned long long tot_ret = 0, tot_cnt = 0;
@@ -183,6 +216,7 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : 1) rollout_defer
         const uint32_t t_end = p.t0 + p.T;
         FoldedKeys ka[2], kr[2];
         LinearW own[POLICY == 6 ? 2 : 1];
+        uint32_t window[2] = {};  // GIVEN: the actions from t[j] on, first one on top
         uint32_t t[2], cnt[2], begin[2];
         bool act[2];
         State z0[2];
@@ -249,6 +283,61 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : 1) rollout_defer
                 atomicOr(p.done_bits + (int64_t)(t_done - p.t0) * words + word0 + j, 1u << lane);
         };
 
+        // Row `row` of the caller's start states ([T][4][n]) for slot j's environment.
+        auto supplied_start = [&](int j, uint32_t row) {
+            int64_t idx = base + j * 32 + lane;
+            if (idx >= p.n) idx = p.n - 1;
+            const float *src = p.start_in + (int64_t)row * 4 * p.n + idx;
+            State f;
+            f.x = __ldg(src);
+            f.xd = __ldg(src + p.n);
+            f.th = __ldg(src + 2 * p.n);
+            f.thd = __ldg(src + 3 * p.n);
+            return f;
+        };
+
+        // GIVEN: blocks [0, hi) of 32 steps have been put into the ring (the last kRing are there);
+        // raw holds this lane's row of block hi, requested a whole block ahead of its use.
+        uint32_t hi = 0u, raw[2] = {};
+        const uint32_t blocks = (p.T + 31u) >> 5;
+        auto (*const ring)[2][32] = s_ring[GIVEN ? threadIdx.x >> 5 : 0];
+        auto request_block = [&](uint32_t b) {  // reversed: the block's first step becomes bit 31
+            const uint32_t row = b * 32u + 31u - lane;
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                raw[j] = row < p.T && word0 + j < words ? __ldg(p.action_bits_in + (int64_t)row * words + word0 + j) : 0u;
+        };
+        auto load_windows = [&]() {
+            const uint32_t r0 = t[0] - p.t0, r1 = t[1] - p.t0;
+            // the block of the slot that is furthest ahead, retired ones aside
+            const uint32_t first = __reduce_max_sync(0xffffffffu, max(r0 < p.T ? r0 : 0u, r1 < p.T ? r1 : 0u)) >> 5;
+            while (hi < blocks && hi < first + 2u) {  // warp-uniform
+                ring[hi % kRing][0][lane] = transpose32(raw[0], lane);
+                ring[hi % kRing][1][lane] = transpose32(raw[1], lane);
+                ++hi;
+                request_block(hi);
+            }
+            // every lane reads its own column only: no barrier
+            bool behind = false;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const uint32_t r = j ? r1 : r0, b = r >> 5;
+                window[j] = __funnelshift_l(ring[(b + 1u) % kRing][j][lane], ring[b % kRing][j][lane], r & 31u);
+                behind = behind || b + kRing < hi;
+            }
+            if (__any_sync(0xffffffffu, behind)) {
+#pragma unroll 1
+                for (int j = 0; j < 2; ++j) {
+                    const uint32_t r = j ? r1 : r0;
+                    if ((r >> 5) + kRing >= hi || word0 + j >= words) continue;
+                    uint32_t w = 0u;
+                    for (uint32_t i = 0; i < 32u && r + i < p.T; ++i)
+                        w |= ((__ldg(p.action_bits_in + (int64_t)(r + i) * words + word0 + j) >> lane) & 1u) << (31u - i);
+                    window[j] = w;
+                }
+            }
+        };
+
         uint32_t trips = 0;  // trips made; no slot's clock is more than one step ahead of t0 + trips
 
         // Slot j has done its last step (its clock reached t_end) and retires. cnt / begin are
@@ -267,7 +356,7 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : 1) rollout_defer
                 State a, b;
                 unpack_states(zz, a, b);
                 State mine = j ? b : a;
-                if (done_now) mine = start_state_folded(kr[j], fold16(4u * t_end));
+                if (done_now) mine = START_IN ? supplied_start(j, p.T - 1u) : start_state_folded(kr[j], fold16(4u * t_end));
                 const int64_t idx = base + j * 32 + lane;
                 if (idx < p.n) {
                     p.out_planes[idx] = mine.x;
@@ -319,6 +408,8 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : 1) rollout_defer
         // linear policies' 80-step episodes the test only costs: 4,194,304 x 100 with streams
         // 0.828 -> 0.878 ms.)
         constexpr bool FORESIGHT = is_network(POLICY);
+        int passes = 0;     // GIVEN: since the windows were loaded
+        bool wide = false;  // START_IN, warp-uniform: a slot stands at a start state beyond the polynomial range
         auto restart_pass = [&](auto tail) {
             constexpr bool TAIL = decltype(tail)::value;
             if (FORESIGHT) {
@@ -338,69 +429,106 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : 1) rollout_defer
                     }
                 }
             }
+            if (START_IN) {
+                State f[2];  // both slots' loads are in flight before either is used
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                if (!act[j] && (!TAIL || t[j] != t_end)) {
-                    cnt[j] += 1u;
-                    begin[j] = t[j];
-                    set_done_bit(j, t[j] - 1u);
-                    State a, b;
-                    unpack_states(zz, a, b);
-                    (j ? b : a) = start_state_folded(kr[j], fold16(4u * t[j]));
-                    zz = pack_states(a, b);
-                    act[j] = true;
+                for (int j = 0; j < 2; ++j)
+                    if (!act[j] && (!TAIL || t[j] != t_end)) f[j] = supplied_start(j, t[j] - 1u - p.t0);
+                State a, b;
+                unpack_states(zz, a, b);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (!act[j] && (!TAIL || t[j] != t_end)) {
+                        cnt[j] += 1u;
+                        begin[j] = t[j];
+                        set_done_bit(j, t[j] - 1u);
+                        (j ? b : a) = f[j];
+                        act[j] = true;
+                    }
                 }
+                zz = pack_states(a, b);
+                wide = __any_sync(0xffffffffu, (act[0] && !(fabsf(a.th) <= kSmallAngle)) || (act[1] && !(fabsf(b.th) <= kSmallAngle)));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (!act[j] && (!TAIL || t[j] != t_end)) {
+                        cnt[j] += 1u;
+                        begin[j] = t[j];
+                        set_done_bit(j, t[j] - 1u);
+                        State a, b;
+                        unpack_states(zz, a, b);
+                        (j ? b : a) = start_state_folded(kr[j], fold16(4u * t[j]));
+                        zz = pack_states(a, b);
+                        act[j] = true;
+                    }
+                }
+            }
+            if (GIVEN && ++passes == 32 / K) {  // no slot has used more than the 32 actions of its window
+                load_windows();
+                passes = 0;
             }
         };
 
         uint32_t row = 0;  // trips made so far = the row of the reward plane the next trip writes
-        auto trip = [&](auto tail) {
+        // general: states that may hold any angle, stepped by the general scalar step
+        auto trip = [&](auto tail, auto general) {
             if (RD) reward_row(tail, row++);
             uint32_t sb0, sb1;
-            deferred_actions<POLICY, SHORT, CONTRACT>(p, ka, own, t, zz, sb0, sb1);
+            deferred_actions<POLICY, SHORT, CONTRACT>(p, ka, own, t, act, window, zz, sb0, sb1);
             bool d0, d1;
-            const f32x2 force = pack2(force_from_signbit(sb0), force_from_signbit(sb1));
-            if (CONTRACT) euler_step_contracted_pair(zz, force, d0, d1);
-            else euler_step_pair(zz, force, d0, d1);
+            if (decltype(general)::value) {
+                State a, b;
+                unpack_states(zz, a, b);
+                d0 = CONTRACT ? euler_step_contracted<false>(a, force_from_signbit(sb0)) : euler_step<false>(a, force_from_signbit(sb0));
+                d1 = CONTRACT ? euler_step_contracted<false>(b, force_from_signbit(sb1)) : euler_step<false>(b, force_from_signbit(sb1));
+                zz = pack_states(a, b);
+            } else {
+                const f32x2 force = pack2(force_from_signbit(sb0), force_from_signbit(sb1));
+                if (CONTRACT) euler_step_contracted_pair(zz, force, d0, d1);
+                else euler_step_pair(zz, force, d0, d1);
+            }
             after_step(tail, 0, d0);
             after_step(tail, 1, d1);
         };
+        // The K trips between two restart passes (a network policy's trip is 600 instructions or more:
+        // its trips stay a loop).
+        constexpr int kUnroll = is_network(POLICY) ? 1 : K;
+        auto trip_block = [&](auto tail) {
+            if (START_IN && wide) {  // only the first trip after a pass can meet such an angle
+                trip(tail, std::true_type{});
+                wide = false;
+#pragma unroll 1
+                for (int k = 1; k < K; ++k) trip(tail, std::false_type{});
+            } else {
+#pragma unroll kUnroll
+                for (int k = 0; k < K; ++k) trip(tail, std::false_type{});
+            }
+        };
 
+        if (GIVEN) {
+            request_block(0u);
+            load_windows();
+        }
         if (p.init_planes) {
             // A caller's states may hold any angle: the first trip uses the general scalar step.
             // From then on every stepping slot is a survivor (|theta| <= 0.2095) or a fresh
             // start state (|theta| <= 0.05), which is the packed step's domain.
-            if (RD) reward_row(std::false_type{}, row++);
-            uint32_t sb0, sb1;
-            deferred_actions<POLICY, SHORT, CONTRACT>(p, ka, own, t, zz, sb0, sb1);
-            State a, b;
-            unpack_states(zz, a, b);
-            const bool d0 = CONTRACT ? euler_step_contracted<false>(a, force_from_signbit(sb0))
-                                     : euler_step<false>(a, force_from_signbit(sb0));
-            const bool d1 = CONTRACT ? euler_step_contracted<false>(b, force_from_signbit(sb1))
-                                     : euler_step<false>(b, force_from_signbit(sb1));
-            zz = pack_states(a, b);
-            after_step(std::true_type{}, 0, d0);
-            after_step(std::true_type{}, 1, d1);
+            trip(std::true_type{}, std::true_type{});
             trips = 1;
             restart_pass(std::true_type{});
         }
         // Main part: after these trips no clock can have reached t_end yet (clocks run at most one
         // step ahead of the trips), so no slot can retire.
-        // (a network policy's trip is 600 instructions or more: its K trips stay a loop)
-        constexpr int kUnroll = is_network(POLICY) ? 1 : K;
         while (trips + K + (FORESIGHT ? 1u : 0u) <= p.T - 1u) {
-#pragma unroll kUnroll
-            for (int k = 0; k < K; ++k) trip(std::false_type{});
+            trip_block(std::false_type{});
             trips += K;
             restart_pass(std::false_type{});
         }
-        // Tail: slots retire as their clocks reach t_end. Every block of K trips advances every
+        // Tail: slots retire as their clocks reach t_end. Every block of trips advances every
         // unretired slot by at least one step, so p.T blocks always suffice.
         for (uint32_t block = 0; block <= p.T; ++block) {
             if (__all_sync(0xffffffffu, t[0] == t_end && t[1] == t_end)) break;
-#pragma unroll kUnroll
-            for (int k = 0; k < K; ++k) trip(std::true_type{});
+            trip_block(std::true_type{});
             if (FORESIGHT) trips += K;
             restart_pass(std::true_type{});
         }
@@ -445,30 +573,37 @@ __global__ void __launch_bounds__(256) clear_words_kernel(uint32_t *w, int64_t n
     }
 }
 
-template <int POLICY, bool SHORT, bool LIMIT, bool RD>
-cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
+// The grid of a launch (0: too many environments), and the cleared done plane where it is cleared apart.
+inline unsigned deferred_grid(RolloutParams &p, cudaStream_t s) {
     p.n_tasks = (p.n + 63) / 64;
-    int64_t grid = (p.n_tasks + 7) / 8;
-    if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    if (RD && p.T >= kClearApartFrom) {
+    const int64_t grid = (p.n_tasks + 7) / 8;
+    if (grid > 0x7fffffffLL) return 0;
+    if (p.done_bits && p.T >= kClearApartFrom) {  // rollout_deferred_applies: then the reward plane is written too
         const int64_t n_words = (int64_t)p.T * ((p.n + 31) >> 5);
         const int64_t clear_grid = (n_words + 1023) / 1024;
-        if (clear_grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        if (clear_grid > 0x7fffffffLL) return 0;
         clear_words_kernel<<<(unsigned)clear_grid, 256, 0, s>>>(p.done_bits, n_words);
         count_launch();
     }
+    return (unsigned)grid;
+}
+
+template <int POLICY, bool SHORT, bool LIMIT, bool RD>
+cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
+    const unsigned grid = deferred_grid(p, s);
+    if (grid == 0) return cudaErrorInvalidConfiguration;
     if (contracted) {  // the optional arithmetic comes at the default trip spacing only
         constexpr int kC = is_network(POLICY) ? 2 : 6;
-        rollout_deferred_kernel<POLICY, kC, SHORT, LIMIT, RD, true><<<(unsigned)grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, kC, SHORT, LIMIT, RD, true><<<grid, 256, 0, s>>>(p);
     } else if constexpr (is_wide_network(POLICY)) {  // and so do the wider and deeper networks
-        rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<(unsigned)grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p);
     } else {
         switch (k) {
-            case 2: rollout_deferred_kernel<POLICY, 2, SHORT, LIMIT, RD, false><<<(unsigned)grid, 256, 0, s>>>(p); break;
-            case 3: rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<(unsigned)grid, 256, 0, s>>>(p); break;
-            case 6: rollout_deferred_kernel<POLICY, 6, SHORT, LIMIT, RD, false><<<(unsigned)grid, 256, 0, s>>>(p); break;
-            case 8: rollout_deferred_kernel<POLICY, 8, SHORT, LIMIT, RD, false><<<(unsigned)grid, 256, 0, s>>>(p); break;
-            default: rollout_deferred_kernel<POLICY, 4, SHORT, LIMIT, RD, false><<<(unsigned)grid, 256, 0, s>>>(p); break;
+            case 2: rollout_deferred_kernel<POLICY, 2, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
+            case 3: rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
+            case 6: rollout_deferred_kernel<POLICY, 6, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
+            case 8: rollout_deferred_kernel<POLICY, 8, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
+            default: rollout_deferred_kernel<POLICY, 4, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
         }
     }
     count_launch();

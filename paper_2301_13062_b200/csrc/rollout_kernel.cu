@@ -5,6 +5,9 @@
 namespace cp {
 
 cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool contracted, cudaStream_t s) {
+    // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
+    // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
+    if (const int lanes = rollout_lanes_for(p, policy, streams)) return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
     // The deferred-restart kernel (rollout_deferred.cu) by default: from one 64-env warp per
     // scheduler on (37,888 envs on 148 SMs) for hashed actions and the linear policies, from seven
     // warps per SM on (66,304 envs) for the tanh networks, launches of at least a dozen steps,
@@ -13,14 +16,14 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // 131,072 0.163 / 0.251; linear policy 47,360 0.088 / 0.100, 131,072 0.154 / 0.212; network
     // 56,832 0.483 / 0.427, 75,776 0.483 / 0.545. rollout_coop = 5 forces it wherever it
     // applies, any other forced shape keeps the other kernels.
-    // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
-    // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
-    if (const int lanes = rollout_lanes_for(p, policy, streams)) return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
-    const int64_t warps64 = (p.n + 63) / 64;
+    // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
+    // below, and from 48 steps on (supplied actions, 65,536 x 64: 19 / 23 us, x 250: 52 / 70; 200,003 x
+    // 250 120 / 147, with supplied start states too 140 / 290; 1,048,576 x 16 61 / 46).
+    const int64_t warps32 = (p.n + 31) / 32, warps64 = (p.n + 63) / 64, sms = sm_count();
+    const bool data = p.action_bits_in || p.start_in;
     const bool network = policy == 2 || policy == 4 || policy == 5 || policy == 7;
-    const bool enough = network ? warps64 >= (int64_t)sm_count() * 7 : warps64 >= (int64_t)sm_count() * 4;
-    const bool by_default = g_tuning.rollout_coop == 0 && g_tuning.rollout_ept == 0 && enough && p.T >= 12u &&
-                            (policy == 0 || policy == 1 || policy == 6 || network);
+    const bool enough = data ? warps32 > sms * 10 && p.T >= 48u : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
+    const bool by_default = g_tuning.rollout_coop == 0 && g_tuning.rollout_ept == 0 && enough;
     if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams))
         return launch_rollout_deferred(p, policy, contracted, s);
     // very small batches, unless a network acts: a helper warp per stepping warp (rollout_assisted.cu)
