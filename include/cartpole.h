@@ -304,7 +304,9 @@ int cp_rollout_host(int64_t n_envs, int64_t T, uint32_t seed, const cp_policy *p
 int cp_rollout_host_shard(uint32_t env_offset, int64_t n_envs, int64_t T, uint32_t seed, const cp_policy *policy,
                           float *h_ep_return_sum, uint32_t *h_ep_count, uint64_t *h_totals);
 /* cp_step_host: h_planes_in/out [4][n_envs] (stride n_envs), h_action [n_envs] or NULL,
- * h_reward [n_envs], h_done [n_envs]; the step at global time t of envs 0..n_envs-1. */
+ * h_reward [n_envs], h_done [n_envs]; the step at global time t of envs 0..n_envs-1. Out may be in
+ * (a step in place). On page-locked buffers that do not otherwise overlap, calls of fewer than
+ * 262,144 environments are one kernel that works on host memory directly. */
 int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_planes_in,
                  const uint8_t *h_action, float *h_planes_out, float *h_reward, uint8_t *h_done);
 /* Free the library-owned staging buffers (synchronises the device). */

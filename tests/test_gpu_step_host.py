@@ -1,0 +1,52 @@
+"""cp_step_host on page-locked buffers (the kernel works on host memory) gives what it gives on pageable
+ones (copies), with and without actions, in place, at ragged sizes, from misaligned and overlapping buffers."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def cp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_13062_b200 import binding, build
+    build.build()
+    binding.lib()
+    torch.cuda.set_device(0)
+    return binding
+
+
+def buffers(n, pinned, offset, form):
+    from paper_2301_13062_b200 import inputs
+
+    def make(count, dtype):
+        t = torch.full((count + 4,), 7, dtype=dtype)
+        return (t.pin_memory() if pinned else t)[offset:offset + count]
+
+    z = torch.from_numpy(inputs.random_states(n, 6, "edge")).reshape(-1)
+    planes = make(4 * n, torch.float32)
+    planes.copy_(z)
+    out = planes if form == "in place" else make(4 * n, torch.float32)
+    reward, done = make(n, torch.float32), make(n, torch.uint8)
+    if form == "overlap":  # reward lies in the input planes: only the copies' order is defined
+        reward = planes[:n]
+    action = make(n, torch.uint8)
+    action.copy_(torch.from_numpy(inputs.random_actions(n, 3)))
+    for t in (planes, out, reward, done, action):
+        assert t.is_pinned() == pinned
+    return planes, action, out, reward, done
+
+
+@pytest.mark.parametrize("n", [1, 33, 4099, 70_001, 262_143, 262_145])
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("form", ["apart", "in place", "overlap"])
+@pytest.mark.parametrize("given", [False, True])
+def test_page_locked_equals_pageable(cp, n, offset, form, given):
+    got = []
+    for pinned in (True, False):
+        planes, action, out, reward, done = buffers(n, pinned, offset, form)
+        cp.cp_step_host(n, 9, 4, planes, action if given else None, out, reward, done)
+        got.append([t.numpy().tobytes() for t in (planes, out, reward, done)])
+    assert got[0] == got[1]
