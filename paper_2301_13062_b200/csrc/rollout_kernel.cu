@@ -17,12 +17,15 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // 56,832 0.483 / 0.427, 75,776 0.483 / 0.545. rollout_coop = 5 forces it wherever it
     // applies, any other forced shape keeps the other kernels.
     // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
-    // below, and from 48 steps on (supplied actions, 65,536 x 64: 19 / 23 us, x 250: 52 / 70; 200,003 x
-    // 250 120 / 147, with supplied start states too 140 / 290; 1,048,576 x 16 61 / 46).
+    // below, and from 96 steps on (general kernel / this one, us: supplied actions 60,000 x 140 44 / 35,
+    // 200,003 x 250 147 / 120, with supplied start states too 85 / 58 and 290 / 140; but 100,000 x 64
+    // 30 / 32 and 31 / 35, 1,048,576 x 16 46 / 61). With the reward plane and done bits, supplied
+    // actions alone gain from 66,304 envs on (47,360 x 250 68 / 71, 70,000 x 140 49 / 45).
     const int64_t warps32 = (p.n + 31) / 32, warps64 = (p.n + 63) / 64, sms = sm_count();
     const bool data = p.action_bits_in || p.start_in;
     const bool network = policy == 2 || policy == 4 || policy == 5 || policy == 7;
-    const bool enough = data ? warps32 > sms * 10 && p.T >= 48u : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
+    const bool enough = data ? warps32 > sms * 10 && (!streams || p.start_in || warps64 >= sms * 7) && p.T >= 96u
+                             : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
     const bool by_default = g_tuning.rollout_coop == 0 && g_tuning.rollout_ept == 0 && enough;
     if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams))
         return launch_rollout_deferred(p, policy, contracted, s);

@@ -107,10 +107,12 @@ def test_linear_policies(cp, kind, n, T, contracted):
 
 @pytest.mark.parametrize("kind", [0, LINEAR, PER_ENV, MLP])
 @pytest.mark.parametrize("given", [False, True])
-@pytest.mark.parametrize("n,T", [(1, 17), (33, 1), (1000, 16), (4801, 47)])
+@pytest.mark.parametrize("n,T", [(1, 17), (33, 1), (1000, 16), (4801, 47), (2049, 97)])
 def test_supplied_starts(cp, kind, given, n, T):
     bits = torch.from_numpy(np.random.default_rng(2).integers(-2**31, 2**31, (T, (n + 31) // 32)).astype(np.int32)).cuda()
     for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("reward_stream", "done_bits"), 0, None),
                                    (("done_bits",), 0, "edge")):
         args = dict(streams=streams, limit=limit, spread=spread, starts=start_rows(T, n), given=bits if given else None)
-        assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
+        general = rollout(cp, 2, kind, n, T, **args)
+        for coop in (0, 4):  # what a caller gets; helper warps, which take such calls from 96 steps on
+            assert_same_bits(rollout(cp, coop, kind, n, T, **args), general)
