@@ -4,6 +4,24 @@
 
 namespace cp {
 
+// Do two ranges share memory? (A null pointer's shares none.)
+static bool share_memory(const void *a, int64_t a_bytes, const void *b, int64_t b_bytes) {
+    const char *x = static_cast<const char *>(a), *y = static_cast<const char *>(b);
+    return x && y && x < y + b_bytes && y < x + a_bytes;
+}
+
+// A call may write its per-step outputs over the actions or start states it reads (the done bits of a
+// recording where its actions were): the kernels that step a warp's environments together have read
+// a row by the time they write it. The deferred-restart kernel has not: it clears the done bits before
+// the first step, and its environments read rows that the warp's reward rows have passed.
+static bool outputs_over_data(const RolloutParams &p) {
+    const int64_t T = p.T, word_rows = T * ((p.n + 31) / 32) * 4, env_rows = T * p.n * 4;
+    return share_memory(p.done_bits, word_rows, p.action_bits_in, word_rows) ||
+           share_memory(p.done_bits, word_rows, p.start_in, 4 * env_rows) ||
+           share_memory(p.reward_stream, env_rows, p.action_bits_in, word_rows) ||
+           share_memory(p.reward_stream, env_rows, p.start_in, 4 * env_rows);
+}
+
 cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool contracted, cudaStream_t s) {
     // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
     // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
@@ -27,7 +45,7 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     const bool enough = data ? warps32 > sms * 10 && (!streams || p.start_in || warps64 >= sms * 7) && p.T >= 96u
                              : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
     const bool by_default = g_tuning.rollout_coop == 0 && g_tuning.rollout_ept == 0 && enough;
-    if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams))
+    if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams) && !outputs_over_data(p))
         return launch_rollout_deferred(p, policy, contracted, s);
     // very small batches, unless a network acts: a helper warp per stepping warp (rollout_assisted.cu)
     if (rollout_assisted_applies(p, policy, streams)) return launch_rollout_assisted(p, policy, contracted, s);

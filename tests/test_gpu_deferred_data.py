@@ -111,3 +111,35 @@ def test_environments_far_apart(cp, starts):
     general = rollout(cp, 2, n, T, **args)
     assert_same_bits(rollout(cp, 5, n, T, **args), general)
     assert general["ep_count"][::3].max() <= 1 and general["ep_count"][1::3].min() > T // 15
+
+
+@pytest.mark.parametrize("coop", [0, 5])
+@pytest.mark.parametrize("n,T", [(100_003, 200), (4099, 40)])   # what a caller gets, and the kernel asked for
+def test_done_bits_written_over_the_actions(cp, coop, n, T):
+    """A recording's actions replaced by the done bits of the call that plays it."""
+    bits = action_rows(T, n)
+    apart, over = torch.zeros_like(bits), bits.clone()
+    reward, ret = torch.empty(T, n, device="cuda"), [torch.empty(n, device="cuda") for _ in range(2)]
+    for given, done, r in ((bits, apart, ret[0]), (over, over, ret[1])):
+        with H.rollout_shape(cp, 0, coop):
+            cp.cp_rollout_ex(n_envs=n, T=T, seed=9, action_bits_in=given, done_bits=done, reward_stream=reward, ep_return_sum=r)
+    assert torch.equal(apart, over) and torch.equal(*ret)
+
+
+@pytest.mark.parametrize("coop", [0, 5])
+def test_rewards_written_over_the_start_states(cp, coop):
+    """Reward row r lies over start states of row r / 4, read by the step before or not at all. Episodes of one
+    step (x beyond its threshold), so that every row is read; x overwritten by a reward would not end them."""
+    n, T = 50_001, 200
+    starts = torch.from_numpy(np.random.default_rng(4).uniform(-0.05, 0.05, (T, 4, n)).astype(np.float32)).cuda()
+    starts[:, 0] += 3.0
+    got = []
+    for over in (False, True):
+        s = starts.clone()
+        reward = s.view(-1)[:T * n].view(T, n) if over else torch.empty(T, n, device="cuda")
+        done = torch.empty(T, (n + 31) // 32, dtype=torch.int32, device="cuda")
+        final = torch.empty(4, n, device="cuda")
+        with H.rollout_shape(cp, 0, coop):
+            cp.cp_rollout_ex(n_envs=n, T=T, seed=9, start_states_in=s, done_bits=done, reward_stream=reward, final_state=final)
+        got.append((done, final))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
