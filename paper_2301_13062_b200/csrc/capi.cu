@@ -8,9 +8,12 @@
 #include <mutex>
 #include <new>
 
+#include <cuda.h>  // types of the driver call in pinned_span; its library is not linked
+
 #include "../../include/cartpole.h"
 #include "cartpole_device.cuh"
 #include "cartpole_internal.h"
+#include "pinned_range.h"
 
 struct cp_state {
     int64_t n;
@@ -214,22 +217,35 @@ int staging_reserve(size_t bytes, void **out) {
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Device-side address of a page-locked host range [p, p + bytes), or nullptr if the range is
-// pageable (or not wholly inside one registered allocation).
-void *device_view_of_pinned(void *p, size_t bytes) {
-    cudaPointerAttributes a0, a1;
-    if (cudaPointerGetAttributes(&a0, p) != cudaSuccess || a0.type != cudaMemoryTypeHost || !a0.devicePointer) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    if (cudaPointerGetAttributes(&a1, static_cast<char *>(p) + bytes - 1) != cudaSuccess ||
-        a1.type != cudaMemoryTypeHost || !a1.devicePointer ||
-        static_cast<char *>(a1.devicePointer) - static_cast<char *>(a0.devicePointer) != (ptrdiff_t)(bytes - 1)) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    return a0.devicePointer;
+// The page-locked allocation or registration around host address q, by the driver's own query: only
+// that one tells the extent. (A thread whose first CUDA call this is may get no answer: not page-locked.)
+bool pinned_span(char *q, cp::PinnedSpan &span) {
+    static const auto query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 7000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr)>(fn);
+    }();
+    if (!query) return false;
+    unsigned type = 0;
+    CUdeviceptr at = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[4] = {&type, &at, &start, &size};
+    if (query(4, what, to, reinterpret_cast<CUdeviceptr>(q)) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || !at ||
+        at < start || at - start >= size)
+        return false;
+    span = cp::PinnedSpan{reinterpret_cast<char *>(at), size - (size_t)(at - start)};
+    return true;
 }
+
+// Device-side address of a host range, or nullptr unless all of it is page-locked.
+void *device_view_of_pinned(void *p, size_t bytes) { return cp::pinned_view(p, bytes, pinned_span); }
 
 }  // namespace
 
