@@ -167,9 +167,15 @@ __global__ void __launch_bounds__(32 * kLaneWarps<G, STREAMS>) rollout_lanes_ker
     int64_t idx = base + e;
     const bool valid = idx < p.n;
     if (!valid) idx = p.n - 1;  // idle lanes shadow the last environment and store nothing
+    // A warp that lies wholly past the end must not read what the last environment's warp rewrites at its
+    // end (a batch advanced in place, its episode lengths): nothing orders the two. Its lanes step
+    // along from a hashed state instead. (Per lane without per-step outputs, per warp with them: the
+    // order of the kernel's instructions hangs on it. 4-16-2, 128 steps: 1.00 of the time without the test
+    // and 1.03 the other way round; contracted 4-32-2 with outputs 1.00 and 1.07.)
+    const bool owned = STREAMS ? base < p.n : valid;
     const FoldedKeys kr = fold_keys(make_keys(p.salt_r, p.env_offset + (uint32_t)idx));
     State z;
-    if (p.init_planes) {
+    if (p.init_planes && owned) {
         z.x = p.init_planes[idx];
         z.xd = p.init_planes[p.init_stride + idx];
         z.th = p.init_planes[2 * p.init_stride + idx];
@@ -179,7 +185,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps<G, STREAMS>) rollout_lanes_ker
     }
     LaneNetwork<NET, G> net;
     net.load(p, g);
-    const uint32_t carried = p.ep_len_io ? p.ep_len_io[idx] : 0u;
+    const uint32_t carried = p.ep_len_io && owned ? p.ep_len_io[idx] : 0u;
     // begin: global time at which the running episode began (as in the general kernel)
     uint32_t cnt = 0u, begin = p.t0 - carried;
     const int64_t words = (p.n + 31) >> 5;

@@ -94,6 +94,17 @@ def test_networks_contracted_and_supplied_starts(cp, kind, n):
         assert_same_bits(rollout(cp, 0, kind, n, 50, **args), rollout(cp, 2, kind, n, 50, **args))
 
 
+@pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
+@pytest.mark.parametrize("n", [1, 8, 9, 17, 25, 1217])
+def test_networks_in_place_with_warps_past_the_end(cp, kind, n):
+    """A batch advanced in place whose last CTA has warps without environments: those read neither its states
+    nor its episode lengths, which another warp rewrites. (That they do not is seen in the kernel; here that
+    everything else is as before.)"""
+    for streams in ((), ALL):
+        args = dict(streams=streams, limit=60, spread="edge")
+        assert_same_bits(rollout(cp, 0, kind, n, 70, **args), rollout(cp, 2, kind, n, 70, **args))
+
+
 @pytest.mark.parametrize("kind", [LINEAR, PER_ENV])
 @pytest.mark.parametrize("n,T", [(1, 15), (33, 32), (2049, 33), (4737, 16), (4801, 65)])
 @pytest.mark.parametrize("contracted", [False, True])
