@@ -23,6 +23,10 @@ static bool outputs_over_data(const RolloutParams &p) {
 }
 
 cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool contracted, cudaStream_t s) {
+    // Supplied actions replace whatever policy was named: from here on the call is the same with and
+    // without one (3, the name the kernels have for it). A network named beside them used to bring its own
+    // spacing of the restart passes and its weights, paired, into the launch.
+    if (p.action_bits_in) policy = 3;
     // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
     // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
     if (const int lanes = rollout_lanes_for(p, policy, streams)) return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
