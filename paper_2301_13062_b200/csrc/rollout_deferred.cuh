@@ -24,9 +24,10 @@
 // ragged end.
 //
 // Scope: hashed or supplied actions, the shared linear policy, the shared 4-16-2 tanh network or one
-// linear policy per environment; hashed start states, or (but for the network) supplied ones; either arithmetic; with or without the episode step limit; per-step
-// outputs either none or exactly the reward plane + done bitmask (the action bitmask and the
-// trajectory are rows of global time that half the lanes would have to touch every step). The
+// linear policy per environment; hashed start states, or (but for the network) supplied ones; either
+// arithmetic; with or without the episode step limit; per-step outputs either none or exactly the reward
+// plane + done bitmask (the action bitmask and the trajectory are rows of global time that half the
+// lanes would have to touch every step). The
 // wider and deeper networks (4-32-2, 4-64-2, 4-16-16-2) too, for the plain call: no step limit,
 // no per-step outputs. Everything else takes the general kernel.
 //
@@ -164,7 +165,9 @@ __device__ __forceinline__ void deferred_actions(const RolloutParams &p, const F
     }
 }
 
-// 32x32 bit transpose over a warp: in, lane l holds row l; out, bit r of lane l is bit l of row r.
+// 32x32 bit transpose over a warp: in, lane l holds row l; out, bit r of lane l is bit l of row r. (The
+// recursive exchange of off-diagonal blocks, halved in size from stage to stage, as in Warren's
+// "Hacker's Delight", section 7-3, with a shuffle in place of the word pairs.)
 __device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
     uint32_t m = 0x0000ffffu;
 #pragma unroll
@@ -180,8 +183,8 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
 // every trip. Instead a warp reads 32 rows at a time, one per lane, transposes the 32x32 bits, and
 // keeps the last kRing such blocks in shared memory: one word per environment with its next 32
 // actions. Every 32 trips or so a lane takes 32 actions from its clock on out of two such words.
-// An environment more than kRing - 1 blocks behind the warp's first one (never seen with
-// actions drawn at random) collects its bits from the caller's rows itself.
+// The ring reaches one block past the warp's first environment: one that is more than kRing - 2 blocks
+// behind that (never seen with actions drawn at random) collects its bits from the caller's rows itself.
 // What bounds it: the float32 pipe, as with hashed actions (1,048,576 x 250: 490 us, hashed 475; the
 // general kernel, which reads a word per warp and step, 617), and with supplied start states the
 // gather of 16 bytes per episode from rows that no two environments of a warp share at a time:
@@ -189,8 +192,19 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
 // start states, at 1 / 2 / 3: 236 / 171 / 140 us; the general kernel 290).
 constexpr int kRing = 8;
 
+// Restart passes of the instances with supplied start states. Their episodes may be of any length, and where
+// they are shorter than the K trips between two passes nearly every slot waits most of the time (start
+// states that end in one step: 6 trips for one). So a pass counts the slots it restarts: from kMany on
+// the following passes come as soon as kEnough slots wait, until one restarts fewer than kFew. Counting
+// in every trip of every launch instead costs launches with 20-step episodes a quarter of their time;
+// counting in the passes costs those nothing with hashed or supplied actions and 8-12 % with the linear
+// policies, whose episodes are shorter. us, general kernel / fixed spacing / this, 200,003 x 250 and
+// 1,048,576 x 250 with supplied actions: one-step episodes 398 / 992 / 528 and 1,523 / 9,840 / 4,026,
+// one to three steps 347 / 480 / 252 and 1,307 / 3,640 / 2,356, 20 steps 285 / 134 / 137 and 1,098 / 588 / 596.
+constexpr int kMany = 40, kEnough = 24, kFew = 16;  // of the warp's 64
+
 // POLICY: 0 hashed actions, 1 shared linear policy, 2 / 4 / 5 / 7 a shared tanh network (is_network),
-// 6 one linear policy per environment.
+// 3 supplied actions, 6 one linear policy per environment.
 // K: trips between restart passes. LIMIT: episodes are cut off after p.max_steps steps.
 // RD: the reward plane and the done bitmask are written (see the comment at reward_row).
 // START_IN: finished environments continue from the caller's start states, which may hold any angle.
@@ -408,8 +422,13 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
         // linear policies' 80-step episodes the test only costs: 4,194,304 x 100 with streams
         // 0.828 -> 0.878 ms.)
         constexpr bool FORESIGHT = is_network(POLICY);
-        int passes = 0;     // GIVEN: since the windows were loaded
-        bool wide = false;  // START_IN, warp-uniform: a slot stands at a start state beyond the polynomial range
+        int used = 0;        // GIVEN: trips since the windows were loaded
+        bool wide = false;   // START_IN, warp-uniform: a slot stands at a start state beyond the polynomial range
+        bool early = false;  // START_IN, warp-uniform: episodes are short (see kMany)
+        auto waiting = [&]() {  // slots whose episode has ended and that have steps to do, warp-uniform
+            return __popc(__ballot_sync(0xffffffffu, !act[0] && t[0] != t_end)) +
+                   __popc(__ballot_sync(0xffffffffu, !act[1] && t[1] != t_end));
+        };
         auto restart_pass = [&](auto tail) {
             constexpr bool TAIL = decltype(tail)::value;
             if (FORESIGHT) {
@@ -430,6 +449,9 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
                 }
             }
             if (START_IN) {
+                const int ended = waiting();
+                if (ended >= kMany) early = true;
+                else if (ended < kFew) early = false;
                 State f[2];  // both slots' loads are in flight before either is used
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
@@ -463,9 +485,9 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
                     }
                 }
             }
-            if (GIVEN && ++passes == 32 / K) {  // no slot has used more than the 32 actions of its window
+            if (GIVEN && used + K > 32) {  // the next block would run past the 32 actions of a window
                 load_windows();
-                passes = 0;
+                used = 0;
             }
         };
 
@@ -490,19 +512,29 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
             after_step(tail, 0, d0);
             after_step(tail, 1, d1);
         };
-        // The K trips between two restart passes (a network policy's trip is 600 instructions or more:
+        // The trips between two restart passes: K, or fewer where many slots wait (a network policy's trip is 600 instructions or more:
         // its trips stay a loop).
         constexpr int kUnroll = is_network(POLICY) ? 1 : K;
-        auto trip_block = [&](auto tail) {
-            if (START_IN && wide) {  // only the first trip after a pass can meet such an angle
-                trip(tail, std::true_type{});
-                wide = false;
+        auto trip_block = [&](auto tail) {  // returns the trips made
+            int made = K;
+            if (START_IN && (wide || early)) {
+                made = 0;
+                if (wide) {  // only the first trip after a pass can meet such an angle
+                    trip(tail, std::true_type{});
+                    wide = false;
+                    made = 1;
+                }
 #pragma unroll 1
-                for (int k = 1; k < K; ++k) trip(tail, std::false_type{});
+                while (made < K && !(early && made > 0 && waiting() >= kEnough)) {
+                    trip(tail, std::false_type{});
+                    ++made;
+                }
             } else {
 #pragma unroll kUnroll
                 for (int k = 0; k < K; ++k) trip(tail, std::false_type{});
             }
+            if (GIVEN) used += made;
+            return (uint32_t)made;
         };
 
         if (GIVEN) {
@@ -515,21 +547,21 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
             // start state (|theta| <= 0.05), which is the packed step's domain.
             trip(std::true_type{}, std::true_type{});
             trips = 1;
+            used = 1;
             restart_pass(std::true_type{});
         }
         // Main part: after these trips no clock can have reached t_end yet (clocks run at most one
         // step ahead of the trips), so no slot can retire.
         while (trips + K + (FORESIGHT ? 1u : 0u) <= p.T - 1u) {
-            trip_block(std::false_type{});
-            trips += K;
+            trips += trip_block(std::false_type{});
             restart_pass(std::false_type{});
         }
         // Tail: slots retire as their clocks reach t_end. Every block of trips advances every
         // unretired slot by at least one step, so p.T blocks always suffice.
         for (uint32_t block = 0; block <= p.T; ++block) {
             if (__all_sync(0xffffffffu, t[0] == t_end && t[1] == t_end)) break;
-            trip_block(std::true_type{});
-            if (FORESIGHT) trips += K;
+            const uint32_t made = trip_block(std::true_type{});
+            if (FORESIGHT) trips += made;
             restart_pass(std::true_type{});
         }
 #pragma unroll

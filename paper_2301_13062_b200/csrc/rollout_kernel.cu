@@ -39,14 +39,29 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // 56,832 0.483 / 0.427, 75,776 0.483 / 0.545. rollout_coop = 5 forces it wherever it
     // applies, any other forced shape keeps the other kernels.
     // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
-    // below, and from 96 steps on (general kernel / this one, us: supplied actions 60,000 x 140 44 / 35,
-    // 200,003 x 250 147 / 120, with supplied start states too 85 / 58 and 290 / 140; but 100,000 x 64
-    // 30 / 32 and 31 / 35, 1,048,576 x 16 46 / 61). With the reward plane and done bits, supplied
-    // actions alone gain from 66,304 envs on (47,360 x 250 68 / 71, 70,000 x 140 49 / 45).
+    // below, and where every sort of data that was tried gains or nearly (time of this kernel over the
+    // general kernel's; random actions / actions that end every episode after ten steps / those of a
+    // balancing policy in every third environment):
+    //   actions alone, T = 96, 128, 192: 48,000 envs 0.91 / 1.04 / 1.05, 0.88 / 1.00 / 1.02, 0.89 / 0.89 /
+    //   0.92; 60,000 0.79 / 0.89 / 0.91 at 96, 100,003 0.91 / 1.05 / 1.06, 200,003 0.86 / 0.85 / 0.92;
+    //   with reward plane and done bits, T = 96, 160, 192: 100,003 envs 1.04 / 1.16 / 1.19, 1.02 / 1.13 /
+    //   1.13, 0.94 / 0.95 / 0.96; 200,003 0.91 / 0.92 / 0.97 at 96; below 66,304 envs nothing gained;
+    //   start states of 10- to 20-step episodes, T = 96, 128: 48,000 envs 0.92-1.28, 0.74-1.06; 60,000
+    //   0.82-1.07, 0.68-0.82; 100,003 0.78-1.01, 0.76-0.97; 200,003 0.52-0.71 at 96;
+    //   with a step limit of 1, 5, 8, 12, 13, 16 at T = 250 (every episode costs whole blocks of trips): 200,003
+    //   envs 2.87, 0.99, 1.31, 0.70, 0.96, 0.82, 100,003 envs with outputs 4.47, 1.25, 1.41, 0.82, 1.16, 0.92.
+    // Start states whose episodes last one to three steps lose (see kMany), and nothing here can see
+    // them. With the reward plane and start states of 2 GB and more the time depends on where
+    // the memory lies (500,000 x 250, general kernel 746 us, this one 435 or 984 in different processes;
+    // 1,048,576 x 128 687, 456 or 787; up to 1.6 GB always the lower one), so those stay there too.
     const int64_t warps32 = (p.n + 31) / 32, warps64 = (p.n + 63) / 64, sms = sm_count();
     const bool data = p.action_bits_in || p.start_in;
     const bool network = policy == 2 || policy == 4 || policy == 5 || policy == 7;
-    const bool enough = data ? warps32 > sms * 10 && (!streams || p.start_in || warps64 >= sms * 7) && p.T >= 96u
+    uint32_t from = 96u;
+    if (p.start_in && warps64 < sms * 7) from = 128u;
+    if (!p.start_in && streams && warps64 < sms * 20) from = 192u;
+    const bool streams_gain = !streams || (p.start_in ? p.n * (int64_t)p.T <= 100000000 : warps64 >= sms * 7);
+    const bool enough = data ? p.T >= from && warps32 > sms * 10 && streams_gain && !(p.max_steps && p.max_steps < 12u)
                              : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
     const bool by_default = g_tuning.rollout_coop == 0 && g_tuning.rollout_ept == 0 && enough;
     if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams) && !outputs_over_data(p))

@@ -96,6 +96,23 @@ def test_supplied_starts(cp, kind, given, n, T):
             assert_same_bits(rollout(cp, 5, n, T, defer=defer, **args), general)
 
 
+@pytest.mark.parametrize("kind,given", [(0, False), (0, True), (1, False), (6, False)])
+@pytest.mark.parametrize("theta", [0.3, 0.2, None])   # episodes of one step; of one to three; rows of either sort and of twenty steps
+@pytest.mark.parametrize("n,T", [(65, 33), (4099, 200)])
+def test_short_episodes_from_supplied_starts(cp, kind, given, theta, n, T):
+    """The passes come closer together while episodes are short, and apart again."""
+    rng = np.random.default_rng(8)
+    s = rng.uniform(-0.05, 0.05, (T, 4, n)).astype(np.float32)
+    s[:, 2] = theta if theta else np.array([0.3, 0.2, 0.0])[(np.arange(T) // 16) % 3][:, None]
+    s[:, 3] = rng.uniform(0.1, 0.5, (T, n))
+    bits = action_rows(T, n) if given else None
+    for streams, limit, contracted in (((), 0, False), (RD, 2, False), (RD, 0, True)):
+        args = dict(kind=kind, streams=streams, limit=limit, given=bits, starts=torch.from_numpy(s).cuda(), contracted=contracted)
+        general = rollout(cp, 2, n, T, **args)
+        for defer in (2, 6):
+            assert_same_bits(rollout(cp, 5, n, T, defer=defer, **args), general)
+
+
 @pytest.mark.parametrize("starts", [False, True])
 def test_environments_far_apart(cp, starts):
     """Constant actions end an episode after ten steps; the recorded actions of a policy that balances end
