@@ -94,7 +94,7 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
 cudaError_t launch_rollout_deferred_data(RolloutParams &p, int policy, int k, bool contracted, cudaStream_t s);
 cudaError_t launch_rollout_deferred_wide(RolloutParams &p, int policy, bool contracted, cudaStream_t s);  // policies 4, 5, 7
 // the lane-split kernel of the network policies: lanes per environment it would use for a call, 0 = not its call
-int rollout_lanes_for(const RolloutParams &p, int policy, bool streams);
+int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool contracted);
 cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s);
 // the MLP policies (kinds 2, 4, 5, 7), canonical and contracted arithmetic; mode and shape as
 // chosen by launch_rollout_arith

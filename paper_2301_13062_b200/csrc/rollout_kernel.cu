@@ -29,7 +29,8 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     if (p.action_bits_in) policy = 3;
     // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
     // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
-    if (const int lanes = rollout_lanes_for(p, policy, streams)) return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
+    if (const int lanes = rollout_lanes_for(p, policy, streams, contracted))
+        return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
     // The deferred-restart kernel (rollout_deferred.cu) by default: from one 64-env warp per
     // scheduler on (37,888 envs on 148 SMs) for hashed actions and the linear policies, from seven
     // warps per SM on (66,304 envs) for the tanh networks, launches of at least a dozen steps,
