@@ -47,6 +47,7 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     //   0.92; 60,000 0.79 / 0.89 / 0.91 at 96, 100,003 0.91 / 1.05 / 1.06, 200,003 0.86 / 0.85 / 0.92;
     //   with reward plane and done bits, T = 96, 160, 192: 100,003 envs 1.04 / 1.16 / 1.19, 1.02 / 1.13 /
     //   1.13, 0.94 / 0.95 / 0.96; 200,003 0.91 / 0.92 / 0.97 at 96; below 66,304 envs nothing gained;
+    //   in the contracted arithmetic 70,000 and 100,003 envs 0.81-0.87 at 128 already;
     //   start states of 10- to 20-step episodes, T = 96, 128: 48,000 envs 0.92-1.28, 0.74-1.06; 60,000
     //   0.82-1.07, 0.68-0.82; 100,003 0.78-1.01, 0.76-0.97; 200,003 0.52-0.71 at 96;
     //   with a step limit of 1, 5, 8, 12, 13, 16 at T = 250 (every episode costs whole blocks of trips): 200,003
@@ -60,7 +61,7 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     const bool network = policy == 2 || policy == 4 || policy == 5 || policy == 7;
     uint32_t from = 96u;
     if (p.start_in && warps64 < sms * 7) from = 128u;
-    if (!p.start_in && streams && warps64 < sms * 20) from = 192u;
+    if (!p.start_in && streams && warps64 < sms * 20) from = contracted ? 128u : 192u;
     const bool streams_gain = !streams || (p.start_in ? p.n * (int64_t)p.T <= 100000000 : warps64 >= sms * 7);
     const bool enough = data ? p.T >= from && warps32 > sms * 10 && streams_gain && !(p.max_steps && p.max_steps < 12u)
                              : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
