@@ -18,6 +18,13 @@ bool rollout_assisted_applies(const RolloutParams &p, int policy, bool streams) 
     // behind, keep the general kernel (a linear policy, 20,011 envs x 16: 9.2 us against 11.1, x 64 with
     // the reward plane and done bits 19 against 21, x 400 107 against 100)
     if (p.start_in && p.T < 96u) return false;
+    // a linear policy, short launches with more than a warp's pair per SM: the first chunk of start states is
+    // hashed before anything is stepped (general kernel / this, us: 45,000 envs x 2, 4, 8 steps 2.7 / 3.1,
+    // 3.2 / 3.7, 4.6 / 4.8, 9,000 x 3 2.9 / 3.1); with the action bits or the trajectory among the outputs,
+    // which the general kernel tests for one by one, only the largest lose, up to three steps (45,000 x 2
+    // 1.12 of the general kernel's time, x 4 1.00, 37,000 x 2 0.99)
+    const bool linear = policy == 1 || policy == 6, tested = p.action_bits || p.trajectory;
+    if (linear && p.T <= (tested ? 3u : 8u) && (p.n + 31) / 32 > (int64_t)sm_count() * (tested ? 8 : 1)) return false;
     // up to ten pairs per SM (five CTAs of two pairs: 200 KB of shared memory; a sixth CTA would
     // wait for a second wave). Measured against the general kernel's best shape, ms per launch:
     // x 5,000 steps 9,472 envs 0.25 / 0.61, 18,944 envs 0.45 / 0.61, 28,416 envs 0.57 / 0.74,
