@@ -542,12 +542,12 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
     if (rc != CP_OK) return rc;
     if (!h_planes_in || !h_planes_out || !h_reward || !h_done) return fail(CP_EINVAL, "a host pointer is NULL");
     if (t >= (1u << 30)) return fail(CP_EINVAL, "global step out of range");
-    // Page-locked buffers, up to the batches that the one-environment-per-thread kernel serves: the kernel
-    // reads and writes host memory itself, in one launch instead of a launch and up to five copies, each
-    // after the other (us per call, copies / this: 2,000 envs 51 / 26, 20,000 64 / 35, 100,000 117 / 89,
-    // 200,000 188 / 158; 300,001 260 / 272 and 4,000,001 3,027 / 3,277, where the copy engine's
-    // bandwidth counts). Buffers that overlap, other than a step in place, keep the copies' order.
-    if (n_envs < 262144) {
+    // Page-locked buffers, small and middling batches: the kernel reads and writes host memory itself, in
+    // one launch instead of a launch and up to five copies, each after the other (us per call, copies /
+    // this: 2,000 envs 41 / 22, 20,000 57 / 31, 100,000 118 / 85, 200,000 188 / 157, 240,000 211 / 188,
+    // 250,000 212 / 205, 262,143 222 / 230, the last three with actions; 300,001 260 / 272 and 4,000,001
+    // 3,027 / 3,277, where the copy engine's bandwidth counts). Buffers that overlap, other than a step in place, keep the copies' order.
+    if (n_envs <= 250000) {
         const size_t n = (size_t)n_envs;
         const struct { void *p; size_t bytes; } buf[5] = {{const_cast<float *>(h_planes_in), 16 * n},
             {const_cast<uint8_t *>(h_action), n}, {h_planes_out, 16 * n}, {h_reward, 4 * n}, {h_done, n}};
