@@ -305,8 +305,8 @@ int cp_rollout_host_shard(uint32_t env_offset, int64_t n_envs, int64_t T, uint32
                           float *h_ep_return_sum, uint32_t *h_ep_count, uint64_t *h_totals);
 /* cp_step_host: h_planes_in/out [4][n_envs] (stride n_envs), h_action [n_envs] or NULL,
  * h_reward [n_envs], h_done [n_envs]; the step at global time t of envs 0..n_envs-1. Out may be in
- * (a step in place). On page-locked buffers that do not otherwise overlap, calls of fewer than
- * 262,144 environments are one kernel that works on host memory directly. */
+ * (a step in place). On buffers that are page-locked throughout and do not otherwise overlap, calls of
+ * up to 250,000 environments are one kernel that works on host memory directly. */
 int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_planes_in,
                  const uint8_t *h_action, float *h_planes_out, float *h_reward, uint8_t *h_done);
 /* Free the library-owned staging buffers (synchronises the device). */
@@ -334,17 +334,23 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * actions only, otherwise as 2), 4 = a helper warp per stepping warp hashes every step's action
  * and start state ahead into shared memory, or fetches the supplied ones (hashed or supplied
  * actions and the linear policies; otherwise as 2), 2, 3 and 4 only with one environment per
- * thread; 0 = default: helper warps for up to ten warps of environments per SM, the hidden units
- * of a network spread over several lanes for up to two warps per scheduler, per lane for
+ * thread; 0 = default: helper warps for up to ten warps of environments per SM (a linear policy's
+ * shortest launches aside), the hidden units of a network spread over several lanes for up to two warps
+ * per scheduler and from 3 to 8 steps on, per lane for
  * other batches too small to fill the GPU (ahead for the smaller ones), deferred (5) from one
  * 64-environment warp per scheduler on (37,888 environments on 148 SMs) where that form applies,
- * by the warp otherwise;
+ * with supplied actions or start states only beyond the helper warps' batches, from 96, 128 or 192 steps on
+ * by batch size and outputs, without a step limit below 12, and, beside a reward plane, with at most 1.6 GB of
+ * start states; by the warp otherwise;
  * 5 = two environments per thread with a clock per environment and restarts deferred to every
- * few loop trips (per-step outputs none or reward plane + done bits; hashed or supplied actions, a
- * linear policy, hashed or supplied start states, or the 4-16-2 network with hashed ones; the wider and deeper networks without step limit and per-step
+ * few loop trips (per-step outputs none or reward plane + done bits, not over the call's own actions or
+ * start states; hashed or supplied actions, a linear policy, hashed or supplied start states, or the
+ * 4-16-2 network with hashed ones; the wider and deeper networks without step limit and per-step
  * outputs; otherwise the default); every choice gives the same bits), "rollout_defer" (loop
  * trips between the restart passes of that deferred form: 2, 3, 4, 6 or 8; 0 = default: 2, 4 or
- * 6 by the number of steps, 3 with a network policy; the wider and deeper networks always use 3),
+ * 6 by the number of steps, 3 with a network policy; the wider and deeper networks always use 3, calls with
+ * supplied actions or start states have 2, 4 and 6 only (3 runs as 4, 8 as 6), and the contracted arithmetic
+ * always uses 6, with a network 2),
  * "rollout_ctas_per_sm" (0 = default: one 32*ept-environment task per warp and as many
  * CTAs as that takes; k > 0 = persistent grid of k CTAs per SM looping over tasks), "step_block"
  * (32..256, default 64), "step_vec_min_envs" (batches smaller than this use the one-env-per-thread

@@ -18,9 +18,9 @@
 // Where a thread owns two environments (SHAPE 2) and the arithmetic is the canonical one, both
 // are stepped by the packed float32 instructions of sm_100a (euler_step_pair). Batches that fill
 // the chip mostly go to the deferred-restart kernel of rollout_deferred.cu instead; this
-// kernel keeps every call that one does not cover (action bit stream or trajectory written,
-// supplied actions or start states, the wider and deeper networks, very short launches, batches
-// too small to fill the chip) and is the form the others are compared with bit for bit.
+// kernel keeps every call that one does not cover (action bit stream or trajectory written, the
+// wider and deeper networks with a step limit or outputs, very short launches, batches too small to fill
+// the chip, supplied actions or start states where that kernel does not gain) and is the form the others are compared with bit for bit.
 //
 // This header holds the kernel template and its dispatch; rollout_kernel.cu and
 // rollout_networks.cu instantiate it for the canonical (one rounding per op) arithmetic,
