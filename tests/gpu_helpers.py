@@ -22,13 +22,16 @@ BAND = 1e-5
 REL_TOL = 2e-6
 
 
-# The rollout kernel's work shapes as (rollout_ept, rollout_coop) tuning values: one env per
-# thread with per-lane restarts, the same with start states computed ahead every step, one env
-# per thread with restarts by the whole warp, two envs per thread (always by the warp), and the
-# kernel whose helper warps hash actions and start states ahead of the stepping warps (it covers
-# hashed actions without streams or step limit; other calls fall to the first shape). The
-# library picks one by batch size and policy; tests force each of them on small batches.
+# The rollout kernels' work shapes as (rollout_ept, rollout_coop) tuning values: one env per thread with
+# per-lane restarts, the same with start states computed ahead every step, one env per thread with
+# restarts by the whole warp, two envs per thread (always by the warp), the kernel whose helper warps
+# hash or fetch actions and start states ahead of the stepping warps (every call but a network's; that
+# one falls to the first shape), and the one with a clock per environment and deferred restarts. The
+# library picks one by batch size, policy and outputs; tests force each of them on small batches.
 SHAPES = [(1, 2), (1, 3), (1, 1), (2, 1), (1, 4), (2, 5)]
+# Nothing forced: what a caller gets, and the only way to the network kernel that spreads an environment's
+# hidden units over several lanes.
+DEFAULT = (0, 0)
 
 
 @contextlib.contextmanager

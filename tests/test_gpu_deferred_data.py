@@ -39,7 +39,7 @@ def rollout(cp, coop, n, T, kind=0, streams=(), limit=0, contracted=False, start
           "arithmetic": cp.CP_ARITH_CONTRACTED if contracted else cp.CP_ARITH_EXACT, "start_states_in": starts}
     cp.cp_tune("rollout_defer", defer)
     try:
-        with H.rollout_shape(cp, 2 if coop == 5 else 1, coop):
+        with H.rollout_shape(cp, {0: 0, 5: 2}.get(coop, 1), coop):
             if spread:
                 planes = torch.from_numpy(inputs.random_states(n, 5, spread)).cuda()
                 ep_len = torch.arange(n, dtype=torch.int32, device="cuda") % 37
@@ -111,6 +111,22 @@ def test_short_episodes_from_supplied_starts(cp, kind, given, theta, n, T):
         general = rollout(cp, 2, n, T, **args)
         for defer in (2, 6):
             assert_same_bits(rollout(cp, 5, n, T, defer=defer, **args), general)
+
+
+@pytest.mark.parametrize("kind,given,starts", [(0, True, False), (0, True, True), (0, False, True), (1, False, True), (6, False, True)])
+@pytest.mark.parametrize("n,T", [(70_001, 200), (47_361, 250)])
+def test_what_a_caller_gets(cp, kind, given, starts, n, T):
+    """Nothing forced: large enough for this kernel, which is told by the launch of its own that clears the done
+    bits (actions alone with outputs take it from 66,304 environments on)."""
+    bits = action_rows(T, n) if given else None
+    rows = torch.rand(T, 4, n, generator=torch.Generator("cuda").manual_seed(5), device="cuda") * 0.1 - 0.05 if starts else None
+    for streams, limit, spread in (((), 0, None), (RD, 0, "wide"), (RD, 11, None)):
+        args = dict(kind=kind, streams=streams, limit=limit, spread=spread, given=bits, starts=rows)
+        general = rollout(cp, 2, n, T, **args)
+        before = cp.cp_launch_count()
+        assert_same_bits(rollout(cp, 0, n, T, **args), general)
+        cleared = streams == RD and limit != 11 and (starts or n > 66_304)
+        assert cp.cp_launch_count() - before == (2 if cleared else 1)
 
 
 @pytest.mark.parametrize("starts", [False, True])

@@ -40,6 +40,16 @@ POLICY_SEEDS = {1: 4, 2: 6, 4: 3, 5: 3, 7: 7}
 
 @pytest.mark.parametrize("case", range(int(os.environ.get("CARTPOLE_FUZZ_CASES", "36"))))   # more for a soak run
 def test_random_combination_against_oracle(cp, oracle, case):
+    check_combination(cp, oracle, case, None)
+
+
+@pytest.mark.parametrize("case", range(500, 536))
+def test_random_combination_in_the_default_shape(cp, oracle, case):
+    """The kernel that a caller gets, the lane-split networks among them."""
+    check_combination(cp, oracle, case, H.DEFAULT)
+
+
+def check_combination(cp, oracle, case, forced):
     rng = np.random.default_rng(1000 + case)
     n = int(rng.choice([1, 31, 32, 33, 97, 1000, 4097, 20011]))
     T = int(rng.integers(1, 90))
@@ -47,7 +57,7 @@ def test_random_combination_against_oracle(cp, oracle, case):
     t0 = int(rng.choice([0, 1, 17, 100000]))
     off = int(rng.choice([0, 5, 1 << 20]))
     kind = int(rng.choice([0, 0, 1, 2, 4, 5, 6, 7]))
-    shape = H.SHAPES[int(rng.integers(0, len(H.SHAPES)))]
+    shape = forced or H.SHAPES[int(rng.integers(0, len(H.SHAPES)))]
     limit = int(rng.choice([0, 0, 1, 5, 40]))
     supplied_actions = kind == 0 and rng.random() < 0.35
     supplied_starts = rng.random() < 0.3

@@ -94,7 +94,7 @@ def test_step_and_ladder_stay_inside_their_outputs(cp, n):
 
 
 @pytest.mark.parametrize("n", SIZES)
-@pytest.mark.parametrize("shape", H.SHAPES)
+@pytest.mark.parametrize("shape", [*H.SHAPES, H.DEFAULT])
 def test_rollouts_stay_inside_their_outputs(cp, n, shape):
     T, words = 37, (n + 31) // 32
     w = inputs.policy_weights(1, 1)
@@ -127,3 +127,68 @@ def test_rollouts_stay_inside_their_outputs(cp, n, shape):
     torch.cuda.synchronize()
     check_plane_tails(planes, n, "rollout state planes")
     ep_len.check("rollout ep_len"), ret.check("rollout ep_return_sum (from state)")
+
+
+def guarded_outputs(n, T, outputs):
+    words = (n + 31) // 32
+    out = {"ep_return_sum": Guarded((n,), torch.float32), "ep_count": Guarded((n,), torch.int32),
+           "totals": Guarded((2,), torch.int64), "final_state": Guarded((4, n), torch.float32)}
+    if outputs != "none":
+        out.update(reward_stream=Guarded((T, n), torch.float32), done_bits=Guarded((T, words), torch.int32))
+    if outputs == "all":
+        out.update(action_bits=Guarded((T, words), torch.int32), trajectory=Guarded((T, 4, n), torch.float32))
+    out["totals"].t.zero_()
+    return out
+
+
+def check_outputs(out, n, what):
+    torch.cuda.synchronize()
+    for k, g in out.items():
+        g.check(f"rollout {k} ({what})")
+    assert int(out["totals"].t[1]) == int(out["ep_count"].t.sum())
+    for k in ("done_bits", "action_bits"):
+        assert k not in out or not (n % 32) or not np.any(out[k].t.cpu().numpy().view(np.uint32)[:, -1] >> (n % 32)), k
+
+
+@pytest.mark.parametrize("n", [1, 9, 33, 1025, 2371, 4164, 9465])   # every number of lanes per environment, and past them
+@pytest.mark.parametrize("kind", [2, 4, 5, 6, 7])
+@pytest.mark.parametrize("outputs", ["none", "rd", "all"])
+def test_feedback_policies_stay_inside_their_outputs(cp, n, kind, outputs):
+    T = 37
+    weights = torch.from_numpy(inputs.per_env_linear_weights(n, 2)).cuda() if kind == 6 else inputs.policy_weights(kind, 2)
+    pol = cp.policy(kind, weights)
+    for limit in (0, 9):
+        out = guarded_outputs(n, T, outputs)
+        cp.cp_rollout_ex(n_envs=n, T=T, seed=2, env_offset=3, policy=pol, max_episode_steps=limit,
+                         **{k: g.t for k, g in out.items()})
+        check_outputs(out, n, f"policy {kind}, outputs {outputs}, limit {limit}")
+    # in place, with carried episode lengths
+    planes, ep_len = Guarded((4, n + 5), torch.float32), Guarded((n,), torch.int32)
+    planes.t[:, :n] = torch.from_numpy(inputs.random_states(n, seed=1, spread="live")).cuda()
+    ep_len.t.zero_()
+    out = guarded_outputs(n, T, outputs)
+    del out["final_state"]
+    cp.cp_rollout_ex(T=T, state=cp.cp_wrap(planes.t, n, 4, 9), ep_len=ep_len.t, policy=pol, **{k: g.t for k, g in out.items()})
+    check_outputs(out, n, f"policy {kind}, outputs {outputs}, in place")
+    check_plane_tails(planes, n, "rollout state planes")
+    ep_len.check("rollout ep_len")
+
+
+@pytest.mark.parametrize("n,T,shape", [(1, 37, (1, 4)), (33, 37, (1, 4)), (4164, 37, (1, 4)), (1, 37, (2, 5)), (33, 37, (2, 5)),
+                                       (4164, 70, (2, 5)), (33, 130, H.DEFAULT), (4164, 130, H.DEFAULT), (70001, 130, H.DEFAULT)])
+@pytest.mark.parametrize("kind", [0, 1, 6])
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("starts", [False, True])
+def test_data_fed_calls_stay_inside_their_outputs(cp, n, T, shape, kind, given, starts):
+    words = (n + 31) // 32
+    g = torch.Generator("cuda").manual_seed(3)
+    weights = torch.from_numpy(inputs.per_env_linear_weights(n, 2)).cuda() if kind == 6 else inputs.policy_weights(kind, 2)
+    data = {"action_bits_in": torch.randint(-2**31, 2**31, (T, words), generator=g, device="cuda", dtype=torch.int64).to(torch.int32)
+            if given else None,
+            "start_states_in": torch.rand(T, 4, n, generator=g, device="cuda") * 0.6 - 0.3 if starts else None}
+    for outputs in ("none", "rd", "all"):
+        out = guarded_outputs(n, T, outputs)
+        with H.rollout_shape(cp, *shape):
+            cp.cp_rollout_ex(n_envs=n, T=T, seed=2, policy=cp.policy(kind, weights) if kind else None, **data,
+                             **{k: g.t for k, g in out.items()})
+        check_outputs(out, n, f"policy {kind}, outputs {outputs}, given {given}, starts {starts}")
