@@ -414,6 +414,15 @@ int cp_selftest_tame_div(uint32_t den_step, uint64_t *out);
  * which the packed and scalar steps of CP_ARITH_CONTRACTED differ (must stay 0). */
 int cp_selftest_pair(uint64_t count, uint32_t seed, uint64_t *out);
 
+/* Diagnostics (no counterpart in the paper): the rollout kernels decide most actions of a network policy
+ * from an estimate of logit[1] - logit[0] built on the special-function unit's tanh, and compute the defined
+ * logits only where the estimate lies within its error bound of zero. The bound rests on that tanh's
+ * distance from the defined ones, at most 8.0e-6; this measures it over all 2^32 float bit patterns. out
+ * DEVICE [3] uint64, caller zeroes, in units of 1e-12: out[0] largest distance from the tanh of
+ * CP_ARITH_EXACT, out[1] from that of CP_ARITH_CONTRACTED; out[2] += patterns for which one of the three is
+ * NaN and another is not (must stay 0). */
+int cp_selftest_screen(uint64_t *out);
+
 /* Calibration of the roofline denominators (a measurement aid; the paper has no counterpart):
  * enqueue one launch in which every thread executes
  * iters rounds of eight independent chains of one instruction kind — 0: float32 fused

@@ -681,6 +681,12 @@ int cp_selftest_pair(uint64_t count, uint32_t seed, uint64_t *out) {
     return e == cudaSuccess ? CP_OK : cuda_fail(e, "self-test launch");
 }
 
+int cp_selftest_screen(uint64_t *out) {
+    if (!out || !is_aligned(out, 8)) return fail(CP_EINVAL, "out is NULL or misaligned");
+    cudaError_t e = cp::launch_screen_selftest(reinterpret_cast<unsigned long long *>(out), tl_stream);
+    return e == cudaSuccess ? CP_OK : cuda_fail(e, "self-test launch");
+}
+
 int cp_selftest_tame_div(uint32_t den_step, uint64_t *out) {
     if (!out || !is_aligned(out, 8)) return fail(CP_EINVAL, "out is NULL or misaligned");
     if (den_step == 0) return fail(CP_EINVAL, "den_step must be >= 1");

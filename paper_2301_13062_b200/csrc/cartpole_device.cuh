@@ -511,14 +511,6 @@ struct LinearW {
     float w[2][4];
     float b[2];
 };
-template <int H>
-struct MlpWT {  // 4 -> H (tanh) -> 2
-    float w1[H][4];
-    float b1[H];
-    float w2[2][H];
-    float b2[2];
-};
-using MlpW = MlpWT<16>;
 
 // Returns the action in sign-bit form (0x80000000 = push right).
 __device__ __forceinline__ uint32_t linear_action(const LinearW &p, const State &z) {
@@ -534,8 +526,6 @@ __device__ __forceinline__ uint32_t linear_action(const LinearW &p, const State 
     return (l1 > l0) ? 0x80000000u : 0u;
 }
 
-// Hidden activations are consumed as they are produced (two running logits), so no array of
-// H values is ever live; every weight is an immediate operand from the launch parameters.
 // tanh for the contracted-arithmetic variant: 1 - 2 / (exp(2x) + 1) with the hardware exp2 and
 // reciprocal approximations (five instructions instead of the library routine's ~18). Small
 // arguments lose RELATIVE accuracy to the cancellation in 1 - (...), which a policy does not
@@ -614,56 +604,6 @@ __device__ __forceinline__ f32x2 tanh_contracted_pair(f32x2 x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d0));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d1));
     return fma2(splat2(-2.0f), pack2(r0, r1), splat2(1.0f));
-}
-
-template <int H, bool FAST_TANH = false>
-__device__ __forceinline__ uint32_t mlp_action(const MlpWT<H> &p, const State &z) {
-    float l0 = p.b2[0], l1 = p.b2[1];
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        float acc = p.b1[j];
-        acc = __fmaf_rn(p.w1[j][0], z.x, acc);
-        acc = __fmaf_rn(p.w1[j][1], z.xd, acc);
-        acc = __fmaf_rn(p.w1[j][2], z.th, acc);
-        acc = __fmaf_rn(p.w1[j][3], z.thd, acc);
-        float h = FAST_TANH ? tanh_contracted(acc) : tanh_canonical(acc);
-        l0 = __fmaf_rn(p.w2[0][j], h, l0);
-        l1 = __fmaf_rn(p.w2[1][j], h, l1);
-    }
-    return (l1 > l0) ? 0x80000000u : 0u;
-}
-
-// Two hidden layers, 4 -> 16 (tanh) -> 16 (tanh) -> 2. The sixteen first-layer activations stay
-// in registers; second-layer units are consumed by the two logit chains as they are produced
-// (ascending unit order, the chains start from the biases: the order of the definition).
-struct MlpDeepW {
-    float w1[16][4], b1[16];
-    float w2[16][16], b2[16];
-    float w3[2][16], b3[2];
-};
-template <bool FAST_TANH = false>
-__device__ __forceinline__ uint32_t mlp_deep_action(const MlpDeepW &p, const State &z) {
-    float h1[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float acc = p.b1[j];
-        acc = __fmaf_rn(p.w1[j][0], z.x, acc);
-        acc = __fmaf_rn(p.w1[j][1], z.xd, acc);
-        acc = __fmaf_rn(p.w1[j][2], z.th, acc);
-        acc = __fmaf_rn(p.w1[j][3], z.thd, acc);
-        h1[j] = FAST_TANH ? tanh_contracted(acc) : tanh_canonical(acc);
-    }
-    float l0 = p.b3[0], l1 = p.b3[1];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        float acc = p.b2[k];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc = __fmaf_rn(p.w2[k][j], h1[j], acc);
-        const float h2 = FAST_TANH ? tanh_contracted(acc) : tanh_canonical(acc);
-        l0 = __fmaf_rn(p.w3[0][k], h2, l0);
-        l1 = __fmaf_rn(p.w3[1][k], h2, l1);
-    }
-    return (l1 > l0) ? 0x80000000u : 0u;
 }
 
 }  // namespace cp

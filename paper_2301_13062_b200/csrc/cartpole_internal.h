@@ -23,6 +23,8 @@ struct StepParams {
     uint32_t max_steps;     // episode step limit (needs ep_len), 0 = none
 };
 
+constexpr int kMaxPolicyFloats = 900;
+
 // Parameters of one rollout launch. Weights travel in the launch parameters
 // (constant bank), so every policy FMA reads its weight as an immediate operand.
 struct RolloutParams {
@@ -45,9 +47,12 @@ struct RolloutParams {
     const uint32_t *action_bits_in;  // [T][words] supplied actions or nullptr
     const float *start_in;           // [T][4][n] supplied start states or nullptr
     const float *env_weights;        // [10][n] one linear policy per env (policy kind 6) or nullptr
+    // the network policies' estimate of l1 - l0 (policy_screen.cuh): its constant term, and its largest
+    // distance from the logits' difference
+    float screen_base, screen_bound;
     // largest policy: the network with 64 hidden units, 7*64 + 2 floats; twice the room, because the
-    // deferred-restart kernel reads every shared weight as a (w, w) pair
-    float w[900];
+    // deferred-restart kernel reads shared weights as (w, w) pairs
+    alignas(8) float w[kMaxPolicyFloats];
 };
 
 struct LaunchTuning {
@@ -108,6 +113,12 @@ cudaError_t launch_tanh_accuracy(uint32_t lo_bits, uint32_t hi_bits, unsigned lo
 cudaError_t launch_pipe_rate(int kind, const float *seed, float *sink, int iters, int *threads, cudaStream_t s);
 cudaError_t launch_arith_selftest(unsigned long long *out, cudaStream_t s);
 cudaError_t launch_pair_selftest(unsigned long long count, uint32_t seed, unsigned long long *out, cudaStream_t s);
+cudaError_t launch_screen_selftest(unsigned long long *out, cudaStream_t s);
+// A network's weights in RolloutParams::w rearranged for its estimate, for two environments per thread or
+// for one, with the bound the estimate needs (policy_screen.cu).
+void screen_pairs(RolloutParams &p, int policy);
+void screen_units(RolloutParams &p, int policy);
+void screen_bound(RolloutParams &p, int policy);  // the bound alone, weights as the caller gave them
 cudaError_t launch_tame_div_selftest(uint32_t den_step, unsigned long long *out, cudaStream_t s);
 
 // The per-op ladder. Workspace layout is private to ladder_kernels.cu.

@@ -1,0 +1,187 @@
+// The shared network policies decide an action by the larger of two logits, and the logits
+// themselves go nowhere. So every kernel first takes an estimate of l1 - l0 that is cheap and has
+// a proven bound on its distance from the defined logits' difference: where it is larger than the
+// bound, its sign is the action. Only where it is not are the defined logits computed, in their
+// defined order, by the environment that needs them. The actions are those of the definition,
+// always; what changes is how many operations most of them take.
+//
+//   estimate = (b1 - b0) + sum_j (w1[j] - w0[j]) * h~_j     h~_j: the special-function unit's tanh
+//
+// One result of that unit per hidden unit instead of two, no polynomial beside it, one
+// multiply-add instead of two, and no order to keep. The bound (screen_policy, in policy_screen.cu)
+// grows with the weights and with kTanhScreenError; with the weight distributions of inputs.py it
+// sends one to two environments in 10,000 steps to the defined logits, at most one in 1,000.
+//
+// NaN anywhere makes the comparison with the bound fail, which sends the environment to the defined
+// logits; so do weights beyond the range the bound was derived for (its bound is infinite then).
+#pragma once
+#include "cartpole_device.cuh"
+#include "cartpole_internal.h"
+
+namespace cp {
+
+// tanh by the special-function unit, one instruction. Its distance from either arithmetic's tanh is at
+// most kTanhScreenError over every float32 (measured: 7.987e-6 for both, cp_selftest_screen).
+constexpr double kTanhScreenError = 8.0e-6;
+__device__ __forceinline__ float tanh_screen(float x) {
+    float r;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ f32x2 tanh_screen2(f32x2 x) {
+    float a, b;
+    unpack2(x, a, b);
+    return pack2(tanh_screen(a), tanh_screen(b));
+}
+
+// The shared tanh networks: 2 (4-16-2), 4 (4-32-2), 5 (4-64-2), 7 (4-16-16-2).
+__host__ __device__ constexpr bool is_network(int policy) { return policy == 2 || policy == 4 || policy == 5 || policy == 7; }
+
+template <int NET>
+struct NetShape {
+    static constexpr int H = NET == 4 ? 32 : NET == 5 ? 64 : 16;
+    static constexpr bool kDeep = NET == 7;
+    // floats before the second hidden layer, and before the logits (W[2][H], b[2]), as the caller gives them
+    static constexpr int kSecond = 5 * H;
+    static constexpr int kLogits = kSecond + (kDeep ? H * (H + 1) : 0);
+    static constexpr int kCount = kLogits + 2 * H + 2;
+    // RolloutParams::w for two environments per thread (screen_pairs): every hidden layer's weight and
+    // every w1[j] - w0[j] as a pair, then the logits' weights
+    static constexpr int kPairSteps = 2 * kLogits, kPairLogits = kPairSteps + 2 * H;
+    // and for one (screen_units): the caller's weights, the first layer again with the weights of units
+    // 2q and 2q + 1 side by side (input 0, .., input 3, bias), then w1[j] - w0[j]
+    static constexpr int kUnitFirst = kCount, kUnitSteps = kUnitFirst + 5 * H;
+    static_assert(kPairLogits + 2 * H + 2 <= kMaxPolicyFloats && kUnitSteps + H <= kMaxPolicyFloats, "RolloutParams::w holds either layout");
+    static_assert(kUnitFirst % 2 == 0 && kUnitSteps % 2 == 0, "pairs are read as such");
+};
+
+// The action by the defined logits: every sum left to right from its bias. w: the hidden layers' weights,
+// STRIDE floats apart; logits: W[2][H], b[2]. Two units at a time, whose tanhs share their instructions;
+// few environments come here, so the code is kept short: loops over the units, not unrolled.
+template <int NET, bool CONTRACT, int STRIDE>
+__device__ __forceinline__ uint32_t defined_action(const float *w, const float *logits, const State &z) {
+    using S = NetShape<NET>;
+    constexpr int H = S::H;
+    auto first = [&](int j) {
+        float acc = w[(4 * H + j) * STRIDE];
+        acc = __fmaf_rn(w[(4 * j + 0) * STRIDE], z.x, acc);
+        acc = __fmaf_rn(w[(4 * j + 1) * STRIDE], z.xd, acc);
+        acc = __fmaf_rn(w[(4 * j + 2) * STRIDE], z.th, acc);
+        return __fmaf_rn(w[(4 * j + 3) * STRIDE], z.thd, acc);
+    };
+    auto tanh2 = [](float a, float b, float &ha, float &hb) {
+        const f32x2 v = pack2(a, b);
+        unpack2(CONTRACT ? tanh_contracted_pair(v) : tanh_pair(v), ha, hb);
+    };
+    float l0 = logits[2 * H], l1 = logits[2 * H + 1];
+    auto logit_terms = [&](int j, float a, float b) {  // of units j and j + 1
+        float ha, hb;
+        tanh2(a, b, ha, hb);
+        l0 = __fmaf_rn(logits[j], ha, l0);
+        l1 = __fmaf_rn(logits[H + j], ha, l1);
+        l0 = __fmaf_rn(logits[j + 1], hb, l0);
+        l1 = __fmaf_rn(logits[H + j + 1], hb, l1);
+    };
+    if constexpr (S::kDeep) {
+        const float *w2 = w + S::kSecond * STRIDE, *b2 = w2 + H * H * STRIDE;
+        float h1[H];
+#pragma unroll
+        for (int j = 0; j < H; j += 2) tanh2(first(j), first(j + 1), h1[j], h1[j + 1]);
+#pragma unroll 1
+        for (int k = 0; k < H; k += 2) {
+            float a = b2[k * STRIDE], b = b2[(k + 1) * STRIDE];
+#pragma unroll
+            for (int j = 0; j < H; ++j) {
+                a = __fmaf_rn(w2[(H * k + j) * STRIDE], h1[j], a);
+                b = __fmaf_rn(w2[(H * (k + 1) + j) * STRIDE], h1[j], b);
+            }
+            logit_terms(k, a, b);
+        }
+    } else {
+#pragma unroll 2
+        for (int j = 0; j < H; j += 2) logit_terms(j, first(j), first(j + 1));
+    }
+    return (l1 > l0) ? 0x80000000u : 0u;
+}
+
+// Estimates for the two environments of a thread, from the pairs of screen_pairs.
+template <int NET>
+__device__ __forceinline__ f32x2 screen_estimate_pair(const f32x2 *w, f32x2 base, const StatePair &z) {
+    using S = NetShape<NET>;
+    constexpr int H = S::H;
+    const f32x2 *steps = w + S::kLogits;
+    auto unit = [&](int j) {
+        f32x2 acc = w[4 * H + j];
+        acc = fma2(w[4 * j + 0], z.x, acc);
+        acc = fma2(w[4 * j + 1], z.xd, acc);
+        acc = fma2(w[4 * j + 2], z.th, acc);
+        acc = fma2(w[4 * j + 3], z.thd, acc);
+        return tanh_screen2(acc);
+    };
+    f32x2 est = base;
+    if constexpr (S::kDeep) {
+        const f32x2 *w2 = w + S::kSecond, *b2 = w2 + H * H;
+        f32x2 h1[H];
+#pragma unroll
+        for (int j = 0; j < H; ++j) h1[j] = unit(j);
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            f32x2 acc = b2[k];
+#pragma unroll
+            for (int j = 0; j < H; ++j) acc = fma2(w2[H * k + j], h1[j], acc);
+            est = fma2(steps[k], tanh_screen2(acc), est);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < H; ++j) est = fma2(steps[j], unit(j), est);
+    }
+    return est;
+}
+
+// Estimate for one environment, two hidden units per packed operation, from the layout of screen_units.
+template <int NET>
+__device__ __forceinline__ float screen_estimate(const float *w, float base, const State &z) {
+    using S = NetShape<NET>;
+    constexpr int H = S::H;
+    const f32x2 *first = reinterpret_cast<const f32x2 *>(w + S::kUnitFirst);
+    const f32x2 x = splat2(z.x), xd = splat2(z.xd), th = splat2(z.th), thd = splat2(z.thd);
+    auto units = [&](int q) {  // 2q and 2q + 1
+        f32x2 acc = first[5 * q + 4];
+        acc = fma2(first[5 * q + 0], x, acc);
+        acc = fma2(first[5 * q + 1], xd, acc);
+        acc = fma2(first[5 * q + 2], th, acc);
+        acc = fma2(first[5 * q + 3], thd, acc);
+        return tanh_screen2(acc);
+    };
+    float lo, hi;
+    if constexpr (S::kDeep) {
+        const f32x2 *w2 = reinterpret_cast<const f32x2 *>(w + S::kSecond);
+        const float *b2 = w + S::kSecond + H * H, *steps = w + S::kUnitSteps;
+        f32x2 h1[H / 2];
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) h1[q] = units(q);
+        float est = base;
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            f32x2 acc = pack2(b2[k], 0.0f);
+#pragma unroll
+            for (int q = 0; q < H / 2; ++q) acc = fma2(w2[H / 2 * k + q], h1[q], acc);
+            unpack2(acc, lo, hi);
+            est = __fmaf_rn(steps[k], tanh_screen(__fadd_rn(lo, hi)), est);
+        }
+        return est;
+    } else {
+        const f32x2 *steps = reinterpret_cast<const f32x2 *>(w + S::kUnitSteps);
+        f32x2 est = pack2(base, 0.0f);
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) est = fma2(steps[q], units(q), est);
+        unpack2(est, lo, hi);
+        return __fadd_rn(lo, hi);
+    }
+}
+
+// Does the estimate decide? (false for NaN, and for every estimate where the bound is infinite)
+__device__ __forceinline__ bool screen_decides(float estimate, float bound) { return fabsf(estimate) > bound; }
+__device__ __forceinline__ uint32_t screen_action(float estimate) { return estimate > 0.0f ? 0x80000000u : 0u; }
+
+}  // namespace cp

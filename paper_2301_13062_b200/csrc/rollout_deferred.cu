@@ -19,9 +19,9 @@ bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams) 
 cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracted, cudaStream_t s) {
     // measured on 1,048,576 x 500 at K = 3 / 4 / 6 / 8: hashed actions (22-step episodes) 0.996 /
     // 0.987 / 0.965 / 0.987 ms, the linear policy (80-step episodes) 0.945 / 0.924 / 0.907 / 0.908 ms
-    // The 4-16-2 network of config 5 ends its episodes after 9-10 steps, so waiting costs more and
-    // a restart pass less (next to a 600-instruction trip): 16,777,216 x 200 takes 38.4 / 38.0 /
-    // 41.5 ms at K = 2 / 3 / 4 (the general kernel: 43.2 ms).
+    // The network policies' trips are long, so waiting costs more and a restart pass less. 4-16-2,
+    // 4,194,304 x 200 at K = 2 / 3 / 4: 4,842 / 4,915 / 5,170 us for a policy of 20-step episodes, 4,438 / 4,438 /
+    // 4,559 for one of 9-step episodes, 4,174 / 4,199 / 4,268 and 4,288 / 4,249 / 4,371 for ones of 200 and 16.
     // Short launches (chunked rollouts of a batch in place) pay the ragged end on every call, so
     // the passes come closer together (us per step of 1,048,576 envs at K = 2 / 4 / 6, hashed
     // actions: T = 16: 3.39 / 3.65 / 4.03, T = 64: 2.41 / 2.38 / 2.45, T = 256: 2.17 / 2.02 / 2.00;
@@ -34,14 +34,14 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
     // kernel, by counting the waiting slots every second trip or after every pass, cost 6 to 14 % of
     // every launch.
     const int by_length = p.T < 48u ? 2 : p.T < 192u ? 4 : 6;
-    const int k = g_tuning.rollout_defer > 0 ? g_tuning.rollout_defer : (is_network(policy) ? 3 : by_length);
+    const int k = g_tuning.rollout_defer > 0 ? g_tuning.rollout_defer : (policy == 2 ? 2 : is_network(policy) ? 3 : by_length);
     // the action hash folds the time's upper half into the lower one: nothing to do below 2^16
     const bool short_times = (uint64_t)p.t0 + p.T <= 65536u;
-    if (policy == 1 || is_network(policy)) {  // every shared weight twice: one packed operand for both slots
-        const int count = policy == 1 ? 10 : policy == 2 ? 114 : policy == 4 ? 226 : policy == 5 ? 450 : 386;
-        static_assert(sizeof(p.w) >= 2 * 450 * sizeof(float), "the launch parameters hold the largest policy twice");
-        for (int i = count - 1; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
-    }
+    // shared weights twice: one packed operand for both slots
+    if (policy == 1)
+        for (int i = 9; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
+    else if (is_network(policy))
+        screen_pairs(p, policy);
     if (p.action_bits_in || p.start_in) return launch_rollout_deferred_data(p, p.action_bits_in ? 3 : policy, k, contracted, s);
     switch (policy) {
         case 0: return short_times ? launch_limit<0, true>(p, k, contracted, s) : launch_limit<0, false>(p, k, contracted, s);

@@ -38,6 +38,7 @@
 
 #include "cartpole_device.cuh"
 #include "cartpole_internal.h"
+#include "policy_screen.cuh"
 
 namespace cp {
 
@@ -67,61 +68,35 @@ __device__ __forceinline__ void linear_action_pair(const f32x2 *w, const StatePa
     l1 = fma2(w[7], z.thd, l1);
     argmax_pair(l0, l1, sb0, sb1);
 }
-template <int H, bool CONTRACT>
-__device__ __forceinline__ void mlp_action_pair(const f32x2 *w, const StatePair &z, uint32_t &sb0, uint32_t &sb1) {
-    // w: W1[H][4], b1[H], W2[2][H], b2[2], as pairs
-    const f32x2 *w1 = w, *b1 = w + 4 * H, *w2 = w + 5 * H, *b2 = w + 7 * H;
-    f32x2 l0 = b2[0], l1 = b2[1];
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        f32x2 acc = b1[j];
-        acc = fma2(w1[4 * j + 0], z.x, acc);
-        acc = fma2(w1[4 * j + 1], z.xd, acc);
-        acc = fma2(w1[4 * j + 2], z.th, acc);
-        acc = fma2(w1[4 * j + 3], z.thd, acc);
-        const f32x2 h = CONTRACT ? tanh_contracted_pair(acc) : tanh_pair(acc);
-        l0 = fma2(w2[j], h, l0);
-        l1 = fma2(w2[H + j], h, l1);
+// The networks: the sign of the estimate where it decides, the defined logits where it does not (a
+// waiting slot's state is nobody's, so it never asks for them). What bounds a 4-16-2 trip now: 256 cycles of
+// the special-function pipe (32 tanhs), about 250 of the float32 pipe (80 multiply-adds of the estimate and the
+// 37 packed operations of the step), of 350 measured; with two results and 13 packed operations per
+// tanh it was 512 and 590 of 800 (16,777,216 x 40: 8.59 -> 4.35 ms, contracted 5.48 -> 3.68).
+template <int NET, bool CONTRACT>
+__device__ __forceinline__ void network_action_pair(const RolloutParams &p, const bool (&act)[2], const StatePair &z,
+                                                    uint32_t &sb0, uint32_t &sb1) {
+    using S = NetShape<NET>;
+    float e[2];
+    unpack2(screen_estimate_pair<NET>(reinterpret_cast<const f32x2 *>(p.w), splat2(p.screen_base), z), e[0], e[1]);
+    sb0 = screen_action(e[0]);
+    sb1 = screen_action(e[1]);
+    const bool open0 = act[0] && !screen_decides(e[0], p.screen_bound), open1 = act[1] && !screen_decides(e[1], p.screen_bound);
+    if (open0 || open1) {
+        State a, b;
+        unpack_states(z, a, b);
+#pragma unroll 1
+        for (int j = open0 ? 0 : 1; j < (open1 ? 2 : 1); ++j) {
+            const uint32_t sb = defined_action<NET, CONTRACT, 2>(p.w, p.w + S::kPairLogits, j ? b : a);
+            (j ? sb1 : sb0) = sb;
+        }
     }
-    argmax_pair(l0, l1, sb0, sb1);
 }
 
-// 4-16-16-2 (MlpDeepW as pairs: W1[16][4], b1[16], W2[16][16], b2[16], W3[2][16], b3[2]): the
-// sixteen first-layer activations of both slots stay in registers, second-layer units feed the
-// logit chains as they are produced — mlp_deep_action's order, half by half.
-template <bool CONTRACT>
-__device__ __forceinline__ void mlp_deep_action_pair(const f32x2 *w, const StatePair &z, uint32_t &sb0, uint32_t &sb1) {
-    const f32x2 *w1 = w, *b1 = w + 64, *w2 = w + 80, *b2 = w + 336, *w3 = w + 352, *b3 = w + 384;
-    f32x2 h1[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        f32x2 acc = b1[j];
-        acc = fma2(w1[4 * j + 0], z.x, acc);
-        acc = fma2(w1[4 * j + 1], z.xd, acc);
-        acc = fma2(w1[4 * j + 2], z.th, acc);
-        acc = fma2(w1[4 * j + 3], z.thd, acc);
-        h1[j] = CONTRACT ? tanh_contracted_pair(acc) : tanh_pair(acc);
-    }
-    f32x2 l0 = b3[0], l1 = b3[1];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        f32x2 acc = b2[k];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc = fma2(w2[16 * k + j], h1[j], acc);
-        const f32x2 h2 = CONTRACT ? tanh_contracted_pair(acc) : tanh_pair(acc);
-        l0 = fma2(w3[k], h2, l0);
-        l1 = fma2(w3[16 + k], h2, l1);
-    }
-    argmax_pair(l0, l1, sb0, sb1);
-}
-
-// The shared tanh networks: 2 (4-16-2), 4 (4-32-2), 5 (4-64-2), 7 (4-16-16-2).
-__host__ __device__ constexpr bool is_network(int policy) { return policy == 2 || policy == 4 || policy == 5 || policy == 7; }
 // The networks wider or deeper than 4-16-2 (4, 5, 7): built for the plain call only — no step limit,
-// no per-step outputs, default trip spacing (a kernel of theirs takes up to a minute to compile).
-// Against the general kernel with one environment per thread, 16,777,216 x 200: 4-32-2 77.3 ->
-// 70.0 ms, 4-64-2 145.1 -> 135.3 ms, 4-16-16-2 94.9 -> 88.7 ms (contracted arithmetic 54.4 ->
-// 51.0, 103.8 -> 98.5, 72.4 -> 59.0 ms).
+// no per-step outputs, default trip spacing. With the estimate (policy_screen.cuh) against the defined logits on
+// every step, 4,194,304 x 40: 4-32-2 3.59 -> 1.58 ms, 4-64-2 7.99 -> 3.41, 4-16-16-2 4.95 -> 2.54 (contracted
+// arithmetic 3.03 -> 2.26).
 __host__ __device__ constexpr bool is_wide_network(int policy) { return is_network(policy) && policy != 2; }
 
 // The done bit plane of a launch that sets its bits by atomic OR has to be zeroed first.
@@ -149,14 +124,8 @@ __device__ __forceinline__ void deferred_actions(const RolloutParams &p, const F
         if (act[1]) window[1] <<= 1;
     } else if (POLICY == 1) {
         linear_action_pair(pairs, zz, sb0, sb1);
-    } else if (POLICY == 2) {
-        mlp_action_pair<16, CONTRACT>(pairs, zz, sb0, sb1);
-    } else if (POLICY == 4) {
-        mlp_action_pair<32, CONTRACT>(pairs, zz, sb0, sb1);
-    } else if (POLICY == 5) {
-        mlp_action_pair<64, CONTRACT>(pairs, zz, sb0, sb1);
-    } else if (POLICY == 7) {
-        mlp_deep_action_pair<CONTRACT>(pairs, zz, sb0, sb1);
+    } else if constexpr (is_network(POLICY)) {
+        network_action_pair<POLICY, CONTRACT>(p, act, zz, sb0, sb1);
     } else {
         State a, b;
         unpack_states(zz, a, b);
@@ -215,9 +184,9 @@ constexpr int kMany = 40, kEnough = 24, kFew = 16;  // of the warp's 64
 // that are otherwise re-materialised every trip (1,048,576 x 500: 1.032 -> 0.988 ms; with the
 // reward plane and done bits, 4,194,304 x 100: 0.936 -> 0.828 ms; forcing 3 or 4 CTAs per SM
 // measured 1.04 / 1.01 and 0.87 / 0.93 ms).
-// (The network policies are the exception: their hidden units are latency — exp2 and
-// reciprocal on the special-function pipe — that only more resident warps hide: 16,777,216 x
-// 200 takes 53.1 / 41.1 / 39.9 / 39.4 / 40.8 ms at 1 / 2 / 3 / 4 / 5 CTAs per SM.)
+// (The network policies are the exception: their hidden units are latency — tanh on the
+// special-function pipe — that only more resident warps hide: 4,194,304 x 200, 4-16-2, at 3 / 4 / 5 CTAs per
+// SM 4,949 / 4,954 / 4,910 us, with the reward plane and done bits 5,639 / 5,657 / 5,859.)
 template <int POLICY, int K, bool SHORT, bool LIMIT, bool RD, bool CONTRACT, bool START_IN = false>
 __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || START_IN ? 3 : 1) rollout_deferred_kernel(const __grid_constant__ RolloutParams p) {
     constexpr bool GIVEN = POLICY == 3;
@@ -515,9 +484,11 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
             after_step(tail, 0, d0);
             after_step(tail, 1, d1);
         };
-        // The trips between two restart passes: K, or fewer where many slots wait (a network policy's trip is 600 instructions or more:
-        // its trips stay a loop).
-        constexpr int kUnroll = is_network(POLICY) ? 1 : K;
+        // The trips between two restart passes: K, or fewer where many slots wait. The 4-16-2 network's are
+        // unrolled up to three (4,194,304 x 200 at K = 2, 3, 4: 4,954 -> 4,842, 4,992 -> 4,915, 5,170 -> 5,569
+        // us), the larger networks' stay a loop (1,048,576 x 100, unrolled: 4-32-2 1,019 -> 1,147, 4-64-2 1,979 ->
+        // 2,484, 4-16-16-2 1,528 -> 2,803).
+        constexpr int kUnroll = !is_network(POLICY) || (POLICY == 2 && K <= 3) ? K : 1;
         auto trip_block = [&](auto tail) {  // returns the trips made
             int made = K;
             if (START_IN && (wide || early)) {

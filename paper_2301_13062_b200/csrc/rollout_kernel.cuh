@@ -29,6 +29,7 @@
 #pragma once
 #include "cartpole_device.cuh"
 #include "cartpole_internal.h"
+#include "policy_screen.cuh"
 
 namespace cp {
 
@@ -43,14 +44,12 @@ __device__ __forceinline__ uint32_t policy_signbit(const RolloutParams &p, const
         return action_signbit_folded(ka, folded_t);
     } else if (POLICY == 1) {
         return linear_action(*reinterpret_cast<const LinearW *>(p.w), z);
-    } else if (POLICY == 2) {
-        return mlp_action<16, CONTRACT>(*reinterpret_cast<const MlpWT<16> *>(p.w), z);
-    } else if (POLICY == 4) {
-        return mlp_action<32, CONTRACT>(*reinterpret_cast<const MlpWT<32> *>(p.w), z);
-    } else if (POLICY == 7) {
-        return mlp_deep_action<CONTRACT>(*reinterpret_cast<const MlpDeepW *>(p.w), z);
+    } else if constexpr (is_network(POLICY)) {
+        const float estimate = screen_estimate<POLICY>(p.w, p.screen_base, z);
+        if (screen_decides(estimate, p.screen_bound)) return screen_action(estimate);
+        return defined_action<POLICY, CONTRACT, 1>(p.w, p.w + NetShape<POLICY>::kLogits, z);
     } else {
-        return mlp_action<64, CONTRACT>(*reinterpret_cast<const MlpWT<64> *>(p.w), z);
+        return 0u;  // 3 and 6: the kernel has the action itself
     }
 }
 
@@ -505,6 +504,7 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
 
 template <bool CONTRACT>
 cudaError_t launch_networks_arith(RolloutParams &p, int policy, int mode, int shape, cudaStream_t s) {
+    screen_units(p, policy);
     switch (policy) {
         case 2: return launch_mode<2, CONTRACT>(p, mode, shape, s);
         case 4: return launch_mode<4, CONTRACT>(p, mode, shape, s);

@@ -23,17 +23,9 @@
 #pragma once
 #include "cartpole_device.cuh"
 #include "cartpole_internal.h"
+#include "policy_screen.cuh"
 
 namespace cp {
-
-template <int NET>
-struct NetShape {
-    static constexpr int H = NET == 4 ? 32 : NET == 5 ? 64 : 16;
-    static constexpr bool kDeep = NET == 7;
-    // floats before the second hidden layer, and before the logits (W[2][H], b[2])
-    static constexpr int kSecond = 5 * H;
-    static constexpr int kLogits = kSecond + (kDeep ? H * (H + 1) : 0);
-};
 
 // Keeps the compiler from reading a lane's weight again in every step (the launch parameters are
 // constant memory, which serves one address per warp and access).
