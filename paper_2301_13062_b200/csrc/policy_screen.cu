@@ -18,20 +18,21 @@ namespace {
 //    (n + 1) u (|b| + sum |w|), the operands differ by E1, tanh does not stretch distances, and the
 //    definition's own tanh misses the real one by less than E1: E2_k = E1 sum_j |w2[k][j]| +
 //    2 (n + 2) u (|b2[k]| + sum_j |w2[k][j]|) + 2 E1.
-//  * The logits of the definition miss the exact sums over h_j by (H + 1) u (|b_i| + sum_j |w_i[j]|)
-//    each; the estimate rounds v_j and b1 - b0 once, and its sum by (H + 2) u (|b1 - b0| + sum |v_j|).
-// Estimate and l1 - l0 then differ by at most
-//    sum_j E_j |v_j| + (H + 4) u (|b1 - b0| + sum |v_j|) + (H + 2) u sum_i (|b_i| + sum_j |w_i[j]|);
-// 1/16 more for the second-order terms and this computation itself, and 1e-37 for results too small
+//  * A sum over h_j rounds each of its partial sums once. Those of a defined logit, left to right, are at
+//    most |b_i| + |w_i[0]| + .. + |w_i[k]|, so the logit misses its exact sum by u times the sum of these over k.
+//  * The estimate's order depends on the kernel; `rounds` says how many roundings a term goes through at
+//    most, each of a partial sum of at most |b1 - b0| + sum |v_j|, two more for v_j and b1 - b0 themselves.
+// Estimate and l1 - l0 then differ by at most the sum of all that and sum_j E_j |v_j|; 1/16 more for
+// the second-order terms and this computation itself, and 1e-37 for results too small
 // to be normal numbers. Weights of 1e30 and more in sum (or not finite) could overflow in the estimate where
 // they do not in the logits: their bound is infinite.
 template <int NET>
-void screen(RolloutParams &p, float *steps) {
+void screen(RolloutParams &p, float *steps, int rounds) {
     using S = NetShape<NET>;
     constexpr int H = S::H;
     const double u = std::ldexp(1.0, -24), e1 = kTanhScreenError;
     const float *logits = p.w + S::kLogits;
-    double moved = 0.0, total = std::fabs((double)logits[2 * H]) + std::fabs((double)logits[2 * H + 1]);
+    double moved = 0.0, total = std::fabs((double)logits[2 * H]) + std::fabs((double)logits[2 * H + 1]), partial = 0.0;
     const double base = (double)logits[2 * H + 1] - (double)logits[2 * H];
     double span = std::fabs(base);
     for (int j = 0; j < H; ++j) {
@@ -46,8 +47,9 @@ void screen(RolloutParams &p, float *steps) {
         moved += e * std::fabs(v);
         span += std::fabs(v);
         total += std::fabs((double)logits[j]) + std::fabs((double)logits[H + j]);
+        partial += total;
     }
-    const double bound = 1.0625 * (moved + (H + 4) * u * span + (H + 2) * u * total) + 1e-37;
+    const double bound = 1.0625 * (moved + (rounds + 2) * u * span + u * partial) + 1e-37;
     p.screen_base = (float)base;
     p.screen_bound = bound < 1e30 && total < 1e30 ? std::nextafter((float)bound, INFINITY) : INFINITY;
 }
@@ -57,7 +59,7 @@ void pairs(RolloutParams &p) {
     using S = NetShape<NET>;
     constexpr int H = S::H;
     float steps[H];
-    screen<NET>(p, steps);
+    screen<NET>(p, steps, H);
     std::memmove(p.w + S::kPairLogits, p.w + S::kLogits, (2 * H + 2) * sizeof(float));
     for (int i = S::kLogits - 1; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
     for (int j = 0; j < H; ++j) p.w[S::kPairSteps + 2 * j] = p.w[S::kPairSteps + 2 * j + 1] = steps[j];
@@ -67,15 +69,15 @@ template <int NET>
 void units(RolloutParams &p) {
     using S = NetShape<NET>;
     constexpr int H = S::H;
-    screen<NET>(p, p.w + S::kUnitSteps);
+    screen<NET>(p, p.w + S::kUnitSteps, S::kDeep ? H : H / 2 + 1);
     for (int j = 0; j < H; ++j)
         for (int i = 0; i < 5; ++i) p.w[S::kUnitFirst + 10 * (j / 2) + 2 * i + j % 2] = p.w[i < 4 ? 4 * j + i : 4 * H + j];
 }
 
 template <int NET>
-void bound_alone(RolloutParams &p) {
+void bound_alone(RolloutParams &p) {  // four or eight lanes: H / 4 or H / 8 terms, two or three shuffles, the base
     float steps[NetShape<NET>::H];
-    screen<NET>(p, steps);
+    screen<NET>(p, steps, NetShape<NET>::H / 4 + 3);
 }
 
 }  // namespace

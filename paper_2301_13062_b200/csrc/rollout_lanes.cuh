@@ -3,24 +3,34 @@
 // the chip.
 //
 // One lane per environment evaluates the hidden units one after another; with a few warps per
-// scheduler nothing hides that, and a step of a 4-64-2 network takes 2,250 cycles although its
-// longest dependency chain is a fifth of that. Here lane = g * E + e: the G lanes g of environment e
-// (E = 32 / G environments per warp)
+// scheduler nothing hides that. Here lane = g * E + e: the G lanes g of environment e (E = 32 / G
+// environments per warp)
 //   * all hold the state and all step it (the same instructions for every lane: no cost);
-//   * evaluate H / G hidden units each, side by side, their weights in registers;
-//   * exchange the activations through a row of shared memory per environment, and all run the two
-//     logit chains (whose order is part of the definition; they are what bounds the step now).
-// Every operation is the scalar one of mlp_action / mlp_deep_action on the same operands in the same
-// order, so the action has the same bits. (Two units or both logits per packed operation halve the
-// issue slots but measured slower: latency is what is paid here, and a packed operation's is longer.)
+//   * evaluate H / G hidden units each, side by side, their weights in registers, and sum their part of the
+//     estimate of l1 - l0 (policy_screen.cuh); a deep network's first activations go through a row of
+//     shared memory per environment;
+//   * add the parts pairwise by shuffles. Where a warp has a sum that does not decide, its lanes compute
+//     the defined logits together (lanes_defined_action): one lane by itself takes several thousand cycles,
+//     and one such environment after another lengthened launches by up to a fifth (4-64-2, 4,096 x 500, twelve
+//     policies: 139 .. 162 us against 133 .. 143). The deep network's lanes go by themselves: together they
+//     cost every launch 16 us for the few that gain (133 .. 154 against 148 .. 156).
+// With the defined logits in every step, whose order is a chain of one multiply-add per hidden unit, the 4-64-2
+// network's step took 1,190 cycles on 4,096 environments; it takes 510 (500 steps: 303 -> 133 us).
 // The start state an environment would continue from is hashed on every step ahead of the network,
-// by four lanes, one component each: that work fills issue slots the chains leave empty, and a
+// by four lanes, one component each: that work fills issue slots the network leaves empty, and a
 // finished environment just takes it.
+//
+// One warp per scheduler also waits for its instructions: the loop holds nothing that most steps do not
+// need. The first step from a caller's states and all steps from supplied start states, whose angles need the
+// library's sine and cosine, are a copy of the step of their own (128 steps on 4,096 environments, in
+// one loop / apart: 4-16-2 37 / 27 us, 4-32-2 49 / 35, 4-64-2 41 / 35, 4-16-16-2 49 / 39).
 //
 // Warps only exchange data when bit planes are written: the G warps of a CTA then hold the 32
 // environments of one bit-plane word, leave their bits of 32 steps in shared memory and write the
 // words together. All of a CTA's warps make the same T steps, so they meet the same barriers.
 #pragma once
+#include <type_traits>
+
 #include "cartpole_device.cuh"
 #include "cartpole_internal.h"
 #include "policy_screen.cuh"
@@ -34,107 +44,137 @@ __device__ __forceinline__ float in_register(float v) {
     return v;
 }
 
-// A layer's weights of one lane. The layer's units come in BLOCKS equal runs, each run shared out to
-// the G lanes, U units each: unit (block * G + g) * U + u.
-template <int U, int BLOCKS, int IN>
+// U units of a layer with IN inputs, on one lane: unit g * U + u of the layer.
+template <int U, int IN>
 struct LaneLayer {
-    float w[BLOCKS][U][IN], b[BLOCKS][U];
+    float w[U][IN], b[U];
     // layer: w[units][IN] then b[units], as the caller gave them
-    __device__ __forceinline__ void load(const float *layer, int units, int lanes, uint32_t g) {
+    __device__ __forceinline__ void load(const float *layer, int units, uint32_t g) {
 #pragma unroll
-        for (int k = 0; k < BLOCKS; ++k) {
+        for (int u = 0; u < U; ++u) {
+            const int unit = (int)g * U + u;
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int unit = (k * lanes + (int)g) * U + u;
-#pragma unroll
-                for (int i = 0; i < IN; ++i) w[k][u][i] = in_register(layer[unit * IN + i]);
-                b[k][u] = in_register(layer[units * IN + unit]);
-            }
+            for (int i = 0; i < IN; ++i) w[u][i] = in_register(layer[unit * IN + i]);
+            b[u] = in_register(layer[units * IN + unit]);
         }
     }
-    // activations of this lane's units of one block from the inputs, left at `mine`
-    template <bool CONTRACT>
-    __device__ __forceinline__ void run(int k, const float (&in)[IN], float *mine) const {
-        float h[U];
+    // Sums of this lane's units, left to right from the bias; SPLIT: few long chains, each as two.
+    template <bool SPLIT>
+    __device__ __forceinline__ void sums(const float (&in)[IN], float (&h)[U]) const {
+        constexpr int HALF = SPLIT ? IN / 2 : IN;
 #pragma unroll
-        for (int u = 0; u < U; ++u) h[u] = b[k][u];
+        for (int u = 0; u < U; ++u) h[u] = b[u];
 #pragma unroll
-        for (int i = 0; i < IN; ++i) {
+        for (int i = 0; i < HALF; ++i) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) h[u] = __fmaf_rn(w[k][u][i], in[i], h[u]);
+            for (int u = 0; u < U; ++u) h[u] = __fmaf_rn(w[u][i], in[i], h[u]);
         }
+        if constexpr (SPLIT) {
+            float rest[U] = {};
 #pragma unroll
-        for (int u = 0; u < U; ++u) h[u] = CONTRACT ? tanh_contracted(h[u]) : tanh_canonical(h[u]);
-        if constexpr (U % 4 == 0) {
+            for (int i = HALF; i < IN; ++i) {
 #pragma unroll
-            for (int u = 0; u < U; u += 4) *reinterpret_cast<float4 *>(mine + u) = make_float4(h[u], h[u + 1], h[u + 2], h[u + 3]);
-        } else if constexpr (U == 2) {
-            *reinterpret_cast<float2 *>(mine) = make_float2(h[0], h[1]);
-        } else {
-            mine[0] = h[0];
+                for (int u = 0; u < U; ++u) rest[u] = __fmaf_rn(w[u][i], in[i], rest[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) h[u] = __fadd_rn(h[u], rest[u]);
         }
     }
 };
 template <int NET, int G>
 struct LaneNetwork {
     using S = NetShape<NET>;
-    static constexpr int BLOCKS = S::H >= 64 ? 2 : 1;  // (measured slower with 32 units: the halves are too short)
-    static constexpr int U = S::H / G / BLOCKS;
-    LaneLayer<U, BLOCKS, 4> first;
-    LaneLayer<S::kDeep ? U : 1, 1, S::kDeep ? S::H : 1> second;  // unused unless the network is deep
-    float out[S::H], bias;                                       // this lane's logit: even lanes 0, odd lanes 1
+    static constexpr int U = S::H / G;
+    LaneLayer<U, 4> first;
+    LaneLayer<S::kDeep ? U : 1, S::kDeep ? S::H : 1> second;  // unused unless the network is deep
+    float step[U];                                           // w1[j] - w0[j] of this lane's last-layer units
     __device__ __forceinline__ void load(const RolloutParams &p, uint32_t g) {
-        first.load(p.w, S::H, G, g);
-        if constexpr (S::kDeep) second.load(p.w + S::kSecond, S::H, G, g);
-        const float *logits = p.w + S::kLogits;
+        first.load(p.w, S::H, g);
+        if constexpr (S::kDeep) second.load(p.w + S::kSecond, S::H, g);
+        const float *logits = p.w + S::kLogits + g * U;
 #pragma unroll
-        for (int j = 0; j < S::H; ++j) out[j] = in_register(logits[(g & 1u) * S::H + j]);
-        bias = in_register(logits[2 * S::H + (g & 1u)]);
+        for (int u = 0; u < U; ++u) step[u] = in_register(__fsub_rn(logits[S::H + u], logits[u]));
     }
 };
 
-// Floats per environment's row: 16 bytes more than the activations, so that the 16-byte reads of
-// up to eight environments' rows fall into different banks.
+// Floats per environment's row of shared memory: 16 bytes more than the activations, so that the 16-byte
+// reads of up to eight environments' rows fall into different banks.
 template <int H>
 constexpr int kRow = H + 4;
 
+// The activations of all H units of an environment, from its lanes' U each.
+template <int H, int U>
+__device__ __forceinline__ void share_activations(float *row, uint32_t g, const float (&mine)[U], float (&all)[H]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) row[g * U + u] = mine[u];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < H; j += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(row + j);
+        all[j] = v.x;
+        all[j + 1] = v.y;
+        all[j + 2] = v.z;
+        all[j + 3] = v.w;
+    }
+    __syncwarp();  // the row is read before it is written again
+}
+
+// The action by the defined logits of a network with one hidden layer, by all lanes of the environment
+// together: their units' activations side by side, then one of the two logits each, left to right from its bias.
 template <int NET, int G, bool CONTRACT>
-__device__ __forceinline__ uint32_t lanes_action(const LaneNetwork<NET, G> &net, const State &z, float *row, uint32_t g) {
+__device__ __forceinline__ uint32_t lanes_defined_action(const RolloutParams &p, const LaneNetwork<NET, G> &net, const State &z, float *row, uint32_t g) {
     using S = NetShape<NET>;
-    using N = LaneNetwork<NET, G>;
-    constexpr int H = S::H, PER = H / N::BLOCKS;  // units per block
+    constexpr int H = S::H, U = LaneNetwork<NET, G>::U;
     const float obs[4] = {z.x, z.xd, z.th, z.thd};
-    float h[PER];
-    auto read_block = [&](int k) {
-        __syncwarp();
+    float h[U];
+    net.first.template sums<false>(obs, h);
 #pragma unroll
-        for (int j = 0; j < PER; j += 4) {
-            const float4 v = *reinterpret_cast<const float4 *>(row + k * PER + j);
-            h[j] = v.x;
-            h[j + 1] = v.y;
-            h[j + 2] = v.z;
-            h[j + 3] = v.w;
-        }
-    };
-    net.first.template run<CONTRACT>(0, obs, row + (int)g * N::U);
-    if constexpr (S::kDeep) {
-        read_block(0);
-        __syncwarp();  // the row is read before the next layer overwrites it
-        net.second.template run<CONTRACT>(0, h, row + (int)g * N::U);
-    }
-    float mine = net.bias;
-#pragma unroll
-    for (int k = 0; k < N::BLOCKS; ++k) {
-        read_block(k);
-        // the next block's units do not depend on this block's part of the chain: they overlap
-        if (k + 1 < N::BLOCKS) net.first.template run<CONTRACT>(k + 1, obs, row + (k + 1) * PER + (int)g * N::U);
-#pragma unroll
-        for (int j = 0; j < PER; ++j) mine = __fmaf_rn(net.out[k * PER + j], h[j], mine);
-    }
-    __syncwarp();  // the row is read before the next step overwrites it
+    for (int u = 0; u < U; ++u) row[g * U + u] = CONTRACT ? tanh_contracted(h[u]) : tanh_canonical(h[u]);
+    __syncwarp();
+    const float *logits = p.w + S::kLogits, *w = logits + (g & 1u) * H;
+    float mine = logits[2 * H + (g & 1u)];
+#pragma unroll 4
+    for (int j = 0; j < H; ++j) mine = __fmaf_rn(w[j], row[j], mine);
+    __syncwarp();
     const float other = __shfl_xor_sync(0xffffffffu, mine, 32 / G);  // the neighbouring lane of the environment
     const bool right = (g & 1u) ? mine > other : other > mine;
     return right ? 0x80000000u : 0u;
+}
+
+// The action of this lane's environment. Every lane sums its own units' part of the estimate; the
+// parts are added pairwise over the environment's lanes, so that all of them hold the same sum.
+template <int NET, int G, bool CONTRACT>
+__device__ __forceinline__ uint32_t lanes_action(const RolloutParams &p, const LaneNetwork<NET, G> &net, const State &z, float *row, uint32_t g) {
+    using S = NetShape<NET>;
+    constexpr int U = LaneNetwork<NET, G>::U;
+    const float obs[4] = {z.x, z.xd, z.th, z.thd};
+    float h[U];
+    net.first.template sums<false>(obs, h);
+#pragma unroll
+    for (int u = 0; u < U; ++u) h[u] = tanh_screen(h[u]);
+    if constexpr (S::kDeep) {
+        float all[S::H];
+        share_activations(row, g, h, all);
+        net.second.template sums<U <= 2>(all, h);
+#pragma unroll
+        for (int u = 0; u < U; ++u) h[u] = tanh_screen(h[u]);
+    }
+    float part = 0.0f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) part = __fmaf_rn(net.step[u], h[u], part);
+#pragma unroll
+    for (int o = 32 / G; o < 32; o <<= 1) part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, o));
+    const float estimate = __fadd_rn(p.screen_base, part);
+    uint32_t sb = screen_action(estimate);
+    const bool open = !screen_decides(estimate, p.screen_bound);
+    if constexpr (S::kDeep) {
+        if (open) sb = defined_action<NET, CONTRACT, 1>(p.w, p.w + S::kLogits, z);
+        __syncwarp();
+    } else if (__any_sync(0xffffffffu, open)) {  // warp-uniform
+        const uint32_t defined = lanes_defined_action<NET, G, CONTRACT>(p, net, z, row, g);
+        if (open) sb = defined;
+    }
+    return sb;
 }
 
 // Warps of a CTA: one per scheduler, and as many as hold the 32 environments of a bit-plane word
@@ -143,8 +183,8 @@ template <int G, bool STREAMS>
 constexpr int kLaneWarps = STREAMS ? G : 4;
 
 // NET: 2 (4-16-2), 4 (4-32-2), 5 (4-64-2), 7 (4-16-16-2). G: lanes per environment. STREAMS: any
-// combination of the per-step outputs. Step limit, supplied start states and caller's initial states
-// are run-time options: next to a network's evaluation their tests cost nothing.
+// combination of the per-step outputs. The step limit is a run-time option: next to a network's evaluation
+// its test costs nothing.
 template <int NET, int G, bool STREAMS, bool CONTRACT>
 __global__ void __launch_bounds__(32 * kLaneWarps<G, STREAMS>) rollout_lanes_kernel(const __grid_constant__ RolloutParams p) {
     static_assert(G >= 4, "four lanes of an environment hash the components of its start state");
@@ -184,23 +224,20 @@ __global__ void __launch_bounds__(32 * kLaneWarps<G, STREAMS>) rollout_lanes_ker
     float *tr = STREAMS && p.trajectory ? p.trajectory + (int64_t)c * p.n + idx : nullptr;
     const float *start = p.start_in ? p.start_in + (int64_t)c * p.n + idx : nullptr;
 
-    for (uint32_t k = 0; k < p.T; ++k) {
+    // general: a state may hold any angle
+    auto step = [&](auto general, uint32_t k) {
         const uint32_t t1 = p.t0 + k + 1u;
         float fresh;
-        if (start) {
+        if (decltype(general)::value && start) {
             fresh = __ldg(start);
             start += 4 * p.n;
         } else {
             fresh = start_component_folded(kr, fold16(4u * t1), c);
         }
-        const uint32_t sb = lanes_action<NET, G, CONTRACT>(net, z, row, g);
+        const uint32_t sb = lanes_action<NET, G, CONTRACT>(p, net, z, row, g);
         const float force = force_from_signbit(sb);
-        // a caller's states may hold any angle: its initial ones on the first step, supplied start states always
-        bool done;
-        if (p.start_in || (k == 0u && p.init_planes))
-            done = CONTRACT ? euler_step_contracted<false>(z, force) : euler_step<false>(z, force);
-        else
-            done = CONTRACT ? euler_step_contracted<true>(z, force) : euler_step<true>(z, force);
+        constexpr bool SMALL = !decltype(general)::value;
+        bool done = CONTRACT ? euler_step_contracted<SMALL>(z, force) : euler_step<SMALL>(z, force);
         if (p.max_steps) done |= (t1 - begin) >= p.max_steps;
         const float fx = __shfl_sync(0xffffffffu, fresh, e), fxd = __shfl_sync(0xffffffffu, fresh, e + E);
         const float fth = __shfl_sync(0xffffffffu, fresh, e + 2 * E), fthd = __shfl_sync(0xffffffffu, fresh, e + 3 * E);
@@ -244,7 +281,14 @@ __global__ void __launch_bounds__(32 * kLaneWarps<G, STREAMS>) rollout_lanes_ker
                 }
             }
         }
+    };
+    uint32_t k = 0u;
+    if (p.start_in) {
+        for (; k < p.T; ++k) step(std::true_type{}, k);
+    } else if (p.init_planes && p.T) {
+        step(std::true_type{}, k++);
     }
+    for (; k < p.T; ++k) step(std::false_type{}, k);
 
     unsigned long long tot_ret = 0, tot_cnt = 0;
     if (valid && g == 0u) {
@@ -288,12 +332,9 @@ cudaError_t launch_lanes_one(RolloutParams &p, cudaStream_t s) {
 
 template <int NET, bool STREAMS, bool CONTRACT>
 cudaError_t launch_lanes_g(RolloutParams &p, int g, cudaStream_t s) {
-    if constexpr (STREAMS) {  // rollout_lanes_for: four lanes wherever per-step outputs are written
+    if constexpr (STREAMS)  // rollout_lanes_for: four lanes wherever per-step outputs are written
         return launch_lanes_one<NET, 4, true, CONTRACT>(p, s);
-    } else if constexpr (NetShape<NET>::H >= 32) {
-        if (g == 16) return launch_lanes_one<NET, 16, STREAMS, CONTRACT>(p, s);
-    }
-    if constexpr (!STREAMS)
+    else
         return g == 4 ? launch_lanes_one<NET, 4, false, CONTRACT>(p, s) : launch_lanes_one<NET, 8, false, CONTRACT>(p, s);
 }
 
