@@ -5,7 +5,7 @@
 
 namespace cp {
 
-void launch_assisted_linear(const RolloutParams &p, int policy, bool two, bool contracted, cudaStream_t s);
+void launch_assisted_linear(const RolloutParams &p, int policy, bool contracted, cudaStream_t s);
 void launch_assisted_starts(const RolloutParams &p, int policy, bool contracted, cudaStream_t s);
 
 bool rollout_assisted_applies(const RolloutParams &p, int policy, bool streams) {
@@ -25,8 +25,8 @@ bool rollout_assisted_applies(const RolloutParams &p, int policy, bool streams) 
     // 1.12 of the general kernel's time, x 4 1.00, 37,000 x 2 0.99)
     const bool linear = policy == 1 || policy == 6, tested = p.action_bits || p.trajectory;
     if (linear && p.T <= (tested ? 3u : 8u) && (p.n + 31) / 32 > (int64_t)sm_count() * (tested ? 8 : 1)) return false;
-    // up to ten pairs per SM (five CTAs of two pairs: 200 KB of shared memory; a sixth CTA would
-    // wait for a second wave). Measured against the general kernel's best shape, ms per launch:
+    // up to ten pairs per SM (at 20 KB of shared memory each; an eleventh would wait for a second
+    // wave). Measured against the general kernel's best shape, ms per launch:
     // x 5,000 steps 9,472 envs 0.25 / 0.61, 18,944 envs 0.45 / 0.61, 28,416 envs 0.57 / 0.74,
     // 37,888 envs 0.70 / 0.74; x 4,000 steps 47,360 envs (ten pairs per SM) 0.72 / 0.83,
     // 56,832 envs (twelve) 0.88 / 0.82. The linear policies (whose larger batches the deferred kernel
@@ -39,14 +39,13 @@ bool rollout_assisted_applies(const RolloutParams &p, int policy, bool streams) 
 
 cudaError_t launch_rollout_assisted(RolloutParams &p, int policy, bool contracted, cudaStream_t s) {
     p.n_tasks = (p.n + 31) / 32;
-    const bool two = g_tuning.rollout_block ? g_tuning.rollout_block >= 128 : p.n_tasks > sm_count();
     if (p.action_bits_in) policy = 0;
     if (p.start_in)
         launch_assisted_starts(p, policy, contracted, s);
     else if (policy == 0)
-        launch_assisted_pairs<0, false>(p, two, contracted, s);
+        launch_assisted_chunk<0, false>(p, contracted, s);
     else
-        launch_assisted_linear(p, policy, two, contracted, s);
+        launch_assisted_linear(p, policy, contracted, s);
     count_launch();
     return cudaGetLastError();
 }

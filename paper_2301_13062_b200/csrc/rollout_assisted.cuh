@@ -12,7 +12,7 @@
 //
 // Synchronisation: one hardware barrier per consumer/producer pair (bar.sync with the pair's own
 // id, 64 threads), once per chunk, double-buffered. Both warps of a pair execute exactly
-// 1 + ceil(T / kChunk) barriers, a number fixed by the launch parameters alone; there is no flag,
+// 1 + ceil(T / chunk) barriers, a number fixed by the launch parameters alone; there is no flag,
 // no spin and no dependence on data, so neither warp can wait for an arrival that does not come.
 //
 // Scope: hashed or supplied actions (the producer turns the caller's action words into forces) and
@@ -29,10 +29,11 @@ namespace cp {
 
 namespace {
 
-// Steps per hand-over: 40 KB of static shared memory per CTA either way (640 bytes per step, two
-// buffers). Measured on 2,048 x 10,000: 8 steps 0.543 ms, 16 steps 0.512 ms.
-template <int PAIRS>
-constexpr int kChunkOf = PAIRS == 1 ? 32 : 16;
+// Steps per hand-over: 40 KB of shared memory per pair (640 bytes per step, two buffers) while at most five
+// pairs share an SM, 20 KB beyond that. (2,048 x 10,000 at 8, 16, 32 steps: 0.543, 0.512, 0.481 ms; 500 steps on
+// 17,000 environments, supplied actions, 32 / 16 steps: 41.0 / 45.0 us; on 27,000, where five pairs
+// of 32 steps fill an SM and the sixth waits, 71.5 / 63.5.)
+constexpr int kLongChunk = 32, kShortChunk = 16;
 
 // Steps per trip of the consumer's loop over a chunk. Measured on 2,048 x 10,000 (ms per launch):
 // 1: 0.666, 2: 0.481, 3: 0.487, 4: 0.503, 8: 0.504, 16: 0.506, whole chunk: 0.506.
@@ -44,8 +45,8 @@ struct PairBuffers {
     float force[2][CHUNK][32];   // +-F of the action at time t
 };
 
-// Barrier 1 for pair 0, barrier 2 for pair 1 (immediates: a register id makes the kernel claim
-// all sixteen barriers).
+// One hand-over: barrier 1 for pair 0, barrier 2 for pair 1 (immediates: a register id makes the kernel
+// claim all sixteen barriers).
 template <int PAIRS>
 __device__ __forceinline__ void pair_barrier(uint32_t pair) {
     __syncwarp();
@@ -53,6 +54,31 @@ __device__ __forceinline__ void pair_barrier(uint32_t pair) {
         asm volatile("bar.sync 1, 64;" ::: "memory");
     else
         asm volatile("bar.sync 2, 64;" ::: "memory");
+}
+
+// Pairs per CTA: one, but two, whose first two warps step, for supplied start states without per-step
+// outputs, whose helpers fetch instead of hashing (500 steps with supplied actions, 27,000 environments two / one:
+// 88.1 / 92.2 us, 45,000 130.9 / 138.5; with reward and done bits 111 / 113, 161 / 164, but 12,000 79.9 / 71.7).
+template <bool START_IN, int STREAMS>
+constexpr int kPairs = START_IN && STREAMS == 0 ? 2 : 1;
+
+// Which of the two warps of a CTA of one pair steps (0 or 1). A warp's place among an SM's warps decides which of the four
+// schedulers it has: a CTA of two warps has schedulers 0 and 1 or 2 and 3. The first warp stepping
+// everywhere, schedulers 0 and 2 would have every stepping warp, whose step is the longer one, and 1 and 3 the
+// helpers; so the roles change places from one group of four warp places to the next. The place is read, not
+// assumed: whatever it is, the result is the same.
+// us per launch of 500 steps, roles by place against two pairs per CTA with a fixed place each (start states
+// hashed in two operations fewer on both sides): hashed actions 12,000 environments 39.9 / 47.1, with
+// all outputs 55.3 / 65.6, 27,000 57.5 / 59.4, 77.9 / 82.0; one linear policy each, all outputs, 17,000 57.4 / 75.9,
+// 33,000 106.5 / 118.8.
+__device__ __forceinline__ uint32_t stepping_warp(uint32_t &shared) {
+    if (threadIdx.x == 0) {
+        uint32_t place;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(place));
+        shared = place >> 2 & 1u;
+    }
+    __syncthreads();
+    return shared;
 }
 
 // Where the consumer's per-step outputs go (only read when STREAMS; NULL = not wanted): one pointer
@@ -111,13 +137,17 @@ __device__ __forceinline__ void consume_step(const RolloutParams &p, const PairB
 }
 
 // START_IN: the start states are the caller's data and may hold any angle.
-template <int POLICY, bool START_IN, int PAIRS, bool LIMIT, bool CONTRACT, int STREAMS>
-__global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
-    constexpr int kChunk = kChunkOf<PAIRS>;
+// kChunk: steps per hand-over.
+template <int POLICY, bool START_IN, int kChunk, bool LIMIT, bool CONTRACT, int STREAMS>
+__global__ void __launch_bounds__(64 * kPairs<START_IN, STREAMS>) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
+    constexpr int PAIRS = kPairs<START_IN, STREAMS>;
     __shared__ PairBuffers<kChunk> s_buf[PAIRS];
+    __shared__ uint32_t s_stepping;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const bool producer = warp >= (uint32_t)PAIRS;
-    const uint32_t pair = producer ? warp - PAIRS : warp;
+    bool producer;
+    if constexpr (PAIRS == 1) producer = warp != stepping_warp(s_stepping);
+    else producer = warp >= (uint32_t)PAIRS;
+    const uint32_t pair = PAIRS == 1 ? 0u : warp % PAIRS;
     const int64_t task = (int64_t)blockIdx.x * PAIRS + pair;
     // Both warps of a pair leave here together, before their first barrier; no other pair uses
     // their barrier. Nothing that differs between the two warps of a pair (or between lanes) may
@@ -274,39 +304,36 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
     }
 }
 
-// One pair per CTA (PAIRS 1) spreads the pairs over the SMs; beyond one pair per SM, two pairs per CTA
-// put the four warps of a CTA on the four schedulers of one SM.
-template <int POLICY, bool START_IN, int PAIRS, bool CONTRACT, int STREAMS>
-void launch_assisted_limit(const RolloutParams &p, unsigned grid, cudaStream_t s) {
+template <int POLICY, bool START_IN, int CHUNK, bool CONTRACT, int STREAMS>
+void launch_assisted_limit(const RolloutParams &p, cudaStream_t s) {
+    constexpr int pairs = kPairs<START_IN, STREAMS>;
+    const unsigned grid = (unsigned)((p.n_tasks + pairs - 1) / pairs);
     if (p.max_steps)
-        rollout_assisted_kernel<POLICY, START_IN, PAIRS, true, CONTRACT, STREAMS><<<grid, 64 * PAIRS, 0, s>>>(p);
+        rollout_assisted_kernel<POLICY, START_IN, CHUNK, true, CONTRACT, STREAMS><<<grid, 64 * pairs, 0, s>>>(p);
     else
-        rollout_assisted_kernel<POLICY, START_IN, PAIRS, false, CONTRACT, STREAMS><<<grid, 64 * PAIRS, 0, s>>>(p);
+        rollout_assisted_kernel<POLICY, START_IN, CHUNK, false, CONTRACT, STREAMS><<<grid, 64 * pairs, 0, s>>>(p);
 }
-template <int POLICY, bool START_IN, int PAIRS, bool CONTRACT>
-void launch_assisted_streams(const RolloutParams &p, unsigned grid, cudaStream_t s) {
+template <int POLICY, bool START_IN, int CHUNK, bool CONTRACT>
+void launch_assisted_streams(const RolloutParams &p, cudaStream_t s) {
     const bool rd = p.reward_stream && p.done_bits;
     if (rd && !p.action_bits && !p.trajectory)
-        launch_assisted_limit<POLICY, START_IN, PAIRS, CONTRACT, 1>(p, grid, s);
+        launch_assisted_limit<POLICY, START_IN, CHUNK, CONTRACT, 1>(p, s);
     else if (rd && p.action_bits && p.trajectory)
-        launch_assisted_limit<POLICY, START_IN, PAIRS, CONTRACT, 3>(p, grid, s);
+        launch_assisted_limit<POLICY, START_IN, CHUNK, CONTRACT, 3>(p, s);
     else if (p.reward_stream || p.done_bits || p.action_bits || p.trajectory)
-        launch_assisted_limit<POLICY, START_IN, PAIRS, CONTRACT, 2>(p, grid, s);
+        launch_assisted_limit<POLICY, START_IN, CHUNK, CONTRACT, 2>(p, s);
     else
-        launch_assisted_limit<POLICY, START_IN, PAIRS, CONTRACT, 0>(p, grid, s);
+        launch_assisted_limit<POLICY, START_IN, CHUNK, CONTRACT, 0>(p, s);
 }
+// Supplied start states come in short chunks at all sizes (build time).
 template <int POLICY, bool START_IN>
-void launch_assisted_pairs(const RolloutParams &p, bool two, bool contracted, cudaStream_t s) {
-    const unsigned grid = (unsigned)(two ? (p.n_tasks + 1) / 2 : p.n_tasks);
-    if constexpr (START_IN) {
-        contracted ? launch_assisted_streams<POLICY, true, 2, true>(p, grid, s)
-                   : launch_assisted_streams<POLICY, true, 2, false>(p, grid, s);
-    } else if (two) {
-        contracted ? launch_assisted_streams<POLICY, false, 2, true>(p, grid, s)
-                   : launch_assisted_streams<POLICY, false, 2, false>(p, grid, s);
+void launch_assisted_chunk(const RolloutParams &p, bool contracted, cudaStream_t s) {
+    if (!START_IN && p.n_tasks <= (int64_t)sm_count() * 5) {
+        contracted ? launch_assisted_streams<POLICY, START_IN, START_IN ? kShortChunk : kLongChunk, true>(p, s)
+                   : launch_assisted_streams<POLICY, START_IN, START_IN ? kShortChunk : kLongChunk, false>(p, s);
     } else {
-        contracted ? launch_assisted_streams<POLICY, false, 1, true>(p, grid, s)
-                   : launch_assisted_streams<POLICY, false, 1, false>(p, grid, s);
+        contracted ? launch_assisted_streams<POLICY, START_IN, kShortChunk, true>(p, s)
+                   : launch_assisted_streams<POLICY, START_IN, kShortChunk, false>(p, s);
     }
 }
 

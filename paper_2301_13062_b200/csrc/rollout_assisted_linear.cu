@@ -3,9 +3,9 @@
 
 namespace cp {
 
-void launch_assisted_linear(const RolloutParams &p, int policy, bool two, bool contracted, cudaStream_t s) {
-    if (policy == 1) launch_assisted_pairs<1, false>(p, two, contracted, s);
-    else launch_assisted_pairs<6, false>(p, two, contracted, s);
+void launch_assisted_linear(const RolloutParams &p, int policy, bool contracted, cudaStream_t s) {
+    if (policy == 1) launch_assisted_chunk<1, false>(p, contracted, s);
+    else launch_assisted_chunk<6, false>(p, contracted, s);
 }
 
 }  // namespace cp
