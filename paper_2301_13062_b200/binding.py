@@ -138,7 +138,7 @@ def _dptr(t, dtype=None):
         raise TypeError("expected a contiguous tensor")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"expected dtype {dtype}, got {t.dtype}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _hptr(a):
@@ -152,8 +152,10 @@ def _hptr(a):
 
 
 def _use_current_stream() -> None:
+    # The handle alone: torch.cuda.current_stream() builds a Stream object around it, which costs more than
+    # the rest of a call's marshalling (a step of a small batch is bound by that).
     import torch
-    lib().cp_set_stream(C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    lib().cp_set_stream(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def cp_set_allocator(alloc=None, release=None) -> None:
