@@ -107,13 +107,18 @@ __device__ __forceinline__ float start_from_bits_reference(uint32_t bits) {
     float u = __fmul_rn(__uint2float_rn(bits), 5.9604644775390625e-08f);  // * 2^-24, exact
     return __fmul_rn(__fsub_rn(u, 0.5f), 0.1f);
 }
+// Fewer operations still from the hash itself: bits = h >> 8, so float(h with its low byte cleared) is
+// 256 * bits exactly, and one fused multiply-add takes that to (bits - 2^23) * (0.1f * 2^-24): the same real
+// number (0.05f' = 0.5 * 0.1f), rounded once. The hash's last xorshift and the masking are one logic operation;
+// two of eleven operations per component fall away, both from the half-rate integer pipe.
 // (A conversion-free form — f = 0x4B000000 | low 23 bits, then one fused multiply-add with
 // -0.1f or -0.1f/2 chosen by bit 23 — gives the same bits but was measured slower everywhere:
 // the conversion runs on the otherwise idle special-function pipe, the two logic operations
 // that replace it on the half-rate integer pipe.)
-__device__ __forceinline__ float start_from_bits(uint32_t bits) {
-    return __fmul_rn(__int2float_rn((int)bits - (1 << 23)), 5.9604645663569045e-09f);  // 0.1f * 2^-24
+__device__ __forceinline__ float start_from_masked(uint32_t h) {  // low byte clear
+    return __fmaf_rn(__uint2float_rn(h), 2.3283064712e-11f, -0.5f * 0.1f);  // 0.1f * 2^-32
 }
+__device__ __forceinline__ float start_from_bits(uint32_t bits) { return start_from_masked(bits << 8); }
 
 // Component j of the start state of an episode beginning at global time t.
 __device__ __forceinline__ float start_value(Keys kr, uint32_t t, uint32_t j) {
@@ -128,30 +133,26 @@ struct State {
 // the first xorshift of step_hash (h ^ h>>16) leaves low bits of the counter untouched by the
 // shifted half, so (K0 ^ (4t+j)) ^ ((K0 ^ (4t+j)) >> 16) == m ^ j with m computed once from
 // 4t. The rest of each hash is step_hash's own sequence; results equal start_value(kr, t, j).
-__device__ __forceinline__ uint32_t step_hash_tail(Keys k, uint32_t m) {
-    uint32_t h = m * kMA + k.k1;
+__device__ __forceinline__ float start_from_tail(uint32_t k1, uint32_t m) {
+    uint32_t h = m * kMA + k1;
     h = (h ^ (h >> 15)) * kMB;
-    h ^= h >> 16;
-    return h;
+    return start_from_masked((h ^ (h >> 16)) & 0xffffff00u);
 }
 __device__ __forceinline__ State start_state(Keys kr, uint32_t t) {
     const uint32_t h0 = kr.k0 ^ (4u * t);
     const uint32_t m = h0 ^ (h0 >> 16);
     State z;
-    z.x = start_from_bits(step_hash_tail(kr, m) >> 8);
-    z.xd = start_from_bits(step_hash_tail(kr, m ^ 1u) >> 8);
-    z.th = start_from_bits(step_hash_tail(kr, m ^ 2u) >> 8);
-    z.thd = start_from_bits(step_hash_tail(kr, m ^ 3u) >> 8);
+    z.x = start_from_tail(kr.k1, m);
+    z.xd = start_from_tail(kr.k1, m ^ 1u);
+    z.th = start_from_tail(kr.k1, m ^ 2u);
+    z.thd = start_from_tail(kr.k1, m ^ 3u);
     return z;
 }
 
 // The same from folded keys; folded_4t = fold16(4 * t). The counters 4t + j (j < 4) fold to
 // fold16(4t) ^ j because 4t has its two low bits clear and j >> 16 == 0.
 __device__ __forceinline__ float start_component_folded(FoldedKeys kr, uint32_t folded_4t, uint32_t j) {
-    Keys k;
-    k.k0 = 0u;  // not used by the tail
-    k.k1 = kr.k1;
-    return start_from_bits(step_hash_tail(k, kr.f0 ^ folded_4t ^ j) >> 8);
+    return start_from_tail(kr.k1, kr.f0 ^ folded_4t ^ j);
 }
 __device__ __forceinline__ State start_state_folded(FoldedKeys kr, uint32_t folded_4t) {
     State z;
