@@ -27,6 +27,8 @@
 // rollout_contracted.cu and rollout_networks_contracted.cu for the contracted arithmetic (the
 // *_networks files hold the MLP policies), so that the kernel families compile side by side.
 #pragma once
+#include <type_traits>
+
 #include "cartpole_device.cuh"
 #include "cartpole_internal.h"
 #include "policy_screen.cuh"
@@ -168,10 +170,17 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
             for (int j = 0; j < EPT; ++j) act_word[j] = __ldg(act_ptr[j]);
         }
         const uint32_t t_end = p.t0 + p.T;
-        // Is every angle of this warp within the polynomial range of sine and cosine? After the
-        // first step it is: a survivor has |theta| <= 0.2095 and a restarted env |theta| <= 0.05
-        // (unless the start states are the caller's data). A warp-uniform flag instead of a
-        // per-lane angle test every step: no divergent branch in the loop.
+        // Is every angle within the polynomial range of sine and cosine? After the first step it is: a
+        // survivor has |theta| <= 0.2095 and a restarted env |theta| <= 0.05 (unless the start states
+        // are the caller's data). So the first step from a caller's states is a copy of its own, and the
+        // loop holds neither a test nor the library's functions: what one warp or two per scheduler wait
+        // for is also their instructions (us, in one loop / apart: hashed actions 100,003 envs x 40 with reward,
+        // done and action bits 28.3 / 26.6, 70,001 x 9 8.2 / 6.2, linear policy 60,000 x 40 with all outputs 23.0 /
+        // 20.7, 4-64-2 50,001 x 128 likewise 164 / 159). The canonical warp-restart shapes keep one loop with a
+        // warp-uniform flag (FLAG): apart they measured slower (1,048,576 x 64 with all outputs 307 / 336,
+        // 500,000 x 10 with reward and done bits 20.5 / 22.6, 4-16-2 50,001 x 128 88 / 92).
+        constexpr bool FLAG = COOP && !CONTRACT;
+        constexpr bool APART = !FLAG && !START_IN && !(COOP && is_network(POLICY));  // (contracted 4-16-2: 512 / 522)
         bool small_mine = true;
 #pragma unroll
         for (int j = 0; j < EPT; ++j) small_mine = small_mine && fabsf(z[j].th) <= kSmallAngle;
@@ -180,8 +189,9 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
         // little more to overlap (2,048 x 10,000: 1.30 -> 1.22 ms). The other shapes gain nothing
         // from it or lose (SHAPE 0 at 65,536 envs: 4 % slower; four steps per trip: slower everywhere).
         constexpr int kTimeUnroll = AHEAD ? 2 : 1;
-#pragma unroll kTimeUnroll
-        for (uint32_t t = p.t0; t < t_end; ++t) {
+        // anywhere: a state may hold any angle (read by the shapes without the flag)
+        auto step = [&](auto anywhere, uint32_t t) {
+            [[maybe_unused]] constexpr bool ANYWHERE = decltype(anywhere)::value;
             const uint32_t t1 = t + 1u;
             const uint32_t folded_t = fold16(t), folded_4t1 = fold16(4u * t1);  // warp-uniform
             bool done[EPT];
@@ -210,12 +220,10 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
                 }
                 if (PAIR && small_all) continue;  // both envs step together below
                 const float force = force_from_signbit(sb[j]);
-                // warp-uniform; the per-lane shapes and the contracted arithmetic keep the per-lane
-                // test (measured faster there: 2,048 x 10,000 loses 6 % with the flag)
-                if (COOP && !CONTRACT && small_all)
-                    done[j] = CONTRACT ? euler_step_contracted<true>(z[j], force) : euler_step<true>(z[j], force);
+                if constexpr (FLAG)
+                    done[j] = small_all ? euler_step<true>(z[j], force) : euler_step<false>(z[j], force);
                 else
-                    done[j] = CONTRACT ? euler_step_contracted<false>(z[j], force) : euler_step<false>(z[j], force);
+                    done[j] = CONTRACT ? euler_step_contracted<!ANYWHERE>(z[j], force) : euler_step<!ANYWHERE>(z[j], force);
                 if (LIMIT) done[j] |= (t1 - begin[j]) >= p.max_steps;
                 if (!COOP && done[j]) {
                     cnt[j] += 1u;
@@ -362,7 +370,15 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
                     word_off[j] += words;
                 }
             }
-            small_all = true;  // only read by the warp-restart shapes, which always restart from the hash
+            small_all = true;  // only read under FLAG: shapes that always restart from the hash
+        };
+        uint32_t t = p.t0;
+        if constexpr (FLAG) {
+            for (; t < t_end; ++t) step(std::true_type{}, t);
+        } else {
+            if (APART && p.init_planes && t < t_end) step(std::true_type{}, t++);
+#pragma unroll kTimeUnroll
+            for (; t < t_end; ++t) step(std::bool_constant<!APART>{}, t);
         }
 
 #pragma unroll
@@ -482,7 +498,10 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
     // 2,048 x 10,000 1.49 vs 1.65 ms, 32,768 x 5,000 0.75 vs 0.83 ms; slower from 65,536 envs on,
     // and with the linear policy, whose episodes are long)
     const bool tiny = (p.n + 31) / 32 <= (int64_t)sm_count() * 4 * 2;
-    if (coop == 0) coop = (small && ept == 1) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
+    // (the 4-16-2 network with action bits or trajectory among its outputs restarts by the warp on smaller batches
+    // too: 50,001 x 128 88 us against 92, 20,011 74 against 76, but with reward and done bits 59 against 56)
+    const bool tested = policy == 2 && (p.action_bits || p.trajectory);
+    if (coop == 0) coop = (small && ept == 1 && !tested) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
     // two envs per thread are always cooperative; supplied start states are read by the lane that
     // needs them, so they always take the per-lane shape that reads them (4)
     // (coop 4 asks for the producer-assisted kernel of rollout_assisted.cu; a call it does not
