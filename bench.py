@@ -42,25 +42,25 @@ SMS = 148
 # states of the 4.5 % of env-steps that restart, 8 more for the linear policy).
 # COUNTED_AT = build.kernel_hash() of the sources these were captured from (a test compares it
 # with the current sources, so that the fractions cannot go stale unnoticed).
-COUNTED_AT = "3bd3e07629b34c83"
+COUNTED_AT = "e899333fe9c276f7"
 # pipe_busy: sm__pipe_fmaheavy_cycles_active (share of the launch's cycles) in the same captures — the
 # resource that bounds these kernels; it counts idle slots' arithmetic and the integer multiply-adds too.
 ROLLOUT_OPS = {
     # slots: 1,048,576 x 500 (the deferred kernel's ragged end makes them depend a little on T)
-    "random": {"thread": 60.2, "slot": 47.5, "fp32": 37.2, "pipe_busy": 0.835, "kernel": "rollout_deferred_kernel"},
+    "random": {"thread": 60.2, "slot": 47.5, "fp32": 37.2, "pipe_busy": 0.834, "kernel": "rollout_deferred_kernel"},
     "linear": {"thread": 61.7, "slot": 40.2, "fp32": 45.2, "pipe_busy": 0.827, "kernel": "rollout_deferred_kernel"},
     # slots: 1,048,576 x 1,000 with the reward plane and the done bitmask
-    "linear+streams": {"thread": 81.0, "slot": 46.8, "fp32": 45.2, "pipe_busy": 0.807, "kernel": "rollout_deferred_kernel"},
+    "linear+streams": {"thread": 81.0, "slot": 46.8, "fp32": 45.2, "pipe_busy": 0.804, "kernel": "rollout_deferred_kernel"},
     # slots: 2,097,152 x 200; one estimate of the logits' difference, the defined logits where it is too close to zero
-    "mlp": {"thread": 151.5, "slot": 155.3, "pipe_busy": 0.683, "kernel": "rollout_deferred_kernel"},
-    "random+contracted": {"thread": 46.3, "slot": 38.7, "fp32": 22.2, "pipe_busy": 0.809, "kernel": "rollout_deferred_kernel"},
+    "mlp": {"thread": 151.5, "slot": 155.3, "pipe_busy": 0.679, "kernel": "rollout_deferred_kernel"},
+    "random+contracted": {"thread": 46.3, "slot": 38.7, "fp32": 22.2, "pipe_busy": 0.806, "kernel": "rollout_deferred_kernel"},
 }
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch in the same captures (the per-env
-# results stay in L2); with the per-step streams: bytes per env-step (4,385.1 MB for 1,048,576 x
+# results stay in L2); with the per-step streams: bytes per env-step (4,384.9 MB for 1,048,576 x
 # 1,000; the algorithmic figure is 4.125), which scale with N*T; the launch that zeroes the done bit
 # plane before the rollout writes another 0.125 B per env-step.
-ROLLOUT_DRAM_BYTES = {"random": 125.7e3, "linear": 53.0e3, "mlp": 63.2e3, "random+contracted": 53.0e3}
-STREAM_DRAM_BYTES_PER_ENV_STEP = 4.1819
+ROLLOUT_DRAM_BYTES = {"random": 54.0e3, "linear": 53.2e3, "mlp": 60.4e3, "random+contracted": 53.2e3}
+STREAM_DRAM_BYTES_PER_ENV_STEP = 4.1817
 STEP_DRAM_BYTES_16M = 567.2e6  # step_kernel at 16,777,216 envs, same kind of capture
 # Algorithmic HBM bytes per env-step of the step paths.
 LAST_TIMING: dict = {}  # median / best / worst of the per-iteration event times of the last timed() call

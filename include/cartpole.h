@@ -335,20 +335,21 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * and start state ahead into shared memory, or fetches the supplied ones (hashed or supplied
  * actions and the linear policies; otherwise as 2), 2, 3 and 4 only with one environment per
  * thread; 0 = default: helper warps for up to ten warps of environments per SM (a linear policy's
- * shortest launches aside), the hidden units of a network spread over several lanes for up to two warps
- * per scheduler and from 3 to 8 steps on, per lane for
+ * shortest launches aside), the hidden units of a network spread over several lanes for up to two and a
+ * half warps per scheduler and from 3 to 8 steps on, per lane for
  * other batches too small to fill the GPU (ahead for the smaller ones), deferred (5) from one
- * 64-environment warp per scheduler on (37,888 environments on 148 SMs) where that form applies,
+ * 64-environment warp per scheduler on (37,888 environments on 148 SMs; the networks only on larger batches)
+ * where that form applies,
  * with supplied actions or start states only beyond the helper warps' batches, from 96, 128 or 192 steps on
  * by batch size and outputs, without a step limit below 12, and, beside a reward plane, with at most 1.6 GB of
  * start states; by the warp otherwise;
  * 5 = two environments per thread with a clock per environment and restarts deferred to every
  * few loop trips (per-step outputs none or reward plane + done bits, not over the call's own actions or
  * start states; hashed or supplied actions, a linear policy, hashed or supplied start states, or the
- * 4-16-2 network with hashed ones; the wider and deeper networks without step limit and per-step
+ * 4-16-2 network with hashed ones; the 4-16-16-2 network without step limit and per-step
  * outputs; otherwise the default); every choice gives the same bits), "rollout_defer" (loop
  * trips between the restart passes of that deferred form: 2, 3, 4, 6 or 8; 0 = default: 2, 4 or
- * 6 by the number of steps, 3 with a network policy; the wider and deeper networks always use 3, calls with
+ * 6 by the number of steps, 2 with the 4-16-2 network; the 4-16-16-2 network always uses 3, calls with
  * supplied actions or start states have 2, 4 and 6 only (3 runs as 4, 8 as 6), and the contracted arithmetic
  * always uses 6, with a network 2),
  * "rollout_ctas_per_sm" (0 = default: one 32*ept-environment task per warp and as many

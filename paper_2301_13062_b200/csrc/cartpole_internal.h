@@ -97,7 +97,7 @@ bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams);
 cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracted, cudaStream_t s);
 // policies 0, 1, 3 (supplied actions), 6 where actions or start states are the caller's data
 cudaError_t launch_rollout_deferred_data(RolloutParams &p, int policy, int k, bool contracted, cudaStream_t s);
-cudaError_t launch_rollout_deferred_wide(RolloutParams &p, int policy, bool contracted, cudaStream_t s);  // policies 4, 5, 7
+cudaError_t launch_rollout_deferred_deep(RolloutParams &p, bool contracted, cudaStream_t s);  // policy 7
 // the lane-split kernel of the network policies: lanes per environment it would use for a call, 0 = not its call
 int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool contracted);
 cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s);

@@ -1,7 +1,6 @@
 // The deferred-restart rollout kernel (rollout_deferred.cuh) for hashed actions, the linear
-// policies and the 4-16-2 network, and the entry that picks the instance for a call; the wider
-// and deeper networks are instantiated in rollout_deferred_networks.cu and
-// rollout_deferred_mlp64.cu (build time).
+// policies and the 4-16-2 network, and the entry that picks the instance for a call; the deeper
+// network is instantiated in rollout_deferred_networks.cu (build time).
 #include "rollout_deferred.cuh"
 
 namespace cp {
@@ -12,7 +11,7 @@ bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams) 
     if (!outputs_ok) return false;
     if (p.action_bits_in) return true;  // supplied actions replace whatever policy was named
     if (p.start_in) return policy == 0 || policy == 1 || policy == 6;
-    if (is_wide_network(policy)) return !streams && !p.max_steps;
+    if (is_deep_network(policy)) return !streams && !p.max_steps;
     return policy == 0 || policy == 1 || policy == 2 || policy == 6;
 }
 
@@ -33,7 +32,12 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
     // better (981, 935) and others worse (31-step mixtures 949 at 6; 1,080, 1,199). Choosing in the
     // kernel, by counting the waiting slots every second trip or after every pass, cost 6 to 14 % of
     // every launch.
-    const int by_length = p.T < 48u ? 2 : p.T < 192u ? 4 : 6;
+    // One wave of two 64-env warps per scheduler leaves issue slots for passes that come closer together (hashed
+    // actions without outputs, 50,000 and 75,000 x 500 at K = 4 / 6: 82.1 / 86.2 us; with one warp, 37,888, 57.1 /
+    // 55.5, with more, 100,003, 120.4 / 119.0).
+    const int64_t warps64 = (p.n + 63) / 64, sms = sm_count();
+    const bool two_warps = policy == 0 && !p.start_in && !p.reward_stream && warps64 > sms * 4 && warps64 <= sms * 8;
+    const int by_length = p.T < 48u ? 2 : p.T < 192u || two_warps ? 4 : 6;
     const int k = g_tuning.rollout_defer > 0 ? g_tuning.rollout_defer : (policy == 2 ? 2 : is_network(policy) ? 3 : by_length);
     // the action hash folds the time's upper half into the lower one: nothing to do below 2^16
     const bool short_times = (uint64_t)p.t0 + p.T <= 65536u;
@@ -48,7 +52,7 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
         case 1: return launch_limit<1, false>(p, k, contracted, s);
         case 2: return launch_limit<2, false>(p, k, contracted, s);
         case 6: return launch_limit<6, false>(p, k, contracted, s);
-        default: return launch_rollout_deferred_wide(p, policy, contracted, s);  // 4, 5, 7: weights already paired
+        default: return launch_rollout_deferred_deep(p, contracted, s);  // 7: weights already paired
     }
 }
 

@@ -28,8 +28,8 @@
 // arithmetic; with or without the episode step limit; per-step outputs either none or exactly the reward
 // plane + done bitmask (the action bitmask and the trajectory are rows of global time that half the
 // lanes would have to touch every step). The
-// wider and deeper networks (4-32-2, 4-64-2, 4-16-16-2) too, for the plain call: no step limit,
-// no per-step outputs. Everything else takes the general kernel.
+// 4-16-16-2 network too, for the plain call: no step limit, no per-step outputs. Everything else takes
+// the general kernel.
 //
 // No warp waits for another one and nothing spins: the loop's trip count is bounded by the
 // launch parameters (every trip block advances every unfinished slot by at least one step).
@@ -93,11 +93,10 @@ __device__ __forceinline__ void network_action_pair(const RolloutParams &p, cons
     }
 }
 
-// The networks wider or deeper than 4-16-2 (4, 5, 7): built for the plain call only — no step limit,
-// no per-step outputs, default trip spacing. With the estimate (policy_screen.cuh) against the defined logits on
-// every step, 4,194,304 x 40: 4-32-2 3.59 -> 1.58 ms, 4-64-2 7.99 -> 3.41, 4-16-16-2 4.95 -> 2.54 (contracted
-// arithmetic 3.03 -> 2.26).
-__host__ __device__ constexpr bool is_wide_network(int policy) { return is_network(policy) && policy != 2; }
+// The networks of this kernel: 4-16-2, and 4-16-16-2 for the plain call only — no step limit, no per-step
+// outputs, default trip spacing. (4-32-2 and 4-64-2 are faster in the general kernel at every size since
+// their trips are short: 1,000,000 x 100, there / here, 868 / 948 and 1,657 / 2,333 us.)
+__host__ __device__ constexpr bool is_deep_network(int policy) { return policy == 7; }
 
 // The done bit plane of a launch that sets its bits by atomic OR has to be zeroed first.
 // A warp that clears its own words inside the rollout writes 4 bytes into each of T separate
@@ -172,7 +171,7 @@ constexpr int kRing = 8;
 // one to three steps 347 / 480 / 252 and 1,307 / 3,640 / 2,356, 20 steps 285 / 134 / 137 and 1,098 / 588 / 596.
 constexpr int kMany = 40, kEnough = 24, kFew = 16;  // of the warp's 64
 
-// POLICY: 0 hashed actions, 1 shared linear policy, 2 / 4 / 5 / 7 a shared tanh network (is_network),
+// POLICY: 0 hashed actions, 1 shared linear policy, 2 / 7 a shared tanh network,
 // 3 supplied actions, 6 one linear policy per environment.
 // K: trips between restart passes. LIMIT: episodes are cut off after p.max_steps steps.
 // RD: the reward plane and the done bitmask are written (see the comment at reward_row).
@@ -486,8 +485,7 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
         };
         // The trips between two restart passes: K, or fewer where many slots wait. The 4-16-2 network's are
         // unrolled up to three (4,194,304 x 200 at K = 2, 3, 4: 4,954 -> 4,842, 4,992 -> 4,915, 5,170 -> 5,569
-        // us), the larger networks' stay a loop (1,048,576 x 100, unrolled: 4-32-2 1,019 -> 1,147, 4-64-2 1,979 ->
-        // 2,484, 4-16-16-2 1,528 -> 2,803).
+        // us), the deeper network's stay a loop (1,048,576 x 100: 1,528 -> 2,803).
         constexpr int kUnroll = !is_network(POLICY) || (POLICY == 2 && K <= 3) ? K : 1;
         auto trip_block = [&](auto tail) {  // returns the trips made
             int made = K;
@@ -579,10 +577,19 @@ __global__ void __launch_bounds__(256) clear_words_kernel(uint32_t *w, int64_t n
     }
 }
 
-// The grid of a launch (0: too many environments), and the cleared done plane where it is cleared apart.
-inline unsigned deferred_grid(RolloutParams &p, cudaStream_t s) {
+// The CTA size and grid of a launch (grid 0: too many environments), and the cleared done plane where it is
+// cleared apart. CTAs of eight warps, but of four where that leaves the fullest SM with fewer warps, on batches
+// that one wave holds: it is what the launch waits for (250 steps, supplied actions, 100,003 environments, 196 CTAs
+// of eight warps or 391 of four on 148 SMs: 89.5 / 73.9 us, with reward and done bits 113.2 / 97.5; hashed actions
+// 37,888 x 500, 74 or 148 CTAs, 84.2 / 55.5; where the fullest SM has as many either way four cost up to 5 %,
+// supplied actions on 200,003 environments 127.6 / 130.9).
+inline unsigned deferred_grid(RolloutParams &p, unsigned &block, cudaStream_t s) {
     p.n_tasks = (p.n + 63) / 64;
-    const int64_t grid = (p.n_tasks + 7) / 8;
+    const int64_t sms = sm_count();
+    auto fullest = [&](int64_t warps) { return ((p.n_tasks + warps - 1) / warps + sms - 1) / sms * warps; };
+    const int warps = p.n_tasks <= sms * 16 && fullest(4) < fullest(8) ? 4 : 8;
+    block = 32u * warps;
+    const int64_t grid = (p.n_tasks + warps - 1) / warps;
     if (grid > 0x7fffffffLL) return 0;
     if (p.done_bits && p.T >= kClearApartFrom) {  // rollout_deferred_applies: then the reward plane is written too
         const int64_t n_words = (int64_t)p.T * ((p.n + 31) >> 5);
@@ -596,20 +603,21 @@ inline unsigned deferred_grid(RolloutParams &p, cudaStream_t s) {
 
 template <int POLICY, bool SHORT, bool LIMIT, bool RD>
 cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
-    const unsigned grid = deferred_grid(p, s);
+    unsigned block;
+    const unsigned grid = deferred_grid(p, block, s);
     if (grid == 0) return cudaErrorInvalidConfiguration;
     if (contracted) {  // the optional arithmetic comes at the default trip spacing only
         constexpr int kC = is_network(POLICY) ? 2 : 6;
-        rollout_deferred_kernel<POLICY, kC, SHORT, LIMIT, RD, true><<<grid, 256, 0, s>>>(p);
-    } else if constexpr (is_wide_network(POLICY)) {  // and so do the wider and deeper networks
-        rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, kC, SHORT, LIMIT, RD, true><<<grid, block, 0, s>>>(p);
+    } else if constexpr (is_deep_network(POLICY)) {  // and so does the deeper network
+        rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p);
     } else {
         switch (k) {
-            case 2: rollout_deferred_kernel<POLICY, 2, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
-            case 3: rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
-            case 6: rollout_deferred_kernel<POLICY, 6, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
-            case 8: rollout_deferred_kernel<POLICY, 8, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
-            default: rollout_deferred_kernel<POLICY, 4, SHORT, LIMIT, RD, false><<<grid, 256, 0, s>>>(p); break;
+            case 2: rollout_deferred_kernel<POLICY, 2, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p); break;
+            case 3: rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p); break;
+            case 6: rollout_deferred_kernel<POLICY, 6, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p); break;
+            case 8: rollout_deferred_kernel<POLICY, 8, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p); break;
+            default: rollout_deferred_kernel<POLICY, 4, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p); break;
         }
     }
     count_launch();
@@ -618,7 +626,7 @@ cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
 
 template <int POLICY, bool SHORT>
 cudaError_t launch_limit(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
-    if constexpr (is_wide_network(POLICY)) {
+    if constexpr (is_deep_network(POLICY)) {
         return launch_k<POLICY, SHORT, false, false>(p, k, contracted, s);  // rollout_deferred_applies: nothing else gets here
     } else {
         const bool rd = p.reward_stream != nullptr;  // rollout_deferred_applies: then done_bits too, nothing else

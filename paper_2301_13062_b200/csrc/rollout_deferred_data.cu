@@ -8,16 +8,17 @@ namespace {
 
 template <int POLICY, bool START_IN, bool LIMIT, bool RD>
 cudaError_t launch_data(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
-    const unsigned grid = deferred_grid(p, s);
+    unsigned block;
+    const unsigned grid = deferred_grid(p, block, s);
     if (grid == 0) return cudaErrorInvalidConfiguration;
     if (contracted)
-        rollout_deferred_kernel<POLICY, 6, false, LIMIT, RD, true, START_IN><<<grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, 6, false, LIMIT, RD, true, START_IN><<<grid, block, 0, s>>>(p);
     else if (k <= 2)
-        rollout_deferred_kernel<POLICY, 2, false, LIMIT, RD, false, START_IN><<<grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, 2, false, LIMIT, RD, false, START_IN><<<grid, block, 0, s>>>(p);
     else if (k <= 4)
-        rollout_deferred_kernel<POLICY, 4, false, LIMIT, RD, false, START_IN><<<grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, 4, false, LIMIT, RD, false, START_IN><<<grid, block, 0, s>>>(p);
     else
-        rollout_deferred_kernel<POLICY, 6, false, LIMIT, RD, false, START_IN><<<grid, 256, 0, s>>>(p);
+        rollout_deferred_kernel<POLICY, 6, false, LIMIT, RD, false, START_IN><<<grid, block, 0, s>>>(p);
     count_launch();
     return cudaGetLastError();
 }

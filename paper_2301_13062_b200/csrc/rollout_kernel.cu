@@ -32,13 +32,19 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     if (const int lanes = rollout_lanes_for(p, policy, streams, contracted))
         return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
     // The deferred-restart kernel (rollout_deferred.cu) by default: from one 64-env warp per
-    // scheduler on (37,888 envs on 148 SMs) for hashed actions and the linear policies, from seven
-    // warps per SM on (66,304 envs) for the tanh networks, launches of at least a dozen steps,
-    // per-step outputs none or reward plane + done bits. Measured at T = 500, this kernel against
-    // the kernels below: hashed actions 37,888 envs 0.093 / 0.096 ms, 65,536 0.098 / 0.142,
-    // 131,072 0.163 / 0.251; linear policy 47,360 0.088 / 0.100, 131,072 0.154 / 0.212; network
-    // 56,832 0.483 / 0.427, 75,776 0.483 / 0.545. rollout_coop = 5 forces it wherever it
-    // applies, any other forced shape keeps the other kernels.
+    // scheduler on (37,888 envs on 148 SMs) for hashed actions and the linear policies, launches of at
+    // least a dozen steps, per-step outputs none or reward plane + done bits. Measured at T = 500, this kernel
+    // against the general one: hashed actions 65,536 envs 0.098 / 0.142 ms, 131,072 0.163 / 0.251; linear policy
+    // 47,360 0.088 / 0.100, 131,072 0.154 / 0.212. Against the helper warps, hashed actions and the shared linear
+    // policy gain from eight pairs of theirs per SM on, in launches of 192 steps and more (37,800 envs: x 500
+    // 55 / 72 and 64 / 72 us, with reward and done bits 72 / 82 and 80 / 88, x 96 16.4 / 18.4 and 24.6 / 20.7;
+    // 28,000 x 500 with outputs 74 / 64; one linear policy each 70 / 74, but with outputs 92 / 84).
+    // The networks' trips are short next to their waits since the estimate decides (policy_screen.cuh). This
+    // kernel's time over the general one's, three policies each, T = 100 .. 400: 4-16-2 200,003 envs 0.98 to 1.04,
+    // 1,000,000 0.99 to 1.03 and with reward and done bits 1.03 to 1.07, 4,000,000 with them 0.98 to 1.02, 16,777,216
+    // without 0.95 to 0.99; 4-32-2 1.07 to 1.2 and 4-64-2 1.3 to 1.7 from 67,000 to 1,000,000; 4-16-16-2 1,000,000 0.92 to
+    // 1.28, the latter where more estimates do not decide, contracted 113,000 1.11, 200,003 0.96, 500,000 0.91.
+    // rollout_coop = 5 forces it wherever it applies, any other forced shape keeps the other kernels.
     // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
     // below, and where every sort of data that was tried gains or nearly (time of this kernel over the
     // general kernel's; random actions / actions that end every episode after ten steps / those of a
@@ -58,13 +64,16 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // 1,048,576 x 128 687, 456 or 787; up to 1.6 GB always the lower one), so those stay there too.
     const int64_t warps32 = (p.n + 31) / 32, warps64 = (p.n + 63) / 64, sms = sm_count();
     const bool data = p.action_bits_in || p.start_in;
-    const bool network = policy == 2 || policy == 4 || policy == 5 || policy == 7;
     uint32_t from = 96u;
     if (p.start_in && warps64 < sms * 7) from = 128u;
     if (!p.start_in && streams && warps64 < sms * 20) from = contracted ? 128u : 192u;
     const bool streams_gain = !streams || (p.start_in ? p.n * (int64_t)p.T <= 100000000 : warps64 >= sms * 7);
+    int64_t least = sms * 4;  // 64-env warps
+    if (policy == 2) least = sms * 448;
+    if (policy == 4 || policy == 5 || policy == 7) least = policy == 7 && contracted ? sms * 20 : INT64_MAX;
+    if ((policy == 0 || policy == 1) && p.T >= 192u) least = sms * 7 / 2;
     const bool enough = data ? p.T >= from && warps32 > sms * 10 && streams_gain && !(p.max_steps && p.max_steps < 12u)
-                             : warps64 >= sms * (network ? 7 : 4) && p.T >= 12u;
+                             : warps64 >= least && p.T >= 12u;
     const bool by_default = g_tuning.rollout_coop == 0 && g_tuning.rollout_ept == 0 && enough;
     if ((by_default || g_tuning.rollout_coop == 5) && rollout_deferred_applies(p, policy, streams) && !outputs_over_data(p))
         return launch_rollout_deferred(p, policy, contracted, s);

@@ -19,8 +19,8 @@
 // are stepped by the packed float32 instructions of sm_100a (euler_step_pair). Batches that fill
 // the chip mostly go to the deferred-restart kernel of rollout_deferred.cu instead; this
 // kernel keeps every call that one does not cover (action bit stream or trajectory written, the
-// wider and deeper networks with a step limit or outputs, very short launches, batches too small to fill
-// the chip, supplied actions or start states where that kernel does not gain) and is the form the others are compared with bit for bit.
+// 4-32-2 and 4-64-2 networks, the deeper one with a step limit or outputs, very short launches, batches too
+// small to fill the chip, supplied actions or start states where that kernel does not gain) and is the form the others are compared with bit for bit.
 //
 // This header holds the kernel template and its dispatch; rollout_kernel.cu and
 // rollout_networks.cu instantiate it for the canonical (one rounding per op) arithmetic,
@@ -501,7 +501,10 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
     // (the 4-16-2 network with action bits or trajectory among its outputs restarts by the warp on smaller batches
     // too: 50,001 x 128 88 us against 92, 20,011 74 against 76, but with reward and done bits 59 against 56)
     const bool tested = policy == 2 && (p.action_bits || p.trajectory);
-    if (coop == 0) coop = (small && ept == 1 && !tested) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
+    // (the larger networks restart per lane on every batch: 1,000,000 x 100 4-64-2 1,657 us against 1,741, 4-16-16-2
+    // 1,573 against 1,624, 4-32-2 868 against 869)
+    const bool wide = policy == 4 || policy == 5 || policy == 7;
+    if (coop == 0) coop = ((small || wide) && ept == 1 && !tested) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
     // two envs per thread are always cooperative; supplied start states are read by the lane that
     // needs them, so they always take the per-lane shape that reads them (4)
     // (coop 4 asks for the producer-assisted kernel of rollout_assisted.cu; a call it does not
