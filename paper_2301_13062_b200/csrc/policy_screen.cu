@@ -1,57 +1,19 @@
-// Host side of the network policies' screen (policy_screen.cuh): the bound of a policy's estimate,
-// the layouts the kernels read, and the self-test of the special-function unit's tanh.
+// Host side of the network policies' screen (policy_screen.cuh): the layouts the kernels read, with the bound
+// of a policy's estimate (policy_bound.h), and the self-test of the special-function unit's tanh.
+#include "policy_bound.h"
 #include "policy_screen.cuh"
 
-#include <cmath>
 #include <cstring>
 
 namespace cp {
 
 namespace {
 
-// The bound. Let u = 2^-24 (half an ulp), h_j the activations of the definition (|h_j| <= 1), and
-// v_j = w1[j] - w0[j].
-//  * First layer: the estimate's arguments have the bits of the definition's (same operands, same
-//    order), so |h~_j - h_j| <= E1 = kTanhScreenError, which covers both arithmetics' tanh
-//    (cp_selftest_screen compares over every float32).
-//  * A second hidden layer of n units sums in another order: both sums miss the exact one by at most
-//    (n + 1) u (|b| + sum |w|), the operands differ by E1, tanh does not stretch distances, and the
-//    definition's own tanh misses the real one by less than E1: E2_k = E1 sum_j |w2[k][j]| +
-//    2 (n + 2) u (|b2[k]| + sum_j |w2[k][j]|) + 2 E1.
-//  * A sum over h_j rounds each of its partial sums once. Those of a defined logit, left to right, are at
-//    most |b_i| + |w_i[0]| + .. + |w_i[k]|, so the logit misses its exact sum by u times the sum of these over k.
-//  * The estimate's order depends on the kernel; `rounds` says how many roundings a term goes through at
-//    most, each of a partial sum of at most |b1 - b0| + sum |v_j|, two more for v_j and b1 - b0 themselves.
-// Estimate and l1 - l0 then differ by at most the sum of all that and sum_j E_j |v_j|; 1/16 more for
-// the second-order terms and this computation itself, and 1e-37 for results too small
-// to be normal numbers. Weights of 1e30 and more in sum (or not finite) could overflow in the estimate where
-// they do not in the logits: their bound is infinite.
 template <int NET>
 void screen(RolloutParams &p, float *steps, int rounds) {
-    using S = NetShape<NET>;
-    constexpr int H = S::H;
-    const double u = std::ldexp(1.0, -24), e1 = kTanhScreenError;
-    const float *logits = p.w + S::kLogits;
-    double moved = 0.0, total = std::fabs((double)logits[2 * H]) + std::fabs((double)logits[2 * H + 1]), partial = 0.0;
-    const double base = (double)logits[2 * H + 1] - (double)logits[2 * H];
-    double span = std::fabs(base);
-    for (int j = 0; j < H; ++j) {
-        double e = e1;
-        if (S::kDeep) {
-            double row = 0.0;
-            for (int i = 0; i < H; ++i) row += std::fabs((double)p.w[S::kSecond + H * j + i]);
-            e = e1 * (row + 2.0) + 2.0 * (H + 2) * u * (row + std::fabs((double)p.w[S::kSecond + H * H + j]));
-        }
-        const double v = (double)logits[H + j] - (double)logits[j];
-        steps[j] = (float)v;
-        moved += e * std::fabs(v);
-        span += std::fabs(v);
-        total += std::fabs((double)logits[j]) + std::fabs((double)logits[H + j]);
-        partial += total;
-    }
-    const double bound = 1.0625 * (moved + (rounds + 2) * u * span + u * partial) + 1e-37;
-    p.screen_base = (float)base;
-    p.screen_bound = bound < 1e30 && total < 1e30 ? std::nextafter((float)bound, INFINITY) : INFINITY;
+    const PolicyBound b = policy_bound(p.w, NetShape<NET>::H, NetShape<NET>::kDeep, rounds, steps);
+    p.screen_base = b.base;
+    p.screen_bound = b.bound;
 }
 
 template <int NET>

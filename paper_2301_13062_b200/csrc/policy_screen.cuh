@@ -8,7 +8,7 @@
 //   estimate = (b1 - b0) + sum_j (w1[j] - w0[j]) * h~_j     h~_j: the special-function unit's tanh
 //
 // One result of that unit per hidden unit instead of two, no polynomial beside it, one
-// multiply-add instead of two, and no order to keep. The bound (screen_policy, in policy_screen.cu)
+// multiply-add instead of two, and no order to keep. The bound (policy_bound, in policy_bound.h)
 // grows with the weights and with kTanhScreenError; with the weight distributions of inputs.py it
 // sends one to two environments in 10,000 steps to the defined logits, at most one in 1,000.
 //
@@ -21,8 +21,7 @@
 namespace cp {
 
 // tanh by the special-function unit, one instruction. Its distance from either arithmetic's tanh is at
-// most kTanhScreenError over every float32 (measured: 7.987e-6 for both, cp_selftest_screen).
-constexpr double kTanhScreenError = 8.0e-6;
+// most kTanhScreenError (policy_bound.h) over every float32 (measured: 7.987e-6 for both, cp_selftest_screen).
 __device__ __forceinline__ float tanh_screen(float x) {
     float r;
     asm("tanh.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
