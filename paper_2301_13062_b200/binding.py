@@ -152,10 +152,12 @@ def _hptr(a):
 
 
 def _use_current_stream() -> None:
-    # The handle alone: torch.cuda.current_stream() builds a Stream object around it, which costs more than
-    # the rest of a call's marshalling (a step of a small batch is bound by that).
+    # The handle alone where torch has the function for it: torch.cuda.current_stream() builds a Stream object
+    # around it, which costs more than the rest of a call's marshalling (a step of a small batch is bound by that).
     import torch
-    lib().cp_set_stream(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    device = torch.cuda.current_device()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    lib().cp_set_stream(raw(device) if raw else torch.cuda.current_stream(device).cuda_stream)
 
 
 def cp_set_allocator(alloc=None, release=None) -> None:

@@ -193,6 +193,24 @@ def test_wrap_bookkeeping_needs_no_gpu(cp):
     st.close()
 
 
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_reaches_the_library_without_torchs_private_name(cp, monkeypatch, raw):
+    """torch's raw-handle function is quicker than its Stream object, but not part of its public interface: a torch
+    without it must do as well."""
+    import types
+    torch = pytest.importorskip("torch")
+    seen = []
+    monkeypatch.setattr(cp, "lib", lambda: types.SimpleNamespace(cp_set_stream=seen.append))
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: types.SimpleNamespace(cuda_stream=4096 + (device or 0)))
+    if raw:
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 4096 + device, raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    cp._use_current_stream()
+    assert seen == [4099]
+
+
 def test_missing_library_fails_loudly(cp, monkeypatch):
     monkeypatch.setattr(cp, "_lib", None)
     monkeypatch.setattr(cp, "LIB_PATH", os.path.join(ROOT, "does_not_exist.so"))
