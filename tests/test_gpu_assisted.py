@@ -1,11 +1,9 @@
 """The producer-assisted rollout kernel (very small batches: a helper warp hashes actions and start
 states ahead of each stepping warp). It must give the same bits as the general kernel, which the
 other files pin to the oracle, and it is compared with the oracle directly as well. Cases: ragged
-batch sizes, horizons around the 16- and 32-step hand-overs, both CTA forms with an odd number of warp
-tasks, a caller's initial state with angles outside the polynomial range, carried episode lengths
-and the step limit."""
-import contextlib
-
+batch sizes, horizons around the 16- and 32-step hand-overs, both lengths of a hand-over (32 steps up to five
+warp tasks per SM, 16 beyond) under every policy and output, a caller's initial state with angles
+outside the polynomial range, carried episode lengths and the step limit."""
 import numpy as np
 import pytest
 
@@ -29,17 +27,11 @@ def cp():
     return binding
 
 
-@contextlib.contextmanager
-def kernel(cp, coop, block=0):
-    cp.cp_tune("rollout_block", block)
-    try:
-        with H.rollout_shape(cp, 1, coop):
-            yield
-    finally:
-        cp.cp_tune("rollout_block", 0)
+def kernel(cp, coop):
+    return H.rollout_shape(cp, 1 if coop else 0, coop)
 
 
-def rollout(cp, coop, n, T, seed, block=0, streams=(), **kw):
+def rollout(cp, coop, n, T, seed, streams=(), **kw):
     words = (n + 31) // 32
     out = {"ep_return_sum": torch.full((n,), -1.0, device="cuda"),
            "ep_count": torch.full((n,), -1, dtype=torch.int32, device="cuda"),
@@ -49,7 +41,7 @@ def rollout(cp, coop, n, T, seed, block=0, streams=(), **kw):
               "reward_stream": ((T, n), torch.float32), "trajectory": ((T, 4, n), torch.float32)}
     for name in streams:
         out[name] = torch.full(shapes[name][0], 7, dtype=shapes[name][1], device="cuda")
-    with kernel(cp, coop, block):
+    with kernel(cp, coop):
         cp.cp_rollout_ex(n_envs=n, T=T, seed=seed, **kw, **out)
     torch.cuda.synchronize()
     return {k: v.cpu().numpy() for k, v in out.items()}
@@ -66,9 +58,7 @@ def assert_same_bits(a, b):
 def test_same_bits_as_general_kernel_and_oracle(cp, oracle, n, T):
     seed, t0, off = 12, 5, 77
     general = rollout(cp, PER_LANE, n, T, seed, t0=t0, env_offset=off)
-    for block in (64, 128):                      # one pair and two pairs per CTA (4737 envs: 149 tasks, odd)
-        got = rollout(cp, ASSISTED, n, T, seed, block, t0=t0, env_offset=off)
-        assert_same_bits(got, general)
+    assert_same_bits(rollout(cp, ASSISTED, n, T, seed, t0=t0, env_offset=off), general)
     auto = rollout(cp, 0, n, T, seed, t0=t0, env_offset=off)      # what a caller gets
     assert_same_bits(auto, general)
     o = oracle.rollout(n, T, seed, env_offset=off, t0=t0, min_gap=True)
@@ -83,8 +73,7 @@ def test_contracted_arithmetic_same_bits_as_general_kernel(cp, oracle, limit):
     n, T, seed = 3001, 150, 5
     kw = {"arithmetic": cp.CP_ARITH_CONTRACTED, "max_episode_steps": limit, "t0": 3}
     general = rollout(cp, PER_LANE, n, T, seed, **kw)
-    for block in (64, 128):
-        assert_same_bits(rollout(cp, ASSISTED, n, T, seed, block, **kw), general)
+    assert_same_bits(rollout(cp, ASSISTED, n, T, seed, **kw), general)
     auto = rollout(cp, 0, n, T, seed, **kw)
     assert_same_bits(auto, general)
     canonical = rollout(cp, 0, n, T, seed, max_episode_steps=limit, t0=3)
@@ -106,8 +95,7 @@ def test_streams_and_supplied_actions(cp, oracle, streams, supplied):
         kw["action_bits_in"] = torch.from_numpy(bits.view(np.int32)).cuda()
         ora_kw["action_bits_in"] = bits
     general = rollout(cp, PER_LANE, n, T, seed, streams=streams, **kw)
-    for block in (64, 128):
-        assert_same_bits(rollout(cp, ASSISTED, n, T, seed, block, streams=streams, **kw), general)
+    assert_same_bits(rollout(cp, ASSISTED, n, T, seed, streams=streams, **kw), general)
     auto = rollout(cp, 0, n, T, seed, streams=streams, **kw)
     assert_same_bits(auto, general)
     o = oracle.rollout(n, T, seed, t0=2, env_offset=9, max_episode_steps=limit, done_bits=True, action_bits=True,
@@ -122,6 +110,34 @@ def test_streams_and_supplied_actions(cp, oracle, streams, supplied):
         assert np.all(auto["reward_stream"] == 1.0)
     if "trajectory" in streams:
         assert np.array_equal(auto["trajectory"][-1], auto["final_state"])
+
+
+ALL = ("done_bits", "action_bits", "reward_stream", "trajectory")
+
+
+@pytest.mark.parametrize("kind", ["hashed", "supplied", "linear", "per_env"])
+@pytest.mark.parametrize("limit", [0, 12])
+@pytest.mark.parametrize("contracted", [False, True])
+def test_both_hand_over_lengths(cp, kind, limit, contracted):
+    """One batch on either side of the size from which a hand-over holds 16 steps instead of 32, forced and as a
+    caller gets it: no outputs, the reward plane and done bits alone, one output tested for, and all of them."""
+    from paper_2301_13062_b200 import inputs
+    last_long = torch.cuda.get_device_properties(0).multi_processor_count * 5 * 32
+    for n, T in ((last_long, 33), (last_long + 1, 17), (last_long + 1, 33), (last_long + 3321, 16)):
+        kw = {"t0": 4, "env_offset": 3, "max_episode_steps": limit,
+              "arithmetic": cp.CP_ARITH_CONTRACTED if contracted else cp.CP_ARITH_EXACT}
+        if kind == "supplied":
+            bits = np.random.default_rng(n).integers(0, 1 << 32, (T, (n + 31) // 32), dtype=np.uint64)
+            kw["action_bits_in"] = torch.from_numpy(bits.astype(np.uint32).view(np.int32)).cuda()
+        elif kind == "linear":
+            kw["policy"] = cp.policy(cp.CP_POLICY_LINEAR, inputs.policy_weights(cp.CP_POLICY_LINEAR, 4))
+        elif kind == "per_env":
+            kw["policy"] = cp.policy(cp.CP_POLICY_LINEAR_PER_ENV, torch.from_numpy(inputs.per_env_linear_weights(n, 3)).cuda())
+        for streams in ((), ("reward_stream", "done_bits"), ("done_bits",), ALL):
+            general = rollout(cp, PER_LANE, n, T, 6, streams=streams, **kw)
+            assert general["ep_count"].max() > 0
+            for coop in (ASSISTED, 0):
+                assert_same_bits(rollout(cp, coop, n, T, 6, streams=streams, **kw), general)
 
 
 def test_forced_on_a_large_batch_and_at_the_end_of_time(cp, oracle):
