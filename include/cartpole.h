@@ -326,8 +326,9 @@ void cp_set_stream(void *cuda_stream);
 int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
 
 /* Launch tuning, process-wide (no counterpart in the paper; its analogue is XLA's flag for
- * switching passes off, Sec. III). key: "rollout_block" (threads per CTA, 32..256, multiple of 32;
- * 0 = default: 128 for very small batches, else 256), "rollout_ept" (environments per thread: 1 or 2; 0 = default, 2 for large
+ * switching passes off, Sec. III). key: "rollout_block" (threads per CTA of the kernels that
+ * step a warp's environments together, 1, 2 and 3 below; 32..256, multiple of 32; 0 = default: 128 for very small
+ * batches, else 256; any value but 0 keeps a network from being spread over lanes), "rollout_ept" (environments per thread: 1 or 2; 0 = default, 2 for large
  * batches except with the MLP policies), "rollout_coop" (how finished environments get their
  * start state: 1 = by the whole warp through shared memory, 2 = each lane its own when its env
  * finishes, 3 = each lane computes it every step ahead of the dynamics (hashed or supplied
@@ -338,18 +339,17 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * shortest launches aside), the hidden units of a network spread over several lanes for up to two and a
  * half warps per scheduler and from 3 to 8 steps on, per lane for
  * other batches too small to fill the GPU (ahead for the smaller ones), deferred (5) from one
- * 64-environment warp per scheduler on (37,888 environments on 148 SMs; the networks only on larger batches)
- * where that form applies,
+ * 64-environment warp per scheduler on (37,825 environments on 148 SMs; 33,089 with hashed actions or the shared
+ * linear policy from 192 steps on; the 4-16-2 network on the largest batches) where that form applies,
  * with supplied actions or start states only beyond the helper warps' batches, from 96, 128 or 192 steps on
  * by batch size and outputs, without a step limit below 12, and, beside a reward plane, with at most 1.6 GB of
- * start states; by the warp otherwise;
+ * start states; per lane with the larger networks, by the warp otherwise;
  * 5 = two environments per thread with a clock per environment and restarts deferred to every
  * few loop trips (per-step outputs none or reward plane + done bits, not over the call's own actions or
  * start states; hashed or supplied actions, a linear policy, hashed or supplied start states, or the
- * 4-16-2 network with hashed ones; the 4-16-16-2 network without step limit and per-step
- * outputs; otherwise the default); every choice gives the same bits), "rollout_defer" (loop
+ * 4-16-2 network with hashed ones; otherwise the default); every choice gives the same bits), "rollout_defer" (loop
  * trips between the restart passes of that deferred form: 2, 3, 4, 6 or 8; 0 = default: 2, 4 or
- * 6 by the number of steps, 2 with the 4-16-2 network; the 4-16-16-2 network always uses 3, calls with
+ * 6 by the number of steps, 2 with the 4-16-2 network; calls with
  * supplied actions or start states have 2, 4 and 6 only (3 runs as 4, 8 as 6), and the contracted arithmetic
  * always uses 6, with a network 2),
  * "rollout_ctas_per_sm" (0 = default: one 32*ept-environment task per warp and as many

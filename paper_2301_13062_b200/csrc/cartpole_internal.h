@@ -23,7 +23,7 @@ struct StepParams {
     uint32_t max_steps;     // episode step limit (needs ep_len), 0 = none
 };
 
-constexpr int kMaxPolicyFloats = 900;
+constexpr int kMaxPolicyFloats = 834;
 
 // Parameters of one rollout launch. Weights travel in the launch parameters
 // (constant bank), so every policy FMA reads its weight as an immediate operand.
@@ -50,8 +50,8 @@ struct RolloutParams {
     // the network policies' estimate of l1 - l0 (policy_screen.cuh): its constant term, and its largest
     // distance from the logits' difference
     float screen_base, screen_bound;
-    // largest policy: the network with 64 hidden units, 7*64 + 2 floats; twice the room, because the
-    // deferred-restart kernel reads shared weights as (w, w) pairs
+    // the policy as the caller gave it, or in the layout a kernel reads (policy_screen.cuh): at most the network
+    // with 64 hidden units, 7*64 + 2 floats, and 6*64 more for its estimate
     alignas(8) float w[kMaxPolicyFloats];
 };
 
@@ -97,7 +97,6 @@ bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams);
 cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracted, cudaStream_t s);
 // policies 0, 1, 3 (supplied actions), 6 where actions or start states are the caller's data
 cudaError_t launch_rollout_deferred_data(RolloutParams &p, int policy, int k, bool contracted, cudaStream_t s);
-cudaError_t launch_rollout_deferred_deep(RolloutParams &p, bool contracted, cudaStream_t s);  // policy 7
 // the lane-split kernel of the network policies: lanes per environment it would use for a call, 0 = not its call
 int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool contracted);
 cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s);
@@ -114,9 +113,9 @@ cudaError_t launch_pipe_rate(int kind, const float *seed, float *sink, int iters
 cudaError_t launch_arith_selftest(unsigned long long *out, cudaStream_t s);
 cudaError_t launch_pair_selftest(unsigned long long count, uint32_t seed, unsigned long long *out, cudaStream_t s);
 cudaError_t launch_screen_selftest(unsigned long long *out, cudaStream_t s);
-// A network's weights in RolloutParams::w rearranged for its estimate, for two environments per thread or
-// for one, with the bound the estimate needs (policy_screen.cu).
-void screen_pairs(RolloutParams &p, int policy);
+// A network's weights in RolloutParams::w rearranged for its estimate, for two environments per thread (4-16-2)
+// or for one, with the bound the estimate needs (policy_screen.cu).
+void screen_pairs(RolloutParams &p);
 void screen_units(RolloutParams &p, int policy);
 void screen_bound(RolloutParams &p, int policy);  // the bound alone, weights as the caller gave them
 cudaError_t launch_tame_div_selftest(uint32_t den_step, unsigned long long *out, cudaStream_t s);

@@ -44,13 +44,13 @@ struct NetShape {
     static constexpr int kSecond = 5 * H;
     static constexpr int kLogits = kSecond + (kDeep ? H * (H + 1) : 0);
     static constexpr int kCount = kLogits + 2 * H + 2;
-    // RolloutParams::w for two environments per thread (screen_pairs): every hidden layer's weight and
+    // RolloutParams::w for two environments per thread (screen_pairs, one hidden layer): every weight of it and
     // every w1[j] - w0[j] as a pair, then the logits' weights
     static constexpr int kPairSteps = 2 * kLogits, kPairLogits = kPairSteps + 2 * H;
     // and for one (screen_units): the caller's weights, the first layer again with the weights of units
     // 2q and 2q + 1 side by side (input 0, .., input 3, bias), then w1[j] - w0[j]
     static constexpr int kUnitFirst = kCount, kUnitSteps = kUnitFirst + 5 * H;
-    static_assert(kPairLogits + 2 * H + 2 <= kMaxPolicyFloats && kUnitSteps + H <= kMaxPolicyFloats, "RolloutParams::w holds either layout");
+    static_assert(kUnitSteps + H <= kMaxPolicyFloats, "RolloutParams::w holds the layout");
     static_assert(kUnitFirst % 2 == 0 && kUnitSteps % 2 == 0, "pairs are read as such");
 };
 
@@ -108,31 +108,17 @@ template <int NET>
 __device__ __forceinline__ f32x2 screen_estimate_pair(const f32x2 *w, f32x2 base, const StatePair &z) {
     using S = NetShape<NET>;
     constexpr int H = S::H;
+    static_assert(!S::kDeep && S::kPairLogits + 2 * H + 2 <= kMaxPolicyFloats, "one hidden layer, as pairs");
     const f32x2 *steps = w + S::kLogits;
-    auto unit = [&](int j) {
+    f32x2 est = base;
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
         f32x2 acc = w[4 * H + j];
         acc = fma2(w[4 * j + 0], z.x, acc);
         acc = fma2(w[4 * j + 1], z.xd, acc);
         acc = fma2(w[4 * j + 2], z.th, acc);
         acc = fma2(w[4 * j + 3], z.thd, acc);
-        return tanh_screen2(acc);
-    };
-    f32x2 est = base;
-    if constexpr (S::kDeep) {
-        const f32x2 *w2 = w + S::kSecond, *b2 = w2 + H * H;
-        f32x2 h1[H];
-#pragma unroll
-        for (int j = 0; j < H; ++j) h1[j] = unit(j);
-#pragma unroll
-        for (int k = 0; k < H; ++k) {
-            f32x2 acc = b2[k];
-#pragma unroll
-            for (int j = 0; j < H; ++j) acc = fma2(w2[H * k + j], h1[j], acc);
-            est = fma2(steps[k], tanh_screen2(acc), est);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < H; ++j) est = fma2(steps[j], unit(j), est);
+        est = fma2(steps[j], tanh_screen2(acc), est);
     }
     return est;
 }

@@ -1,6 +1,5 @@
 // The deferred-restart rollout kernel (rollout_deferred.cuh) for hashed actions, the linear
-// policies and the 4-16-2 network, and the entry that picks the instance for a call; the deeper
-// network is instantiated in rollout_deferred_networks.cu (build time).
+// policies and the 4-16-2 network, and the entry that picks the instance for a call.
 #include "rollout_deferred.cuh"
 
 namespace cp {
@@ -11,7 +10,6 @@ bool rollout_deferred_applies(const RolloutParams &p, int policy, bool streams) 
     if (!outputs_ok) return false;
     if (p.action_bits_in) return true;  // supplied actions replace whatever policy was named
     if (p.start_in) return policy == 0 || policy == 1 || policy == 6;
-    if (is_deep_network(policy)) return !streams && !p.max_steps;
     return policy == 0 || policy == 1 || policy == 2 || policy == 6;
 }
 
@@ -38,21 +36,20 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
     const int64_t warps64 = (p.n + 63) / 64, sms = sm_count();
     const bool two_warps = policy == 0 && !p.start_in && !p.reward_stream && warps64 > sms * 4 && warps64 <= sms * 8;
     const int by_length = p.T < 48u ? 2 : p.T < 192u || two_warps ? 4 : 6;
-    const int k = g_tuning.rollout_defer > 0 ? g_tuning.rollout_defer : (policy == 2 ? 2 : is_network(policy) ? 3 : by_length);
+    const int k = g_tuning.rollout_defer > 0 ? g_tuning.rollout_defer : (policy == 2 ? 2 : by_length);
     // the action hash folds the time's upper half into the lower one: nothing to do below 2^16
     const bool short_times = (uint64_t)p.t0 + p.T <= 65536u;
     // shared weights twice: one packed operand for both slots
     if (policy == 1)
         for (int i = 9; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
-    else if (is_network(policy))
-        screen_pairs(p, policy);
+    else if (policy == 2)
+        screen_pairs(p);
     if (p.action_bits_in || p.start_in) return launch_rollout_deferred_data(p, p.action_bits_in ? 3 : policy, k, contracted, s);
     switch (policy) {
         case 0: return short_times ? launch_limit<0, true>(p, k, contracted, s) : launch_limit<0, false>(p, k, contracted, s);
         case 1: return launch_limit<1, false>(p, k, contracted, s);
         case 2: return launch_limit<2, false>(p, k, contracted, s);
-        case 6: return launch_limit<6, false>(p, k, contracted, s);
-        default: return launch_rollout_deferred_deep(p, contracted, s);  // 7: weights already paired
+        default: return launch_limit<6, false>(p, k, contracted, s);
     }
 }
 

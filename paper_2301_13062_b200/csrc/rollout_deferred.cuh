@@ -28,8 +28,7 @@
 // arithmetic; with or without the episode step limit; per-step outputs either none or exactly the reward
 // plane + done bitmask (the action bitmask and the trajectory are rows of global time that half the
 // lanes would have to touch every step). The
-// 4-16-16-2 network too, for the plain call: no step limit, no per-step outputs. Everything else takes
-// the general kernel.
+// larger networks and everything else take the general kernel.
 //
 // No warp waits for another one and nothing spins: the loop's trip count is bounded by the
 // launch parameters (every trip block advances every unfinished slot by at least one step).
@@ -92,11 +91,6 @@ __device__ __forceinline__ void network_action_pair(const RolloutParams &p, cons
         }
     }
 }
-
-// The networks of this kernel: 4-16-2, and 4-16-16-2 for the plain call only — no step limit, no per-step
-// outputs, default trip spacing. (4-32-2 and 4-64-2 are faster in the general kernel at every size since
-// their trips are short: 1,000,000 x 100, there / here, 868 / 948 and 1,657 / 2,333 us.)
-__host__ __device__ constexpr bool is_deep_network(int policy) { return policy == 7; }
 
 // The done bit plane of a launch that sets its bits by atomic OR has to be zeroed first.
 // A warp that clears its own words inside the rollout writes 4 bytes into each of T separate
@@ -171,7 +165,7 @@ constexpr int kRing = 8;
 // one to three steps 347 / 480 / 252 and 1,307 / 3,640 / 2,356, 20 steps 285 / 134 / 137 and 1,098 / 588 / 596.
 constexpr int kMany = 40, kEnough = 24, kFew = 16;  // of the warp's 64
 
-// POLICY: 0 hashed actions, 1 shared linear policy, 2 / 7 a shared tanh network,
+// POLICY: 0 hashed actions, 1 shared linear policy, 2 the shared 4-16-2 network,
 // 3 supplied actions, 6 one linear policy per environment.
 // K: trips between restart passes. LIMIT: episodes are cut off after p.max_steps steps.
 // RD: the reward plane and the done bitmask are written (see the comment at reward_row).
@@ -384,7 +378,7 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
         // more than one step ahead of the trip counter, without it none ahead at all: the main part
         // of the loop relies on that) a slot that is already ahead does not look ahead, and neither
         // does one whose next step is its last.
-        // (Only for the network policies — config 5's episodes last 9 steps: 39.4 -> 38.0 ms.
+        // (Only for the network, whose episodes may be short: 16,777,216 x 200 with 9-step ones 39.4 -> 38.0 ms.
         // With hashed actions (22-step episodes) the saved waiting and the cost of the test in
         // every pass cancel — 1,048,576 x 500: 0.947 ms without, 0.956 ms with it — and with the
         // linear policies' 80-step episodes the test only costs: 4,194,304 x 100 with streams
@@ -483,10 +477,9 @@ __global__ void __launch_bounds__(256, is_network(POLICY) ? 4 : POLICY == 3 || S
             after_step(tail, 0, d0);
             after_step(tail, 1, d1);
         };
-        // The trips between two restart passes: K, or fewer where many slots wait. The 4-16-2 network's are
-        // unrolled up to three (4,194,304 x 200 at K = 2, 3, 4: 4,954 -> 4,842, 4,992 -> 4,915, 5,170 -> 5,569
-        // us), the deeper network's stay a loop (1,048,576 x 100: 1,528 -> 2,803).
-        constexpr int kUnroll = !is_network(POLICY) || (POLICY == 2 && K <= 3) ? K : 1;
+        // The trips between two restart passes: K, or fewer where many slots wait. The network's are
+        // unrolled up to three (4,194,304 x 200 at K = 2, 3, 4: 4,954 -> 4,842, 4,992 -> 4,915, 5,170 -> 5,569 us).
+        constexpr int kUnroll = !is_network(POLICY) || K <= 3 ? K : 1;
         auto trip_block = [&](auto tail) {  // returns the trips made
             int made = K;
             if (START_IN && (wide || early)) {
@@ -609,8 +602,6 @@ cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
     if (contracted) {  // the optional arithmetic comes at the default trip spacing only
         constexpr int kC = is_network(POLICY) ? 2 : 6;
         rollout_deferred_kernel<POLICY, kC, SHORT, LIMIT, RD, true><<<grid, block, 0, s>>>(p);
-    } else if constexpr (is_deep_network(POLICY)) {  // and so does the deeper network
-        rollout_deferred_kernel<POLICY, 3, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p);
     } else {
         switch (k) {
             case 2: rollout_deferred_kernel<POLICY, 2, SHORT, LIMIT, RD, false><<<grid, block, 0, s>>>(p); break;
@@ -626,16 +617,12 @@ cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
 
 template <int POLICY, bool SHORT>
 cudaError_t launch_limit(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
-    if constexpr (is_deep_network(POLICY)) {
-        return launch_k<POLICY, SHORT, false, false>(p, k, contracted, s);  // rollout_deferred_applies: nothing else gets here
-    } else {
-        const bool rd = p.reward_stream != nullptr;  // rollout_deferred_applies: then done_bits too, nothing else
-        if (p.max_steps)
-            return rd ? launch_k<POLICY, SHORT, true, true>(p, k, contracted, s)
-                      : launch_k<POLICY, SHORT, true, false>(p, k, contracted, s);
-        return rd ? launch_k<POLICY, SHORT, false, true>(p, k, contracted, s)
-                  : launch_k<POLICY, SHORT, false, false>(p, k, contracted, s);
-    }
+    const bool rd = p.reward_stream != nullptr;  // rollout_deferred_applies: then done_bits too, nothing else
+    if (p.max_steps)
+        return rd ? launch_k<POLICY, SHORT, true, true>(p, k, contracted, s)
+                  : launch_k<POLICY, SHORT, true, false>(p, k, contracted, s);
+    return rd ? launch_k<POLICY, SHORT, false, true>(p, k, contracted, s)
+              : launch_k<POLICY, SHORT, false, false>(p, k, contracted, s);
 }
 
 }  // namespace

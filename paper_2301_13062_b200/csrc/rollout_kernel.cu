@@ -44,7 +44,7 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // 1,000,000 0.99 to 1.03 and with reward and done bits 1.03 to 1.07, 4,000,000 with them 0.98 to 1.02, 16,777,216
     // without 0.95 to 0.99; 4-32-2 1.07 to 1.2 and 4-64-2 1.3 to 1.7 from 67,000 to 1,000,000; 4-16-16-2 1,000,000 0.92 to
     // 1.28, the latter where more estimates do not decide (contracted 0.88 to 1.13, 1,048,576 x 100 1.41 to 2.00 against 1.58 to 1.77 ms; defined
-    // logits in every step 1.94).
+    // logits in every step 1.94): the larger networks have no instance of it any more.
     // rollout_coop = 5 forces it wherever it applies, any other forced shape keeps the other kernels.
     // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
     // below, and where every sort of data that was tried gains or nearly (time of this kernel over the
@@ -71,7 +71,6 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     const bool streams_gain = !streams || (p.start_in ? p.n * (int64_t)p.T <= 100000000 : warps64 >= sms * 7);
     int64_t least = sms * 4;  // 64-env warps
     if (policy == 2) least = sms * 448;
-    if (policy == 4 || policy == 5 || policy == 7) least = INT64_MAX;
     if ((policy == 0 || policy == 1) && p.T >= 192u) least = sms * 7 / 2;
     const bool enough = data ? p.T >= from && warps32 > sms * 10 && streams_gain && !(p.max_steps && p.max_steps < 12u)
                              : warps64 >= least && p.T >= 12u;

@@ -19,7 +19,7 @@
 // are stepped by the packed float32 instructions of sm_100a (euler_step_pair). Batches that fill
 // the chip mostly go to the deferred-restart kernel of rollout_deferred.cu instead; this
 // kernel keeps every call that one does not cover (action bit stream or trajectory written, the
-// 4-32-2 and 4-64-2 networks, the deeper one with a step limit or outputs, very short launches, batches too
+// larger networks on batches beyond the lane-split kernel's, very short launches, batches too
 // small to fill the chip, supplied actions or start states where that kernel does not gain) and is the form the others are compared with bit for bit.
 //
 // This header holds the kernel template and its dispatch; rollout_kernel.cu and

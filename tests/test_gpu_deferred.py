@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-WIDE = (inputs.POLICY_MLP32, inputs.POLICY_MLP64, inputs.POLICY_MLP_DEEP)  # 4-32-2, 4-64-2, 4-16-16-2
+LARGER = (inputs.POLICY_MLP32, inputs.POLICY_MLP64, inputs.POLICY_MLP_DEEP)  # 4-32-2, 4-64-2, 4-16-16-2
 GENERAL = (2, 1)   # two envs per thread, restarts by the whole warp after every step
 DEFERRED = (2, 5)
 
@@ -47,7 +47,7 @@ def make_policy(cp, kind, n):
     if kind in (1, 2):
         w = inputs.policy_weights(kind, kind)
         return cp.policy(kind, w), w
-    if kind in WIDE:  # weight draws for which the network uses both actions
+    if kind in LARGER:  # weight draws for which the network uses both actions
         w = inputs.policy_weights(kind, 7 if kind == inputs.POLICY_MLP_DEEP else 3)
         return cp.policy(kind, w), w
     w = inputs.per_env_linear_weights(n, 11)
@@ -88,24 +88,33 @@ def test_same_bits_as_the_general_kernel(cp, kind, n, T, t0, off, limit):
     assert n < 4000 or not np.array_equal(want_c["final_state"], want["final_state"])
 
 
-@pytest.mark.parametrize("kind", WIDE)
+@pytest.mark.parametrize("kind", LARGER)
 @pytest.mark.parametrize("n,T,t0,off", [(1, 1, 0, 0), (63, 2, 0, 5), (4099, 61, 3, 77), (70001, 120, 0, 0),
                                         (20000, 90, 70000, 1 << 20)])
-def test_wider_and_deeper_networks_same_bits_as_the_general_kernel(cp, kind, n, T, t0, off):
-    """The deferred kernel covers these networks for the plain call (no step limit, no per-step
-    outputs), in both arithmetics; with a limit the call must still come out right (it takes the
-    general kernel)."""
+def test_larger_networks_same_bits_as_two_environments_per_thread(cp, kind, n, T, t0, off):
+    """The deferred kernel does not cover these networks: asked for, such a call takes the general kernel. By
+    default they take the lane-split kernel (the three small batches) or the general kernel's per-lane restarts,
+    with and without per-step outputs; both must give the bits of its two environments per thread."""
     pol, _ = make_policy(cp, kind, n)
+    streams = {"reward_stream": lambda: torch.full((T, n), -7.0, device="cuda"),
+               "done_bits": lambda: torch.full((T, (n + 31) // 32), -1, dtype=torch.int32, device="cuda"),
+               "action_bits": lambda: torch.full((T, (n + 31) // 32), -1, dtype=torch.int32, device="cuda")}
     for arith in (cp.CP_ARITH_EXACT, cp.CP_ARITH_CONTRACTED):
         for limit in (0, 17):
-            kw = dict(n_envs=n, T=T, seed=8, t0=t0, env_offset=off, policy=pol, max_episode_steps=limit, arithmetic=arith)
-            want = run(cp, GENERAL, 0, **kw)
-            before = cp.cp_launch_count()
-            got = run(cp, DEFERRED, 0, **kw)
-            assert cp.cp_launch_count() - before == 1
-            for key in want:
-                assert np.array_equal(want[key], got[key]), (key, arith, limit)
-        assert want["ep_count"].max() > 0 or T < 8
+            for names in ((), ("reward_stream", "done_bits"), tuple(streams)):
+                res = {}
+                for shape in (GENERAL, DEFERRED, H.DEFAULT):
+                    out = {**outputs(n), **{k: streams[k]() for k in names}}
+                    with H.rollout_shape(cp, *shape):
+                        before = cp.cp_launch_count()
+                        cp.cp_rollout_ex(n_envs=n, T=T, seed=8, t0=t0, env_offset=off, policy=pol, max_episode_steps=limit,
+                                         arithmetic=arith, **out)
+                        assert cp.cp_launch_count() - before == 1
+                    res[shape] = fetch(out)
+                for shape in (DEFERRED, H.DEFAULT):
+                    for key in res[GENERAL]:
+                        assert np.array_equal(res[GENERAL][key], res[shape][key]), (key, arith, limit, names, shape)
+                assert res[GENERAL]["ep_count"].max() > 0 or T < 8
 
 
 @pytest.mark.parametrize("kind", [0, 1, 2])
@@ -148,11 +157,11 @@ def test_chunks_from_a_callers_states(cp, kind, limit, streams, n):
     assert sum(int(c["ep_count"].sum()) for c in results["deferred"][0::2]) > n // 4
 
 
-@pytest.mark.parametrize("kind", [0, 1, 2, 6, *WIDE])
+@pytest.mark.parametrize("kind", [0, 1, 2, 6, *LARGER])
 def test_returns_against_the_oracle(cp, oracle, kind):
     n, T, seed = 50001, 300, 2
     pol, w = make_policy(cp, kind, n)
-    r = run(cp, DEFERRED, 0, n_envs=n, T=T, seed=seed, policy=pol)
+    r = run(cp, H.DEFAULT if kind in LARGER else DEFERRED, 0, n_envs=n, T=T, seed=seed, policy=pol)
     o = oracle.rollout(n, T, seed, inputs.POLICY_LINEAR_PER_ENV if kind == 6 else kind, w, final_state=True,
                        min_gap=True, nthreads=8)
     excuse = (o["min_gap"] < 1e-5) if kind else None
