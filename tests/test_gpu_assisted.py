@@ -1,8 +1,8 @@
 """The producer-assisted rollout kernel (very small batches: a helper warp hashes actions and start
 states ahead of each stepping warp). It must give the same bits as the general kernel, which the
 other files pin to the oracle, and it is compared with the oracle directly as well. Cases: ragged
-batch sizes, horizons around the 16- and 32-step hand-overs, both lengths of a hand-over (32 steps up to five
-warp tasks per SM, 16 beyond) under every policy and output, a caller's initial state with angles
+batch sizes, horizons around the 16- and 32-step hand-overs, both lengths of a hand-over on either side of every
+size and horizon at which the choice changes, under every policy and output, a caller's initial state with angles
 outside the polynomial range, carried episode lengths and the step limit."""
 import numpy as np
 import pytest
@@ -54,7 +54,7 @@ def assert_same_bits(a, b):
 
 
 @pytest.mark.parametrize("n", [1, 33, 1000, 4737])
-@pytest.mark.parametrize("T", [1, 15, 16, 17, 32, 33, 100])
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 32, 33, 100, 200])
 def test_same_bits_as_general_kernel_and_oracle(cp, oracle, n, T):
     seed, t0, off = 12, 5, 77
     general = rollout(cp, PER_LANE, n, T, seed, t0=t0, env_offset=off)
@@ -119,11 +119,14 @@ ALL = ("done_bits", "action_bits", "reward_stream", "trajectory")
 @pytest.mark.parametrize("limit", [0, 12])
 @pytest.mark.parametrize("contracted", [False, True])
 def test_both_hand_over_lengths(cp, kind, limit, contracted):
-    """One batch on either side of the size from which a hand-over holds 16 steps instead of 32, forced and as a
-    caller gets it: no outputs, the reward plane and done bits alone, one output tested for, and all of them."""
+    """Hand-overs of 16 and of 32 steps on either side of every line between them (24, 64 and 192 steps, two and five
+    warp tasks per SM), forced and as a caller gets it: no outputs, the reward plane and done bits alone, one output
+    tested for, and all of them."""
     from paper_2301_13062_b200 import inputs
-    last_long = torch.cuda.get_device_properties(0).multi_processor_count * 5 * 32
-    for n, T in ((last_long, 33), (last_long + 1, 17), (last_long + 1, 33), (last_long + 3321, 16)):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    two, five = sms * 2 * 32, sms * 5 * 32
+    for n, T in ((97, 23), (97, 24), (two, 65), (two, 191), (two, 192), (two + 1, 63), (two + 1, 65), (five, 33), (five, 65),
+                 (five + 1, 17), (five + 1, 65), (five + 3321, 16)):
         kw = {"t0": 4, "env_offset": 3, "max_episode_steps": limit,
               "arithmetic": cp.CP_ARITH_CONTRACTED if contracted else cp.CP_ARITH_EXACT}
         if kind == "supplied":
