@@ -65,11 +65,21 @@ __device__ __forceinline__ void pair_barrier(uint32_t pair) {
         asm volatile("bar.sync 2, 64;" ::: "memory");
 }
 
-// Pairs per CTA: one, but two, whose first two warps step, for supplied start states without per-step
-// outputs, whose helpers fetch instead of hashing (500 steps with supplied actions, 27,000 environments two / one:
-// 88.1 / 92.2 us, 45,000 130.9 / 138.5; with reward and done bits 111 / 113, 161 / 164, but 12,000 79.9 / 71.7).
-template <bool START_IN, int STREAMS>
-constexpr int kPairs = START_IN && STREAMS == 0 ? 2 : 1;
+// Pairs per CTA: one, but two, whose first two warps step, for supplied start states, whose helpers fetch instead of
+// hashing: without per-step outputs always (500 steps with supplied actions, 27,000 environments two / one: 88.1 /
+// 92.2 us, 45,000 130.9 / 138.5), and with the reward plane and done bits, in the contracted arithmetic also with all
+// outputs, beyond five pairs per SM where the fullest SM gets no more pairs that way (two_pairs). Time of one over two
+// there, actions supplied, hashed and by a policy per environment, 96, 200, 500 steps: reward and done bits, 26,001
+// environments 1.05-1.08, 1.05-1.09, 1.03-1.07, 36,001 1.00-1.03, 1.01-1.05, 1.00-1.04, 45,001 0.99-1.04, 1.04-1.08, 1.03-1.07;
+// all outputs, contracted 26,001 1.06-1.08, 1.07-1.09, 1.00-1.01, 45,001 1.06-1.07, 1.03-1.05, 0.95-0.97, canonical 0.94-0.98,
+// 1.01-1.02, 0.96-0.97 and 1.02-1.04, 1.00-1.02, 0.93-0.98. Where the fullest SM gets more, 33,100, 0.94-1.03, and below five
+// pairs 3,001 to 23,001 0.74-1.07 (mean 0.95). One shared linear policy 0.91-1.03 at all sizes: one pair.
+template <int POLICY, bool START_IN, bool CONTRACT, int STREAMS>
+constexpr bool kMayPair = START_IN && POLICY != 1 && (STREAMS == 1 || (STREAMS == 3 && CONTRACT));
+inline bool two_pairs(const RolloutParams &p) {
+    const int64_t sms = sm_count(), pairs = p.n_tasks, ctas = (pairs + 1) / 2;
+    return pairs > sms * 5 && (ctas + sms - 1) / sms * 2 == (pairs + sms - 1) / sms;
+}
 
 // Which of the two warps of a CTA of one pair steps (0 or 1). A warp's place among an SM's warps decides which of the four
 // schedulers it has: a CTA of two warps has schedulers 0 and 1 or 2 and 3. The first warp stepping
@@ -147,9 +157,8 @@ __device__ __forceinline__ void consume_step(const RolloutParams &p, const PairB
 
 // START_IN: the start states are the caller's data and may hold any angle.
 // kChunk: steps per hand-over.
-template <int POLICY, bool START_IN, int kChunk, bool LIMIT, bool CONTRACT, int STREAMS>
-__global__ void __launch_bounds__(64 * kPairs<START_IN, STREAMS>) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
-    constexpr int PAIRS = kPairs<START_IN, STREAMS>;
+template <int POLICY, bool START_IN, int PAIRS, int kChunk, bool LIMIT, bool CONTRACT, int STREAMS>
+__global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
     __shared__ PairBuffers<kChunk> s_buf[PAIRS];
     __shared__ uint32_t s_stepping;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -313,14 +322,20 @@ __global__ void __launch_bounds__(64 * kPairs<START_IN, STREAMS>) rollout_assist
     }
 }
 
+template <int POLICY, bool START_IN, int PAIRS, int CHUNK, bool CONTRACT, int STREAMS>
+void launch_assisted_pairs(const RolloutParams &p, cudaStream_t s) {
+    const unsigned grid = (unsigned)((p.n_tasks + PAIRS - 1) / PAIRS);
+    if (p.max_steps)
+        rollout_assisted_kernel<POLICY, START_IN, PAIRS, CHUNK, true, CONTRACT, STREAMS><<<grid, 64 * PAIRS, 0, s>>>(p);
+    else
+        rollout_assisted_kernel<POLICY, START_IN, PAIRS, CHUNK, false, CONTRACT, STREAMS><<<grid, 64 * PAIRS, 0, s>>>(p);
+}
 template <int POLICY, bool START_IN, int CHUNK, bool CONTRACT, int STREAMS>
 void launch_assisted_limit(const RolloutParams &p, cudaStream_t s) {
-    constexpr int pairs = kPairs<START_IN, STREAMS>;
-    const unsigned grid = (unsigned)((p.n_tasks + pairs - 1) / pairs);
-    if (p.max_steps)
-        rollout_assisted_kernel<POLICY, START_IN, CHUNK, true, CONTRACT, STREAMS><<<grid, 64 * pairs, 0, s>>>(p);
-    else
-        rollout_assisted_kernel<POLICY, START_IN, CHUNK, false, CONTRACT, STREAMS><<<grid, 64 * pairs, 0, s>>>(p);
+    if constexpr (kMayPair<POLICY, START_IN, CONTRACT, STREAMS>) {
+        if (two_pairs(p)) return launch_assisted_pairs<POLICY, START_IN, 2, CHUNK, CONTRACT, STREAMS>(p, s);
+    }
+    launch_assisted_pairs<POLICY, START_IN, START_IN && STREAMS == 0 ? 2 : 1, CHUNK, CONTRACT, STREAMS>(p, s);
 }
 template <int POLICY, bool START_IN, int CHUNK, bool CONTRACT>
 void launch_assisted_streams(const RolloutParams &p, cudaStream_t s) {

@@ -143,6 +143,28 @@ def test_both_hand_over_lengths(cp, kind, limit, contracted):
                 assert_same_bits(rollout(cp, coop, n, T, 6, streams=streams, **kw), general)
 
 
+@pytest.mark.parametrize("kind", ["hashed", "supplied", "per_env"])
+@pytest.mark.parametrize("contracted", [False, True])
+def test_two_pairs_per_block_with_outputs(cp, kind, contracted):
+    """Supplied start states with per-step outputs on either side of the sizes at which a block gets two pairs: the
+    last of five pairs per SM, the odd and even counts of pairs after it, and where two would load an SM more."""
+    from paper_2301_13062_b200 import inputs
+    sms, T = torch.cuda.get_device_properties(0).multi_processor_count, 97
+    for n in (sms * 160, sms * 160 + 1, sms * 160 + 33, sms * 192, sms * 192 + 1):
+        starts = torch.rand(T, 4, n, device="cuda", generator=torch.Generator("cuda").manual_seed(n)) * 0.1 - 0.05
+        kw = {"t0": 4, "env_offset": 3, "max_episode_steps": 15 * (n % 2), "start_states_in": starts,
+              "arithmetic": cp.CP_ARITH_CONTRACTED if contracted else cp.CP_ARITH_EXACT}
+        if kind == "supplied":
+            bits = np.random.default_rng(n).integers(0, 1 << 32, (T, (n + 31) // 32), dtype=np.uint64)
+            kw["action_bits_in"] = torch.from_numpy(bits.astype(np.uint32).view(np.int32)).cuda()
+        elif kind == "per_env":
+            kw["policy"] = cp.policy(cp.CP_POLICY_LINEAR_PER_ENV, torch.from_numpy(inputs.per_env_linear_weights(n, 3)).cuda())
+        for streams in (("reward_stream", "done_bits"), ALL):
+            general = rollout(cp, PER_LANE, n, T, 6, streams=streams, **kw)
+            for coop in (ASSISTED, 0):
+                assert_same_bits(rollout(cp, coop, n, T, 6, streams=streams, **kw), general)
+
+
 def test_forced_on_a_large_batch_and_at_the_end_of_time(cp, oracle):
     """Far more pairs than fit on the chip at once (CTAs in waves), and the last steps the
     32-bit step counter allows (the counter 4 * (t + 1) of the last start state wraps to 0 on
