@@ -33,15 +33,18 @@ namespace {
 // pairs share an SM, 20 KB beyond that. (2,048 x 10,000 at 8, 16, 32 steps: 0.543, 0.512, 0.481 ms; 500 steps on
 // 17,000 environments, supplied actions, 32 / 16 steps: 41.0 / 45.0 us; on 27,000, where five pairs
 // of 32 steps fill an SM and the sixth waits, 71.5 / 63.5.) Nothing is stepped before the first hand-over, so a launch
-// of 24 to 63 steps takes the short one, and up to 191 with at most two pairs per SM, where the helpers have
+// of 32 to 63 steps takes the short one, and one of 24 to 127 with at most two pairs per SM, where the helpers have
 // schedulers to themselves. 32 over 16 steps per hand-over, all policies, without outputs, with reward and done bits
 // and with all outputs, at T = 17, 24, 32, 48, 64, 96, 128, 200, 500: 3,001 to 9,001 environments 0.96-1.00, 1.02-1.08,
 // 1.08-1.16, 1.06-1.13, 1.03-1.09, 1.01-1.06, 0.99-1.05, 0.95-1.03, 0.92-1.01; 11,001 to 18,001 0.96-0.99, 0.98-1.03,
-// 1.01-1.09, 1.00-1.05, 0.94-1.02, 0.94-1.03, 0.95-1.08, 0.95-1.07, 0.94-1.06.
+// 1.01-1.09, 1.00-1.05, 0.94-1.02, 0.94-1.03, 0.95-1.08, 0.95-1.07, 0.94-1.06. The contracted arithmetic, whose step is
+// shorter, waits for its helper sooner: up to 9,001 environments 0.98-1.12 at 50 steps, 0.94-1.03 at 150, so up to 95
+// there, and 0.94-1.06 at 50 steps on 14,001 and 23,001, so never beyond two pairs.
 constexpr int kLongChunk = 32, kShortChunk = 16;
-inline bool long_chunks(const RolloutParams &p) {
+inline bool long_chunks(const RolloutParams &p, bool contracted) {
     const int64_t sms = sm_count();
-    return p.n_tasks <= sms * 5 && (p.T < 24u || p.T >= (p.n_tasks <= sms * 2 ? 192u : 64u));
+    if (p.n_tasks <= sms * 2) return p.T < 24u || p.T >= (contracted ? 96u : 128u);
+    return p.n_tasks <= sms * 5 && (contracted || p.T < 32u || p.T >= 64u);
 }
 
 // Steps per trip of the consumer's loop over a chunk. Measured on 2,048 x 10,000 (ms per launch):
@@ -352,7 +355,7 @@ void launch_assisted_streams(const RolloutParams &p, cudaStream_t s) {
 // Supplied start states come in short chunks at all sizes (build time).
 template <int POLICY, bool START_IN>
 void launch_assisted_chunk(const RolloutParams &p, bool contracted, cudaStream_t s) {
-    if (!START_IN && long_chunks(p)) {
+    if (!START_IN && long_chunks(p, contracted)) {
         contracted ? launch_assisted_streams<POLICY, START_IN, START_IN ? kShortChunk : kLongChunk, true>(p, s)
                    : launch_assisted_streams<POLICY, START_IN, START_IN ? kShortChunk : kLongChunk, false>(p, s);
     } else {

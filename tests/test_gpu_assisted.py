@@ -119,13 +119,14 @@ ALL = ("done_bits", "action_bits", "reward_stream", "trajectory")
 @pytest.mark.parametrize("limit", [0, 12])
 @pytest.mark.parametrize("contracted", [False, True])
 def test_both_hand_over_lengths(cp, kind, limit, contracted):
-    """Hand-overs of 16 and of 32 steps on either side of every line between them (24, 64 and 192 steps, two and five
-    warp tasks per SM), forced and as a caller gets it: no outputs, the reward plane and done bits alone, one output
+    """Hand-overs of 16 and of 32 steps on either side of every line between them (24, 32, 64, 96 and 128 steps, two and
+    five warp tasks per SM), forced and as a caller gets it: no outputs, the reward plane and done bits alone, one output
     tested for, and all of them."""
     from paper_2301_13062_b200 import inputs
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     two, five = sms * 2 * 32, sms * 5 * 32
-    for n, T in ((97, 23), (97, 24), (two, 65), (two, 191), (two, 192), (two + 1, 63), (two + 1, 65), (five, 33), (five, 65),
+    for n, T in ((97, 23), (97, 24), (two, 65), (two, 95), (two, 97), (two, 127), (two, 129), (two + 1, 31), (two + 1, 33),
+                 (two + 1, 63), (two + 1, 65), (five, 33), (five, 65),
                  (five + 1, 17), (five + 1, 65), (five + 3321, 16)):
         kw = {"t0": 4, "env_offset": 3, "max_episode_steps": limit,
               "arithmetic": cp.CP_ARITH_CONTRACTED if contracted else cp.CP_ARITH_EXACT}
