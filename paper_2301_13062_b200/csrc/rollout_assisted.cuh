@@ -70,18 +70,20 @@ __device__ __forceinline__ void pair_barrier(uint32_t pair) {
 
 // Pairs per CTA: one, but two, whose first two warps step, for supplied start states, whose helpers fetch instead of
 // hashing: without per-step outputs always (500 steps with supplied actions, 27,000 environments two / one: 88.1 /
-// 92.2 us, 45,000 130.9 / 138.5), and with the reward plane and done bits, in the contracted arithmetic also with all
-// outputs, beyond five pairs per SM where the fullest SM gets no more pairs that way (two_pairs). Time of one over two
-// there, actions supplied, hashed and by a policy per environment, 96, 200, 500 steps: reward and done bits, 26,001
-// environments 1.05-1.08, 1.05-1.09, 1.03-1.07, 36,001 1.00-1.03, 1.01-1.05, 1.00-1.04, 45,001 0.99-1.04, 1.04-1.08, 1.03-1.07;
-// all outputs, contracted 26,001 1.06-1.08, 1.07-1.09, 1.00-1.01, 45,001 1.06-1.07, 1.03-1.05, 0.95-0.97, canonical 0.94-0.98,
-// 1.01-1.02, 0.96-0.97 and 1.02-1.04, 1.00-1.02, 0.93-0.98. Where the fullest SM gets more, 33,100, 0.94-1.03, and below five
-// pairs 3,001 to 23,001 0.74-1.07 (mean 0.95). One shared linear policy 0.91-1.03 at all sizes: one pair.
+// 92.2 us, 45,000 130.9 / 138.5), and with the reward plane and done bits, in the contracted arithmetic up to 256 steps
+// also with all outputs, beyond five pairs per SM where the fullest SM gets no more pairs that way (two_pairs). Time of
+// one over two there, actions supplied, hashed and by a policy per environment, 96, 200, 500 steps: reward and done bits,
+// 26,001 environments 1.05-1.08, 1.05-1.09, 1.03-1.07, 36,001 1.00-1.03, 1.01-1.05, 1.00-1.04, 45,001 0.99-1.04, 1.04-1.08,
+// 1.03-1.07; all outputs, contracted 26,001 1.06-1.08, 1.07-1.09, 0.94-1.01, 45,001 1.06-1.07, 1.03-1.05, 0.92-0.97, canonical
+// 0.94-0.98, 1.01-1.02, 0.96-0.97 and 1.02-1.04, 1.00-1.02, 0.93-0.98. Where the fullest SM gets more, 33,100, 0.94-1.03, and
+// below five pairs 3,001 to 23,001 0.74-1.07 (mean 0.95). One shared linear policy with reward and done bits: canonical
+// 0.94-1.03, one pair; contracted 26,001 and 45,001 x 200 1.05-1.06.
 template <int POLICY, bool START_IN, bool CONTRACT, int STREAMS>
-constexpr bool kMayPair = START_IN && POLICY != 1 && (STREAMS == 1 || (STREAMS == 3 && CONTRACT));
-inline bool two_pairs(const RolloutParams &p) {
+constexpr bool kMayPair = START_IN && (STREAMS == 1 ? POLICY != 1 || CONTRACT : STREAMS == 3 && CONTRACT && POLICY != 1);
+template <int STREAMS>
+bool two_pairs(const RolloutParams &p) {
     const int64_t sms = sm_count(), pairs = p.n_tasks, ctas = (pairs + 1) / 2;
-    return pairs > sms * 5 && (ctas + sms - 1) / sms * 2 == (pairs + sms - 1) / sms;
+    return pairs > sms * 5 && (ctas + sms - 1) / sms * 2 == (pairs + sms - 1) / sms && (STREAMS != 3 || p.T <= 256u);
 }
 
 // Which of the two warps of a CTA of one pair steps (0 or 1). A warp's place among an SM's warps decides which of the four
@@ -336,7 +338,7 @@ void launch_assisted_pairs(const RolloutParams &p, cudaStream_t s) {
 template <int POLICY, bool START_IN, int CHUNK, bool CONTRACT, int STREAMS>
 void launch_assisted_limit(const RolloutParams &p, cudaStream_t s) {
     if constexpr (kMayPair<POLICY, START_IN, CONTRACT, STREAMS>) {
-        if (two_pairs(p)) return launch_assisted_pairs<POLICY, START_IN, 2, CHUNK, CONTRACT, STREAMS>(p, s);
+        if (two_pairs<STREAMS>(p)) return launch_assisted_pairs<POLICY, START_IN, 2, CHUNK, CONTRACT, STREAMS>(p, s);
     }
     launch_assisted_pairs<POLICY, START_IN, START_IN && STREAMS == 0 ? 2 : 1, CHUNK, CONTRACT, STREAMS>(p, s);
 }

@@ -144,7 +144,7 @@ def test_both_hand_over_lengths(cp, kind, limit, contracted):
                 assert_same_bits(rollout(cp, coop, n, T, 6, streams=streams, **kw), general)
 
 
-@pytest.mark.parametrize("kind", ["hashed", "supplied", "per_env"])
+@pytest.mark.parametrize("kind", ["hashed", "supplied", "linear", "per_env"])
 @pytest.mark.parametrize("contracted", [False, True])
 def test_two_pairs_per_block_with_outputs(cp, kind, contracted):
     """Supplied start states with per-step outputs on either side of the sizes at which a block gets two pairs: the
@@ -158,6 +158,8 @@ def test_two_pairs_per_block_with_outputs(cp, kind, contracted):
         if kind == "supplied":
             bits = np.random.default_rng(n).integers(0, 1 << 32, (T, (n + 31) // 32), dtype=np.uint64)
             kw["action_bits_in"] = torch.from_numpy(bits.astype(np.uint32).view(np.int32)).cuda()
+        elif kind == "linear":
+            kw["policy"] = cp.policy(cp.CP_POLICY_LINEAR, inputs.policy_weights(cp.CP_POLICY_LINEAR, 4))
         elif kind == "per_env":
             kw["policy"] = cp.policy(cp.CP_POLICY_LINEAR_PER_ENV, torch.from_numpy(inputs.per_env_linear_weights(n, 3)).cuda())
         for streams in (("reward_stream", "done_bits"), ALL):
