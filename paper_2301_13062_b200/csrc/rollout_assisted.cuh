@@ -105,6 +105,15 @@ __device__ __forceinline__ uint32_t stepping_warp(uint32_t &shared) {
     return shared;
 }
 
+// Instances that take the role, which comes from shared memory, once more from a lane of the warp, as a value that the
+// compiler sees to be the same for all lanes. With / without, 150 and 400 or 500 steps, 2,001 to 30,001 environments:
+// a policy per environment and the shared linear one, action bits among the outputs 0.90-0.96, all outputs canonical
+// 0.90-1.04, contracted 0.88-1.14; reward and done bits, a policy per environment 0.89-1.00, hashed and supplied actions
+// canonical 0.93-1.01, contracted 0.93-1.03, the shared linear policy 0.98-1.09; without outputs 0.95-1.05.
+template <int POLICY, bool START_IN, bool CONTRACT, int STREAMS>
+constexpr bool kUniformRole = !START_IN && (POLICY == 0 ? STREAMS == 1 && !CONTRACT
+                                                        : STREAMS == 2 || (STREAMS == 3 && !CONTRACT) || (STREAMS == 1 && POLICY == 6));
+
 // Where the consumer's per-step outputs go (only read when STREAMS; NULL = not wanted): one pointer
 // per output, advanced by a row per step.
 struct StreamCursor {
@@ -168,9 +177,14 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
     __shared__ uint32_t s_stepping;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     bool producer;
-    if constexpr (PAIRS == 1) producer = warp != stepping_warp(s_stepping);
-    else producer = warp >= (uint32_t)PAIRS;
-    const uint32_t pair = PAIRS == 1 ? 0u : warp % PAIRS;
+    uint32_t pair = 0u;
+    if constexpr (PAIRS == 1) {
+        producer = warp != stepping_warp(s_stepping);
+        if constexpr (kUniformRole<POLICY, START_IN, CONTRACT, STREAMS>) producer = __shfl_sync(0xffffffffu, (int)producer, 0) != 0;
+    } else {
+        producer = warp >= (uint32_t)PAIRS;
+        pair = producer ? warp - PAIRS : warp;  // (not warp % PAIRS: 9,401 x 400, step limit, start states given, 41.9 / 44.8 us)
+    }
     const int64_t task = (int64_t)blockIdx.x * PAIRS + pair;
     // Both warps of a pair leave here together, before their first barrier; no other pair uses
     // their barrier. Nothing that differs between the two warps of a pair (or between lanes) may
