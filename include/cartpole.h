@@ -336,8 +336,8 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * and start state ahead into shared memory, or fetches the supplied ones (hashed or supplied
  * actions and the linear policies; otherwise as 2), 2, 3 and 4 only with one environment per
  * thread; 0 = default: helper warps for up to ten warps of environments per SM (a linear policy's
- * shortest launches aside), the hidden units of a network spread over several lanes for up to two and a
- * half warps per scheduler and from 3 to 8 steps on, per lane for
+ * shortest launches aside), the hidden units of a network spread over several lanes for up to one, two or three
+ * warps per scheduler by network, outputs and steps, and from 3 to 8 steps on, per lane for
  * other batches too small to fill the GPU (ahead for the smaller ones), deferred (5) from one
  * 64-environment warp per scheduler on (37,825 environments on 148 SMs; 33,089 with hashed actions or the shared
  * linear policy from 192 steps on; the 4-16-2 network on the largest batches) where that form applies,

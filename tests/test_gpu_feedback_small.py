@@ -2,8 +2,8 @@
 (linear policies, supplied starts) and the network kernel that spreads hidden units over lanes. Both
 must give the bits of the general kernel's per-lane shape, which the other files pin to the oracle.
 Sizes: around the 32 environments of a bit-plane word, odd warp tasks, and either side of the bounds
-at which the network kernel takes more lanes or leaves the call (148 SMs: 1,184, 2,368, 4,736 and
-9,472 environments). Horizons: around the 32-step hand-overs of both kernels."""
+at which the network kernel takes more lanes or leaves the call (148 SMs: 2,368, 4,736, 9,472 and 14,208
+environments). Horizons: around the 32-step hand-overs of both kernels."""
 import numpy as np
 import pytest
 
@@ -77,7 +77,7 @@ def start_rows(T, n):
 
 @pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
 @pytest.mark.parametrize("n,T", [(1, 33), (31, 64), (33, 5), (1184, 40), (1185, 31), (2369, 32), (4737, 31),
-                                 (9465, 65), (9472, 33), (9473, 33)])
+                                 (9465, 65), (9472, 33), (9473, 33), (9473, 129), (14208, 129), (14209, 129)])
 def test_networks(cp, kind, n, T):
     for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("done_bits",), 0, "edge"), (("trajectory",), 9, None)):
         args = dict(streams=streams, limit=limit, spread=spread)
@@ -85,11 +85,17 @@ def test_networks(cp, kind, n, T):
 
 
 @pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
-@pytest.mark.parametrize("n", [97, 1500, 4097])
-def test_networks_contracted_and_supplied_starts(cp, kind, n):
-    for streams in ((), ALL):
+@pytest.mark.parametrize("n,T", [(97, 50), (1500, 50), (4097, 50), (9473, 64), (14208, 128), (14209, 128)])
+def test_networks_contracted(cp, kind, n, T):
+    for streams in ((), ALL, ("reward_stream", "done_bits")):
         args = dict(streams=streams, limit=15, contracted=True)
-        assert_same_bits(rollout(cp, 0, kind, n, 50, **args), rollout(cp, 2, kind, n, 50, **args))
+        assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
+
+
+@pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
+@pytest.mark.parametrize("n", [97, 1500, 4097])
+def test_networks_from_supplied_starts(cp, kind, n):
+    for streams in ((), ALL):
         args = dict(streams=streams, starts=start_rows(50, n), spread="edge")
         assert_same_bits(rollout(cp, 0, kind, n, 50, **args), rollout(cp, 2, kind, n, 50, **args))
 
