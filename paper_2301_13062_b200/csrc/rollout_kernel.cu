@@ -27,24 +27,27 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // without one (3, the name the kernels have for it). A network named beside them used to bring its own
     // spacing of the restart passes and its weights, paired, into the launch.
     if (p.action_bits_in) policy = 3;
-    // a network policy on a batch that leaves schedulers idle, or with outputs that the deferred kernel
-    // does not write: its hidden units spread over several lanes (rollout_lanes.cu)
+    // a network policy on a batch that leaves schedulers idle: its hidden units spread over several lanes
+    // (rollout_lanes.cu)
     if (const int lanes = rollout_lanes_for(p, policy, streams, contracted))
         return launch_rollout_lanes(p, policy, lanes, streams, contracted, s);
     // The deferred-restart kernel (rollout_deferred.cu) by default: from one 64-env warp per
-    // scheduler on (37,888 envs on 148 SMs) for hashed actions and the linear policies, launches of at
+    // scheduler on (37,825 envs on 148 SMs) for hashed actions and the linear policies, launches of at
     // least a dozen steps, per-step outputs none or reward plane + done bits. Measured at T = 500, this kernel
     // against the general one: hashed actions 65,536 envs 0.098 / 0.142 ms, 131,072 0.163 / 0.251; linear policy
     // 47,360 0.088 / 0.100, 131,072 0.154 / 0.212. Against the helper warps, hashed actions and the shared linear
-    // policy gain from eight pairs of theirs per SM on, in launches of 192 steps and more (37,800 envs: x 500
-    // 55 / 72 and 64 / 72 us, with reward and done bits 72 / 82 and 80 / 88, x 96 16.4 / 18.4 and 24.6 / 20.7;
-    // 28,000 x 500 with outputs 74 / 64; one linear policy each 70 / 74, but with outputs 92 / 84).
+    // policy gain from 33,089 environments on (three and a half 64-env warps per SM), in launches of 192 steps and more
+    // (this kernel's time over theirs, 33,100 envs x 200 / 500: 0.85 / 0.75 and 0.72 / 0.69, with reward and done bits
+    // 1.01 / 0.88 and 0.78 / 0.72, contracted 0.77 / 0.69 and 0.62 / 0.60, 1.02 / 0.88 and 0.77 / 0.72; 37,800 x 96 16.4 / 18.4
+    // and 24.6 / 20.7 us; 28,000 x 500 with outputs 74 / 64; one linear policy each 70 / 74, but with outputs 92 / 84).
     // The networks' trips are short next to their waits since the estimate decides (policy_screen.cuh). This
-    // kernel's time over the general one's, three policies each, T = 100 .. 400: 4-16-2 200,003 envs 0.98 to 1.04,
-    // 1,000,000 0.99 to 1.03 and with reward and done bits 1.03 to 1.07, 4,000,000 with them 0.98 to 1.02, 16,777,216
-    // without 0.95 to 0.99; 4-32-2 1.07 to 1.2 and 4-64-2 1.3 to 1.7 from 67,000 to 1,000,000; 4-16-16-2 1,000,000 0.92 to
-    // 1.28, the latter where more estimates do not decide (contracted 0.88 to 1.13, 1,048,576 x 100 1.41 to 2.00 against 1.58 to 1.77 ms; defined
-    // logits in every step 1.94): the larger networks have no instance of it any more.
+    // kernel's time over the general one's, three policies each: 4-16-2 x 100 1,000,003 envs 0.99 to 1.01, 2,000,003 0.97
+    // to 0.99, 4,200,001 0.96 to 0.98, 16,777,216 0.95 to 0.97, contracted 0.96 to 0.98, 0.94 to 0.96, 0.93 to 0.95, 0.92 to
+    // 0.94; with reward and done bits x 40 1.02 to 1.05, 1.00 to 1.03, 0.99 to 1.01, 0.98 to 1.01, contracted 1.00 to 1.03,
+    // 0.99 to 1.01, 0.97 to 1.00, 0.96 to 0.99: from 4.24 million on no form loses more than 1 %. T = 100 .. 400, 4-32-2
+    // 1.07 to 1.2 and 4-64-2 1.3 to 1.7 from 67,000 to 1,000,000, 4-16-16-2 at 1,000,000 0.92 to 1.28, the latter where
+    // more estimates do not decide (contracted 0.88 to 1.13; 1,048,576 x 100 1.41 to 2.00 against 1.58 to 1.77 ms, defined
+    // logits in every step 1.94): the larger networks have no instance of it.
     // rollout_coop = 5 forces it wherever it applies, any other forced shape keeps the other kernels.
     // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
     // below, and where every sort of data that was tried gains or nearly (time of this kernel over the

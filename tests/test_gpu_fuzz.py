@@ -49,9 +49,15 @@ def test_random_combination_in_the_default_shape(cp, oracle, case):
     check_combination(cp, oracle, case, H.DEFAULT)
 
 
-def check_combination(cp, oracle, case, forced):
+@pytest.mark.parametrize("case", range(700, 718))
+def test_random_combination_on_larger_batches(cp, oracle, case):
+    """The same at sizes that the kernels for small batches hand over to one another or to the larger ones'."""
+    check_combination(cp, oracle, case, H.DEFAULT, [9473, 14207, 23681, 33089, 37825, 47361])
+
+
+def check_combination(cp, oracle, case, forced, sizes=(1, 31, 32, 33, 97, 1000, 4097, 20011)):
     rng = np.random.default_rng(1000 + case)
-    n = int(rng.choice([1, 31, 32, 33, 97, 1000, 4097, 20011]))
+    n = int(rng.choice(sizes))
     T = int(rng.integers(1, 90))
     seed = int(rng.integers(0, 1 << 31))
     t0 = int(rng.choice([0, 1, 17, 100000]))
