@@ -156,8 +156,11 @@ def _use_current_stream() -> None:
     # around it, which costs more than the rest of a call's marshalling (a step of a small batch is bound by that).
     import torch
     device = torch.cuda.current_device()
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    lib().cp_set_stream(raw(device) if raw else torch.cuda.current_stream(device).cuda_stream)
+    try:
+        handle = torch._C._cuda_getCurrentRawStream(device)
+    except AttributeError:
+        handle = torch.cuda.current_stream(device).cuda_stream
+    lib().cp_set_stream(handle)
 
 
 def cp_set_allocator(alloc=None, release=None) -> None:
