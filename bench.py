@@ -506,7 +506,7 @@ def measure_paths(cp, inputs, torch, timed, peaks, peak_inst, args) -> dict:
         torch.cuda.empty_cache()
     out["fused_step_sweep"] = sweep
 
-    # config 2: 65,536 envs, per-step launches (launch-bound), 1,000 steps per timed iteration
+    # the per-step workload: 65,536 envs, per-step launches (launch-bound), 1,000 steps per timed iteration
     w2 = inputs.WORKLOADS["c2"]
     n = w2.n_envs
     a, b, sa, sb, reward, done = step_setup(n)
@@ -632,7 +632,7 @@ def measure_paths(cp, inputs, torch, timed, peaks, peak_inst, args) -> dict:
     del outs, act, pop, starts
     torch.cuda.empty_cache()
 
-    # wider in-kernel policies on config 5's shape (16,777,216 envs x 200 steps)
+    # wider in-kernel policies on the network workload's shape (16,777,216 envs x 200 steps)
     w5 = inputs.WORKLOADS["c5"]
     n, T = w5.n_envs, w5.T
     outs = {"ep_return_sum": torch.empty(n, device="cuda"), "ep_count": torch.empty(n, dtype=torch.int32, device="cuda"),
@@ -648,7 +648,7 @@ def measure_paths(cp, inputs, torch, timed, peaks, peak_inst, args) -> dict:
         ms /= 2
         out[key] = {"n_envs": n, "T": T, "hidden": inputs.HIDDEN_OF.get(kind, "16+16"), "ms_per_launch": ms,
                     "env_steps_per_sec": n * T / (ms * 1e-3)}
-    # config 5 itself in the contracted arithmetic (FMA dynamics and the five-instruction tanh)
+    # the network workload itself in the contracted arithmetic (FMA dynamics and the five-instruction tanh)
     pol = cp.policy(w5.policy, inputs.policy_weights(w5.policy, w5.policy_seed))
 
     def c5_contracted():
