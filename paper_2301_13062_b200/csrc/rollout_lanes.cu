@@ -1,6 +1,7 @@
 // The lane-split network rollout (rollout_lanes.cuh): the 4-16-2 network, and the entry that picks
 // the instance for a call. The other networks are in files of their own (build time).
 #include "rollout_lanes.cuh"
+#include <algorithm>
 
 namespace cp {
 
@@ -8,52 +9,55 @@ cudaError_t launch_lanes_mlp32(RolloutParams &p, int g, bool streams, bool contr
 cudaError_t launch_lanes_mlp64(RolloutParams &p, int g, bool streams, bool contracted, cudaStream_t s);
 cudaError_t launch_lanes_deep(RolloutParams &p, int g, bool streams, bool contracted, cudaStream_t s);
 
-// Four lanes per environment: one warp per scheduler up to 4,736 environments on 148 SMs, two up to 9,472, three
-// up to 14,208 (the time only changes from one to the next: 9,473 and 14,001 take the same); beyond that the general
-// kernel's one lane per environment keeps the schedulers busy with fewer instructions. us per launch of 500 steps,
-// general kernel / this one, canonical:
-//     environments        1,000          4,096          8,192         14,001         16,001
-//     4-16-2            127 / 81       128 / 79       127 / 95       127 / 121      128 / 155
-//     4-32-2            165 / 87       166 / 90       165 / 115      166 / 148      166 / 193
-//     4-64-2            271 / 100      278 / 133      278 / 177      281 / 236      282 / 345
-//     4-16-16-2         241 / 119      244 / 131      245 / 174      245 / 228      245 / 343
-//     with all four per-step outputs:
-//     4-16-2            213 / 143      214 / 143      214 / 171      215 / 203      214 / 253
-//     4-32-2            261 / 149      262 / 149      263 / 181      263 / 235      263 / 298
-//     4-64-2            365 / 167      372 / 170      373 / 216      376 / 284      376 / 427
-//     4-16-16-2         323 / 190      327 / 190      327 / 247      328 / 324      327 / 490
-// Two warps from 32 steps on (this kernel's time over the general one's, 8,192 environments, at 16 and 100 steps: 4-16-2
-// 0.99 and 0.79, contracted 1.03 and 0.85, 4-16-16-2 0.95 and 0.75, with reward and done bits 1.07 and 0.89). Not
-// for the two smaller networks with reward plane and done bits alone, for which the general kernel has an instance
-// without tests: 6,001 environments at 32, 128, 500 steps: 4-16-2 1.15, 1.06, 1.04, 4-32-2 1.04, 0.96, 0.94.
-// Three warps (14,001 environments at 32, 64, 128, 500 steps): 4-64-2 in every form from 32 steps on (0.73 to 0.92); 4-32-2
-// from 64 (1.06, 0.98, 0.93, 0.89), contracted from 32 (0.97, 0.89, 0.84, 0.80); 4-16-2 from 128 (1.10, 1.03, 0.99, 0.95;
-// contracted 1.11, 1.05, 1.00, 0.95; all outputs 1.04, 0.99, 0.97, 0.94), contracted with outputs from 32 (0.97, 0.92, 0.89,
-// 0.84); 4-16-16-2 from 128 without outputs (1.08, 1.01, 0.97, 0.93) and contracted with them from 32 (0.99, 0.94,
-// 0.91, 0.88), but not the other way round (contracted 1.18, 1.11, 1.07, 1.03; all outputs 1.10, 1.04, 1.02, 0.99), and
-// these three not with reward plane and done bits alone (1.08 to 1.34).
-// Launches of one to seven steps do not earn back the loads of a lane's weights, which differ from lane to
-// lane; the two smaller networks with reward plane and done bits alone need eight steps.
-// Eight lanes for the smallest batches, as long as every warp has a scheduler to itself (500 steps, 1,000
-// environments at four / eight lanes: 4-16-2 92 / 86, 4-32-2 119 / 101, 4-64-2 147 / 120, 4-16-16-2 133 / 127, but
-// contracted 152 / 187; with per-step outputs four are better everywhere: 4-64-2 168 / 190).
+// How many lanes an environment gets, and from how many steps on. A warp of this kernel takes its step's latency
+// whatever it holds, until its scheduler has a second one: so as many lanes as leave every scheduler its one warp,
+// and two or three warps where that is still quicker than the general kernel. Four lanes for up to 4,736 environments on 148 SMs
+// (more measured the same or slower, but for the smallest batches without outputs: 1,000 environments x 300, eight over four
+// lanes, 4-32-2 1.04, 4-64-2 1.20, 4-16-16-2 1.10, contracted 4-16-16-2 0.69, 4-16-2 0.95), two and one beyond them where a
+// lane's registers hold its weights (4-32-2: two lanes, 4-16-2: one). us per launch, general kernel / this one,
+// canonical, 300 steps without outputs, then with reward and done bits, then with all four:
+//     environments         4,096                  9,001                  18,900                 37,800
+//     4-16-2        78 / 41  82 / 49 129 / 50   78 / 49  99 / 62 129 / 64   88 / 62  99 / 76 140 / 80   103 / 96 115 / 109 155 / 115
+//     4-32-2        97 / 51 117 / 60 145 / 60   97 / 64 117 / 80 145 / 82  108 / 88 119 / 108 166 / 109      (not taken)
+//     4-64-2       163 / 62 165 / 72 219 / 72  164 / 88 165 / 111 220 / 111     (not taken)
+//     4-16-16-2    144 / 68 165 / 84 194 / 85  144 / 101 165 / 120 195 / 119    (not taken)
+// Time of the general kernel over this one's around the lines, at the step counts given:
+//   one warp per scheduler: 4 lanes without outputs x 3 1.03-1.05, contracted x 4 1.05, plain (reward and done bits alone, for
+//     which the general kernel has an instance without tests) x 6 1.04-1.19; 2 lanes x 6 1.05-1.08, plain x 8 1.05-1.08;
+//     1 lane x 24 1.03-1.15, with action bits or trajectory x 6 1.04
+//   two: 4-16-2 x 64 1.01-1.04, plain canonical x 96 1.01 (contracted never more than 1.01), tested x 12 1.03; 4-32-2 x 24
+//     1.03-1.09, plain x 48 1.00-1.04, tested x 12 1.07-1.12; 4-64-2 x 16 1.06-1.34; 4-16-16-2 x 24 1.06-1.29
+//   three: 4-16-2 tested x 48 1.05-1.09 (otherwise at most 1.00); 4-32-2 x 64 1.05-1.10, tested x 24 1.06 (plain at most
+//     1.00); 4-64-2 x 32 1.04-1.15; 4-16-16-2 x 64 1.00-1.17 (plain canonical at most 0.96)
+// Launches shorter than that do not earn back the loads of a lane's weights. Supplied start states without outputs, whose steps
+// are not split in two (see euler_both_ways), gain nothing from fewer lanes (14,001 x 200, 4-32-2, four over two 0.93).
 int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool contracted) {
     if (p.action_bits_in || !is_network(policy)) return 0;
     // a forced shape keeps the other kernels
     if (g_tuning.rollout_coop || g_tuning.rollout_ept || g_tuning.rollout_block || g_tuning.rollout_ctas_per_sm) return 0;
     const int64_t schedulers = (int64_t)sm_count() * 4;
-    const int64_t warps4 = (p.n + 7) / 8, warps8 = (p.n + 3) / 4;
-    // reward plane and done bits alone
-    const bool plain = p.reward_stream && p.done_bits && !p.action_bits && !p.trajectory;
-    const bool small_plain = plain && (policy == 2 || policy == 4);
-    int most = p.T >= 32u && !small_plain ? 2 : 1;  // warps per scheduler
-    const uint32_t three_from = policy == 5 || (contracted && (streams || policy == 4)) ? 32u : policy == 4 ? 64u : 128u;
-    if (p.T >= three_from && (policy == 5 || !plain) && (policy != 7 || streams == contracted)) most = 3;
-    if (warps4 > schedulers * most) return 0;
-    uint32_t from = !contracted ? 3u : policy == 7 || (policy == 2 && streams) ? 6u : 4u;
-    if (small_plain) from = 8u;
-    if (p.T < from) return 0;
-    return streams || warps8 > schedulers || (policy == 7 && contracted) ? 4 : 8;
+    auto warps = [&](int lanes) {  // on the fullest scheduler
+        return (int)std::min<int64_t>(4, ((p.n * lanes + 31) / 32 + schedulers - 1) / schedulers);
+    };
+    const bool small = policy == 2 || policy == 4, four = !small || warps(4) == 1 || (p.start_in && !streams);
+    const int g = four ? 4 : policy == 2 && warps(2) > 1 ? 1 : 2, w = warps(g);
+    const bool tested = p.action_bits || p.trajectory, plain = streams && !tested;
+    uint32_t from = 0u;  // steps; 0: the general kernel
+    if (w == 1)
+        from = g == 4 ? (plain ? 6u : contracted ? 4u : 3u) : g == 2 ? (plain ? 8u : 6u) : tested ? 6u : 24u;
+    else if (w <= 3 && small && four)
+        from = w == 2 ? 32u : policy == 2 ? 128u : contracted ? 32u : 64u;
+    else if (w == 2)
+        from = policy == 2   ? (tested ? 12u : !plain ? 64u : contracted ? 0u : 96u)
+               : policy == 4 ? (tested ? 12u : !plain ? 24u : 48u)
+                             : (policy == 5 ? 16u : 24u);
+    else if (w == 3)
+        from = policy == 2   ? (tested ? 48u : 0u)
+               : policy == 4 ? (tested ? 24u : !plain ? 64u : 0u)
+               : policy == 5 ? 32u
+                             : (plain && !contracted ? 0u : 64u);
+    if (from == 0u || p.T < from) return 0;
+    return !streams && policy != 2 && !(policy == 7 && contracted) && warps(8) == 1 ? 8 : g;
 }
 
 cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s) {
