@@ -11,7 +11,7 @@
 // dynamics function, same bits as the general kernel.
 //
 // Synchronisation: one hardware barrier per consumer/producer pair (bar.sync with the pair's own
-// id, 64 threads), once per chunk, double-buffered. Both warps of a pair execute exactly
+// id, the threads of its two or four warps), once per chunk, double-buffered. All warps of a pair execute exactly
 // 1 + ceil(T / chunk) barriers, a number fixed by the launch parameters alone; there is no flag,
 // no spin and no dependence on data, so neither warp can wait for an arrival that does not come.
 //
@@ -50,6 +50,9 @@ inline bool long_chunks(const RolloutParams &p, bool contracted) {
 // Steps per trip of the consumer's loop over a chunk. Measured on 2,048 x 10,000 (ms per launch):
 // 1: 0.666, 2: 0.481, 3: 0.487, 4: 0.503, 8: 0.504, 16: 0.506, whole chunk: 0.506.
 constexpr int kStepUnroll = 2;
+// The same with the cart one step behind (CartBehind), whose steps overlap. 2,048 x 10,000 with three helpers: 1: 543, 2: 425,
+// 4: 389, 8: 388 us; with one, reward and done bits, x 500 (us) 40.9, 29.7, 27.5, 27.8.
+constexpr int kBehindUnroll = 4;
 
 template <int CHUNK>
 struct PairBuffers {
@@ -57,15 +60,15 @@ struct PairBuffers {
     float force[2][CHUNK][32];   // +-F of the action at time t
 };
 
-// One hand-over: barrier 1 for pair 0, barrier 2 for pair 1 (immediates: a register id makes the kernel
-// claim all sixteen barriers).
-template <int PAIRS>
+// One hand-over among a stepping warp and its HELPERS: barrier 1 for pair 0, barrier 2 for pair 1 (immediates: a register
+// id makes the kernel claim all sixteen barriers).
+template <int PAIRS, int HELPERS>
 __device__ __forceinline__ void pair_barrier(uint32_t pair) {
     __syncwarp();
     if (PAIRS == 1 || pair == 0u)
-        asm volatile("bar.sync 1, 64;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * (1 + HELPERS)) : "memory");
     else
-        asm volatile("bar.sync 2, 64;" ::: "memory");
+        asm volatile("bar.sync 2, %0;" ::"n"(32 * (1 + HELPERS)) : "memory");
 }
 
 // Pairs per CTA: one, but two, whose first two warps step, for supplied start states, whose helpers fetch instead of
@@ -86,7 +89,7 @@ bool two_pairs(const RolloutParams &p) {
     return pairs > sms * 5 && (ctas + sms - 1) / sms * 2 == (pairs + sms - 1) / sms && (STREAMS != 3 || p.T <= 256u);
 }
 
-// Which of the two warps of a CTA of one pair steps (0 or 1). A warp's place among an SM's warps decides which of the four
+// Which warp of a CTA of one pair steps (0 or 1; of four, 0 to 3). A warp's place among an SM's warps decides which of the four
 // schedulers it has: a CTA of two warps has schedulers 0 and 1 or 2 and 3. The first warp stepping
 // everywhere, schedulers 0 and 2 would have every stepping warp, whose step is the longer one, and 1 and 3 the
 // helpers; so the roles change places from one group of four warp places to the next. The place is read, not
@@ -95,11 +98,12 @@ bool two_pairs(const RolloutParams &p) {
 // hashed in two operations fewer on both sides): hashed actions 12,000 environments 39.9 / 47.1, with
 // all outputs 55.3 / 65.6, 27,000 57.5 / 59.4, 77.9 / 82.0; one linear policy each, all outputs, 17,000 57.4 / 75.9,
 // 33,000 106.5 / 118.8.
+template <int HELPERS>
 __device__ __forceinline__ uint32_t stepping_warp(uint32_t &shared) {
     if (threadIdx.x == 0) {
         uint32_t place;
         asm volatile("mov.u32 %0, %%warpid;" : "=r"(place));
-        shared = place >> 2 & 1u;
+        shared = (place >> 2) & (uint32_t)HELPERS;
     }
     __syncthreads();
     return shared;
@@ -169,25 +173,102 @@ __device__ __forceinline__ void consume_step(const RolloutParams &p, const PairB
     }
 }
 
+// The same step with the cart's velocity one step behind. The chain that a step waits for is the pole's: rates, angular
+// acceleration, rates. The cart's acceleration comes after it (seven operations more) and is needed only by the next step's
+// position, so the next step computes it first, while its own angular acceleration is under way; in one step after the
+// other a loop's end waited for it. For actions that are not the state's, without the trajectory among the outputs, and
+// up to two pairs per SM, where latency is the time: hashed actions, 500 steps, before / after (one helper), without outputs and
+// with reward and done bits, 9,400 environments 26.9 / 26.0 and 30.8 / 27.8 us; 20,011 54.6 / 54.7 and 60.4 / 62.5.
+// A batch of one pair per SM gets a helper on each of the three other schedulers: the one helper's 84 cycles per step
+// were as many as the stepping warp's 88. 2,048 x 10,000: 450 -> 389 us, 74 cycles per step, of which 55 are the stepping warp's
+// instructions; contracted 500 steps 24.7 -> 16.9, supplied actions 30.6 -> 23.2. (With two pairs per SM three helpers each
+// are slower, 9,400 x 500 28.7 against 26.0; for a policy, which the stepping warp evaluates, they gain 1-3 %.
+// The reciprocal of the denominator by a polynomial and a Newton step, which gives the same quotients and does not
+// wait for the special-function unit: 389 -> 378, but 26.4 -> 26.9 with outputs; not kept.)
+struct CartBehind {
+    float xd, temp, thacc, c, fresh;  // of the step before: what its new velocity is made of, or is where its episode ended
+    bool done;
+    template <bool CONTRACT>
+    __device__ __forceinline__ float velocity() const {
+        float v;
+        if (CONTRACT) {
+            v = __fmaf_rn(kTau, __fmaf_rn(__fmul_rn(thacc, c), kXaccK, temp), xd);
+        } else {
+            const float p1 = __fmul_rn(__fmul_rn(kPML, thacc), c);
+            v = __fadd_rn(xd, __fmul_rn(kTau, __fsub_rn(temp, div_mtot_core(p1))));
+        }
+        return done ? fresh : v;
+    }
+};
+template <bool LIMIT, bool CONTRACT, int STREAMS, int CHUNK>
+__device__ __forceinline__ void consume_step_behind(const RolloutParams &p, const PairBuffers<CHUNK> &buf, uint32_t b, int s,
+                                                    uint32_t lane, uint32_t t1, StreamCursor &sc, State &z, CartBehind &cart,
+                                                    uint32_t &cnt, uint32_t &begin) {
+    const float4 fresh = buf.start[b][s][lane];
+    const float force = buf.force[b][s][lane];
+    const float xd = cart.velocity<CONTRACT>();
+    const float sn = sin_small(z.th), c = cos_small(z.th);
+    float nx, nth, nthd, temp, thacc;
+    if (CONTRACT) {
+        const float t1_ = __fmul_rn(__fmul_rn(z.thd, z.thd), kPML);
+        temp = __fmul_rn(__fmaf_rn(t1_, sn, force), kRcpMTot);
+        const float num = __fmaf_rn(-c, temp, __fmul_rn(kG, sn));
+        const float den = __fmaf_rn(__fmul_rn(c, c), kDenK, kDenC);
+        float r;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den));
+        thacc = __fmul_rn(num, r);
+        nx = __fmaf_rn(kTau, xd, z.x);
+        nth = __fmaf_rn(kTau, z.thd, z.th);
+        nthd = __fmaf_rn(kTau, thacc, z.thd);
+    } else {
+        const float t2 = __fmul_rn(__fmul_rn(kPML, __fmul_rn(z.thd, z.thd)), sn);
+        temp = div_mtot_core(__fadd_rn(force, t2));
+        const float num = __fsub_rn(__fmul_rn(kG, sn), __fmul_rn(c, temp));
+        const float den = __fsub_rn(0.5f * kFT, div_mtot_core(__fmul_rn(0.5f * kMPole, __fmul_rn(c, c))));
+        thacc = div_tame(num, den);
+        nx = __fadd_rn(z.x, __fmul_rn(kTau, xd));
+        nth = __fadd_rn(z.th, __fmul_rn(kTau, z.thd));
+        nthd = __fadd_rn(z.thd, __fmul_rn(kTau, thacc));
+    }
+    bool done = (fabsf(nx) > kXT) | (fabsf(nth) > kTT);
+    if (LIMIT) done |= (t1 - begin) >= p.max_steps;
+    cart = CartBehind{xd, temp, thacc, c, fresh.y, done};
+    cnt += done ? 1u : 0u;
+    begin = done ? t1 : begin;
+    z.x = done ? fresh.x : nx;
+    z.th = done ? fresh.z : nth;
+    z.thd = done ? fresh.w : nthd;
+    if (STREAMS == 1) {
+        const uint32_t m = __ballot_sync(0xffffffffu, done && sc.valid);
+        if (lane == 0u) *sc.done = m;
+        sc.done += sc.words;
+        if (sc.valid) *sc.rew = 1.0f;
+        sc.rew += sc.n;
+    }
+}
+
 // START_IN: the start states are the caller's data and may hold any angle.
+// HELPERS: warps that hash or fetch for the stepping one, every HELPERS-th step each. BEHIND: see CartBehind.
 // kChunk: steps per hand-over.
-template <int POLICY, bool START_IN, int PAIRS, int kChunk, bool LIMIT, bool CONTRACT, int STREAMS>
-__global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
+template <int POLICY, bool START_IN, int PAIRS, int HELPERS, bool BEHIND, int kChunk, bool LIMIT, bool CONTRACT, int STREAMS>
+__global__ void __launch_bounds__(32 * (1 + HELPERS) * PAIRS) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
     __shared__ PairBuffers<kChunk> s_buf[PAIRS];
     __shared__ uint32_t s_stepping;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     bool producer;
-    uint32_t pair = 0u;
+    uint32_t pair = 0u, helper = 0u;
     if constexpr (PAIRS == 1) {
-        producer = warp != stepping_warp(s_stepping);
+        const uint32_t steps = stepping_warp<HELPERS>(s_stepping);
+        producer = warp != steps;
+        if (HELPERS > 1) helper = warp > steps ? warp - 1u : warp;
         if constexpr (kUniformRole<POLICY, START_IN, CONTRACT, STREAMS>) producer = __shfl_sync(0xffffffffu, (int)producer, 0) != 0;
     } else {
         producer = warp >= (uint32_t)PAIRS;
         pair = producer ? warp - PAIRS : warp;  // (not warp % PAIRS: 9,401 x 400, step limit, start states given, 41.9 / 44.8 us)
     }
     const int64_t task = (int64_t)blockIdx.x * PAIRS + pair;
-    // Both warps of a pair leave here together, before their first barrier; no other pair uses
-    // their barrier. Nothing that differs between the two warps of a pair (or between lanes) may
+    // The warps of a pair leave here together, before their first barrier; no other pair uses
+    // their barrier. Nothing that differs between the warps of a pair (or between lanes) may
     // decide an exit or a barrier from here on: each warp must execute exactly 1 + n_chunks
     // barriers, a count fixed by the launch parameters, or its partner waits for ever.
     if (task >= p.n_tasks) return;
@@ -221,20 +302,21 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
                 }
                 if (START_IN) {
                     // the chunk's rows of [T][4][n], all in flight at once
-                    const float *src = p.start_in + (int64_t)row0 * 4 * p.n + idx;
+                    const float *src = p.start_in + (int64_t)(row0 + helper) * 4 * p.n + idx;
 #pragma unroll 4
-                    for (int s = 0; s < rows; ++s) {
+                    for (int s = helper; s < rows; s += HELPERS) {
                         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&buf.start[b][s][lane]);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * q), "l"(src) : "memory");
                             src += p.n;
                         }
+                        if (HELPERS > 1) src += (HELPERS - 1) * 4 * p.n;
                     }
                 }
                 if (!START_IN || (POLICY == 0 && !given)) {
 #pragma unroll 4
-                    for (int s = 0; s < rows; ++s) {
+                    for (int s = helper; s < rows; s += HELPERS) {
                         const uint32_t t = tc + s;
                         if (!START_IN) {
                             const State f = start_state_folded(kr, fold16(4u * (t + 1u)));
@@ -246,7 +328,7 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
                 }
                 if (given) {
 #pragma unroll 4
-                    for (int s = 0; s < rows; ++s) {
+                    for (int s = helper; s < rows; s += HELPERS) {
                         const uint32_t word = __shfl_sync(0xffffffffu, my_word, s);
                         buf.force[b][s][lane] = force_from_signbit((word << (31u - lane)) & 0x80000000u);
                     }
@@ -254,7 +336,7 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
                 // a lane's own copies have landed before it arrives at the barrier
                 if (START_IN) asm volatile("cp.async.wait_all;" ::: "memory");
             }
-            pair_barrier<PAIRS>(pair);
+            pair_barrier<PAIRS, HELPERS>(pair);
         }
         return;
     }
@@ -287,14 +369,20 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
     sc.traj = p.trajectory ? p.trajectory + idx : nullptr;
     sc.done = p.done_bits ? p.done_bits + task : nullptr;  // one 32-env word per warp task
     sc.act = p.action_bits ? p.action_bits + task : nullptr;
-    pair_barrier<PAIRS>(pair);  // chunk 0 is there
+    pair_barrier<PAIRS, HELPERS>(pair);  // chunk 0 is there
+    static_assert(!BEHIND || (POLICY == 0 && !START_IN && STREAMS <= 1), "see CartBehind");
+    constexpr int kUnroll = BEHIND ? kBehindUnroll : kStepUnroll;
+    CartBehind cart;
     for (uint32_t c = 0; c < n_chunks; ++c) {
         const uint32_t b = c & 1u, tc = p.t0 + c * kChunk;
         const int steps = (int)min((uint32_t)kChunk, t_end - tc);
+        auto one = [&](int s) {
+            if constexpr (BEHIND) consume_step_behind<LIMIT, CONTRACT, STREAMS>(p, buf, b, s, lane, tc + s + 1u, sc, z, cart, cnt, begin);
+            else consume_step<POLICY, !START_IN, LIMIT, CONTRACT, STREAMS>(p, buf, b, s, lane, tc + s + 1u, own, sc, z, cnt, begin);
+        };
         if (c != 0u && steps == kChunk) {
-#pragma unroll kStepUnroll
-            for (int s = 0; s < kChunk; ++s)
-                consume_step<POLICY, !START_IN, LIMIT, CONTRACT, STREAMS>(p, buf, b, s, lane, tc + s + 1u, own, sc, z, cnt, begin);
+#pragma unroll kUnroll
+            for (int s = 0; s < kChunk; ++s) one(s);
         } else {
             // The caller's initial state may hold any angle: the very first step tests it per
             // lane. From the second step on every angle is a survivor's (<= 0.2095) or a start
@@ -302,14 +390,15 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
             int s = 0;
             if (c == 0u) {
                 consume_step<POLICY, false, LIMIT, CONTRACT, STREAMS>(p, buf, b, 0, lane, tc + 1u, own, sc, z, cnt, begin);
+                cart = CartBehind{0.0f, 0.0f, 0.0f, 0.0f, z.xd, true};
                 s = 1;
             }
-#pragma unroll kStepUnroll
-            for (; s < steps; ++s)
-                consume_step<POLICY, !START_IN, LIMIT, CONTRACT, STREAMS>(p, buf, b, s, lane, tc + s + 1u, own, sc, z, cnt, begin);
+#pragma unroll kUnroll
+            for (; s < steps; ++s) one(s);
         }
-        pair_barrier<PAIRS>(pair);
+        pair_barrier<PAIRS, HELPERS>(pair);
     }
+    if (BEHIND && p.T) z.xd = cart.velocity<CONTRACT>();
 
     unsigned long long tot_ret = 0, tot_cnt = 0;
     if (valid) {
@@ -341,13 +430,23 @@ __global__ void __launch_bounds__(64 * PAIRS) rollout_assisted_kernel(const __gr
     }
 }
 
+template <int POLICY, bool START_IN, int PAIRS, int HELPERS, bool BEHIND, int CHUNK, bool CONTRACT, int STREAMS>
+void launch_assisted_helpers(const RolloutParams &p, cudaStream_t s) {
+    const unsigned grid = (unsigned)((p.n_tasks + PAIRS - 1) / PAIRS), block = 32 * (1 + HELPERS) * PAIRS;
+    if (p.max_steps)
+        rollout_assisted_kernel<POLICY, START_IN, PAIRS, HELPERS, BEHIND, CHUNK, true, CONTRACT, STREAMS><<<grid, block, 0, s>>>(p);
+    else
+        rollout_assisted_kernel<POLICY, START_IN, PAIRS, HELPERS, BEHIND, CHUNK, false, CONTRACT, STREAMS><<<grid, block, 0, s>>>(p);
+}
 template <int POLICY, bool START_IN, int PAIRS, int CHUNK, bool CONTRACT, int STREAMS>
 void launch_assisted_pairs(const RolloutParams &p, cudaStream_t s) {
-    const unsigned grid = (unsigned)((p.n_tasks + PAIRS - 1) / PAIRS);
-    if (p.max_steps)
-        rollout_assisted_kernel<POLICY, START_IN, PAIRS, CHUNK, true, CONTRACT, STREAMS><<<grid, 64 * PAIRS, 0, s>>>(p);
-    else
-        rollout_assisted_kernel<POLICY, START_IN, PAIRS, CHUNK, false, CONTRACT, STREAMS><<<grid, 64 * PAIRS, 0, s>>>(p);
+    if constexpr (POLICY == 0 && !START_IN && STREAMS <= 1) {
+        // (from 8 and 32 steps on: shorter launches take 0.05 us longer with either; 2,048 x 1, 8, 16 steps, before / after 0.98,
+        // 1.02, 1.09; 9,472 x 16, 32, 128 with reward and done bits 1.00, 1.02, 1.09)
+        if (p.n_tasks <= sm_count() && p.T >= 8u) return launch_assisted_helpers<0, false, 1, 3, true, CHUNK, CONTRACT, STREAMS>(p, s);
+        if (p.n_tasks <= sm_count() * 2 && p.T >= 32u) return launch_assisted_helpers<0, false, 1, 1, true, CHUNK, CONTRACT, STREAMS>(p, s);
+    }
+    launch_assisted_helpers<POLICY, START_IN, PAIRS, 1, false, CHUNK, CONTRACT, STREAMS>(p, s);
 }
 template <int POLICY, bool START_IN, int CHUNK, bool CONTRACT, int STREAMS>
 void launch_assisted_limit(const RolloutParams &p, cudaStream_t s) {

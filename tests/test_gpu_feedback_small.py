@@ -144,3 +144,16 @@ def test_supplied_starts(cp, kind, given, n, T):
         general = rollout(cp, 2, kind, n, T, **args)
         for coop in (0, 4):  # what a caller gets; helper warps, which take such calls from 96 steps on
             assert_same_bits(rollout(cp, coop, kind, n, T, **args), general)
+
+
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("contracted", [False, True])
+@pytest.mark.parametrize("n,T", [(31, 1), (4736, 2), (4735, 36), (4737, 35), (9472, 34), (9473, 37), (4700, 129)])
+def test_hashed_and_given_actions_by_pairs_per_sm(cp, given, contracted, n, T):
+    """148 SMs: three helper warps up to 4,736 environments, the cart's velocity a step behind up to 9,472, neither beyond;
+    horizons around the hand-overs and the four steps of a trip."""
+    bits = torch.from_numpy(np.random.default_rng(2).integers(-2**31, 2**31, (T, (n + 31) // 32)).astype(np.int32)).cuda()
+    for streams, limit, spread in (((), 0, None), (("reward_stream", "done_bits"), 0, "wide"), ((), 9, "edge"),
+                                   (("reward_stream", "done_bits"), 20, None), (ALL, 0, "edge")):
+        args = dict(streams=streams, limit=limit, spread=spread, contracted=contracted, given=bits if given else None)
+        assert_same_bits(rollout(cp, 0, 0, n, T, **args), rollout(cp, 2, 0, n, T, **args))
