@@ -306,10 +306,11 @@ int cp_rollout_host_shard(uint32_t env_offset, int64_t n_envs, int64_t T, uint32
 /* cp_step_host: h_planes_in/out [4][n_envs] (stride n_envs), h_action [n_envs] or NULL,
  * h_reward [n_envs], h_done [n_envs]; the step at global time t of envs 0..n_envs-1. Out may be in
  * (a step in place). On buffers that are page-locked throughout and do not otherwise overlap, calls of
- * up to 250,000 environments are one kernel that works on host memory directly. */
+ * up to 250,000 environments are one kernel that works on host memory directly, larger ones overlap the
+ * copies in with steps that store into host memory. */
 int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_planes_in,
                  const uint8_t *h_action, float *h_planes_out, float *h_reward, uint8_t *h_done);
-/* Free the library-owned staging buffers (synchronises the device). */
+/* Free the library-owned staging buffers and copy stream (synchronises the device). */
 void cp_shutdown(void);
 
 /* Stream used by this thread's later calls (a cudaStream_t; NULL = legacy default stream). */

@@ -23,7 +23,7 @@ LIB = os.path.join(HERE, "libcartpole.so")
 STAMP = os.path.join(HERE, "libcartpole.so.stamp")
 SOURCES = ["rollout_networks.cu", "rollout_networks_contracted.cu", "rollout_kernel.cu", "rollout_contracted.cu",
            "rollout_assisted.cu", "rollout_assisted_linear.cu", "rollout_assisted_starts.cu", "rollout_deferred.cu", "rollout_deferred_data.cu",
-           "rollout_lanes.cu", "rollout_lanes_mlp32.cu", "rollout_lanes_mlp64.cu", "rollout_lanes_deep.cu", "policy_screen.cu", "capi.cu", "step_kernel.cu", "step_strided.cu", "ladder_kernels.cu", "ladder_noalloc.cu"]
+           "rollout_lanes.cu", "rollout_lanes_mlp32.cu", "rollout_lanes_mlp64.cu", "rollout_lanes_deep.cu", "policy_screen.cu", "capi.cu", "step_kernel.cu", "step_strided.cu", "step_host.cu", "ladder_kernels.cu", "ladder_noalloc.cu"]
 HEADERS = ["cartpole_device.cuh", "cartpole_internal.h", "pinned_range.h", "rollout_kernel.cuh", "rollout_deferred.cuh", "rollout_lanes.cuh", "rollout_assisted.cuh", "policy_screen.cuh", "policy_bound.h", os.path.join("..", "..", "include", "cartpole.h")]
 
 NVCC_FLAGS = [

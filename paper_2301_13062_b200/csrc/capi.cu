@@ -193,7 +193,27 @@ struct Staging {
     std::mutex mu;
     void *buf = nullptr;
     size_t bytes = 0;
+    cudaStream_t copies = nullptr;  // cp_step_host's copies in, beside the caller's stream, on `device`
+    cudaEvent_t event = nullptr;
+    int device = -1;
 } g_staging;
+
+// The stream and event of the copies in, made once; false where there are none for the current device.
+bool staging_stream() {
+    int device;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    if (!g_staging.copies) {
+        if (cudaStreamCreateWithFlags(&g_staging.copies, cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&g_staging.event, cudaEventDisableTiming) != cudaSuccess) {
+            (void)cudaGetLastError();
+            if (g_staging.copies) cudaStreamDestroy(g_staging.copies);
+            g_staging.copies = nullptr;
+            return false;
+        }
+        g_staging.device = device;
+    }
+    return g_staging.device == device;
+}
 
 int staging_reserve(size_t bytes, void **out) {
     if (g_staging.bytes < bytes) {
@@ -547,30 +567,28 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
     // this: 2,000 envs 41 / 22, 20,000 57 / 31, 100,000 118 / 85, 200,000 188 / 157, 240,000 211 / 188,
     // 250,000 212 / 205, 262,143 222 / 230, the last three with actions; 300,001 260 / 272 and 4,000,001
     // 3,027 / 3,277, where the copy engine's bandwidth counts). Buffers that overlap, other than a step in place, keep the copies' order.
-    if (n_envs <= 250000) {
-        const size_t n = (size_t)n_envs;
-        const struct { void *p; size_t bytes; } buf[5] = {{const_cast<float *>(h_planes_in), 16 * n},
-            {const_cast<uint8_t *>(h_action), n}, {h_planes_out, 16 * n}, {h_reward, 4 * n}, {h_done, n}};
-        void *dev[5];
-        bool direct = is_aligned(h_planes_in, 4) && is_aligned(h_planes_out, 4) && is_aligned(h_reward, 4);
-        for (int i = 0; i < 5 && direct; ++i) {
-            dev[i] = buf[i].p ? device_view_of_pinned(buf[i].p, buf[i].bytes) : nullptr;
-            direct = dev[i] || !buf[i].p;
-            for (int j = 0; j < i && direct; ++j) {  // 0 and 1 are read, 2 to 4 written
-                const char *a = static_cast<char *>(buf[i].p), *b = static_cast<char *>(buf[j].p);
-                const bool apart = !a || !b || a + buf[i].bytes <= b || b + buf[j].bytes <= a;
-                direct = apart || i < 2 || (i == 2 && j == 0 && a == b);
-            }
+    const size_t n = (size_t)n_envs;
+    const struct { void *p; size_t bytes; } host[5] = {{const_cast<float *>(h_planes_in), 16 * n},
+        {const_cast<uint8_t *>(h_action), n}, {h_planes_out, 16 * n}, {h_reward, 4 * n}, {h_done, n}};
+    void *dev[5];
+    bool direct = is_aligned(h_planes_in, 4) && is_aligned(h_planes_out, 4) && is_aligned(h_reward, 4);
+    for (int i = 0; i < 5 && direct; ++i) {
+        dev[i] = host[i].p ? device_view_of_pinned(host[i].p, host[i].bytes) : nullptr;
+        direct = dev[i] || !host[i].p;
+        for (int j = 0; j < i && direct; ++j) {  // 0 and 1 are read, 2 to 4 written
+            const char *a = static_cast<char *>(host[i].p), *b = static_cast<char *>(host[j].p);
+            const bool apart = !a || !b || a + host[i].bytes <= b || b + host[j].bytes <= a;
+            direct = apart || i < 2 || (i == 2 && j == 0 && a == b);
         }
-        if (direct) {
-            cp_state in{n_envs, n_envs, seed, t, 0, static_cast<float *>(dev[0]), false, nullptr};
-            cp_state out{n_envs, n_envs, seed, t, 0, static_cast<float *>(dev[2]), false, nullptr};
-            if ((rc = cp_step(&in, static_cast<uint8_t *>(dev[1]), &out, static_cast<float *>(dev[3]),
-                              static_cast<uint8_t *>(dev[4]))) != CP_OK)
-                return rc;
-            const cudaError_t e = cudaStreamSynchronize(tl_stream);
-            return e == cudaSuccess ? CP_OK : cuda_fail(e, "step on host memory");
-        }
+    }
+    if (direct && n_envs <= 250000) {
+        cp_state in{n_envs, n_envs, seed, t, 0, static_cast<float *>(dev[0]), false, nullptr};
+        cp_state out{n_envs, n_envs, seed, t, 0, static_cast<float *>(dev[2]), false, nullptr};
+        if ((rc = cp_step(&in, static_cast<uint8_t *>(dev[1]), &out, static_cast<float *>(dev[3]),
+                          static_cast<uint8_t *>(dev[4]))) != CP_OK)
+            return rc;
+        const cudaError_t e = cudaStreamSynchronize(tl_stream);
+        return e == cudaSuccess ? CP_OK : cuda_fail(e, "step on host memory");
     }
     std::lock_guard<std::mutex> lock(g_staging.mu);
     const int64_t stride = (n_envs + 63) / 64 * 64;
@@ -583,6 +601,42 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
     float *d_reward = reinterpret_cast<float *>(base + 4 * plane_bytes);
     uint8_t *d_done = reinterpret_cast<uint8_t *>(base + 5 * plane_bytes);
     uint8_t *d_action = d_done + byte_plane;
+    // Larger page-locked batches in pieces: the copies in run on a stream of their own, and each piece's step stores
+    // its outputs into host memory itself, by whole lines (step_host.cu), so that both directions of the bus are busy.
+    // A piece costs a start of its copies (10 us and more), so they are few. us per call with actions, copies and step in turn /
+    // in 2, 3, 4, 6 pieces: 250,001 envs 214 / 196, 219, 231, 248; 400,003 324 / 280, 292, 313, 350; 500,000 387-413 / 334,
+    // 322, 338, 361; 1,000,003 722 / 625, 595, 603, 633; 2,000,000 1,396 / 1,178, 1,102, 1,081, 1,071; 4,000,001 2,760 /
+    // 2,362, 2,208, 2,125, 2,068. (The kernel reading the actions from host memory too 10 to 17 % slower; outputs by the step
+    // kernels' own stores, whose lines lie across two where n is odd, 1,000,003 640, 4,000,001 2,865.)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (direct && cudaStreamIsCapturing(tl_stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone && staging_stream()) {
+        const cudaStream_t copies = g_staging.copies;
+        const int pieces = n_envs <= 450000 ? 2 : n_envs <= 800000 ? 3 : n_envs <= 1500000 ? 4 : 6;
+        const int64_t step = ((n_envs + pieces - 1) / pieces + 127) / 128 * 128;
+        // the caller's inputs are what earlier work on its stream has left there
+        cudaError_t e = cudaEventRecord(g_staging.event, tl_stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(copies, g_staging.event, 0);
+        for (int64_t at = 0; at < n_envs && e == cudaSuccess; at += step) {
+            const int64_t len = n_envs - at < step ? n_envs - at : step;
+            e = cudaMemcpy2DAsync(d_planes + at, plane_bytes, h_planes_in + at, n * 4, (size_t)len * 4, 4, cudaMemcpyHostToDevice, copies);
+            if (e == cudaSuccess && h_action)
+                e = cudaMemcpyAsync(d_action + at, h_action + at, (size_t)len, cudaMemcpyHostToDevice, copies);
+            if (e == cudaSuccess) e = cudaEventRecord(g_staging.event, copies);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(tl_stream, g_staging.event, 0);
+            if (e != cudaSuccess) break;
+            cp_state in{len, stride, seed, t, (uint32_t)at, d_planes + at, false, nullptr};
+            cp_state out{len, n_envs, seed, t, (uint32_t)at, static_cast<float *>(dev[2]) + at, false, nullptr};
+            cp::StepParams p;
+            fill_step_params(p, &in, &out, h_action ? d_action + at : nullptr, static_cast<float *>(dev[3]) + at,
+                             static_cast<uint8_t *>(dev[4]) + at);
+            e = cp::launch_step_host(p, tl_stream);
+        }
+        // nothing is in flight when the call returns, whatever came of it
+        const cudaError_t done[2] = {cudaStreamSynchronize(copies), cudaStreamSynchronize(tl_stream)};
+        for (const cudaError_t d : done)
+            if (e == cudaSuccess) e = d;
+        return e == cudaSuccess ? CP_OK : cuda_fail(e, "step on host memory");
+    }
     cudaError_t e = cudaMemcpy2DAsync(d_planes, plane_bytes, h_planes_in, (size_t)n_envs * 4, (size_t)n_envs * 4, 4,
                                       cudaMemcpyHostToDevice, tl_stream);
     if (e == cudaSuccess && h_action)
@@ -605,6 +659,12 @@ void cp_shutdown(void) {
         cudaFree(g_staging.buf);
         g_staging.buf = nullptr;
         g_staging.bytes = 0;
+    }
+    if (g_staging.copies) {
+        cudaStreamSynchronize(g_staging.copies);
+        cudaEventDestroy(g_staging.event);
+        cudaStreamDestroy(g_staging.copies);
+        g_staging.copies = nullptr;
     }
 }
 

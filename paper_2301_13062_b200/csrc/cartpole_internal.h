@@ -83,6 +83,8 @@ int sm_count();
 cudaError_t launch_step(const StepParams &p, bool vec, cudaStream_t s);
 // the step for large batches that cannot be accessed as float4
 cudaError_t launch_step_strided(const StepParams &p, cudaStream_t s);
+// the step whose outputs lie in page-locked host memory
+cudaError_t launch_step_host(const StepParams &p, cudaStream_t s);
 cudaError_t launch_fill_start(float *planes, int64_t stride, int64_t n, uint32_t env_offset, uint32_t salt_r,
                               uint32_t t, cudaStream_t s);
 cudaError_t launch_actions(uint8_t *out, int64_t n, uint32_t env_offset, uint32_t salt_a, uint32_t t,

@@ -1,4 +1,4 @@
-"""cp_step_host on page-locked buffers (the kernel works on host memory) gives what it gives on pageable
+"""cp_step_host on page-locked buffers (the kernel works on host memory, in pieces on large batches) gives what it gives on pageable
 ones (copies), with and without actions, in place, at ragged sizes, from misaligned and overlapping buffers."""
 import pytest
 
@@ -44,6 +44,18 @@ def buffers(n, pinned, offset, form):
 @pytest.mark.parametrize("form", ["apart", "in place", "overlap"])
 @pytest.mark.parametrize("given", [False, True])
 def test_page_locked_equals_pageable(cp, n, offset, form, given):
+    got = []
+    for pinned in (True, False):
+        planes, action, out, reward, done = buffers(n, pinned, offset, form)
+        cp.cp_step_host(n, 9, 4, planes, action if given else None, out, reward, done)
+        got.append([t.numpy().tobytes() for t in (planes, out, reward, done)])
+    assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("n,offset,form", [(450_001, 0, "apart"), (800_003, 1, "in place"), (1_500_001, 1, "apart"), (1_536_000, 0, "in place")])
+@pytest.mark.parametrize("given", [False, True])
+def test_pieces_equal_pageable(cp, n, offset, form, given):
+    """Three, four and six pieces, the last of them ragged, on rows that start anywhere between two lines."""
     got = []
     for pinned in (True, False):
         planes, action, out, reward, done = buffers(n, pinned, offset, form)
