@@ -115,9 +115,7 @@ cudaError_t launch_pipe_rate(int kind, const float *seed, float *sink, int iters
 cudaError_t launch_arith_selftest(unsigned long long *out, cudaStream_t s);
 cudaError_t launch_pair_selftest(unsigned long long count, uint32_t seed, unsigned long long *out, cudaStream_t s);
 cudaError_t launch_screen_selftest(unsigned long long *out, cudaStream_t s);
-// A network's weights in RolloutParams::w rearranged for its estimate, for two environments per thread (4-16-2)
-// or for one, with the bound the estimate needs (policy_screen.cu).
-void screen_pairs(RolloutParams &p);
+// A network's weights in RolloutParams::w rearranged for its estimate, with the bound the estimate needs (policy_screen.cu).
 void screen_units(RolloutParams &p, int policy);
 void screen_bound(RolloutParams &p, int policy);  // the bound alone, weights as the caller gave them
 cudaError_t launch_tame_div_selftest(uint32_t den_step, unsigned long long *out, cudaStream_t s);

@@ -33,16 +33,6 @@ void bound_alone(RolloutParams &p) {  // four or eight lanes: H / 4 or H / 8 ter
 
 }  // namespace
 
-void screen_pairs(RolloutParams &p) {
-    using S = NetShape<2>;
-    constexpr int H = S::H;
-    float steps[H];
-    screen<2>(p, steps, H);
-    std::memmove(p.w + S::kPairLogits, p.w + S::kLogits, (2 * H + 2) * sizeof(float));
-    for (int i = S::kLogits - 1; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
-    for (int j = 0; j < H; ++j) p.w[S::kPairSteps + 2 * j] = p.w[S::kPairSteps + 2 * j + 1] = steps[j];
-}
-
 void screen_units(RolloutParams &p, int policy) {
     switch (policy) {
         case 2: return units<2>(p);

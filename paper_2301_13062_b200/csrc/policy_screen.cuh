@@ -44,10 +44,7 @@ struct NetShape {
     static constexpr int kSecond = 5 * H;
     static constexpr int kLogits = kSecond + (kDeep ? H * (H + 1) : 0);
     static constexpr int kCount = kLogits + 2 * H + 2;
-    // RolloutParams::w for two environments per thread (screen_pairs, one hidden layer): every weight of it and
-    // every w1[j] - w0[j] as a pair, then the logits' weights
-    static constexpr int kPairSteps = 2 * kLogits, kPairLogits = kPairSteps + 2 * H;
-    // and for one (screen_units): the caller's weights, the first layer again with the weights of units
+    // RolloutParams::w (screen_units): the caller's weights, the first layer again with the weights of units
     // 2q and 2q + 1 side by side (input 0, .., input 3, bias), then w1[j] - w0[j]
     static constexpr int kUnitFirst = kCount, kUnitSteps = kUnitFirst + 5 * H;
     static_assert(kUnitSteps + H <= kMaxPolicyFloats, "RolloutParams::w holds the layout");
@@ -103,26 +100,6 @@ __device__ __forceinline__ uint32_t defined_action(const float *w, const float *
     return (l1 > l0) ? 0x80000000u : 0u;
 }
 
-// Estimates for the two environments of a thread, from the pairs of screen_pairs.
-template <int NET>
-__device__ __forceinline__ f32x2 screen_estimate_pair(const f32x2 *w, f32x2 base, const StatePair &z) {
-    using S = NetShape<NET>;
-    constexpr int H = S::H;
-    static_assert(!S::kDeep && S::kPairLogits + 2 * H + 2 <= kMaxPolicyFloats, "one hidden layer, as pairs");
-    const f32x2 *steps = w + S::kLogits;
-    f32x2 est = base;
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        f32x2 acc = w[4 * H + j];
-        acc = fma2(w[4 * j + 0], z.x, acc);
-        acc = fma2(w[4 * j + 1], z.xd, acc);
-        acc = fma2(w[4 * j + 2], z.th, acc);
-        acc = fma2(w[4 * j + 3], z.thd, acc);
-        est = fma2(steps[j], tanh_screen2(acc), est);
-    }
-    return est;
-}
-
 // Estimate for one environment, two hidden units per packed operation, from the layout of screen_units.
 template <int NET>
 __device__ __forceinline__ float screen_estimate(const float *w, float base, const State &z) {
@@ -163,6 +140,36 @@ __device__ __forceinline__ float screen_estimate(const float *w, float base, con
         unpack2(est, lo, hi);
         return __fadd_rn(lo, hi);
     }
+}
+
+// Estimates for the two environments of a thread, from the same layout: every pair of weights is loaded once for both.
+template <int NET>
+__device__ __forceinline__ void screen_estimate_two(const float *w, float base, const State &a, const State &b, float (&e)[2]) {
+    using S = NetShape<NET>;
+    constexpr int H = S::H;
+    static_assert(!S::kDeep, "one hidden layer");
+    const f32x2 *first = reinterpret_cast<const f32x2 *>(w + S::kUnitFirst), *steps = reinterpret_cast<const f32x2 *>(w + S::kUnitSteps);
+    const f32x2 za[4] = {splat2(a.x), splat2(a.xd), splat2(a.th), splat2(a.thd)};
+    const f32x2 zb[4] = {splat2(b.x), splat2(b.xd), splat2(b.th), splat2(b.thd)};
+    f32x2 ea = pack2(base, 0.0f), eb = ea;
+#pragma unroll
+    for (int q = 0; q < H / 2; ++q) {
+        f32x2 ha = first[5 * q + 4], hb = ha;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const f32x2 v = first[5 * q + i];
+            ha = fma2(v, za[i], ha);
+            hb = fma2(v, zb[i], hb);
+        }
+        const f32x2 v = steps[q];
+        ea = fma2(v, tanh_screen2(ha), ea);
+        eb = fma2(v, tanh_screen2(hb), eb);
+    }
+    float lo, hi;
+    unpack2(ea, lo, hi);
+    e[0] = __fadd_rn(lo, hi);
+    unpack2(eb, lo, hi);
+    e[1] = __fadd_rn(lo, hi);
 }
 
 // Does the estimate decide? (false for NaN, and for every estimate where the bound is infinite)

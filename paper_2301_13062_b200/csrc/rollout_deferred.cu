@@ -43,7 +43,7 @@ cudaError_t launch_rollout_deferred(RolloutParams &p, int policy, bool contracte
     if (policy == 1)
         for (int i = 9; i >= 0; --i) p.w[2 * i] = p.w[2 * i + 1] = p.w[i];
     else if (policy == 2)
-        screen_pairs(p);
+        screen_units(p, 2);
     if (p.action_bits_in || p.start_in) return launch_rollout_deferred_data(p, p.action_bits_in ? 3 : policy, k, contracted, s);
     switch (policy) {
         case 0: return short_times ? launch_limit<0, true>(p, k, contracted, s) : launch_limit<0, false>(p, k, contracted, s);

@@ -70,23 +70,25 @@ __device__ __forceinline__ void linear_action_pair(const f32x2 *w, const StatePa
 // The networks: the sign of the estimate where it decides, the defined logits where it does not (a
 // waiting slot's state is nobody's, so it never asks for them). What bounds a 4-16-2 trip now: 256 cycles of
 // the special-function pipe (32 tanhs), about 250 of the float32 pipe (80 multiply-adds of the estimate and the
-// 37 packed operations of the step), of 350 measured; with two results and 13 packed operations per
-// tanh it was 512 and 590 of 800 (16,777,216 x 40: 8.59 -> 4.35 ms, contracted 5.48 -> 3.68).
+// 37 packed operations of the step), of 320 measured; with two results and 13 packed operations per
+// tanh it was 512 and 590 of 800 (16,777,216 x 40: 8.59 -> 4.35 ms, contracted 5.48 -> 3.68). The estimate pairs hidden
+// units, not environments: one load brings the weights of two units for both environments, where a weight
+// paired with itself was loaded for every multiply-add (16,777,216 x 50: 4,717 -> 4,369 us, another policy 4,345 -> 4,069,
+// contracted 4,418 -> 4,081).
 template <int NET, bool CONTRACT>
 __device__ __forceinline__ void network_action_pair(const RolloutParams &p, const bool (&act)[2], const StatePair &z,
                                                     uint32_t &sb0, uint32_t &sb1) {
-    using S = NetShape<NET>;
+    State a, b;
+    unpack_states(z, a, b);
     float e[2];
-    unpack2(screen_estimate_pair<NET>(reinterpret_cast<const f32x2 *>(p.w), splat2(p.screen_base), z), e[0], e[1]);
+    screen_estimate_two<NET>(p.w, p.screen_base, a, b, e);
     sb0 = screen_action(e[0]);
     sb1 = screen_action(e[1]);
     const bool open0 = act[0] && !screen_decides(e[0], p.screen_bound), open1 = act[1] && !screen_decides(e[1], p.screen_bound);
     if (open0 || open1) {
-        State a, b;
-        unpack_states(z, a, b);
 #pragma unroll 1
         for (int j = open0 ? 0 : 1; j < (open1 ? 2 : 1); ++j) {
-            const uint32_t sb = defined_action<NET, CONTRACT, 2>(p.w, p.w + S::kPairLogits, j ? b : a);
+            const uint32_t sb = defined_action<NET, CONTRACT, 1>(p.w, p.w + NetShape<NET>::kLogits, j ? b : a);
             (j ? sb1 : sb0) = sb;
         }
     }
@@ -575,12 +577,15 @@ __global__ void __launch_bounds__(256) clear_words_kernel(uint32_t *w, int64_t n
 // that one wave holds: it is what the launch waits for (250 steps, supplied actions, 100,003 environments, 196 CTAs
 // of eight warps or 391 of four on 148 SMs: 89.5 / 73.9 us, with reward and done bits 113.2 / 97.5; hashed actions
 // 37,888 x 500, 74 or 148 CTAs, 84.2 / 55.5; where the fullest SM has as many either way four cost up to 5 %,
-// supplied actions on 200,003 environments 127.6 / 130.9).
-inline unsigned deferred_grid(RolloutParams &p, unsigned &block, cudaStream_t s) {
+// supplied actions on 200,003 environments 127.6 / 130.9). The networks, of which an SM holds 32 warps, by CTAs of two
+// warps too (152,000 x 128, 4-16-2, general kernel / eight warps / this 1.00 / 1.08 / 0.96).
+inline unsigned deferred_grid(RolloutParams &p, bool network, unsigned &block, cudaStream_t s) {
     p.n_tasks = (p.n + 63) / 64;
     const int64_t sms = sm_count();
     auto fullest = [&](int64_t warps) { return ((p.n_tasks + warps - 1) / warps + sms - 1) / sms * warps; };
-    const int warps = p.n_tasks <= sms * 16 && fullest(4) < fullest(8) ? 4 : 8;
+    int warps = 8;
+    if (p.n_tasks <= sms * (network ? 32 : 16) && fullest(4) < fullest(8)) warps = 4;
+    if (network && p.n_tasks <= sms * 32 && fullest(2) < fullest(warps)) warps = 2;
     block = 32u * warps;
     const int64_t grid = (p.n_tasks + warps - 1) / warps;
     if (grid > 0x7fffffffLL) return 0;
@@ -597,7 +602,7 @@ inline unsigned deferred_grid(RolloutParams &p, unsigned &block, cudaStream_t s)
 template <int POLICY, bool SHORT, bool LIMIT, bool RD>
 cudaError_t launch_k(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
     unsigned block;
-    const unsigned grid = deferred_grid(p, block, s);
+    const unsigned grid = deferred_grid(p, is_network(POLICY), block, s);
     if (grid == 0) return cudaErrorInvalidConfiguration;
     if (contracted) {  // the optional arithmetic comes at the default trip spacing only
         constexpr int kC = is_network(POLICY) ? 2 : 6;

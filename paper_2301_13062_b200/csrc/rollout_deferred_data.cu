@@ -9,7 +9,7 @@ namespace {
 template <int POLICY, bool START_IN, bool LIMIT, bool RD>
 cudaError_t launch_data(RolloutParams &p, int k, bool contracted, cudaStream_t s) {
     unsigned block;
-    const unsigned grid = deferred_grid(p, block, s);
+    const unsigned grid = deferred_grid(p, false, block, s);
     if (grid == 0) return cudaErrorInvalidConfiguration;
     if (contracted)
         rollout_deferred_kernel<POLICY, 6, false, LIMIT, RD, true, START_IN><<<grid, block, 0, s>>>(p);

@@ -40,14 +40,15 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     // (this kernel's time over theirs, 33,100 envs x 200 / 500: 0.85 / 0.75 and 0.72 / 0.69, with reward and done bits
     // 1.01 / 0.88 and 0.78 / 0.72, contracted 0.77 / 0.69 and 0.62 / 0.60, 1.02 / 0.88 and 0.77 / 0.72; 37,800 x 96 16.4 / 18.4
     // and 24.6 / 20.7 us; 28,000 x 500 with outputs 74 / 64; one linear policy each 70 / 74, but with outputs 92 / 84).
-    // The networks' trips are short next to their waits since the estimate decides (policy_screen.cuh). This
-    // kernel's time over the general one's, three policies each: 4-16-2 x 100 1,000,003 envs 0.99 to 1.01, 2,000,003 0.97
-    // to 0.99, 4,200,001 0.96 to 0.98, 16,777,216 0.95 to 0.97, contracted 0.96 to 0.98, 0.94 to 0.96, 0.93 to 0.95, 0.92 to
-    // 0.94; with reward and done bits x 40 1.02 to 1.05, 1.00 to 1.03, 0.99 to 1.01, 0.98 to 1.01, contracted 1.00 to 1.03,
-    // 0.99 to 1.01, 0.97 to 1.00, 0.96 to 0.99: from 4.24 million on no form loses more than 1 %. T = 100 .. 400, 4-32-2
-    // 1.07 to 1.2 and 4-64-2 1.3 to 1.7 from 67,000 to 1,000,000, 4-16-16-2 at 1,000,000 0.92 to 1.28, the latter where
-    // more estimates do not decide (contracted 0.88 to 1.13; 1,048,576 x 100 1.41 to 2.00 against 1.58 to 1.77 ms, defined
-    // logits in every step 1.94): the larger networks have no instance of it.
+    // The networks' trips are short next to their waits since the estimate decides (policy_screen.cuh). Time of the general
+    // kernel over this one's for 4-16-2, each weight loaded once for both environments of a thread, without outputs, contracted,
+    // with reward and done bits, contracted, two policies each: x 128, 230,000 envs 1.06-1.08, 1.11-1.12, 1.00-1.02, 1.03-1.04;
+    // 303,000 (one wave of four CTAs per SM) 1.10, 1.13, 1.03, 1.05; 310,000 (a second one) 1.00, 1.03, 0.93, 0.95; 480,000
+    // 1.03, 1.07, 0.97, 1.00; x 48 to 128, 600,000 1.09-1.12, 1.13-1.15, 1.05-1.08, 1.07-1.09; x 100, 2,000,003 1.10, 1.14, 1.04,
+    // 1.07, 4,200,001 1.11, 1.15, 1.06, 1.08; x 32 from states, 200,000 1.00, 1.04, 0.95, 0.97; x 24, 600,000 1.02, 1.07, 0.97,
+    // 0.99; below one wave 120,000 x 128 1.03, 1.02, 1.00, 0.99, 90,000 x 128 1.00, 0.98, 0.96, 0.94. The larger networks, which the
+    // special-function unit binds in either kernel, were tried in the same form: 4-32-2, 4-64-2 and 4-16-16-2 at 300,000 and
+    // 1,000,003 0.98 to 1.05, at 75,000 and 100,000 0.88 to 1.03: they have no instance of it.
     // rollout_coop = 5 forces it wherever it applies, any other forced shape keeps the other kernels.
     // Calls that bring actions or start states as data: beyond the batches of the helper-warp kernel
     // below, and where every sort of data that was tried gains or nearly (time of this kernel over the
@@ -73,7 +74,10 @@ cudaError_t launch_rollout(RolloutParams &p, int policy, bool streams, bool cont
     if (!p.start_in && streams && warps64 < sms * 20) from = contracted ? 128u : 192u;
     const bool streams_gain = !streams || (p.start_in ? p.n * (int64_t)p.T <= 100000000 : warps64 >= sms * 7);
     int64_t least = sms * 4;  // 64-env warps
-    if (policy == 2) least = sms * 448;
+    // (4-16-2: whole waves, or several)
+    const bool waves = streams ? p.T >= 96u && warps64 >= sms * 64
+                               : p.T >= 64u && (warps64 >= sms * 48 || (warps64 >= sms * 17 && warps64 <= sms * 32));
+    if (policy == 2) least = waves ? 0 : sms * 448;
     if ((policy == 0 || policy == 1) && p.T >= 192u) least = sms * 7 / 2;
     const bool enough = data ? p.T >= from && warps32 > sms * 10 && streams_gain && !(p.max_steps && p.max_steps < 12u)
                              : warps64 >= least && p.T >= 12u;
