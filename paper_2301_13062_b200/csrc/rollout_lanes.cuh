@@ -14,8 +14,9 @@
 //     and one such environment after another lengthened launches by up to a fifth (4-64-2, 4,096 x 500, twelve
 //     policies: 139 .. 162 us against 133 .. 143). The deep network's lanes go by themselves: together they
 //     cost every launch 16 us for the few that gain (133 .. 154 against 148 .. 156).
-// One lane per environment (G = 1) is this kernel for its registers: the general one loads every weight in every
-// step.
+// One lane per environment (G = 1) is this kernel for 4-16-2's weights in registers, where the general one loads every weight in
+// every step, and for the larger networks, whose weights are loaded here too, for the shorter chain below and for per-step
+// outputs without a test of each in every step.
 //
 // What a step waits for is its chain: network, action, acceleration, rates, network. All of the step that does not
 // depend on the action is taken out of it (euler_both_ways: both candidates of the new rates, the termination test and
@@ -145,12 +146,15 @@ struct LaneNetwork {
     // Units 2q and 2q + 1 of the lane by one packed operation: half the instructions of a loop that waits for issue, with
     // one or two lanes per environment; alone on its scheduler a warp waits for latency, which they don't shorten.
     static constexpr bool kPaired = G <= 2;
+    // One lane, and more weights than it has registers: they are read from the launch parameters in every step.
+    static constexpr bool kReads = G == 1 && NET != 2;
     LaneLayer<kPaired ? 1 : U, 4> first;
-    f32x2 paired[kPaired ? U / 2 : 1][5], paired_step[kPaired ? U / 2 : 1];
-    LaneLayer<S::kDeep ? U : 1, S::kDeep ? S::H : 1> second;  // unused unless the network is deep
+    f32x2 paired[kPaired && !kReads ? U / 2 : 1][5], paired_step[kPaired && !kReads ? U / 2 : 1];
+    LaneLayer<S::kDeep && !kPaired ? U : 1, S::kDeep && !kPaired ? S::H : 1> second;  // unused unless the network is deep
     float step[kPaired ? 1 : U];                             // w1[j] - w0[j] of this lane's last-layer units
     __device__ __forceinline__ void load(const RolloutParams &p, uint32_t g) {
-        if constexpr (kPaired) {
+        if constexpr (kReads) {
+        } else if constexpr (kPaired) {
             static_assert(!S::kDeep, "one hidden layer");
             const float *w = p.w + (p.n >> 62), *logits = w + S::kLogits;
 #pragma unroll
@@ -230,9 +234,11 @@ __device__ __forceinline__ uint32_t lanes_defined_action(const RolloutParams &p,
 
 // The first hidden layer's activations of this lane's units.
 template <int NET, int G>
-__device__ __forceinline__ void lanes_activations(const LaneNetwork<NET, G> &net, const State &z, float (&h)[LaneNetwork<NET, G>::U]) {
+__device__ __forceinline__ void lanes_activations(const float *w, float base, const LaneNetwork<NET, G> &net, const State &z, float (&h)[LaneNetwork<NET, G>::U]) {
     constexpr int U = LaneNetwork<NET, G>::U;
-    if constexpr (LaneNetwork<NET, G>::kPaired) {
+    if constexpr (LaneNetwork<NET, G>::kReads) {
+        h[0] = screen_estimate<NET>(w, base, z);
+    } else if constexpr (LaneNetwork<NET, G>::kPaired) {
 #pragma unroll
         for (int q = 0; q < U / 2; ++q) unpack2(tanh_screen2(net.arguments(q, z)), h[2 * q], h[2 * q + 1]);
     } else {
@@ -251,7 +257,9 @@ __device__ __forceinline__ uint32_t lanes_action(const RolloutParams &p, const L
     using S = NetShape<NET>;
     constexpr int U = LaneNetwork<NET, G>::U;
     float part = 0.0f;
-    if constexpr (LaneNetwork<NET, G>::kPaired) {
+    if constexpr (LaneNetwork<NET, G>::kReads) {
+        part = h[0];
+    } else if constexpr (LaneNetwork<NET, G>::kPaired) {
         f32x2 sum = mul2(net.paired_step[0], pack2(h[0], h[1]));
 #pragma unroll
         for (int q = 1; q < U / 2; ++q) sum = fma2(net.paired_step[q], pack2(h[2 * q], h[2 * q + 1]), sum);
@@ -271,7 +279,7 @@ __device__ __forceinline__ uint32_t lanes_action(const RolloutParams &p, const L
     }
 #pragma unroll
     for (int o = 32 / G; o < 32; o <<= 1) part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, o));
-    const float estimate = __fadd_rn(p.screen_base, part);
+    const float estimate = LaneNetwork<NET, G>::kReads ? part : __fadd_rn(p.screen_base, part);
     uint32_t sb = screen_action(estimate);
     const bool open = !screen_decides(estimate, p.screen_bound);
     if constexpr (S::kDeep || G == 1) {
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(128, NET == 7 && !STREAMS ? 0 : 3) rollout_lan
     constexpr int E = 32 / G, W = 4;     // environments per warp; warps of a CTA, one per scheduler
     constexpr int C = G >= 4 ? 1 : 4 / G;  // state components that a lane hashes and stores
     static_assert(!STREAMS || E >= 8, "a warp writes whole bytes of the bit planes");
-    constexpr int ROW = kRow<NetShape<NET>::H>;
+    constexpr int ROW = G == 1 ? 1 : kRow<NetShape<NET>::H>;  // one lane: not used
     __shared__ __align__(16) float s_rows[W * E * ROW];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t e = lane % E, g = lane / E, c = (g * C) & 3u;  // c: the first of the lane's components
@@ -350,10 +358,11 @@ __global__ void __launch_bounds__(128, NET == 7 && !STREAMS ? 0 : 3) rollout_lan
     auto step = [&](auto general, auto given, uint32_t k) {
         const uint32_t t1 = p.t0 + k + 1u;
         float h[LaneNetwork<NET, G>::U];
-        // (One lane per environment, canonical: ahead of the rest in program order too, or the compiler loads the weights
-        // in every step: without outputs 0.59 to 0.84 of the time, with them 0.96 to 1.00; the other forms 0.94 to 1.23.)
-        constexpr bool FIRST = G == 1 && !CONTRACT && !decltype(general)::value;
-        if (FIRST) lanes_activations<NET, G>(net, z, h);
+        // (One lane per environment, canonical: ahead of the rest in program order too, or the compiler loads 4-16-2's weights
+        // in every step: without outputs 0.59 to 0.84 of the time, with them 0.96 to 1.00; the larger networks with outputs 0.96
+        // to 1.00, without 1.00 to 1.03; the other forms 0.94 to 1.23.)
+        constexpr bool FIRST = G == 1 && !CONTRACT && (NET == 2 || STREAMS) && !decltype(general)::value;
+        if (FIRST) lanes_activations<NET, G>(p.w, p.screen_base, net, z, h);
         // the start state that a finished environment continues from: this lane's components of it
         float mine[C];
         if constexpr (decltype(given)::value) asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
@@ -367,7 +376,7 @@ __global__ void __launch_bounds__(128, NET == 7 && !STREAMS ? 0 : 3) rollout_lan
         uint32_t sb;
         bool done;
         if constexpr (decltype(general)::value) {
-            lanes_activations<NET, G>(net, z, h);
+            lanes_activations<NET, G>(p.w, p.screen_base, net, z, h);
             sb = lanes_action<NET, G, CONTRACT>(p, net, z, h, row, g);
             const float force = force_from_signbit(sb);
             done = CONTRACT ? euler_step_contracted<false>(z, force) : euler_step<false>(z, force);
@@ -392,7 +401,7 @@ __global__ void __launch_bounds__(128, NET == 7 && !STREAMS ? 0 : 3) rollout_lan
             thd0 = done ? f.thd : thd0;
             thd1 = done ? f.thd : thd1;
             asm volatile("" : "+f"(x), "+f"(th), "+f"(xd0), "+f"(xd1), "+f"(thd0), "+f"(thd1));  // not after its branch
-            if (!FIRST) lanes_activations<NET, G>(net, z, h);
+            if (!FIRST) lanes_activations<NET, G>(p.w, p.screen_base, net, z, h);
             sb = lanes_action<NET, G, CONTRACT>(p, net, z, h, row, g);
             z.x = x;
             z.xd = sb ? xd1 : xd0;
@@ -499,7 +508,7 @@ cudaError_t launch_lanes_one(RolloutParams &p, cudaStream_t s) {
 // The instances that rollout_lanes_for asks for.
 template <int NET, bool STREAMS, bool CONTRACT>
 cudaError_t launch_lanes_g(RolloutParams &p, int g, cudaStream_t s) {
-    if constexpr (NET == 2)
+    if constexpr (STREAMS || NET == 2 || NET == 5)
         if (g == 1) return launch_lanes_one<NET, 1, STREAMS, CONTRACT>(p, s);
     if constexpr (NET == 2 || NET == 4)
         if (g == 2) return launch_lanes_one<NET, 2, STREAMS, CONTRACT>(p, s);

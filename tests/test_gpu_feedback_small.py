@@ -92,12 +92,12 @@ def test_networks_contracted(cp, kind, n, T):
         assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
 
 
-@pytest.mark.parametrize("kind", [MLP, MLP32])
+@pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
 @pytest.mark.parametrize("contracted", [False, True])
-@pytest.mark.parametrize("n,T", [(4737, 33), (9473, 31), (9487, 97), (18944, 64), (18961, 130), (28417, 65), (37889, 49), (56832, 66)])
+@pytest.mark.parametrize("n,T", [(4737, 33), (9473, 31), (9487, 97), (14209, 8), (18944, 64), (18961, 130), (28417, 65), (37889, 49), (56832, 66)])
 def test_networks_by_two_lanes_and_one(cp, kind, contracted, n, T):
-    """148 SMs: two lanes per environment up to 9,472 (4-16-2) and 28,416 (4-32-2), one up to 37,888 or 56,832
-    (4-16-2); sixteen or eight environments of the last warp or byte present."""
+    """148 SMs: two lanes per environment up to 9,472 (4-16-2) and 28,416 (4-32-2), one up to 37,888 or 56,832, depending on
+    network and outputs; sixteen or eight environments of the last warp or byte present."""
     for streams, limit, spread in (((), 0, "edge"), (ALL, 20, "wide"), (("reward_stream", "done_bits"), 0, None), (("action_bits",), 7, "edge")):
         args = dict(streams=streams, limit=limit, spread=spread, contracted=contracted)
         assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
