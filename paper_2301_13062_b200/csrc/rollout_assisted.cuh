@@ -180,7 +180,7 @@ __device__ __forceinline__ void consume_step(const RolloutParams &p, const PairB
 // up to two pairs per SM, where latency is the time: hashed actions, 500 steps, before / after (one helper), without outputs and
 // with reward and done bits, 9,400 environments 26.9 / 26.0 and 30.8 / 27.8 us; 20,011 54.6 / 54.7 and 60.4 / 62.5.
 // A batch of one pair per SM gets a helper on each of the three other schedulers: the one helper's 84 cycles per step
-// were as many as the stepping warp's 88. 2,048 x 10,000: 450 -> 389 us, 74 cycles per step, of which 55 are the stepping warp's
+// were as many as the stepping warp's 88. 2,048 x 10,000: 450 -> 389 us, 75 cycles per step, of which 50 are the stepping warp's
 // instructions; contracted 500 steps 24.7 -> 16.9, supplied actions 30.6 -> 23.2. (With two pairs per SM three helpers each
 // are slower, 9,400 x 500 28.7 against 26.0; for a policy, which the stepping warp evaluates, they gain 1-3 %.
 // The reciprocal of the denominator by a polynomial and a Newton step, which gives the same quotients and does not

@@ -70,8 +70,8 @@ constexpr int kMaxWarpsPerCta = 8;  // __launch_bounds__(256)
 //   4: as 0, with the start states read from the caller's array instead of hashed (a shape of
 //      its own because even a never-taken run-time test in the restart path cost shape 0
 //      4-6 %).
-// STREAMS: 0 no per-step output; 1 exactly the reward plane and the done bitmask (no run-time
-// tests in the loop); 2 any combination, tested per step.
+// STREAMS: 0 no per-step output; 1 exactly the reward plane and the done bitmask, 3 the action bitmask with them, 4 all
+// four outputs (no run-time tests in the loop, one running pointer per output); 2 any other combination, tested per step.
 // LIMIT: episodes are cut off after p.max_steps steps.
 // CONTRACT: the contracted arithmetic of euler_step_contracted instead of the canonical order.
 template <int POLICY, int SHAPE, int STREAMS, bool LIMIT, bool CONTRACT>
@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
     constexpr bool AHEAD = SHAPE == 3;
     constexpr bool START_IN = SHAPE == 4;
     constexpr bool PAIR = SHAPE == 2 && !CONTRACT;  // packed two-env arithmetic
+    constexpr bool FIXED = STREAMS == 1 || STREAMS >= 3;
     const uint32_t lane = threadIdx.x & 31u;
     // Per warp: key pairs of up to 8 finished envs, and their 8 x 4 start-state components.
     __shared__ uint2 s_keys[COOP ? kMaxWarpsPerCta : 1][8];
@@ -154,13 +155,15 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
             word_off[j] = task * EPT + j;
             const bool in_range = word_off[j] < words;
             word_ok[j] = lane == 0 && in_range;
-            // STREAMS == 1 keeps ONE running pointer per stream: slot j's element lies a constant
+            // fixed outputs keep ONE running pointer per stream: slot j's element lies a constant
             // 32 floats / 1 word behind slot 0's (never dereferenced where the slot has no env)
-            rew_ptr[j] = STREAMS == 1 ? p.reward_stream + (base + lane) : nullptr;
-            done_ptr[j] = STREAMS == 1 ? p.done_bits + task * EPT : nullptr;
+            rew_ptr[j] = FIXED ? p.reward_stream + (base + lane) : nullptr;
+            done_ptr[j] = FIXED ? p.done_bits + task * EPT : nullptr;
             act_ptr[j] = POLICY == 3 ? p.action_bits_in + (in_range ? word_off[j] : 0) : nullptr;
             vmask[j] = __ballot_sync(0xffffffffu, valid[j]);
         }
+        uint32_t *taken_ptr = STREAMS >= 3 ? p.action_bits + task * EPT : nullptr;
+        float *traj_ptr = STREAMS == 4 ? p.trajectory + (base + lane) : nullptr;
         const bool want_done = STREAMS == 2 && p.done_bits, want_act = STREAMS == 2 && p.action_bits;
         const bool want_rew = STREAMS == 2 && p.reward_stream, want_traj = STREAMS == 2 && p.trajectory;
 
@@ -337,13 +340,27 @@ __global__ void __launch_bounds__(256, 1) rollout_kernel(const __grid_constant__
 
 #pragma unroll
             for (int j = 0; j < EPT; ++j) {
-                if (STREAMS == 1) {
+                if (FIXED) {
                     const uint32_t m = COOP ? (dmask[j] & vmask[j]) : __ballot_sync(0xffffffffu, done[j] && valid[j]);
                     if (word_ok[j]) done_ptr[0][j] = m;
-                    if (valid[j]) rew_ptr[0][32 * j] = 1.0f;
+                    if (STREAMS >= 3) {
+                        const uint32_t taken = __ballot_sync(0xffffffffu, (sb[j] != 0u) && valid[j]);
+                        if (word_ok[j]) taken_ptr[j] = taken;
+                    }
+                    if (valid[j]) {
+                        rew_ptr[0][32 * j] = 1.0f;
+                        if (STREAMS == 4) {
+                            traj_ptr[32 * j] = z[j].x;
+                            traj_ptr[p.n + 32 * j] = z[j].xd;
+                            traj_ptr[2 * p.n + 32 * j] = z[j].th;
+                            traj_ptr[3 * p.n + 32 * j] = z[j].thd;
+                        }
+                    }
                     if (j == EPT - 1) {
                         done_ptr[0] += words;
                         rew_ptr[0] += p.n;
+                        if (STREAMS >= 3) taken_ptr += words;
+                        if (STREAMS == 4) traj_ptr += 4 * p.n;
                     }
                 }
                 if (STREAMS == 2) {
@@ -471,6 +488,8 @@ cudaError_t launch_mode(RolloutParams &p, int mode, int shape, cudaStream_t s) {
     switch (mode) {
         case 0: return launch_limit<POLICY, 0, CONTRACT>(p, shape, s);
         case 1: return launch_limit<POLICY, 1, CONTRACT>(p, shape, s);
+        case 3: return launch_limit<POLICY, 3, CONTRACT>(p, shape, s);
+        case 4: return launch_limit<POLICY, 4, CONTRACT>(p, shape, s);
         default: return launch_limit<POLICY, 2, CONTRACT>(p, shape, s);
     }
 }
@@ -506,14 +525,25 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
     // (the larger networks restart per lane on every batch: 1,000,000 x 100 4-64-2 1,657 us against 1,741, 4-16-16-2
     // 1,573 against 1,624, 4-32-2 868 against 869)
     const bool wide = policy == 4 || policy == 5 || policy == 7;
-    if (coop == 0) coop = ((small || wide) && ept == 1 && !tested) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
+    // (contracted, one linear policy each, all four outputs: 300,000 x 64 by the warp 92 us, as with tests, per lane 79)
+    const bool own_all = CONTRACT && policy == 6 && p.reward_stream && p.done_bits && p.action_bits && p.trajectory;
+    if (coop == 0) coop = ((small || wide || own_all) && ept == 1 && !tested) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
     // two envs per thread are always cooperative; supplied start states are read by the lane that
     // needs them, so they always take the per-lane shape that reads them (4)
     // (coop 4 asks for the producer-assisted kernel of rollout_assisted.cu; a call it does not
     // cover lands here and takes the plain per-lane shape)
     const int shape = p.start_in ? 4 : ept == 2 ? 2 : ((coop == 2 || coop == 4) ? 0 : coop == 3 ? 3 : 1);
-    // 0: no per-step output; 1: reward plane + done bitmask only; 2: any other combination
-    const int mode = !streams ? 0 : (p.reward_stream && p.done_bits && !p.action_bits && !p.trajectory) ? 1 : 2;
+    // 0: no per-step output; 1: reward plane + done bitmask, 3: + action bitmask, 4: + trajectory; 2: any other combination
+    // Without tests / with, x 64: reward, done and action bits 60,001 environments hashed actions 19.9 / 23.9 us, one linear policy each
+    // 22.1 / 25.7, shared 20.6 / 24.1, 1,000,003 217 / 258, 244 / 278, 240 / 292, 4-16-2 443 / 472, 4-64-2 1,073 / 1,129; all four 60,001
+    // 24.8 / 27.8, 24.8 / 29.1, 24.7 / 27.7, 600,000 148 / 176, 169 / 194, 163 / 196, 4-64-2 683 / 679. But rows that do not start on
+    // 32 bytes reach memory in parts once a launch writes more than L2 holds, and the faster writer then pays (tests / none,
+    // 200,003 x 64 75 / 68, 80 / 83, 84 / 70, contracted 70 / 74, 81 / 77, 76 / 78; 70,001 x 300 121 / 125, 129 / 130, 126 / 132, 118 / 129,
+    // 122 / 135, 124 / 134; 1,000,003 x 64 305 / 324; but 100,003 x 64 40 / 36, 42 / 39, 40 / 36, contracted 38 / 36, 39 / 40, 38 / 36,
+    // 50,001 x 300 101 / 87, 109 / 89, 105 / 90, 95 / 87, 99 / 91, 99 / 89): all four stay tested there. And so they do with supplied
+    // actions, whose warps drift apart as they read (120,000 x 200 167 / 187, 131,072 x 200 164 / 226, 200,000 x 200 248 / 233).
+    const bool four = p.action_bits && !p.action_bits_in && (p.n % 8 == 0 || p.n * (int64_t)p.T <= 6500000 || (p.n + 31) / 32 <= (int64_t)sm_count() * 12);
+    const int mode = !streams ? 0 : !(p.reward_stream && p.done_bits) ? 2 : p.trajectory ? (four ? 4 : 2) : p.action_bits ? 3 : 1;
     // the network policies are instantiated in translation units of their own (build time)
     if (policy == 2 || policy == 4 || policy == 5 || policy == 7)
         return CONTRACT ? launch_rollout_networks_contracted(p, policy, mode, shape, s)

@@ -157,3 +157,20 @@ def test_hashed_and_given_actions_by_pairs_per_sm(cp, given, contracted, n, T):
                                    (("reward_stream", "done_bits"), 20, None), (ALL, 0, "edge")):
         args = dict(streams=streams, limit=limit, spread=spread, contracted=contracted, given=bits if given else None)
         assert_same_bits(rollout(cp, 0, 0, n, T, **args), rollout(cp, 2, 0, n, T, **args))
+
+
+@pytest.mark.parametrize("kind", [0, LINEAR, PER_ENV, MLP, MLP64])
+@pytest.mark.parametrize("coop", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,T", [(1, 5), (33, 7), (65, 3), (1000, 9), (57_001, 115), (160_001, 3)])
+def test_outputs_together_equal_outputs_apart(cp, kind, coop, n, T):
+    """The general kernel's instances for fixed combinations of outputs (with the action bits, all four) write what the
+    instance that tests for each output writes, in every shape; the size before the last is one where all four stay tested, the last has two environments per thread."""
+    words = (n + 31) // 32
+    bits = torch.from_numpy(np.random.default_rng(4).integers(-2**31, 2**31, (T, words)).astype(np.int32)).cuda()
+    for contracted, limit, given in ((False, 0, None), (True, 4, None), (False, 6, bits if kind == 0 else None)):
+        args = dict(limit=limit, contracted=contracted, given=given, spread="edge")
+        apart = rollout(cp, coop, kind, n, T, streams=("done_bits", "trajectory"), **args)
+        apart |= rollout(cp, coop, kind, n, T, streams=("reward_stream", "action_bits"), **args)
+        for streams in (ALL, ("reward_stream", "done_bits", "action_bits")):
+            got = rollout(cp, coop, kind, n, T, streams=streams, **args)
+            assert_same_bits(got, {k: apart[k] for k in got})
