@@ -42,7 +42,7 @@ SMS = 148
 # states of the 4.5 % of env-steps that restart, 8 more for the linear policy).
 # COUNTED_AT = build.kernel_hash() of the sources these were captured from (a test compares it
 # with the current sources, so that the fractions cannot go stale unnoticed).
-COUNTED_AT = "6e2a5ea35eac1ca0"
+COUNTED_AT = "d4213d0d534c0e03"
 # pipe_busy: sm__pipe_fmaheavy_cycles_active (share of the launch's cycles) in the same captures — the
 # resource that bounds these kernels; it counts idle slots' arithmetic and the integer multiply-adds too.
 ROLLOUT_OPS = {

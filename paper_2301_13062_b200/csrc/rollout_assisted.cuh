@@ -4,7 +4,7 @@
 //
 // Everything random in a rollout depends on (seed, env, time) only, never on the trajectory. So
 // each stepping warp ("consumer") gets a helper warp ("producer") on another scheduler of the
-// same SM that hashes, a chunk of steps ahead, the action force and the start state of every
+// same SM, on the smallest batches one on each of the three others, that hashes, a chunk of steps ahead, the action force and the start state of every
 // step for the consumer's 32 environments into shared memory. The consumer's step is then two
 // shared-memory loads, the dynamics, the termination test and four selects: about 60 instead
 // of 110 instructions, with no integer hashing in its dependency chain. Same hashes, same

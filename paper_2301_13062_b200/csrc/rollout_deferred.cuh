@@ -43,9 +43,9 @@ namespace cp {
 
 namespace {
 
-// Shared policies read their weights as (w, w) pairs: the launcher duplicates every weight in the
+// The shared linear policy reads its weights as (w, w) pairs: the launcher duplicates every weight in the
 // launch parameters, so that one packed fused multiply-add applies it to both environments of a
-// thread. Each half is the scalar chain of linear_action / mlp_action (same order, one rounding per
+// thread. Each half is the scalar chain of linear_action (same order, one rounding per
 // fused operation), hence the same logits bit for bit.
 __device__ __forceinline__ void argmax_pair(f32x2 l0, f32x2 l1, uint32_t &sb0, uint32_t &sb1) {
     float a0, a1, b0, b1;
