@@ -117,7 +117,8 @@ cudaError_t launch_pair_selftest(unsigned long long count, uint32_t seed, unsign
 cudaError_t launch_screen_selftest(unsigned long long *out, cudaStream_t s);
 // A network's weights in RolloutParams::w rearranged for its estimate, with the bound the estimate needs (policy_screen.cu).
 void screen_units(RolloutParams &p, int policy);
-void screen_bound(RolloutParams &p, int policy);  // the bound alone, weights as the caller gave them
+// the bound alone, for an environment's units over `lanes` lanes; weights as the caller gave them
+void screen_bound(RolloutParams &p, int policy, int lanes);
 cudaError_t launch_tame_div_selftest(uint32_t den_step, unsigned long long *out, cudaStream_t s);
 
 // The per-op ladder. Workspace layout is private to ladder_kernels.cu.

@@ -9,6 +9,18 @@ namespace cp {
 // float32 (measured: 7.987e-6 for both, cp_selftest_screen).
 constexpr double kTanhScreenError = 8.0e-6;
 
+// Roundings that a term of the estimate goes through at most, in the kernels' orders.
+// Units 2q and 2q + 1 of one lane side by side, a multiply-add per pair onto the base, then both halves' sum; a second
+// hidden layer's units one after another (screen_estimate, screen_estimate_two).
+constexpr int units_rounds(int units, bool deep) { return deep ? units : units / 2 + 1; }
+// An environment's units spread over `lanes` lanes (rollout_lanes.cuh): with one or two lanes a pair of units per
+// product or multiply-add and both halves' sum, with more one unit each; then a sum per doubling of the lanes and the base.
+constexpr int lanes_rounds(int units, int lanes) {
+    int rounds = (lanes <= 2 ? units / lanes / 2 + 1 : units / lanes) + 1;
+    for (; lanes > 1; lanes /= 2) ++rounds;
+    return rounds;
+}
+
 struct PolicyBound {
     float base;   // the estimate's constant term, b1 - b0
     float bound;  // largest distance of an estimate from l1 - l0; negative: every estimate that is not NaN decides

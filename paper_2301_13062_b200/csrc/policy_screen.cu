@@ -20,15 +20,16 @@ template <int NET>
 void units(RolloutParams &p) {
     using S = NetShape<NET>;
     constexpr int H = S::H;
-    screen<NET>(p, p.w + S::kUnitSteps, S::kDeep ? H : H / 2 + 1);
+    screen<NET>(p, p.w + S::kUnitSteps, units_rounds(H, S::kDeep));
     for (int j = 0; j < H; ++j)
         for (int i = 0; i < 5; ++i) p.w[S::kUnitFirst + 10 * (j / 2) + 2 * i + j % 2] = p.w[i < 4 ? 4 * j + i : 4 * H + j];
 }
 
 template <int NET>
-void bound_alone(RolloutParams &p) {  // four or eight lanes: H / 4 or H / 8 terms, two or three shuffles, the base
-    float steps[NetShape<NET>::H];
-    screen<NET>(p, steps, NetShape<NET>::H / 4 + 3);
+void bound_alone(RolloutParams &p, int lanes) {
+    constexpr int H = NetShape<NET>::H;
+    float steps[H];
+    screen<NET>(p, steps, lanes_rounds(H, lanes));
 }
 
 }  // namespace
@@ -42,12 +43,12 @@ void screen_units(RolloutParams &p, int policy) {
     }
 }
 
-void screen_bound(RolloutParams &p, int policy) {
+void screen_bound(RolloutParams &p, int policy, int lanes) {
     switch (policy) {
-        case 2: return bound_alone<2>(p);
-        case 4: return bound_alone<4>(p);
-        case 5: return bound_alone<5>(p);
-        default: return bound_alone<7>(p);
+        case 2: return bound_alone<2>(p, lanes);
+        case 4: return bound_alone<4>(p, lanes);
+        case 5: return bound_alone<5>(p, lanes);
+        default: return bound_alone<7>(p, lanes);
     }
 }
 

@@ -75,7 +75,7 @@ int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool con
 
 cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s) {
     if (g == 1 && policy != 2) screen_units(p, policy);
-    else screen_bound(p, policy);
+    else screen_bound(p, policy, g);
     switch (policy) {
         case 2: return contracted ? launch_lanes_net<2, true>(p, g, streams, s) : launch_lanes_net<2, false>(p, g, streams, s);
         case 4: return launch_lanes_mlp32(p, g, streams, contracted, s);
