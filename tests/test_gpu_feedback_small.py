@@ -104,11 +104,14 @@ def test_networks_by_two_lanes_and_one(cp, kind, contracted, n, T):
 
 
 @pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
-@pytest.mark.parametrize("n", [97, 1500, 4097])
-def test_networks_from_supplied_starts(cp, kind, n):
-    for streams in ((), ALL):
-        args = dict(streams=streams, starts=start_rows(50, n), spread="edge")
-        assert_same_bits(rollout(cp, 0, kind, n, 50, **args), rollout(cp, 2, kind, n, 50, **args))
+@pytest.mark.parametrize("contracted", [False, True])
+@pytest.mark.parametrize("n,T", [(97, 50), (1500, 50), (4097, 50), (4737, 50), (4745, 9), (9473, 51), (14_209, 50), (18_961, 10)])
+def test_networks_from_supplied_starts(cp, kind, contracted, n, T):
+    """With four lanes per environment and, with outputs beyond 4,736 environments on 148 SMs, with two and one, whose lanes
+    bring two and four components each; angles beyond the polynomial range, NaN and infinities among the start states."""
+    for streams, limit in (((), 0), (ALL, 0), (ALL, 6), (("reward_stream", "done_bits"), 0)):
+        args = dict(streams=streams, limit=limit, starts=start_rows(T, n), spread="edge", contracted=contracted)
+        assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
 
 
 @pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])

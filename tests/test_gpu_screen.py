@@ -50,10 +50,13 @@ def test_estimates_decide_as_the_defined_logits_do(cp, kind, contracted, apart):
     w, last = weights(kind, apart)
     scaled = w.copy()
     scaled[last:] *= np.float32(2.0**100)
-    # sizes: one environment, either side of a bit-plane word, and the kernel a caller gets for larger batches;
-    # coop 2 / 5: the general kernel and the deferred-restart kernel wherever it applies
+    # sizes: one environment, either side of a bit-plane word, and the kernel a caller gets for larger batches (148 SMs:
+    # two lanes per environment at 4,737 for 4-16-2 and 4-32-2, which keeps them without outputs at 9,473; one lane at 9,473
+    # for the others but 4-64-2, for that one at 14,209); coop 2 / 5: the general kernel and the deferred-restart kernel wherever it applies
     for coop, n, T, streams, limit in ((0, 1, 40, (), 0), (0, 33, 33, ALL, 20), (0, 1200, 35, (), 9), (2, 97, 40, ALL, 0),
                                        (2, 65, 40, (), 20), (5, 129, 45, (), 0), (0, 70_001, 14, (), 0),
+                                       (0, 4737, 33, (), 9), (0, 4737, 33, ALL, 0), (0, 9473, 33, (), 0), (0, 9473, 33, ALL, 20),
+                                       (0, 14_209, 33, (), 20), (0, 14_209, 33, ALL, 0),
                                        (5, 129, 45, ("reward_stream", "done_bits"), 20)):
         args = (kind, n, T, streams, limit, contracted)
         assert_same_bits(rollout(cp, coop, w, *args), rollout(cp, coop, scaled, *args))
