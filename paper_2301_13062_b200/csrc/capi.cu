@@ -63,7 +63,10 @@ int fail(int code, const char *fmt, ...) {
     return code;
 }
 
+// (The runtime keeps a call's error for cudaGetLastError too, which the launches ask: taken here, or the next
+// call's first launch would report it once more.)
 int cuda_fail(cudaError_t e, const char *what) {
+    (void)cudaGetLastError();
     return fail(CP_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
