@@ -12,8 +12,10 @@ cudaError_t launch_lanes_deep(RolloutParams &p, int g, bool streams, bool contra
 // How many lanes an environment gets, and from how many steps on. A warp of this kernel takes its step's latency
 // whatever it holds, until its scheduler has a second one: so as many lanes as leave every scheduler its one warp,
 // and more warps where that is still quicker than the general kernel. Four lanes for up to 4,736 environments on 148 SMs
-// (more measured the same or slower, but for the smallest batches without outputs: 1,000 environments x 300, eight over four
-// lanes, 4-32-2 1.04, 4-64-2 1.20, 4-16-16-2 1.10, contracted 4-16-16-2 0.69, 4-16-2 0.95), two and one beyond them.
+// (more measured the same or slower, but for the smallest batches without outputs: 1,000 environments x 300, time of four
+// lanes over eight, 4-32-2 1.04, 4-64-2 1.20, 4-16-16-2 1.10, contracted 4-16-16-2 0.69, 4-16-2 0.95; below twelve steps, 33 to
+// 2,368 environments at 3, 4, 5, 8 steps, 4-64-2 0.94-0.98, 0.94-0.99, 0.95-0.99, 0.97-1.00, 4-16-16-2 0.93-0.99, 0.95-1.00,
+// 0.95-1.00, 0.97-1.01), two and one beyond them.
 // us per launch, general kernel / this one, canonical, 300 steps without outputs, then with reward and done bits, then
 // with all four:
 //     environments         4,096                  9,001                  18,900                 37,800
@@ -23,10 +25,11 @@ cudaError_t launch_lanes_deep(RolloutParams &p, int g, bool streams, bool contra
 //     4-16-16-2    144 / 68 165 / 84 194 / 85  144 / 101 165 / 120 195 / 119    (see below)
 // Time of the general kernel over this one's around the lines, at the step counts given ("plain": reward and done bits alone,
 // for which the general kernel has an instance without tests; "tested": action bits or trajectory too):
-//   one warp per scheduler: 4 lanes without outputs x 3 1.03-1.05, contracted x 4 1.05, plain x 6 1.04-1.19; 2 lanes x 6
-//     1.05-1.08, plain x 8 1.05-1.08; 1 lane x 24 1.03-1.15, tested x 6 1.04
+//   one warp per scheduler: 4 lanes without outputs x 3 1.03-1.05, contracted x 4 1.05, plain x 6 1.04-1.19, 4-64-2 plain x 3
+//     0.99-1.33, x 4 1.07-1.41 (the others x 4 0.89-1.06); 2 lanes 4-16-2 x 6 1.05-1.08, plain x 8 1.05-1.08, 4-32-2 x 6 0.90-1.06,
+//     x 8 0.97-1.12, plain x 8 0.93-1.04, x 12 1.04-1.13; 1 lane x 24 1.03-1.15, tested x 6 1.04
 //   two: 4-16-2 x 64 1.01-1.04, plain canonical x 96 1.01 (contracted never more than 1.01), tested x 12 1.03; 4-32-2 x 24
-//     1.03-1.09, plain x 48 1.00-1.04; 4-64-2 x 16 1.06-1.34; 4-16-16-2 x 24 1.06-1.29
+//     0.95-1.03, contracted 1.01-1.09, plain x 48 1.00-1.04; 4-64-2 x 16 1.06-1.34; 4-16-16-2 x 24 1.06-1.29
 //   three: 4-16-2 tested x 48 1.05-1.09 (otherwise at most 1.00); 4-32-2 x 64 1.05-1.10 (plain at most 1.00);
 //     4-64-2 x 32 1.04-1.15; 4-16-16-2 x 64 1.00-1.09 (plain canonical at most 0.96)
 //   the larger networks by one lane, one / two / three warps: 4-32-2 tested x 8 1.13-1.15, 1.09-1.12, 1.01 (x 32 1.31, 1.20,
@@ -52,12 +55,12 @@ int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool con
     const int w = warps(g);
     uint32_t from = 0u;  // steps; 0: the general kernel
     if (g == 4) {
-        if (w == 1) from = plain ? 6u : contracted ? 4u : 3u;
+        if (w == 1) from = plain ? (policy == 5 ? 3u : 6u) : contracted ? 4u : 3u;
         else if (w == 2) from = policy == 5 ? 16u : policy == 7 ? 24u : 32u;
         else if (w == 3) from = policy == 2 ? 128u : policy == 4 ? (contracted ? 32u : 64u) : policy == 5 ? 32u : plain && !contracted ? 0u : 64u;
     } else if (g == 2) {
-        if (w == 1) from = plain ? 8u : 6u;
-        else if (w == 2) from = plain ? 48u : 24u;
+        if (w == 1) from = policy == 4 ? (plain ? 10u : 8u) : plain ? 8u : 6u;
+        else if (w == 2) from = plain ? 48u : contracted ? 24u : 32u;
         else if (w == 3) from = plain ? 0u : 64u;
     } else if (policy == 2) {
         if (w == 1) from = tested ? 6u : 24u;
@@ -70,7 +73,7 @@ int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool con
         if (w <= 3) from = w <= 2 ? 8u : 32u;
     }
     if (from == 0u || p.T < from) return 0;
-    return !streams && policy != 2 && !(policy == 7 && contracted) && warps(8) == 1 ? 8 : g;
+    return !streams && policy != 2 && !(policy == 7 && contracted) && warps(8) == 1 && (policy == 4 || p.T >= 12u) ? 8 : g;
 }
 
 cudaError_t launch_rollout_lanes(RolloutParams &p, int policy, int g, bool streams, bool contracted, cudaStream_t s) {

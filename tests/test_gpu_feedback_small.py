@@ -76,10 +76,11 @@ def start_rows(T, n):
 
 
 @pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
-@pytest.mark.parametrize("n,T", [(1, 33), (31, 64), (33, 5), (1184, 40), (1185, 31), (2369, 32), (4737, 31),
+@pytest.mark.parametrize("n,T", [(1, 33), (31, 64), (33, 5), (1000, 4), (1184, 11), (1184, 40), (1185, 31), (2369, 32), (4737, 31),
                                  (9465, 65), (9472, 33), (9473, 33), (9473, 129), (14208, 129), (14209, 129)])
 def test_networks(cp, kind, n, T):
-    for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("done_bits",), 0, "edge"), (("trajectory",), 9, None)):
+    for streams, limit, spread in (((), 0, None), (ALL, 20, "wide"), (("done_bits",), 0, "edge"), (("trajectory",), 9, None),
+                                   (("reward_stream", "done_bits"), 0, "edge")):
         args = dict(streams=streams, limit=limit, spread=spread)
         assert_same_bits(rollout(cp, 0, kind, n, T, **args), rollout(cp, 2, kind, n, T, **args))
 
