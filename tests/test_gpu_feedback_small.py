@@ -106,7 +106,7 @@ def test_networks_by_two_lanes_and_one(cp, kind, contracted, n, T):
 
 @pytest.mark.parametrize("kind", [MLP, MLP32, MLP64, DEEP])
 @pytest.mark.parametrize("contracted", [False, True])
-@pytest.mark.parametrize("n,T", [(97, 50), (1500, 50), (4097, 50), (4737, 50), (4745, 9), (9473, 51), (14_209, 50), (18_961, 10)])
+@pytest.mark.parametrize("n,T", [(97, 50), (1500, 50), (4097, 50), (4737, 50), (4745, 17), (9473, 65), (14_209, 64), (18_961, 130)])
 def test_networks_from_supplied_starts(cp, kind, contracted, n, T):
     """With four lanes per environment and, with outputs beyond 4,736 environments on 148 SMs, with two and one, whose lanes
     bring two and four components each; angles beyond the polynomial range, NaN and infinities among the start states."""
