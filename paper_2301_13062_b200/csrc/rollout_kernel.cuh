@@ -497,6 +497,33 @@ cudaError_t launch_mode(RolloutParams &p, int mode, int shape, cudaStream_t s) {
 template <bool CONTRACT>
 cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cudaStream_t s) {
     if (p.action_bits_in) policy = 3;
+    // 0: no per-step output; 1: reward plane + done bitmask, 3: + action bitmask, 4: + trajectory; 2: any other combination
+    // Without tests / with, x 64: reward, done and action bits 60,001 environments hashed actions 19.9 / 23.9 us, one linear policy each
+    // 22.1 / 25.7, shared 20.6 / 24.1, 1,000,003 217 / 258, 244 / 278, 240 / 292, 4-16-2 443 / 472, 4-64-2 1,073 / 1,129; all four 60,001
+    // 24.8 / 27.8, 24.8 / 29.1, 24.7 / 27.7, 600,000 148 / 176, 169 / 194, 163 / 196, 4-64-2 683 / 679. But rows that do not start on
+    // 32 bytes reach memory in parts once a launch writes more than L2 holds (21 bytes per step), and the faster writer then pays
+    // (us, tests / none, 200,003 x 64 75 / 68, 80 / 83, 84 / 70, 70,001 x 300 121 / 125, 129 / 130, 126 / 132, 1,000,003 x 64 305 / 324):
+    // all four stay tested from some number of steps of all environments on. Time without tests over with, around the lines:
+    //   up to twelve warps per SM (48,001 to 56,801 environments), one shared linear policy, 12 to 16 million 0.86-1.00, 17 to 20
+    //     0.96-1.06, 24 to 28 0.96-1.16, contracted 7 to 9 0.84-0.99, 10 to 12 0.93-1.14, 24 to 28 1.13-1.34; the others 18 to 23
+    //     0.82-0.98, 24 to 28 0.88-1.02, contracted 14 to 17 0.86-0.98, 18 to 21 0.93-1.06, 24 to 28 0.98-1.15;
+    //   beyond, 5.0 to 6.45 million, 100,003 to 600,003 environments, canonical and contracted hashed actions 0.83-1.03; contracted
+    //     linear 5.2 to 6.0 0.85-1.05, 6.3 to 6.45 0.90-1.09; one policy each, whose weights L2 holds too, up to 200,003 5.4 to 6.0
+    //     0.86-1.04, 6.3 to 6.45 0.87-1.05, 300,003 to 600,003 5.2 to 6.45 1.00-1.10; one shared linear policy between 30 and 32 warps
+    //     per SM (145,001 to 151,001), where the restarts of a lane by itself end, 0.9 million 0.93-1.04, 1.9 to 6.4 0.91-1.07.
+    // So they do with supplied actions, whose warps drift apart as they read (120,000 x 200 167 / 187, 131,072 x 200 164 / 226,
+    // 200,000 x 200 248 / 233); and contracted ones restarted per lane, 24 to 32 warps per SM, also without the trajectory: 120,000 to
+    // 150,001 x 200, 300, 500 0.88-1.26, 1.01-1.27, 1.08-1.30 (131,072 x 200 143 / 181), up to 25 million steps 0.82-0.94; 110,003 and
+    // 152,000 0.82-0.88.
+    const int64_t warps = (p.n + 31) / 32, sms = sm_count(), steps = p.n * (int64_t)p.T;
+    int64_t most = 6500000;  // steps of all environments
+    if (warps <= sms * 12) most = CONTRACT ? (policy == 1 ? 9900000 : 18000000) : (policy == 1 ? 16000000 : 26000000);
+    else if (policy == 1 && warps > sms * 30 && warps <= sms * 32) most = 1000000;
+    else if (CONTRACT && policy == 1) most = 6200000;
+    else if (CONTRACT && policy == 6) most = warps <= sms * 48 ? 6000000 : 5700000 - 2 * p.n;
+    const bool four = p.action_bits && !p.action_bits_in && (p.n % 8 == 0 || steps <= most);
+    const bool three = !(CONTRACT && policy == 3 && warps > sms * 24 && warps <= sms * 32 && steps > 26000000);
+    const int mode = !streams ? 0 : !(p.reward_stream && p.done_bits) ? 2 : p.trajectory ? (four ? 4 : 2) : p.action_bits ? (three ? 3 : 2) : 1;
     // A batch too small to give every SM sixteen two-env warps is latency-bound: one env per
     // thread over twice as many warps, and per-lane restarts (the cooperative restart adds two
     // shared-memory round trips to every step's dependency chain: 2,048 envs x 10,000 steps
@@ -525,41 +552,16 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
     // (the larger networks restart per lane on every batch: 1,000,000 x 100 4-64-2 1,657 us against 1,741, 4-16-16-2
     // 1,573 against 1,624, 4-32-2 868 against 869)
     const bool wide = policy == 4 || policy == 5 || policy == 7;
-    // (contracted, one linear policy each, all four outputs: 300,000 x 64 by the warp 92 us, as with tests, per lane 79)
-    const bool own_all = CONTRACT && policy == 6 && p.reward_stream && p.done_bits && p.action_bits && p.trajectory;
+    // (contracted, one linear policy each, all four outputs: 300,000 x 64 by the warp 92 us, as with tests, per lane 79, 160,001 to
+    // 600,003 environments 0.82-0.97 of the time by the warp; with tests, on the rows above, per lane over by the warp from 24 steps
+    // on 0.94-1.00, 600,003 to 2,000,003 x 8 and 16 1.01-1.04)
+    const bool own_all = CONTRACT && policy == 6 && p.reward_stream && p.done_bits && p.action_bits && p.trajectory && (four || p.T >= 24u);
     if (coop == 0) coop = ((small || wide || own_all) && ept == 1 && !tested) ? ((tiny && (policy == 0 || policy == 3)) ? 3 : 2) : 1;
     // two envs per thread are always cooperative; supplied start states are read by the lane that
     // needs them, so they always take the per-lane shape that reads them (4)
     // (coop 4 asks for the producer-assisted kernel of rollout_assisted.cu; a call it does not
     // cover lands here and takes the plain per-lane shape)
     const int shape = p.start_in ? 4 : ept == 2 ? 2 : ((coop == 2 || coop == 4) ? 0 : coop == 3 ? 3 : 1);
-    // 0: no per-step output; 1: reward plane + done bitmask, 3: + action bitmask, 4: + trajectory; 2: any other combination
-    // Without tests / with, x 64: reward, done and action bits 60,001 environments hashed actions 19.9 / 23.9 us, one linear policy each
-    // 22.1 / 25.7, shared 20.6 / 24.1, 1,000,003 217 / 258, 244 / 278, 240 / 292, 4-16-2 443 / 472, 4-64-2 1,073 / 1,129; all four 60,001
-    // 24.8 / 27.8, 24.8 / 29.1, 24.7 / 27.7, 600,000 148 / 176, 169 / 194, 163 / 196, 4-64-2 683 / 679. But rows that do not start on
-    // 32 bytes reach memory in parts once a launch writes more than L2 holds (21 bytes per step), and the faster writer then pays
-    // (us, tests / none, 200,003 x 64 75 / 68, 80 / 83, 84 / 70, 70,001 x 300 121 / 125, 129 / 130, 126 / 132, 1,000,003 x 64 305 / 324):
-    // all four stay tested from some number of steps of all environments on. Time without tests over with, around the lines:
-    //   up to twelve warps per SM (48,001 to 56,801 environments), one shared linear policy, 12 to 16 million 0.86-1.00, 17 to 20
-    //     0.96-1.06, 24 to 28 0.96-1.16, contracted 7 to 9 0.84-0.99, 10 to 12 0.93-1.14, 24 to 28 1.13-1.34; the others 18 to 23
-    //     0.82-0.98, 24 to 28 0.88-1.02, contracted 14 to 17 0.86-0.98, 18 to 21 0.93-1.06, 24 to 28 0.98-1.15;
-    //   beyond, 5.0 to 6.45 million, 100,003 to 600,003 environments, canonical and contracted hashed actions 0.83-1.03; contracted
-    //     linear 5.2 to 6.0 0.85-1.05, 6.3 to 6.45 0.90-1.09; one policy each, whose weights L2 holds too, up to 200,003 5.4 to 6.0
-    //     0.86-1.04, 6.3 to 6.45 0.87-1.05, 300,003 to 600,003 5.2 to 6.45 1.00-1.10; one shared linear policy between 30 and 32 warps
-    //     per SM (145,001 to 151,001), where the restarts of a lane by itself end, 0.9 million 0.93-1.04, 1.9 to 6.4 0.91-1.07.
-    // So they do with supplied actions, whose warps drift apart as they read (120,000 x 200 167 / 187, 131,072 x 200 164 / 226,
-    // 200,000 x 200 248 / 233); and contracted ones restarted per lane, 24 to 32 warps per SM, also without the trajectory: 120,000 to
-    // 150,001 x 200, 300, 500 0.88-1.26, 1.01-1.27, 1.08-1.30 (131,072 x 200 143 / 181), up to 25 million steps 0.82-0.94; 110,003 and
-    // 152,000 0.82-0.88.
-    const int64_t warps = (p.n + 31) / 32, sms = sm_count(), steps = p.n * (int64_t)p.T;
-    int64_t most = 6500000;  // steps of all environments
-    if (warps <= sms * 12) most = CONTRACT ? (policy == 1 ? 9900000 : 18000000) : (policy == 1 ? 16000000 : 26000000);
-    else if (policy == 1 && warps > sms * 30 && warps <= sms * 32) most = 1000000;
-    else if (CONTRACT && policy == 1) most = 6200000;
-    else if (CONTRACT && policy == 6) most = warps <= sms * 48 ? 6000000 : 5700000 - 2 * p.n;
-    const bool four = p.action_bits && !p.action_bits_in && (p.n % 8 == 0 || steps <= most);
-    const bool three = !(CONTRACT && policy == 3 && warps > sms * 24 && warps <= sms * 32 && steps > 26000000);
-    const int mode = !streams ? 0 : !(p.reward_stream && p.done_bits) ? 2 : p.trajectory ? (four ? 4 : 2) : p.action_bits ? (three ? 3 : 2) : 1;
     // the network policies are instantiated in translation units of their own (build time)
     if (policy == 2 || policy == 4 || policy == 5 || policy == 7)
         return CONTRACT ? launch_rollout_networks_contracted(p, policy, mode, shape, s)

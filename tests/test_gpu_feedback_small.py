@@ -178,3 +178,13 @@ def test_outputs_together_equal_outputs_apart(cp, kind, coop, n, T):
         for streams in (ALL, ("reward_stream", "done_bits", "action_bits")):
             got = rollout(cp, coop, kind, n, T, streams=streams, **args)
             assert_same_bits(got, {k: apart[k] for k in got})
+
+
+@pytest.mark.parametrize("n,T", [(250_003, 20), (250_003, 26), (450_003, 12)])
+def test_own_policies_with_all_outputs_on_larger_batches(cp, n, T):
+    """Contracted, more than 151,552 environments on 148 SMs: restarts per lane without tests of the outputs, per lane with them on
+    rows off 32 bytes, by the warp on the shortest of those launches."""
+    args = dict(streams=ALL, contracted=True, limit=9, spread="edge")
+    general = rollout(cp, 2, PER_ENV, n, T, **args)
+    for coop in (0, 1):
+        assert_same_bits(rollout(cp, coop, PER_ENV, n, T, **args), general)
