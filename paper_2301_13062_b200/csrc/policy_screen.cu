@@ -3,8 +3,6 @@
 #include "policy_bound.h"
 #include "policy_screen.cuh"
 
-#include <cstring>
-
 namespace cp {
 
 namespace {

@@ -51,19 +51,19 @@ struct NetShape {
     static_assert(kUnitFirst % 2 == 0 && kUnitSteps % 2 == 0, "pairs are read as such");
 };
 
-// The action by the defined logits: every sum left to right from its bias. w: the hidden layers' weights,
-// STRIDE floats apart; logits: W[2][H], b[2]. Two units at a time, whose tanhs share their instructions;
+// The action by the defined logits: every sum left to right from its bias. w: the hidden layers' weights; logits:
+// W[2][H], b[2]. Two units at a time, whose tanhs share their instructions;
 // few environments come here, so the code is kept short: loops over the units, not unrolled.
-template <int NET, bool CONTRACT, int STRIDE>
+template <int NET, bool CONTRACT>
 __device__ __forceinline__ uint32_t defined_action(const float *w, const float *logits, const State &z) {
     using S = NetShape<NET>;
     constexpr int H = S::H;
     auto first = [&](int j) {
-        float acc = w[(4 * H + j) * STRIDE];
-        acc = __fmaf_rn(w[(4 * j + 0) * STRIDE], z.x, acc);
-        acc = __fmaf_rn(w[(4 * j + 1) * STRIDE], z.xd, acc);
-        acc = __fmaf_rn(w[(4 * j + 2) * STRIDE], z.th, acc);
-        return __fmaf_rn(w[(4 * j + 3) * STRIDE], z.thd, acc);
+        float acc = w[4 * H + j];
+        acc = __fmaf_rn(w[4 * j + 0], z.x, acc);
+        acc = __fmaf_rn(w[4 * j + 1], z.xd, acc);
+        acc = __fmaf_rn(w[4 * j + 2], z.th, acc);
+        return __fmaf_rn(w[4 * j + 3], z.thd, acc);
     };
     auto tanh2 = [](float a, float b, float &ha, float &hb) {
         const f32x2 v = pack2(a, b);
@@ -79,17 +79,17 @@ __device__ __forceinline__ uint32_t defined_action(const float *w, const float *
         l1 = __fmaf_rn(logits[H + j + 1], hb, l1);
     };
     if constexpr (S::kDeep) {
-        const float *w2 = w + S::kSecond * STRIDE, *b2 = w2 + H * H * STRIDE;
+        const float *w2 = w + S::kSecond, *b2 = w2 + H * H;
         float h1[H];
 #pragma unroll
         for (int j = 0; j < H; j += 2) tanh2(first(j), first(j + 1), h1[j], h1[j + 1]);
 #pragma unroll 1
         for (int k = 0; k < H; k += 2) {
-            float a = b2[k * STRIDE], b = b2[(k + 1) * STRIDE];
+            float a = b2[k], b = b2[k + 1];
 #pragma unroll
             for (int j = 0; j < H; ++j) {
-                a = __fmaf_rn(w2[(H * k + j) * STRIDE], h1[j], a);
-                b = __fmaf_rn(w2[(H * (k + 1) + j) * STRIDE], h1[j], b);
+                a = __fmaf_rn(w2[H * k + j], h1[j], a);
+                b = __fmaf_rn(w2[H * (k + 1) + j], h1[j], b);
             }
             logit_terms(k, a, b);
         }

@@ -258,7 +258,7 @@ constexpr bool kWrittenOut = CONTRACT && (STREAMS == 1 ? CHUNK == kLongChunk || 
                                                       : STREAMS == 3 && CHUNK == kShortChunk && !LIMIT && POLICY != 1);
 
 // START_IN: the start states are the caller's data and may hold any angle.
-// HELPERS: warps that hash or fetch for the stepping one, every HELPERS-th step each. BEHIND: see CartBehind.
+// HELPERS: warps that hash for the stepping one, every HELPERS-th step each; supplied start states have one. BEHIND: see CartBehind.
 // kChunk: steps per hand-over.
 template <int POLICY, bool START_IN, int PAIRS, int HELPERS, bool BEHIND, int kChunk, bool LIMIT, bool CONTRACT, int STREAMS>
 __global__ void __launch_bounds__(32 * (1 + HELPERS) * PAIRS) rollout_assisted_kernel(const __grid_constant__ RolloutParams p) {
@@ -312,16 +312,16 @@ __global__ void __launch_bounds__(32 * (1 + HELPERS) * PAIRS) rollout_assisted_k
                 }
                 if (START_IN) {
                     // the chunk's rows of [T][4][n], all in flight at once
-                    const float *src = p.start_in + (int64_t)(row0 + helper) * 4 * p.n + idx;
+                    static_assert(!START_IN || HELPERS == 1, "one helper fetches all rows");
+                    const float *src = p.start_in + (int64_t)row0 * 4 * p.n + idx;
 #pragma unroll 4
-                    for (int s = helper; s < rows; s += HELPERS) {
+                    for (int s = 0; s < rows; ++s) {
                         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&buf.start[b][s][lane]);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * q), "l"(src) : "memory");
                             src += p.n;
                         }
-                        if (HELPERS > 1) src += (HELPERS - 1) * 4 * p.n;
                     }
                 }
                 if (!START_IN || (POLICY == 0 && !given)) {

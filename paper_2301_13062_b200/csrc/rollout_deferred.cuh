@@ -88,7 +88,7 @@ __device__ __forceinline__ void network_action_pair(const RolloutParams &p, cons
     if (open0 || open1) {
 #pragma unroll 1
         for (int j = open0 ? 0 : 1; j < (open1 ? 2 : 1); ++j) {
-            const uint32_t sb = defined_action<NET, CONTRACT, 1>(p.w, p.w + NetShape<NET>::kLogits, j ? b : a);
+            const uint32_t sb = defined_action<NET, CONTRACT>(p.w, p.w + NetShape<NET>::kLogits, j ? b : a);
             (j ? sb1 : sb0) = sb;
         }
     }

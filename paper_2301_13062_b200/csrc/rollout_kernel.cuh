@@ -49,7 +49,7 @@ __device__ __forceinline__ uint32_t policy_signbit(const RolloutParams &p, const
     } else if constexpr (is_network(POLICY)) {
         const float estimate = screen_estimate<POLICY>(p.w, p.screen_base, z);
         if (screen_decides(estimate, p.screen_bound)) return screen_action(estimate);
-        return defined_action<POLICY, CONTRACT, 1>(p.w, p.w + NetShape<POLICY>::kLogits, z);
+        return defined_action<POLICY, CONTRACT>(p.w, p.w + NetShape<POLICY>::kLogits, z);
     } else {
         return 0u;  // 3 and 6: the kernel has the action itself
     }

@@ -156,6 +156,8 @@ struct LaneNetwork {
         if constexpr (kReads) {
         } else if constexpr (kPaired) {
             static_assert(!S::kDeep, "one hidden layer");
+            // (+ 0, which the compiler cannot know: from an address it knows it reads one lane's weights again in every step,
+            // 60 to 72 registers instead of 142 to 160)
             const float *w = p.w + (p.n >> 62), *logits = w + S::kLogits;
 #pragma unroll
             for (int q = 0; q < U / 2; ++q) {
@@ -283,7 +285,7 @@ __device__ __forceinline__ uint32_t lanes_action(const RolloutParams &p, const L
     uint32_t sb = screen_action(estimate);
     const bool open = !screen_decides(estimate, p.screen_bound);
     if constexpr (S::kDeep || G == 1) {
-        if (open) sb = defined_action<NET, CONTRACT, 1>(p.w, p.w + S::kLogits, z);
+        if (open) sb = defined_action<NET, CONTRACT>(p.w, p.w + S::kLogits, z);
         __syncwarp();
     } else if (__any_sync(0xffffffffu, open)) {  // warp-uniform
         const uint32_t defined = lanes_defined_action<NET, G, CONTRACT>(p, net, z, row, g);
@@ -332,6 +334,7 @@ __global__ void __launch_bounds__(128, NET == 7 && !STREAMS ? 0 : 3) rollout_lan
     uint32_t cnt = 0u, begin = p.t0 - carried;
     const int64_t words = (p.n + 31) >> 5;
     const float *start = p.start_in ? p.start_in + (int64_t)c * p.n + idx : nullptr;
+    // (Pointers of lanes that write nothing are null and advanced all the same, never followed.)
     // Per-step outputs, by the environment's own warp alone: a lane stores its components of the trajectory, and
     // lane 0 the done bits and lane 1 the action bits of the warp's E environments, which are whole bytes of the row's word.
     const bool keeps = STREAMS && p.trajectory && valid && g < 4u;
