@@ -333,7 +333,7 @@ int cp_set_allocator(void *(*alloc)(size_t), void (*release)(void *));
  * batches except with the MLP policies), "rollout_coop" (how finished environments get their
  * start state: 1 = by the whole warp through shared memory, 2 = each lane its own when its env
  * finishes, 3 = each lane computes it every step ahead of the dynamics (hashed or supplied
- * actions only, otherwise as 2), 4 = a helper warp per stepping warp hashes every step's action
+ * actions only, otherwise as 2), 4 = helper warps beside each stepping warp hash every step's action
  * and start state ahead into shared memory, or fetches the supplied ones (hashed or supplied
  * actions and the linear policies; otherwise as 2), 2, 3 and 4 only with one environment per
  * thread; 0 = default: helper warps for up to ten warps of environments per SM (a linear policy's

@@ -566,10 +566,13 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
     if (!h_planes_in || !h_planes_out || !h_reward || !h_done) return fail(CP_EINVAL, "a host pointer is NULL");
     if (t >= (1u << 30)) return fail(CP_EINVAL, "global step out of range");
     // Page-locked buffers, small and middling batches: the kernel reads and writes host memory itself, in
-    // one launch instead of a launch and up to five copies, each after the other (us per call, copies /
-    // this: 2,000 envs 41 / 22, 20,000 57 / 31, 100,000 118 / 85, 200,000 188 / 157, 240,000 211 / 188,
-    // 250,000 212 / 205, 262,143 222 / 230, the last three with actions; 300,001 260 / 272 and 4,000,001
-    // 3,027 / 3,277, where the copy engine's bandwidth counts). Buffers that overlap, other than a step in place, keep the copies' order.
+    // one launch instead of a launch and up to five copies, each after the other (us per call, copies in turn /
+    // this: 2,000 envs 41 / 22, 20,000 57 / 31, 100,000 118 / 85). Against the pieces below, the same buffers in turn, with
+    // actions, this / two pieces in each of two processes: 100,000 79 / 105, 104; 150,000 125 / 143, 174; 200,000 151 / 223, 253; 250,000
+    // 200 / 197, 248; 300,000 218 / 228, 480; 350,000 256 / 249, 257; odd sizes, whose stores lie across two lines, 140,001 125 /
+    // 129, 213; 220,001 190 / 179, 310; 249,999 217 / 210, 278; 262,143 225 / 213, 206; 320,001 276 / 231, 290. The copies' time
+    // depends on where the buffers lie, up to twice, the kernel's does not: the line lies where the pieces begin to gain in their
+    // better case. Buffers that overlap, other than a step in place, keep the copies' order.
     const size_t n = (size_t)n_envs;
     const struct { void *p; size_t bytes; } host[5] = {{const_cast<float *>(h_planes_in), 16 * n},
         {const_cast<uint8_t *>(h_action), n}, {h_planes_out, 16 * n}, {h_reward, 4 * n}, {h_done, n}};
@@ -607,9 +610,11 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
     // Larger page-locked batches in pieces: the copies in run on a stream of their own, and each piece's step stores
     // its outputs into host memory itself, by whole lines (step_host.cu), so that both directions of the bus are busy.
     // A piece costs a start of its copies (10 us and more), so they are few. us per call with actions, copies and step in turn /
-    // in 2, 3, 4, 6 pieces: 250,001 envs 214 / 196, 219, 231, 248; 400,003 324 / 280, 292, 313, 350; 500,000 387-413 / 334,
-    // 322, 338, 361; 1,000,003 722 / 625, 595, 603, 633; 2,000,000 1,396 / 1,178, 1,102, 1,081, 1,071; 4,000,001 2,760 /
-    // 2,362, 2,208, 2,125, 2,068. (The kernel reading the actions from host memory too 10 to 17 % slower; outputs by the step
+    // in 2, 3, 4, 6, 8 pieces: 250,001 envs 214 / 196, 219, 231, 248; 400,003 324 / 277, 285, 315, 339, 355; 450,001 - / 307, 314, 320,
+    // 359, 385; 480,003 - / 329, 328, 337, 380, 409; 500,000 387-413 / 333, 321, 331, 365, 375; 700,001 - / 448, 437, 450, 489, 518;
+    // 800,003 - / 508, 486, 487, 551, 578; 900,000 - / 558, 527, 538, 543, 581, without actions 538, 529, 500, 493, 518; 1,000,003
+    // 722 / 624, 599, 594, 628, 691; 1,500,001 - / 908, 861, 848, 841, 894; 1,700,000 - / 1,005, 947, 929, 926, 941; 2,000,000 1,396 / 1,178,
+    // 1,103, 1,073, 1,058, 1,088; 4,000,001 2,760 / 2,352, 2,198, 2,119, 2,060, 2,057. (The kernel reading the actions from host memory too 10 to 17 % slower; outputs by the step
     // kernels' own stores, whose lines lie across two where n is odd, 1,000,003 640, 4,000,001 2,865.)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (direct && cudaStreamIsCapturing(tl_stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone && staging_stream()) {

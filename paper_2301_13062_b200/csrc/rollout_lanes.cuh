@@ -23,7 +23,7 @@
 // the restart), so that it runs while the special-function unit works on the activations, and the chain is network,
 // one selection, network. 4-64-2, 4,096 x 500: 510 -> 372 cycles per step (134 -> 97 us), of which 128 are that unit's sixteen
 // results; 4-16-2 324 -> 243; with all outputs 168 -> 117 and 152 -> 80 us (these also by what follows). With one
-// warp per scheduler issue is no bound (235 instructions); with three of 4-16-2's one-lane warps it is: 236
+// warp per scheduler issue is no bound (192 instructions); with three of 4-16-2's one-lane warps it is: 222
 // instructions, the packed ones two slots each, of 370 cycles per warp and step.
 // The start state an environment would continue from is hashed on every step ahead of the network, one
 // component per lane where there are four: that work fills issue slots the network leaves empty, and a
