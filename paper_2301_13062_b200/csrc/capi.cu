@@ -597,27 +597,27 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
         return e == cudaSuccess ? CP_OK : cuda_fail(e, "step on host memory");
     }
     std::lock_guard<std::mutex> lock(g_staging.mu);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const bool in_pieces = direct && cudaStreamIsCapturing(tl_stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone && staging_stream();
     const int64_t stride = (n_envs + 63) / 64 * 64;
     const size_t plane_bytes = (size_t)stride * 4;
     const size_t byte_plane = round_up((size_t)n_envs, 256);
-    void *buf;
-    if ((rc = staging_reserve(5 * plane_bytes + 2 * byte_plane, &buf)) != CP_OK) return rc;
+    void *buf;  // states and actions, then what only the copies out need
+    if ((rc = staging_reserve(4 * plane_bytes + byte_plane + (in_pieces ? 0 : plane_bytes + byte_plane), &buf)) != CP_OK) return rc;
     char *base = static_cast<char *>(buf);
     float *d_planes = reinterpret_cast<float *>(base);
-    float *d_reward = reinterpret_cast<float *>(base + 4 * plane_bytes);
-    uint8_t *d_done = reinterpret_cast<uint8_t *>(base + 5 * plane_bytes);
-    uint8_t *d_action = d_done + byte_plane;
+    uint8_t *d_action = reinterpret_cast<uint8_t *>(base + 4 * plane_bytes);
     // Larger page-locked batches in pieces: the copies in run on a stream of their own, and each piece's step stores
     // its outputs into host memory itself, by whole lines (step_host.cu), so that both directions of the bus are busy.
     // A piece costs a start of its copies (10 us and more), so they are few. us per call with actions, copies and step in turn /
-    // in 2, 3, 4, 6, 8 pieces: 250,001 envs 214 / 196, 219, 231, 248; 400,003 324 / 277, 285, 315, 339, 355; 450,001 - / 307, 314, 320,
-    // 359, 385; 480,003 - / 329, 328, 337, 380, 409; 500,000 387-413 / 333, 321, 331, 365, 375; 700,001 - / 448, 437, 450, 489, 518;
-    // 800,003 - / 508, 486, 487, 551, 578; 900,000 - / 558, 527, 538, 543, 581, without actions 538, 529, 500, 493, 518; 1,000,003
-    // 722 / 624, 599, 594, 628, 691; 1,500,001 - / 908, 861, 848, 841, 894; 1,700,000 - / 1,005, 947, 929, 926, 941; 2,000,000 1,396 / 1,178,
-    // 1,103, 1,073, 1,058, 1,088; 4,000,001 2,760 / 2,352, 2,198, 2,119, 2,060, 2,057. (The kernel reading the actions from host memory too 10 to 17 % slower; outputs by the step
-    // kernels' own stores, whose lines lie across two where n is odd, 1,000,003 640, 4,000,001 2,865.)
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (direct && cudaStreamIsCapturing(tl_stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone && staging_stream()) {
+    // in 2, 3, 4, 6, 8 pieces: 250,001 envs 214 / 196, 219, 231, 248; 400,003 324 / 277, 285, 315, 339, 355; 450,001 - / 307, 314,
+    // 320, 359, 385; 480,003 - / 329, 328, 337, 380, 409; 500,000 387-413 / 333, 321, 331, 365, 375; 700,001 - / 448, 437, 450, 489,
+    // 518; 800,003 - / 508, 486, 487, 551, 578; 900,000 - / 558, 527, 538, 543, 581, without actions 538, 529, 500, 493, 518;
+    // 1,000,003 722 / 624, 599, 594, 628, 691; 1,500,001 - / 908, 861, 848, 841, 894; 1,700,000 - / 1,005, 947, 929, 926, 941;
+    // 2,000,000 1,396 / 1,178, 1,103, 1,073, 1,058, 1,088; 4,000,001 2,760 / 2,352, 2,198, 2,119, 2,060, 2,057. (The kernel
+    // reading the actions from host memory too 10 to 17 % slower; outputs by the step kernels' own stores, whose lines lie
+    // across two where n is odd, 1,000,003 640, 4,000,001 2,865.)
+    if (in_pieces) {
         const cudaStream_t copies = g_staging.copies;
         const int pieces = n_envs <= 450000 ? 2 : n_envs <= 800000 ? 3 : n_envs <= 1500000 ? 4 : 6;
         const int64_t step = ((n_envs + pieces - 1) / pieces + 127) / 128 * 128;
@@ -645,6 +645,8 @@ int cp_step_host(int64_t n_envs, uint32_t seed, uint32_t t, const float *h_plane
             if (e == cudaSuccess) e = d;
         return e == cudaSuccess ? CP_OK : cuda_fail(e, "step on host memory");
     }
+    float *d_reward = reinterpret_cast<float *>(base + 4 * plane_bytes + byte_plane);
+    uint8_t *d_done = reinterpret_cast<uint8_t *>(base + 5 * plane_bytes + byte_plane);
     cudaError_t e = cudaMemcpy2DAsync(d_planes, plane_bytes, h_planes_in, (size_t)n_envs * 4, (size_t)n_envs * 4, 4,
                                       cudaMemcpyHostToDevice, tl_stream);
     if (e == cudaSuccess && h_action)
