@@ -42,18 +42,18 @@ SMS = 148
 # states of the 4.5 % of env-steps that restart, 8 more for the linear policy).
 # COUNTED_AT = build.kernel_hash() of the sources these were captured from (a test compares it
 # with the current sources, so that the fractions cannot go stale unnoticed).
-COUNTED_AT = "c08e3d289d9554e2"
+COUNTED_AT = "1d5466428a8b62d2"
 # pipe_busy: sm__pipe_fmaheavy_cycles_active (share of the launch's cycles) in the same captures — the
 # resource that bounds these kernels; it counts idle slots' arithmetic and the integer multiply-adds too.
 ROLLOUT_OPS = {
     # slots: 1,048,576 x 500 (the deferred kernel's ragged end makes them depend a little on T)
-    "random": {"thread": 60.2, "slot": 47.5, "fp32": 37.2, "pipe_busy": 0.835, "kernel": "rollout_deferred_kernel"},
-    "linear": {"thread": 61.7, "slot": 40.2, "fp32": 45.2, "pipe_busy": 0.826, "kernel": "rollout_deferred_kernel"},
+    "random": {"thread": 60.2, "slot": 47.5, "fp32": 37.2, "pipe_busy": 0.833, "kernel": "rollout_deferred_kernel"},
+    "linear": {"thread": 61.7, "slot": 40.2, "fp32": 45.2, "pipe_busy": 0.824, "kernel": "rollout_deferred_kernel"},
     # slots: 1,048,576 x 1,000 with the reward plane and the done bitmask
-    "linear+streams": {"thread": 81.0, "slot": 46.8, "fp32": 45.2, "pipe_busy": 0.806, "kernel": "rollout_deferred_kernel"},
+    "linear+streams": {"thread": 81.0, "slot": 46.8, "fp32": 45.2, "pipe_busy": 0.804, "kernel": "rollout_deferred_kernel"},
     # slots: 2,097,152 x 200; one estimate of the logits' difference, the defined logits where it is too close to zero
-    "mlp": {"thread": 151.5, "slot": 140.8, "pipe_busy": 0.741, "kernel": "rollout_deferred_kernel"},
-    "random+contracted": {"thread": 46.3, "slot": 38.7, "fp32": 22.2, "pipe_busy": 0.807, "kernel": "rollout_deferred_kernel"},
+    "mlp": {"thread": 151.5, "slot": 140.8, "pipe_busy": 0.737, "kernel": "rollout_deferred_kernel"},
+    "random+contracted": {"thread": 46.3, "slot": 38.7, "fp32": 22.2, "pipe_busy": 0.803, "kernel": "rollout_deferred_kernel"},
 }
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch in the same captures (the per-env
 # results stay in L2); with the per-step streams: bytes per env-step (4,384.9 MB for 1,048,576 x

@@ -508,7 +508,7 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
     //     0.96-1.06, 24 to 28 0.96-1.16, contracted 7 to 9 0.84-0.99, 10 to 12 0.93-1.14, 24 to 28 1.13-1.34; the others 18 to 23
     //     0.82-0.98, 24 to 28 0.88-1.02, contracted 14 to 17 0.86-0.98, 18 to 21 0.93-1.06, 24 to 28 0.98-1.15;
     //   beyond, 5.0 to 6.45 million, 100,003 to 600,003 environments, canonical and contracted hashed actions 0.83-1.03; contracted
-    //     linear 5.2 to 6.0 0.85-1.05, 6.3 to 6.45 0.90-1.09; one policy each, whose weights L2 holds too, up to 200,003 5.4 to 6.0
+    //     linear 5.2 to 6.0 0.85-1.05, 6.3 to 6.45 0.90-1.09; one policy each, whose weights L2 holds too, up to 200,003 5.4 to 6.15
     //     0.86-1.04, 6.3 to 6.45 0.87-1.05, 300,003 to 600,003 5.2 to 6.45 1.00-1.10; one shared linear policy between 30 and 32 warps
     //     per SM (145,001 to 151,001), where the restarts of a lane by itself end, 0.9 million 0.93-1.04, 1.9 to 6.4 0.91-1.07.
     // So they do with supplied actions, whose warps drift apart as they read (120,000 x 200 167 / 187, 131,072 x 200 164 / 226,
@@ -520,7 +520,7 @@ cudaError_t launch_rollout_arith(RolloutParams &p, int policy, bool streams, cud
     if (warps <= sms * 12) most = CONTRACT ? (policy == 1 ? 9900000 : 18000000) : (policy == 1 ? 16000000 : 26000000);
     else if (policy == 1 && warps > sms * 30 && warps <= sms * 32) most = 1000000;
     else if (CONTRACT && policy == 1) most = 6200000;
-    else if (CONTRACT && policy == 6) most = warps <= sms * 48 ? 6000000 : 5700000 - 2 * p.n;
+    else if (CONTRACT && policy == 6) most = warps <= sms * 48 ? 6150000 : 5700000 - 2 * p.n;
     const bool four = p.action_bits && !p.action_bits_in && (p.n % 8 == 0 || steps <= most);
     const bool three = !(CONTRACT && policy == 3 && warps > sms * 24 && warps <= sms * 32 && steps > 26000000);
     const int mode = !streams ? 0 : !(p.reward_stream && p.done_bits) ? 2 : p.trajectory ? (four ? 4 : 2) : p.action_bits ? (three ? 3 : 2) : 1;

@@ -42,11 +42,11 @@ cudaError_t launch_lanes_deep(RolloutParams &p, int g, bool streams, bool contra
 // general kernel fetches the finished environments' part: all at about the same steps where the call begins the episodes, some in
 // every step where it takes up a batch in the middle of them, which costs it more. From the beginning / from the middle:
 // 2 lanes x 8 0.86-1.04 / 1.08-1.30, x 16 1.05-1.25 / 1.28-1.53; 1 lane 4-16-2 tested, one warp x 16 0.80-1.06 / 1.00-1.30, x 24
-// 0.95-1.17 / 1.11-1.30, two (23,001 to 37,800 environments) x 40 0.90-1.08 / 1.14-1.18, x 64 0.96-1.23 / 1.06-1.24, three x 40
+// 0.95-1.17 / 1.11-1.30, two (23,001 to 37,800 environments) x 32 0.84-1.04 / 0.95-1.17, x 64 0.96-1.23 / 1.06-1.24, three x 40
 // 0.94 / 1.00, x 64 0.99-1.57 / 1.38; plain, one x 24 0.85-1.10 / 1.08, x 64 1.00-1.23 / 1.11-1.43, two x 64 0.90-1.10 / 1.16, x 128
 // 0.95-1.29 / 1.16-1.28; on the first batches with two warps (18,945) tested x 64 0.90-0.94, x 128 0.91-1.01 / 1.11, plain x 128
 // 0.91 / 0.94-0.99, x 192 0.94 / 0.99, x 300 1.55 / 1.75; 4-64-2 tested, one to three x 8 0.92-0.98 / 0.97-1.06, x 24 0.99-1.05 /
-// 1.02-1.12, four x 32 0.94, x 64 1.08, seven and more x 16 0.99-1.21; plain, one x 32 0.98 / 1.05, x 64 1.01-1.05 / 1.04-1.09, two
+// 1.02-1.12, four (75,001) x 32 0.94, x 64 1.08, five to sixteen x 8 0.95-1.13 / 0.95-1.16; plain, one x 32 0.98 / 1.05, x 64 1.01-1.05 / 1.04-1.09, two
 // and three x 32 0.94-1.00 / 0.98-1.02, x 128 0.98-1.11 / 0.97-1.17; 4-32-2 and 4-16-16-2 tested, one x 8 0.84-1.01 / 1.03-1.15,
 // x 24 1.02-1.10 / 1.15-1.28, two and three x 8 0.85-0.98 / 0.97-1.12, 4-32-2 x 32 0.94-1.10 / 1.02-1.21, 4-16-16-2 x 40 0.97-1.06 /
 // 1.02-1.11, x 64 1.00-1.19 / 1.04-1.11.
@@ -89,10 +89,10 @@ int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool con
         uint32_t least = 0u;
         if (g == 2) least = middle ? 0u : 16u;
         else if (policy == 2 && w == 2 && p.n * 20 < schedulers * 32 * 23) least = middle ? 128u : 256u;
-        else if (policy == 2 && tested) least = middle ? (w == 1 ? 16u : 40u) : w == 1 ? 24u : 64u;
+        else if (policy == 2 && tested) least = middle ? (w == 1 ? 16u : 32u) : w == 1 ? 24u : 64u;
         else if (middle) least = 0u;
         else if (policy == 2) least = w == 1 ? 48u : 128u;
-        else if (policy == 5) least = tested ? (w <= 3 ? 24u : w <= 6 ? 64u : 16u) : w == 1 ? 64u : 128u;
+        else if (policy == 5) least = tested ? (w <= 3 ? 24u : w == 4 ? 64u : 8u) : w == 1 ? 64u : 128u;
         else least = w == 1 ? 24u : policy == 4 ? 32u : 48u;
         from = std::max(from, least);
     }
