@@ -196,6 +196,7 @@ struct Staging {
     std::mutex mu;
     void *buf = nullptr;
     size_t bytes = 0;
+    int buf_device = -1;            // the device that buf lies on
     cudaStream_t copies = nullptr;  // cp_step_host's copies in, beside the caller's stream, on `device`
     cudaEvent_t event = nullptr;
     int device = -1;
@@ -218,8 +219,12 @@ bool staging_stream() {
     return g_staging.device == device;
 }
 
+// On the current device: a kernel there cannot address what another one holds.
 int staging_reserve(size_t bytes, void **out) {
-    if (g_staging.bytes < bytes) {
+    int device;
+    const cudaError_t asked = cudaGetDevice(&device);
+    if (asked != cudaSuccess) return cuda_fail(asked, "cudaGetDevice");
+    if (g_staging.bytes < bytes || g_staging.buf_device != device) {
         if (g_staging.buf) {
             cudaError_t e = cudaFree(g_staging.buf);
             g_staging.buf = nullptr;
@@ -233,6 +238,7 @@ int staging_reserve(size_t bytes, void **out) {
             return fail(CP_ENOMEM, "cudaMalloc(%zu) for staging failed: %s", bytes, cudaGetErrorString(e));
         }
         g_staging.bytes = bytes;
+        g_staging.buf_device = device;
     }
     *out = g_staging.buf;
     return CP_OK;
