@@ -32,24 +32,26 @@ cudaError_t launch_lanes_deep(RolloutParams &p, int g, bool streams, bool contra
 //     0.95-1.03, contracted 1.01-1.09, plain x 48 1.00-1.04; 4-64-2 x 16 1.06-1.34; 4-16-16-2 x 24 1.06-1.29
 //   three: 4-16-2 tested x 48 1.05-1.09 (otherwise at most 1.00); 4-32-2 x 64 1.05-1.10 (plain at most 1.00);
 //     4-64-2 x 32 1.04-1.15; 4-16-16-2 x 64 1.00-1.09 (plain canonical at most 0.96)
-//   the larger networks by one lane, one / two / three warps: 4-32-2 tested x 8 1.13-1.15, 1.09-1.12, 1.01 (x 32 1.31, 1.20,
-//     1.08; four warps 1.01-1.03; without outputs 0.94-1.08, plain 0.91-1.07); 4-64-2 tested x 8 1.12-1.15, 1.07-1.10, 1.06,
-//     x 128 1.33, 1.19, 1.09, and 1.05-1.12 at 75,000 to 300,000 (sixteen warps x 8 to 100 1.01-1.10; seventeen to 53, 303,200 to
-//     1,000,003 environments, 1.02-1.16 too: the general kernel keeps those until the line is moved); without outputs and plain x 32 1.00-1.10, 1.01-1.06, 1.00-1.04
-//     (75,000 0.96-1.01); 4-16-16-2 tested x 8 1.06, 1.03, 1.03, x 128 1.25, 1.11, 1.04 (four 1.00; without 0.74-1.03)
+//   the larger networks by one lane, one / two / three warps: 4-32-2 tested x 8 1.13-1.15, 1.09-1.12, 1.01 (x 32 1.31,
+//     1.20, 1.08; four warps 1.01-1.03; without outputs 0.94-1.08, plain 0.91-1.07); 4-64-2 tested x 8 1.12-1.15,
+//     1.07-1.10, 1.06, x 128 1.33, 1.19, 1.09, and 1.05-1.12 at 75,000 to 300,000 (sixteen warps x 8 to 100 1.01-1.10;
+//     seventeen to 53, 303,200 to 1,000,003 environments, 1.02-1.16 too, which still go to the general
+//     kernel); without outputs and plain x 32 1.00-1.10, 1.01-1.06, 1.00-1.04 (75,000 0.96-1.01); 4-16-16-2 tested x 8
+//     1.06, 1.03, 1.03, x 128 1.25, 1.11, 1.04 (four 1.00; without 0.74-1.03)
 // Launches shorter than that do not earn back the loads of a lane's weights. Supplied start states without outputs keep
-// four lanes (14,001 x 200, 4-32-2, four over two 0.93). With outputs one lane and two fetch every step's row, of which the
-// general kernel fetches the finished environments' part: all at about the same steps where the call begins the episodes, some in
-// every step where it takes up a batch in the middle of them, which costs it more. From the beginning / from the middle:
-// 2 lanes x 8 0.86-1.04 / 1.08-1.30, x 16 1.05-1.25 / 1.28-1.53; 1 lane 4-16-2 tested, one warp x 16 0.80-1.06 / 1.00-1.30, x 24
-// 0.95-1.17 / 1.11-1.30, two (23,001 to 37,800 environments) x 32 0.84-1.04 / 0.95-1.17, x 64 0.96-1.23 / 1.06-1.24, three x 40
-// 0.94 / 1.00, x 64 0.99-1.57 / 1.38; plain, one x 24 0.85-1.10 / 1.08, x 64 1.00-1.23 / 1.11-1.43, two x 64 0.90-1.10 / 1.16, x 128
-// 0.95-1.29 / 1.16-1.28; on the first batches with two warps (18,945) tested x 64 0.90-0.94, x 128 0.91-1.01 / 1.11, plain x 128
-// 0.91 / 0.94-0.99, x 192 0.94 / 0.99, x 300 1.55 / 1.75; 4-64-2 tested, one to three x 8 0.92-0.98 / 0.97-1.06, x 24 0.99-1.05 /
-// 1.02-1.12, four (75,001) x 32 0.94, x 64 1.08, five to sixteen x 8 0.95-1.13 / 0.95-1.16; plain, one x 32 0.98 / 1.05, x 64 1.01-1.05 / 1.04-1.09, two
-// and three x 32 0.94-1.00 / 0.98-1.02, x 128 0.98-1.11 / 0.97-1.17; 4-32-2 and 4-16-16-2 tested, one x 8 0.84-1.01 / 1.03-1.15,
-// x 24 1.02-1.10 / 1.15-1.28, two and three x 8 0.85-0.98 / 0.97-1.12, 4-32-2 x 32 0.94-1.10 / 1.02-1.21, 4-16-16-2 x 40 0.97-1.06 /
-// 1.02-1.11, x 64 1.00-1.19 / 1.04-1.11.
+// four lanes (14,001 x 200, 4-32-2, four over two 0.93). With outputs one lane and two fetch every step's row, of which
+// the general kernel fetches the finished environments' part: all at about the same steps where the call begins the
+// episodes, some in every step where it takes up a batch in the middle of them, which costs it more. From the beginning /
+// from the middle: 2 lanes x 8 0.86-1.04 / 1.08-1.30, x 16 1.05-1.25 / 1.28-1.53; 1 lane 4-16-2 tested, one warp x 16
+// 0.80-1.06 / 1.00-1.30, x 24 0.95-1.17 / 1.11-1.30, two (23,001 to 37,800 environments) x 32 0.84-1.04 / 0.95-1.17, x 64
+// 0.96-1.23 / 1.06-1.24, three x 40 0.94 / 1.00, x 64 0.99-1.57 / 1.38; plain, one x 24 0.85-1.10 / 1.08, x 64 1.00-1.23
+// / 1.11-1.43, two x 64 0.90-1.10 / 1.16, x 128 0.95-1.29 / 1.16-1.28; on the first batches with two warps (18,945)
+// tested x 64 0.90-0.94, x 128 0.91-1.01 / 1.11, plain x 128 0.91 / 0.94-0.99, x 192 0.94 / 0.99, x 300 1.55 / 1.75;
+// 4-64-2 tested, one to three x 8 0.92-0.98 / 0.97-1.06, x 24 0.99-1.05 / 1.02-1.12, four (75,001) x 32 0.94, x 64 1.08,
+// five to sixteen x 8 0.95-1.13 / 0.95-1.16; plain, one x 32 0.98 / 1.05, x 64 1.01-1.05 / 1.04-1.09, two and three x 32
+// 0.94-1.00 / 0.98-1.02, x 128 0.98-1.11 / 0.97-1.17; 4-32-2 and 4-16-16-2 tested, one x 8 0.84-1.01 / 1.03-1.15, x 24
+// 1.02-1.10 / 1.15-1.28, two and three x 8 0.85-0.98 / 0.97-1.12, 4-32-2 x 32 0.94-1.10 / 1.02-1.21, 4-16-16-2 x 40
+// 0.97-1.06 / 1.02-1.11, x 64 1.00-1.19 / 1.04-1.11.
 int rollout_lanes_for(const RolloutParams &p, int policy, bool streams, bool contracted) {
     if (p.action_bits_in || !is_network(policy)) return 0;
     // a forced shape keeps the other kernels
